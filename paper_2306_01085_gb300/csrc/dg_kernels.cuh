@@ -267,6 +267,7 @@ __global__ void k_grad(long long E, const Ops* __restrict__ ops, PhysT<R> P, con
   R* sQ = sY + EPB * 9 * NP;                // [EPB][3][C][NP]
   R* sL = sQ + EPB * 3 * C * NP;            // [EPB][6][3][NF]: (w n_d dS) u_hat_c of the current c
   load_ops<N, R>(ops, so);
+  if constexpr (BLK) __syncthreads();       // the trace loop reads eL / eR for kappa
   const long long e0 = (long long)blockIdx.x * EPB;
   const long long plane_g = E * 5 * NP, plane_f = E * 30 * NF;
   const long long og = TO ? plane_g : 0, of = TO ? plane_f : 0;   // TO: read the tangent plane
