@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "../../include/dg.h"
+#include "dg_fx.cuh"
 
 namespace dg {
 
@@ -42,8 +43,18 @@ struct Ops {
   double w[MAXN];            // Gauss weights
   double eta[MAXN];          // Gauss points
   double xi[MAXN];           // GLL nodes
+  // with the weights folded in (dg_fx.cuh): Dh[k][i] = D[k][i] w_k / w_i, eh[side][i] = e[i] / w_i,
+  // Bt[q][a] = B[q][a] w_q
+  double Dh[MAXN * MAXN], eh[2][MAXN], Bt[MAXN * MAXN];
+  // fixed-point coefficients: B and Bt with exponent FX_T_B, -Dh and eh with FX_T_D, eL / eR with FX_T_E
+  int2 xB[MAXN * MAXN], xBt[MAXN * MAXN], xDn[MAXN * MAXN], xlift[2][MAXN], xend[2][MAXN];
 };
 void build_ops(int n, Ops* ops);   // host, defined in dg_ops.cu
+// the operators before rounding (end-point rows e[0] at -1, e[1] at +1)
+struct OpsLd {
+  long double B[MAXN * MAXN], Binv[MAXN * MAXN], D[MAXN * MAXN], e[2][MAXN], w[MAXN], eta[MAXN], xi[MAXN];
+};
+void build_ops_ld(int n, OpsLd* ops);
 
 // --------------------------------------------------------------------------------------------
 // physics parameters (nondimensional, Sec. 2.4), passed by value to kernels
@@ -130,6 +141,10 @@ struct dg_mesh {
   dg::Ops* d_ops = nullptr;
   double* x = nullptr;     // [E][3][Np] node coordinates
   double* geo = nullptr;   // [E][10][Np]: G[a][d] = W detJ dxi_a/dx_d (9), W detJ (1)
+  // the same without quadrature weights (FP64 kernels)
+  double* gu = nullptr;    // [E][11][Np]: detJ dxi_a/dx_d (9), detJ, 1 / detJ
+  double* fgu = nullptr;   // [E][6][4][Nf]: n dS (3), |n dS|
+  double* kn = nullptr;    // [E][6][3][Nf]: factors of the cross gradient traces, created with the blocks
   double* acc = nullptr;   // [E][3][Np]: static acceleration g/gamma - Fr^2/gamma w x (w x r)
   double* xg = nullptr;    // [E][3][Np]: Gauss point positions
   double* fgeo = nullptr;  // [E][6][4][Nf]: w n dS (3), w |n dS| (1), outward, own face order
@@ -218,6 +233,7 @@ struct Driver {
   static int mass(dg_mesh* m, const double* v, double* mv, cudaStream_t s, bool f32 = false);
   static int mass_inv(dg_mesh* m, const double* v, double* mv, cudaStream_t s);
   static int mixture(dg_mesh* m);
+  static int cross_kappa(dg_mesh* m, double* kn);   // mesh factors of the cross gradient traces (default stream)
   // J_r probe restricted to each element's own diagonal block (exact, one column per element)
   static int jv_blockdiag(dg_mesh* m, const double* u, const double* probe, double t, double* jv, cudaStream_t s,
                           bool f32 = false, bool tangent_only = false);

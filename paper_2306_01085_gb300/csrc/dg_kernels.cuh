@@ -16,7 +16,9 @@
 // (p-degree polynomials, the same quadrature), so these kernels compute the same discrete
 // operator as a dense nodal implementation, up to rounding.
 //
-// Kernels (one CTA handles EPB elements, one thread per Gauss point; faces one thread per point):
+// Kernels (one CTA handles EPB elements, one thread per Gauss point; faces one thread per point). The
+// kernels of this file named k_interp, k_grad and k_volume are the FP32 ones; their FP64 counterparts
+// k_interp64, k_grad64 and k_volume64 (dg_fp64.cuh) run the contractions in block fixed point.
 //   k_interp   nodal u (and tangent v) -> Gauss values U, face traces UF
 //   k_grad     U, UF (own + neighbour) -> Q in Gauss space, face traces QF
 //   k_faces    UF, QF of both sides -> F_hat . (w n dS) for both element faces (Eq. LDG2)
@@ -32,6 +34,7 @@
 #include <type_traits>
 
 #include "dg_internal.cuh"
+#include "dg_phys64.cuh"
 
 namespace dg {
 
@@ -198,43 +201,25 @@ __global__ void k_interp(const double* __restrict__ u, const double* __restrict_
       if (NC == 2) ug[plane_g + e * 5 * NP + rem] = in[(l * C + 5) * NP + rem];
     }
   }
-  // face traces. FP32: one face point per iteration, its N volume points found once (less index
-  // arithmetic); FP64: the flat loop over (face, c, point), which spreads the FP64 work evenly.
+  // face traces, one face point per iteration, its N volume points found once (less index arithmetic)
   const long long plane_f = E * 6 * 5 * NF;
-  if constexpr (sizeof(R) == 4) {
-    for (int idx = threadIdx.x; idx < EPB * 6 * NF; idx += blockDim.x) {
-      const int l = idx / (6 * NF), phi = (idx / NF) % 6, f = idx % NF;
-      const long long e = e0 + l;
-      if (e >= E) continue;
-      const R* ev = (phi & 1) ? so.eR : so.eL;
-      int vp[N];
+  for (int idx = threadIdx.x; idx < EPB * 6 * NF; idx += blockDim.x) {
+    const int l = idx / (6 * NF), phi = (idx / NF) % 6, f = idx % NF;
+    const long long e = e0 + l;
+    if (e >= E) continue;
+    const R* ev = (phi & 1) ? so.eR : so.eL;
+    int vp[N];
 #pragma unroll
-      for (int k = 0; k < N; ++k) vp[k] = face_vol_point<N>(phi, f, k);
-      for (int pl = 0; pl < NC; ++pl)
+    for (int k = 0; k < N; ++k) vp[k] = face_vol_point<N>(phi, f, k);
+    for (int pl = 0; pl < NC; ++pl)
 #pragma unroll
-        for (int c = 0; c < 5; ++c) {
-          const R* src = in + (l * C + 5 * pl + c) * NP;
-          R acc = R(0);
-#pragma unroll
-          for (int k = 0; k < N; ++k) acc = cm_fma<CM>(ev[k], src[vp[k]], acc);
-          uf[pl * plane_f + e * 30 * NF + (phi * 5 + c) * NF + f] = acc;
-        }
-    }
-  } else {
-    for (int idx = threadIdx.x; idx < EPB * 6 * 5 * NF; idx += blockDim.x) {
-      const int l = idx / (30 * NF), rem = idx % (30 * NF);
-      const int phi = rem / (5 * NF), c = (rem / NF) % 5, f = rem % NF;
-      const long long e = e0 + l;
-      if (e >= E) continue;
-      const R* ev = (phi & 1) ? so.eR : so.eL;
-      for (int pl = 0; pl < NC; ++pl) {
+      for (int c = 0; c < 5; ++c) {
         const R* src = in + (l * C + 5 * pl + c) * NP;
         R acc = R(0);
 #pragma unroll
-        for (int k = 0; k < N; ++k) acc = cm_fma<CM>(ev[k], src[face_vol_point<N>(phi, f, k)], acc);
-        uf[pl * plane_f + e * 30 * NF + rem] = acc;
+        for (int k = 0; k < N; ++k) acc = cm_fma<CM>(ev[k], src[vp[k]], acc);
+        uf[pl * plane_f + e * 30 * NF + (phi * 5 + c) * NF + f] = acc;
       }
-    }
   }
 }
 
@@ -387,10 +372,9 @@ __global__ void k_grad(long long E, const Ops* __restrict__ ops, PhysT<R> P, con
     }
     __syncthreads();
   }
-  // write Q (Gauss space): each thread its own point, the 15 (d, c) entries unrolled. For FP32 the
-  // face traces go one face point per iteration with its N volume points found once (the kernel is
-  // bound by instruction issue, much of it index arithmetic); the FP64 kernel is bound by the FP64
-  // pipe, and there the flat loop over (face, d, c, point) keeps every thread equally busy.
+  // write Q (Gauss space): each thread its own point, the 15 (d, c) entries unrolled; the face traces go
+  // one face point per iteration with its N volume points found once (the kernel is bound by
+  // instruction issue, much of it index arithmetic)
   if (active) {
     const long long e = e0 + el;
     for (int pl = 0; pl < NC; ++pl)
@@ -399,41 +383,23 @@ __global__ void k_grad(long long E, const Ops* __restrict__ ops, PhysT<R> P, con
         qg[(TO ? E * 15 * NP : 0) + pl * E * 15 * NP + e * 15 * NP + dc * NP + g] =
             sQ[((el * 3 + dc / 5) * C + 5 * pl + dc % 5) * NP + g];
   }
-  if constexpr (sizeof(R) == 4) {
-    for (int idx = threadIdx.x; idx < EPB * 6 * NF; idx += blockDim.x) {
-      const int l = idx / (6 * NF), phi = (idx / NF) % 6, f = idx % NF;
-      const long long e = e0 + l;
-      if (e >= E) continue;
-      const R* ev = (phi & 1) ? so.eR : so.eL;
-      int vp[N];
+  for (int idx = threadIdx.x; idx < EPB * 6 * NF; idx += blockDim.x) {
+    const int l = idx / (6 * NF), phi = (idx / NF) % 6, f = idx % NF;
+    const long long e = e0 + l;
+    if (e >= E) continue;
+    const R* ev = (phi & 1) ? so.eR : so.eL;
+    int vp[N];
 #pragma unroll
-      for (int k = 0; k < N; ++k) vp[k] = face_vol_point<N>(phi, f, k);
-      for (int pl = 0; pl < NC; ++pl)
+    for (int k = 0; k < N; ++k) vp[k] = face_vol_point<N>(phi, f, k);
+    for (int pl = 0; pl < NC; ++pl)
 #pragma unroll
-        for (int dc = 0; dc < 15; ++dc) {
-          const R* src = sQ + ((l * 3 + dc / 5) * C + 5 * pl + dc % 5) * NP;
-          R acc = R(0);
-#pragma unroll
-          for (int k = 0; k < N; ++k) acc = cm_fma<CM>(ev[k], src[vp[k]], acc);
-          qf[(TO ? E * 90 * NF : 0) + pl * E * 90 * NF + e * 90 * NF + (phi * 15 + dc) * NF + f] = acc;
-        }
-    }
-  } else {
-    for (int idx = threadIdx.x; idx < EPB * 6 * 15 * NF; idx += blockDim.x) {
-      const int l = idx / (90 * NF), rem = idx % (90 * NF);
-      const int phi = rem / (15 * NF), dc = (rem / NF) % 15, f = rem % NF;
-      const int d = dc / 5, c = dc % 5;
-      const long long e = e0 + l;
-      if (e >= E) continue;
-      const R* ev = (phi & 1) ? so.eR : so.eL;
-      for (int pl = 0; pl < NC; ++pl) {
-        const R* src = sQ + ((l * 3 + d) * C + 5 * pl + c) * NP;
+      for (int dc = 0; dc < 15; ++dc) {
+        const R* src = sQ + ((l * 3 + dc / 5) * C + 5 * pl + dc % 5) * NP;
         R acc = R(0);
 #pragma unroll
-        for (int k = 0; k < N; ++k) acc = cm_fma<CM>(ev[k], src[face_vol_point<N>(phi, f, k)], acc);
-        qf[(TO ? E * 90 * NF : 0) + pl * E * 90 * NF + e * 90 * NF + rem] = acc;
+        for (int k = 0; k < N; ++k) acc = cm_fma<CM>(ev[k], src[vp[k]], acc);
+        qf[(TO ? E * 90 * NF : 0) + pl * E * 90 * NF + e * 90 * NF + (phi * 15 + dc) * NF + f] = acc;
       }
-    }
   }
 }
 
@@ -679,7 +645,7 @@ __device__ __forceinline__ void prefetch_l2(const R* p, long long n) {
 // the value + tangent physics would otherwise take enough registers to halve the resident warps of
 // this latency-bound kernel (FP64 is bound by its pipe instead)
 template <int N, int NC, typename R, int CM = CM_NATIVE>
-__global__ void __launch_bounds__(Epb<N, NC>::value * Shape<N>::NP, sizeof(R) == 4 ? (N == 4 && NC == 2 ? 4 : 2) : 1)
+__global__ void __launch_bounds__(Epb<N, NC>::value * Shape<N>::NP, N == 4 && NC == 2 ? 4 : 2)
 k_volume(long long E, const Ops* __restrict__ ops, PhysT<R> P, R t,
                          const R* __restrict__ geo, const R* __restrict__ accg,
                          const R* __restrict__ xg, const R* __restrict__ ug,
@@ -812,6 +778,12 @@ k_volume(long long E, const Ops* __restrict__ ops, PhysT<R> P, R t,
     }
   }
 }
+
+}  // namespace dg
+
+#include "dg_fp64.cuh"
+
+namespace dg {
 
 // --------------------------------------------------------------------------------------------
 // tensor transforms of nodal q and the mass matrix
@@ -999,7 +971,8 @@ template <int N>
 __global__ void k_geometry(long long E, const Ops* __restrict__ ops, Phys P, int gravity_kind,
                            double g0, double g1, double g2, double g_r0,
                            const double* __restrict__ x, double* __restrict__ geo,
-                           double* __restrict__ accg, double* __restrict__ xg, double* __restrict__ fgeo) {
+                           double* __restrict__ accg, double* __restrict__ xg, double* __restrict__ fgeo,
+                           double* __restrict__ gu, double* __restrict__ fgu) {
   constexpr int NP = Shape<N>::NP, NF = Shape<N>::NF;
   __shared__ SmemOps so;
   __shared__ double w1[MAXN];
@@ -1056,6 +1029,11 @@ __global__ void k_geometry(long long E, const Ops* __restrict__ ops, Phys P, int
     for (int a = 0; a < 3; ++a)
       for (int d = 0; d < 3; ++d) gp[(a * 3 + d) * NP] = wq * cof[d][a];
     gp[9 * NP] = wq * det;
+    double* gq = gu + e * 11 * NP + g;
+    for (int a = 0; a < 3; ++a)
+      for (int d = 0; d < 3; ++d) gq[(a * 3 + d) * NP] = cof[d][a];
+    gq[9 * NP] = det;
+    gq[10 * NP] = 1.0 / det;
     const double X[3] = {x[e * 3 * NP] + in[g], x[e * 3 * NP + NP] + in[NP + g], x[e * 3 * NP + 2 * NP] + in[2 * NP + g]};
     for (int d = 0; d < 3; ++d) xg[e * 3 * NP + d * NP + g] = X[d];
     double gv[3];
@@ -1100,6 +1078,9 @@ __global__ void k_geometry(long long E, const Ops* __restrict__ ops, Phys P, int
       a2n += nv[d] * nv[d];
     }
     fp[3 * NF] = wf * sqrt(a2n);
+    double* fq = fgu + ((e * 6 + phi) * 4) * NF + f;
+    for (int d = 0; d < 3; ++d) fq[d * NF] = side * nv[d];
+    fq[3 * NF] = sqrt(a2n);
   }
 }
 
@@ -1128,69 +1109,111 @@ static int set_smem(K kernel, size_t bytes) {
   return DG_OK;
 }
 
+// FP64: `planes` planes from plane `first` on (u -> first, v -> the next) with k_interp64
+template <int N>
+static int launch_interp64(dg_mesh* m, const double* u, const double* v, int first, cudaStream_t s) {
+  using G = Grp<N>;
+  const int threads = threads64<N>(m->E * (v ? 2 : 1)), per = threads / G::T;
+  const size_t sm = sizeof(cell) * 10 * G::NP * per;
+  int rc = set_smem(k_interp64<N>, sm);
+  if (rc) return rc;
+  prof_begin(m, s, KK_INTERP);
+  k_interp64<N><<<dim3((unsigned)((m->E + per - 1) / per), v ? 2 : 1), threads, sm, s>>>(
+      u, v, m->E, m->d_ops, m->ws.ug + first * m->E * 5 * G::NP, m->ws.uf + first * m->E * 30 * G::NF);
+  prof_end(m, s);
+  DG_LAUNCH_CHECK("k_interp64");
+  return DG_OK;
+}
+
 template <int N, int NC, typename R = double, int CM = CM_NATIVE>
 static int run_interp(dg_mesh* m, const double* u, const double* v, cudaStream_t s) {
   constexpr int EPB = Epb<N, NC>::value, NP = Shape<N>::NP;
-  if constexpr (std::is_same<R, double>::value && CM == CM_NATIVE)
+  if constexpr (std::is_same<R, double>::value) {
     if (m->interp_mode == DG_INTERP_TC) return interp_tc<N, NC>(m, u, v, m->ws.ug, m->ws.uf, s);
-  const size_t sm = Smem<N, NC, R>::interp;
-  int rc = set_smem(k_interp<N, NC, R, CM>, sm);
-  if (rc) return rc;
-  const unsigned blocks = (unsigned)((m->E + EPB - 1) / EPB);
-  const WorkT<R> w = work_of<R>(m);
-  prof_begin(m, s, KK_INTERP);
-  k_interp<N, NC, R, CM><<<blocks, EPB * NP, sm, s>>>(u, v, m->E, m->d_ops, w.ug, w.uf);
-  prof_end(m, s);
-  DG_LAUNCH_CHECK("k_interp");
-  return DG_OK;
+    return launch_interp64<N>(m, u, NC == 2 ? v : nullptr, 0, s);
+  } else {
+    const size_t sm = Smem<N, NC, R>::interp;
+    int rc = set_smem(k_interp<N, NC, R, CM>, sm);
+    if (rc) return rc;
+    const unsigned blocks = (unsigned)((m->E + EPB - 1) / EPB);
+    const WorkT<R> w = work_of<R>(m);
+    prof_begin(m, s, KK_INTERP);
+    k_interp<N, NC, R, CM><<<blocks, EPB * NP, sm, s>>>(u, v, m->E, m->d_ops, w.ug, w.uf);
+    prof_end(m, s);
+    DG_LAUNCH_CHECK("k_interp");
+    return DG_OK;
+  }
 }
 
 template <int N, int NC, bool BLK = false, typename R = double, int CM = CM_NATIVE, bool TO = false>
 static int run_grad(dg_mesh* m, cudaStream_t s) {
-  constexpr int EPB = Epb<N, NC>::value, NP = Shape<N>::NP;
-  const size_t sm = Smem<N, NC, R>::grad;
-  int rc = set_smem(k_grad<N, NC, BLK, R, CM, TO>, sm);
-  if (rc) return rc;
-  const unsigned blocks = (unsigned)((m->E + EPB - 1) / EPB);
-  const WorkT<R> w = work_of<R>(m);
-  prof_begin(m, s, KK_GRAD);
-  k_grad<N, NC, BLK, R, CM, TO><<<blocks, EPB * NP, sm, s>>>(m->E, m->d_ops, phys_as<R>(m->phys), w.geo, w.fgeo,
-                                                          m->nbr, m->nbr_fo, w.ug, w.uf, w.qg, w.qf, w.qx);
-  prof_end(m, s);
-  DG_LAUNCH_CHECK("k_grad");
-  return DG_OK;
+  if constexpr (std::is_same<R, double>::value) {
+    using G = Grp<N>;
+    const int threads = threads64<N>(m->E * NC), per = threads / G::T;
+    const size_t sm = sizeof(cell) * GradCells<N>::size * per;
+    int rc = set_smem(k_grad64<N, BLK>, sm);
+    if (rc) return rc;
+    prof_begin(m, s, KK_GRAD);
+    k_grad64<N, BLK><<<dim3((unsigned)((m->E + per - 1) / per), NC), threads, sm, s>>>(
+        m->E, m->d_ops, m->phys.t_wall, TO ? 1 : 0, m->gu, m->fgu, m->kn, m->nbr, m->nbr_fo, m->ws.ug,
+        m->ws.uf, m->ws.qg, m->ws.qf, m->ws.qx);
+    prof_end(m, s);
+    DG_LAUNCH_CHECK("k_grad64");
+    return DG_OK;
+  } else {
+    constexpr int EPB = Epb<N, NC>::value, NP = Shape<N>::NP;
+    const size_t sm = Smem<N, NC, R>::grad;
+    int rc = set_smem(k_grad<N, NC, BLK, R, CM, TO>, sm);
+    if (rc) return rc;
+    const unsigned blocks = (unsigned)((m->E + EPB - 1) / EPB);
+    const WorkT<R> w = work_of<R>(m);
+    prof_begin(m, s, KK_GRAD);
+    k_grad<N, NC, BLK, R, CM, TO><<<blocks, EPB * NP, sm, s>>>(m->E, m->d_ops, phys_as<R>(m->phys), w.geo, w.fgeo,
+                                                            m->nbr, m->nbr_fo, w.ug, w.uf, w.qg, w.qf, w.qx);
+    prof_end(m, s);
+    DG_LAUNCH_CHECK("k_grad");
+    return DG_OK;
+  }
 }
 
 // the tangent plane of ug, uf (nodal v -> Gauss values and traces), with the NC = 1 kernel
 template <int N, typename R>
 static int run_interp_tangent(dg_mesh* m, const double* v, cudaStream_t s) {
   constexpr int EPB = Epb<N, 1>::value, NP = Shape<N>::NP, NF = Shape<N>::NF;
-  if constexpr (std::is_same<R, double>::value)
+  if constexpr (std::is_same<R, double>::value) {
     if (m->interp_mode == DG_INTERP_TC)
       return interp_tc<N, 1>(m, v, nullptr, m->ws.ug + m->E * 5 * NP, m->ws.uf + m->E * 30 * NF, s);
-  const size_t sm = Smem<N, 1, R>::interp;
-  int rc = set_smem(k_interp<N, 1, R, CM_NATIVE>, sm);
-  if (rc) return rc;
-  const unsigned blocks = (unsigned)((m->E + EPB - 1) / EPB);
-  const WorkT<R> w = work_of<R>(m);
-  prof_begin(m, s, KK_INTERP);
-  k_interp<N, 1, R, CM_NATIVE><<<blocks, EPB * NP, sm, s>>>(v, nullptr, m->E, m->d_ops, w.ug + m->E * 5 * NP,
-                                                             w.uf + m->E * 30 * NF);
-  prof_end(m, s);
-  DG_LAUNCH_CHECK("k_interp(tangent)");
-  return DG_OK;
+    return launch_interp64<N>(m, v, nullptr, 1, s);
+  } else {
+    const size_t sm = Smem<N, 1, R>::interp;
+    int rc = set_smem(k_interp<N, 1, R, CM_NATIVE>, sm);
+    if (rc) return rc;
+    const unsigned blocks = (unsigned)((m->E + EPB - 1) / EPB);
+    const WorkT<R> w = work_of<R>(m);
+    prof_begin(m, s, KK_INTERP);
+    k_interp<N, 1, R, CM_NATIVE><<<blocks, EPB * NP, sm, s>>>(v, nullptr, m->E, m->d_ops, w.ug + m->E * 5 * NP,
+                                                               w.uf + m->E * 30 * NF);
+    prof_end(m, s);
+    DG_LAUNCH_CHECK("k_interp(tangent)");
+    return DG_OK;
+  }
 }
 
 template <int N, int NC, bool BLK = false, typename R = double>
 static int run_faces(dg_mesh* m, cudaStream_t s) {
   constexpr int NF = Shape<N>::NF;
   const long long work = m->nfaces * NF;
-  const int threads = 128;
+  // FP64: one warp per CTA while the faces cannot fill every SM with larger ones
+  const int threads = std::is_same<R, double>::value && work <= 152 * 512 ? 32 : 128;
   const unsigned blocks = (unsigned)((work + threads - 1) / threads);
   const WorkT<R> w = work_of<R>(m);
   prof_begin(m, s, KK_FACES);
-  k_faces<N, NC, BLK, R><<<blocks, threads, 0, s>>>(m->E, m->nfaces, phys_as<R>(m->phys), m->face_e, m->face_f,
-                                                     m->nbr, m->nbr_fo, w.fgeo, w.uf, w.qf, w.qx, w.fh, w.mixf);
+  if constexpr (std::is_same<R, double>::value)
+    k_faces64<N, NC, BLK><<<blocks, threads, 0, s>>>(m->E, m->nfaces, phys_as<R>(m->phys), m->face_e, m->face_f, m->nbr,
+                                                     m->nbr_fo, m->fgu, w.uf, w.qf, w.qx, w.fh, w.mixf);
+  else
+    k_faces<N, NC, BLK, R><<<blocks, threads, 0, s>>>(m->E, m->nfaces, phys_as<R>(m->phys), m->face_e, m->face_f,
+                                                       m->nbr, m->nbr_fo, w.fgeo, w.uf, w.qf, w.qx, w.fh, w.mixf);
   prof_end(m, s);
   DG_LAUNCH_CHECK("k_faces");
   return DG_OK;
@@ -1220,19 +1243,42 @@ inline long long resident_ctas(dg_mesh* m, const void* fn, int threads, size_t s
 
 template <int N, int NC, typename R = double, int CM = CM_NATIVE>
 static int run_volume(dg_mesh* m, double t, double* r, double* jv, cudaStream_t s, double stage_c = 0.0) {
-  constexpr int EPB = Epb<N, NC>::value, NP = Shape<N>::NP;
-  const size_t sm = Smem<N, NC, R>::volume;
-  int rc = set_smem(k_volume<N, NC, R, CM>, sm);
-  if (rc) return rc;
-  const unsigned blocks = (unsigned)((m->E + EPB - 1) / EPB);
-  const WorkT<R> w = work_of<R>(m);
-  // CTAs resident at once (the prefetch distance of the FP32 kernel), per mesh and kernel instance
-  const long long resident = resident_ctas(m, (const void*)k_volume<N, NC, R, CM>, EPB * NP, sm);
-  prof_begin(m, s, KK_VOLUME);
-  k_volume<N, NC, R, CM><<<blocks, EPB * NP, sm, s>>>(m->E, m->d_ops, phys_as<R>(m->phys), (R)t, w.geo, w.acc, w.xg,
-                                                   w.ug, w.qg, w.fh, r, jv, (R)stage_c, w.mixg, resident);
-  prof_end(m, s);
-  DG_LAUNCH_CHECK("k_volume");
+  if constexpr (std::is_same<R, double>::value) {
+    using G = Grp<N>;
+    const int threads = threads64<N>(m->E), per = threads / G::T;
+    const size_t sm = sizeof(cell) * VolCells<N, NC>::size * per;
+    int rc = set_smem(k_volume64<N, NC>, sm);
+    if (rc) return rc;
+    prof_begin(m, s, KK_VOLUME);
+    k_volume64<N, NC><<<(unsigned)((m->E + per - 1) / per), threads, sm, s>>>(
+        m->E, m->d_ops, phys_as<double>(m->phys), t, m->gu, m->acc, m->xg, m->ws.ug, m->ws.qg, m->ws.fh, r, jv, stage_c,
+        stage_c != 0.0 ? 1.0 / stage_c : 0.0, m->mixg);
+    prof_end(m, s);
+    DG_LAUNCH_CHECK("k_volume64");
+    return DG_OK;
+  } else {
+    constexpr int EPB = Epb<N, NC>::value, NP = Shape<N>::NP;
+    const size_t sm = Smem<N, NC, R>::volume;
+    int rc = set_smem(k_volume<N, NC, R, CM>, sm);
+    if (rc) return rc;
+    const unsigned blocks = (unsigned)((m->E + EPB - 1) / EPB);
+    const WorkT<R> w = work_of<R>(m);
+    // CTAs resident at once (the prefetch distance), per mesh and kernel instance
+    const long long resident = resident_ctas(m, (const void*)k_volume<N, NC, R, CM>, EPB * NP, sm);
+    prof_begin(m, s, KK_VOLUME);
+    k_volume<N, NC, R, CM><<<blocks, EPB * NP, sm, s>>>(m->E, m->d_ops, phys_as<R>(m->phys), (R)t, w.geo, w.acc, w.xg,
+                                                     w.ug, w.qg, w.fh, r, jv, (R)stage_c, w.mixg, resident);
+    prof_end(m, s);
+    DG_LAUNCH_CHECK("k_volume");
+    return DG_OK;
+  }
+}
+
+template <int N>
+int Driver<N>::cross_kappa(dg_mesh* m, double* kn) {
+  constexpr int NF = Shape<N>::NF;
+  k_cross_kappa<N><<<(unsigned)((m->E * 6 * NF + 127) / 128), 128>>>(m->E, m->d_ops, m->geo, m->fgeo, kn);
+  DG_LAUNCH_CHECK("k_cross_kappa");
   return DG_OK;
 }
 
@@ -1246,7 +1292,7 @@ int Driver<N>::geometry(dg_mesh* m, cudaStream_t s) {
   prof_begin(m, s, KK_GEOMETRY);
   k_geometry<N><<<(unsigned)m->E, NP < 32 ? 32 : NP, sm, s>>>(m->E, m->d_ops, m->phys, d.gravity_kind, d.gvec[0],
                                                             d.gvec[1], d.gvec[2], d.g_r0, m->x, m->geo, m->acc,
-                                                            m->xg, m->fgeo);
+                                                            m->xg, m->fgeo, m->gu, m->fgu);
   prof_end(m, s);
   DG_LAUNCH_CHECK("k_geometry");
   return DG_OK;

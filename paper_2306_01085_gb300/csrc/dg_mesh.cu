@@ -324,7 +324,7 @@ static void free_mesh(dg_mesh* m) {
   dg_mlp_release(m);
   dg::interp_tc_release(m);
   if (m->w32_base) cudaFree(m->w32_base);
-  void* ptrs[] = {m->d_ops, m->x, m->geo, m->acc, m->xg, m->fgeo, m->mixg, m->mixf, m->nbr, m->nbr_fo, m->face_e,
+  void* ptrs[] = {m->d_ops, m->x, m->geo, m->gu, m->fgu, m->kn, m->acc, m->xg, m->fgeo, m->mixg, m->mixf, m->nbr, m->nbr_fo, m->face_e,
                   m->face_f,
                   m->ws.ug, m->ws.uf, m->ws.qg, m->ws.qf, m->ws.fh, m->ws.tmp, m->ws.red, m->ws.qx};
   for (void* p : ptrs)
@@ -494,6 +494,8 @@ extern "C" int dg_mesh_create(const dg_mesh_desc* desc, const double* nodes, dg_
 
   rc |= dalloc(&m->d_ops, 1);
   rc |= dalloc(&m->geo, E * 10 * NP);
+  rc |= dalloc(&m->gu, E * 11 * NP);
+  rc |= dalloc(&m->fgu, E * 24 * NF);
   rc |= dalloc(&m->acc, E * 3 * NP);
   rc |= dalloc(&m->xg, E * 3 * NP);
   rc |= dalloc(&m->fgeo, E * 6 * 4 * NF);

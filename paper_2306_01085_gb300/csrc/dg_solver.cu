@@ -1291,18 +1291,6 @@ static int solver_get(dg_mesh* m, int restart, Solver** out) {
   return DG_OK;
 }
 
-static int ensure_blocks(dg_mesh* m, Solver* S) {
-  if (S->blocks) return DG_OK;
-  const long long nb = 5LL * m->np;
-  cudaError_t err = cudaMalloc(&S->blocks, sizeof(float) * (size_t)m->E * nb * nb);
-  if (err == cudaSuccess) err = cudaMalloc(&S->piv, sizeof(int) * (size_t)m->E * nb);
-  if (err == cudaSuccess) err = cudaMalloc(&S->info, sizeof(int));
-  if (err == cudaSuccess) err = cudaMalloc(&S->probe, sizeof(double) * (size_t)m->ndof);
-  if (err == cudaSuccess && !m->ws.qx) err = cudaMalloc(&m->ws.qx, sizeof(double) * (size_t)m->E * 90 * m->nf);
-  if (err != cudaSuccess) return fail(DG_ENOMEM, std::string("block-Jacobi storage: ") + cudaGetErrorString(err));
-  return DG_OK;
-}
-
 #define DG_DISPATCH_S(m, call)                                 \
   switch ((m)->n) {                                            \
     case 2: rc = Driver<2>::call; break;                       \
@@ -1311,6 +1299,27 @@ static int ensure_blocks(dg_mesh* m, Solver* S) {
     case 5: rc = Driver<5>::call; break;                       \
     default: rc = fail(DG_EINVAL, "unsupported degree");       \
   }
+
+static int ensure_blocks(dg_mesh* m, Solver* S) {
+  if (S->blocks) return DG_OK;
+  const long long nb = 5LL * m->np;
+  cudaError_t err = cudaMalloc(&S->blocks, sizeof(float) * (size_t)m->E * nb * nb);
+  if (err == cudaSuccess) err = cudaMalloc(&S->piv, sizeof(int) * (size_t)m->E * nb);
+  if (err == cudaSuccess) err = cudaMalloc(&S->info, sizeof(int));
+  if (err == cudaSuccess) err = cudaMalloc(&S->probe, sizeof(double) * (size_t)m->ndof);
+  if (err == cudaSuccess && !m->ws.qx) err = cudaMalloc(&m->ws.qx, sizeof(double) * (size_t)m->E * 90 * m->nf);
+  if (err == cudaSuccess && !m->kn) {
+    err = cudaMalloc(&m->kn, sizeof(double) * (size_t)m->E * 18 * m->nf);
+    if (err == cudaSuccess) {
+      int rc = DG_OK;
+      DG_DISPATCH_S(m, cross_kappa(m, m->kn));
+      if (rc) return rc;
+      err = cudaDeviceSynchronize();   // once per mesh: later sweeps may run on any stream
+    }
+  }
+  if (err != cudaSuccess) return fail(DG_ENOMEM, std::string("block-Jacobi storage: ") + cudaGetErrorString(err));
+  return DG_OK;
+}
 
 static unsigned grid_for(long long n) {
   long long b = (n + 255) / 256;

@@ -422,25 +422,26 @@ template <int N>
 int build_operator(dg_mesh* m) {
   using S = TcShape<N>;
   constexpr int NP = S::NP, NF = S::NF, KT = S::KT, MT = S::MT, ROWS = S::ROWS;
-  const Ops& o = m->ops;
+  OpsLd o;
+  build_ops_ld(N, &o);
   // rows: Gauss values (B x B x B), then face traces phi * NF + f (e_L / e_R along the normal)
   std::vector<long double> A((size_t)MT * TC_M * KT, 0.0L);
   for (int g = 0; g < NP; ++g) {
     const int g0 = g % N, g1 = (g / N) % N, g2 = g / (N * N);
     for (int k = 0; k < NP; ++k) {
       const int k0 = k % N, k1 = (k / N) % N, k2 = k / (N * N);
-      A[(size_t)g * KT + k] = (long double)o.B[g0 * N + k0] * o.B[g1 * N + k1] * o.B[g2 * N + k2];
+      A[(size_t)g * KT + k] = o.B[g0 * N + k0] * o.B[g1 * N + k1] * o.B[g2 * N + k2];
     }
   }
   for (int phi = 0; phi < 6; ++phi) {
     const int axis = phi >> 1;
-    const double* ev = (phi & 1) ? o.eR : o.eL;
+    const long double* ev = o.e[phi & 1];
     for (int f = 0; f < NF; ++f) {
       const int is = f % N, it = f / N;
       for (int j = 0; j < N; ++j) {
         const int i0 = axis == 0 ? j : is, i1 = axis == 0 ? is : (axis == 1 ? j : it), i2 = axis == 2 ? j : it;
         const int g = i0 + N * (i1 + N * i2);
-        for (int k = 0; k < NP; ++k) A[(size_t)(NP + phi * NF + f) * KT + k] += (long double)ev[j] * A[(size_t)g * KT + k];
+        for (int k = 0; k < NP; ++k) A[(size_t)(NP + phi * NF + f) * KT + k] += ev[j] * A[(size_t)g * KT + k];
       }
     }
   }
