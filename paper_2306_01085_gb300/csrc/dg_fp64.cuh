@@ -53,11 +53,11 @@ __device__ __forceinline__ void grp_max(int (&v)[K], int* red) {
       for (int w = 0; w < W; ++w) v[k] = max(v[k], red[w * K + k]);
   }
 }
-// whether every thread that shares a branch with this group (its warp, or its CTA) says yes
+// whether all groups that share this warp or CTA say yes (groups of a warp or more: uniform already)
 template <int N>
 __device__ __forceinline__ bool grp_all(bool yes) {
-  if constexpr (Grp<N>::T <= 32) return __all_sync(0xffffffffu, yes);
-  else return yes;                            // derived from group-wide maxima: uniform in the CTA
+  if constexpr (Grp<N>::T < 32) return __all_sync(0xffffffffu, yes);
+  else return yes;
 }
 
 // a shared cell of 8 bytes holds a double or a split fixed-point value
@@ -223,8 +223,12 @@ __global__ void __launch_bounds__(128) k_interp64(const double* __restrict__ u, 
   }
   double* go = ug + (blockIdx.y ? E * 5 * NP : 0) + e * 5 * NP;
   double* fo = uf + (blockIdx.y ? E * 30 * NF : 0) + e * 30 * NF;
-  if (grp_all<N>(ok)) interp_body<N, true>(so, x, ex, b0, b0 + 5 * NP, g, act, live, go, fo);
-  else interp_slow<N>(so, x, ex, b0, b0 + 5 * NP, g, act, live, go, fo);
+  if (!grp_all<N>(ok)) {
+    interp_slow<N>(so, x, ex, b0, b0 + 5 * NP, g, act, live && !ok, go, fo);
+    if constexpr (T >= 32) return;
+    grp_sync<N>();                           // groups of this warp that passed take the fixed-point path
+  }
+  interp_body<N, true>(so, x, ex, b0, b0 + 5 * NP, g, act, live && ok, go, fo);
 }
 
 // --------------------------------------------------------------------------------------------
@@ -256,7 +260,7 @@ __device__ __noinline__ void grad_slow(const XOps<N>& so, const double* gu, cell
         cells[C::L + (idx / NF * 3 + d) * NF + idx % NF] =
             c_of(c_d(cells[C::Nn + d * 6 * NF + idx]) * c_d(cells[C::Uh + c * 6 * NF + idx]));
     grp_sync<N>();
-    if (act)
+    if (act && live)
       for (int d = 0; d < 3; ++d) {
         double s = 0.0;
         for (int a = 0; a < 3; ++a) {
@@ -266,9 +270,9 @@ __device__ __noinline__ void grad_slow(const XOps<N>& so, const double* gu, cell
             s = fma(so.deh[side][i], c_d(cells[C::L + ((2 * a + side) * 3 + d) * NF + fp]), s);
           for (int k = 0; k < N; ++k) s = fma(-so.dDh[k * N + i], c_d(cells[C::Y + (a * 3 + d) * NP + base + k * st]), s);
         }
-        s *= live ? gu[10 * NP + g] : 0.0;
+        s *= gu[10 * NP + g];
         cells[C::Q + d * NP + g] = c_of(s);
-        if (live) qg[(d * 5 + c) * NP + g] = s;
+        qg[(d * 5 + c) * NP + g] = s;
       }
     grp_sync<N>();
     if (live)
@@ -310,12 +314,13 @@ __global__ void __launch_bounds__(128, 5) k_grad64(long long E, const Ops* __res
   cell *sY = cells + C::Y, *sL = cells + C::L, *sN = cells + C::Nn, *sUh = cells + C::Uh, *sQ = cells + C::Q,
        *sU = cells + C::U;
   const long long e = (long long)blockIdx.x * (blockDim.x / T) + grp;
-  const bool live = e < E, act = g < NP, on = live && act;
+  bool live = e < E;
+  const bool act = g < NP;
   const int plane = plane0 + blockIdx.y;
   const double* ufp = uf + plane * E * 30 * NF;
   const double* gue = gu + e * 11 * NP;
   int mx[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};   // geometry per d, field per c, 1 / |J|
-  if (on) {
+  if (live && act) {
     const double* ugp = ug + (plane * E + e) * 5 * NP;
 #pragma unroll
     for (int k = 0; k < 9; ++k) mx[k % 3] = max(mx[k % 3], fx_mag(gue[k * NP + g]));
@@ -400,12 +405,13 @@ __global__ void __launch_bounds__(128, 5) k_grad64(long long E, const Ops* __res
   double* qge = qg + (plane * E + e) * 15 * NP;
   double* qfe = qf + (plane * E + e) * 90 * NF;
   if (!grp_all<N>(ok)) {
-    grad_slow<N>(so, gue, cells, g, act, live, qge, qfe);
-    return;
+    grad_slow<N>(so, gue, cells, g, act, live && !ok, qge, qfe);
+    if constexpr (T >= 32) return;
   }
+  live = live && ok;
   // fixed point: own entries, so no barrier is needed
   fx G[9], wx{0, 0};
-  if (on) {
+  if (live && act) {
 #pragma unroll
     for (int k = 0; k < 9; ++k) G[k] = fx_split<29>(fx_from<57>(gue[k * NP + g], mx[k % 3]));
     wx = fx_split<27>(fx_from<57>(gue[10 * NP + g], mx[8]));
@@ -431,7 +437,7 @@ __global__ void __launch_bounds__(128, 5) k_grad64(long long E, const Ops* __res
 #pragma unroll 1
   for (int c = 0; c < 5; ++c) {
     // products: G u at the Gauss points, n u_hat at the face points
-    if (on) {
+    if (live && act) {
       const fx ux = c_fx(sU[c * NP + g]);
 #pragma unroll
       for (int k = 0; k < 9; ++k) sY[k * NP + g] = c_split<28>(fx_mul<28>(G[k], ux));
@@ -709,7 +715,7 @@ struct VolCells {
 
 // the FP64 twin of k_volume64 from the pointwise fluxes on
 template <int N, int NC>
-__device__ __noinline__ void volume_slow(const XOps<N>& so, long long e, long long E, int g, bool act, bool live,
+__device__ __noinline__ void volume_slow(const XOps<N>& so, long long e, long long E, int g, bool act, bool own,
                                          const PhysT<double>& P, double t, const double* gu, const double* accg,
                                          const double* xg, const double* ug, const double* qg, const double* fh,
                                          const double* mixg, double stage_c, double inv_stage_c, cell* cells, double* r,
@@ -718,7 +724,7 @@ __device__ __noinline__ void volume_slow(const XOps<N>& so, long long e, long lo
   using C = VolCells<N, NC>;
   constexpr int NP = C::NP, NF = C::NF, T = Grp<N>::T;
   cell *sF = cells, *sS = cells + C::S, *sH = cells + C::H;
-  if (act && live) {
+  if (act) {
     S F[12], src[5];
     volume_load<N, NC, S>(e, E, g, P, t, gu, accg, xg, ug, qg, mixg, inv_stage_c, F, src);
     for (int a = 0; a < 3; ++a)
@@ -739,7 +745,7 @@ __device__ __noinline__ void volume_slow(const XOps<N>& so, long long e, long lo
   const int ig[3] = {g % N, (g / N) % N, g / (N * N)};
   for (int pl = 0; pl < NC; ++pl) {
     grp_sync<N>();
-    if (live)
+    if (own)
       for (int idx = g; idx < 6 * NF; idx += T)
         for (int c = 0; c < 5; ++c)
           sH[c * 6 * NF + idx] = c_of(fh[pl * E * 30 * NF + e * 30 * NF + (idx / NF * 5 + c) * NF + idx % NF]);
@@ -766,7 +772,7 @@ __device__ __noinline__ void volume_slow(const XOps<N>& so, long long e, long lo
     if (act) pass_b<N, 1, true, false, 5>(so, F + 5 * NP, F, g);
     grp_sync<N>();
     if (act) pass_b<N, 2, true, false, 5>(so, F, F + 5 * NP, g);
-    if (act && live)
+    if (act)
       for (int c = 0; c < 5; ++c) {
         const double x = c_d(F[(5 + c) * NP + g]);
         if (pl == 0 && r) r[(e * 5 + c) * NP + g] = x;
@@ -794,7 +800,8 @@ __global__ void __launch_bounds__(128, NC == 2 ? 3 : 4)
   cell* cells = cells_all + (size_t)grp * C::size;
   cell *sF = cells, *sS = cells + C::S, *sH = cells + C::H;
   const long long e = (long long)blockIdx.x * (blockDim.x / T) + grp;
-  const bool live = e < E, act = g < NP, on = live && act;
+  bool live = e < E;
+  const bool act = g < NP;
   // per plane and variable: exponent bound (|x| < 2^(m - 1022)) of the reference fluxes, sources and face
   // fluxes; BAD marks magnitudes for the FP64 twin
   constexpr int BAD = 1 << 20;
@@ -803,7 +810,7 @@ __global__ void __launch_bounds__(128, NC == 2 ? 3 : 4)
   for (int k = 0; k < NC * 5; ++k) mx[k] = 0;
   auto expo = [](int mag) { return mag == 0 ? 0 : fx_ok(mag) ? mag >> 20 : BAD; };
   int eG[3] = {0, 0, 0}, eF[NC][3];          // this point's exponents: geometry rows, flux groups
-  if (on) {
+  if (live && act) {
     S F[12], src[5];
     volume_load<N, NC, S>(e, E, g, P, t, gu, accg, xg, ug, qg, mixg, inv_stage_c, F, src);
     double Gd[9];
@@ -882,9 +889,11 @@ __global__ void __launch_bounds__(128, NC == 2 ? 3 : 4)
     if (mx[k] == 0) mx[k] = 1023;
   }
   if (!grp_all<N>(ok)) {
-    volume_slow<N, NC>(so, e, E, g, act, live, P, t, gu, accg, xg, ug, qg, fh, mixg, stage_c, inv_stage_c, cells, r, jv);
-    return;
+    volume_slow<N, NC>(so, e, E, g, act && live && !ok, live && !ok, P, t, gu, accg, xg, ug, qg, fh, mixg, stage_c, inv_stage_c, cells,
+                       r, jv);
+    if constexpr (T >= 32) return;
   }
+  live = live && ok;
   const int ig[3] = {g % N, (g / N) % N, g / (N * N)};
 #pragma unroll 1
   for (int pl = 0; pl < NC; ++pl) {
