@@ -9,6 +9,7 @@
 // L = mean_b || Bs_b (diag(D) + U V^T) - I ||_F^2 / n with Adam; the gradients are written out by
 // hand (GEMM kernels for the layers, one CTA per sample for the loss). The loss measures P as a
 // RIGHT inverse (|| Bs P - I ||) because GMRES applies it on the right.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <string>
@@ -19,175 +20,315 @@
 namespace dg {
 
 // ------------------------------------------------------------------------------------------
-// FP32 tiled GEMM: C[m][n] = sum_k A(m,k) B(k,n) (+ beta C) (+ bias[n]); optional SiLU copy
+// FP32 tiled GEMM: C[m][n] = sum_k A(m,k) B(k,n)
 // A(m,k) = TA ? A[k lda + m] : A[m lda + k];  B(k,n) = TB ? B[n ldb + k] : B[k ldb + n]
+// The layers are small (a few hundred outputs each way), so K is split over grid.z until every SM has
+// work: dh2 = dout W3 (512 x 256 outputs, K = 4455) took 1.04 ms on 32 CTAs. A split writes partial sums
+// [z][M][N], which k_gemm_finish adds in order with the layer's epilogue. The forward layers (K of a few
+// hundred) are not split: every element's outputs are the same whatever the number of rows. The next
+// tile's global loads are in flight while the current one is multiplied (4 x 4 per thread, 16-byte shared
+// loads).
 // ------------------------------------------------------------------------------------------
 constexpr int GBM = 64, GBN = 64, GBK = 16;
 
+// v (+ bias); times silu'(z) when backward; *h = silu(v) when forward
+__device__ __forceinline__ float gemm_epilogue(float v, const float* bias, int column, const float* Z, long long i, float* H) {
+  if (bias) v += bias[column];
+  if (Z) {
+    const float sg = 1.f / (1.f + expf(-Z[i]));
+    v *= sg * (1.f + Z[i] * (1.f - sg));
+  }
+  if (H) H[i] = v / (1.f + expf(-v));
+  return v;
+}
+
 template <bool TA, bool TB>
-__global__ void __launch_bounds__(256) k_gemm(int M, int N, int K, const float* __restrict__ A, int lda,
-                                              const float* __restrict__ B, int ldb, float* __restrict__ C, int ldc,
-                                              float beta, const float* __restrict__ bias, float* __restrict__ H) {
-  __shared__ float As[GBK][GBM + 4];
-  __shared__ float Bs[GBK][GBN + 4];
+__global__ void __launch_bounds__(256) k_gemm(int M, int N, int K, int kc, const float* __restrict__ A, int lda,
+                                              const float* __restrict__ B, int ldb, float* __restrict__ C,
+                                              const float* __restrict__ bias, float* __restrict__ H,
+                                              const float* __restrict__ Z) {
+  __shared__ __align__(16) float As[2][GBK][GBM + 4];
+  __shared__ __align__(16) float Bs[2][GBK][GBN + 4];
   const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
   const int m0 = blockIdx.y * GBM, n0 = blockIdx.x * GBN;
+  const int kb = blockIdx.z * kc, ke = min(K, kb + kc);
   float acc[4][4] = {};
-  for (int k0 = 0; k0 < K; k0 += GBK) {
-    for (int t = tid; t < GBK * GBM; t += 256) {
-      int kk, mm;
-      if (TA) { mm = t % GBM; kk = t / GBM; } else { kk = t % GBK; mm = t / GBK; }
-      const int gm = m0 + mm, gk = k0 + kk;
-      float v = 0.f;
-      if (gm < M && gk < K) v = TA ? A[(long long)gk * lda + gm] : A[(long long)gm * lda + gk];
-      As[kk][mm] = v;
+  float ra[4], rb[4];
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int t = tid + 256 * q;
+      const int am = TA ? t % GBM : t / GBK, ak = k0 + (TA ? t / GBM : t % GBK);
+      const int bn = TB ? t / GBK : t % GBN, bk = k0 + (TB ? t % GBK : t / GBN);
+      ra[q] = (m0 + am < M && ak < ke) ? (TA ? A[(long long)ak * lda + m0 + am] : A[(long long)(m0 + am) * lda + ak]) : 0.f;
+      rb[q] = (n0 + bn < N && bk < ke) ? (TB ? B[(long long)(n0 + bn) * ldb + bk] : B[(long long)bk * ldb + n0 + bn]) : 0.f;
     }
-    for (int t = tid; t < GBK * GBN; t += 256) {
-      int kk, nn;
-      if (TB) { kk = t % GBK; nn = t / GBK; } else { nn = t % GBN; kk = t / GBN; }
-      const int gn = n0 + nn, gk = k0 + kk;
-      float v = 0.f;
-      if (gn < N && gk < K) v = TB ? B[(long long)gn * ldb + gk] : B[(long long)gk * ldb + gn];
-      Bs[kk][nn] = v;
+  };
+  auto stage = [&](int buf) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int t = tid + 256 * q;
+      As[buf][TA ? t / GBM : t % GBK][TA ? t % GBM : t / GBK] = ra[q];
+      Bs[buf][TB ? t % GBK : t / GBN][TB ? t / GBK : t % GBN] = rb[q];
     }
-    __syncthreads();
+  };
+  fetch(kb);
+  stage(0);
+  __syncthreads();
+  int buf = 0;
+  for (int k0 = kb; k0 < ke; k0 += GBK) {
+    const bool more = k0 + GBK < ke;
+    if (more) fetch(k0 + GBK);
 #pragma unroll
     for (int kk = 0; kk < GBK; ++kk) {
-      float a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx * 4 + j];
+      const float4 a4 = *reinterpret_cast<const float4*>(&As[buf][kk][ty * 4]);
+      const float4 b4 = *reinterpret_cast<const float4*>(&Bs[buf][kk][tx * 4]);
+      const float a[4] = {a4.x, a4.y, a4.z, a4.w}, b[4] = {b4.x, b4.y, b4.z, b4.w};
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
     }
+    if (more) stage(buf ^ 1);                // the other buffer: its readers passed the last barrier
     __syncthreads();
+    buf ^= 1;
   }
+  float* out = C + (long long)blockIdx.z * M * N;
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const int gm = m0 + ty * 4 + i, gn = n0 + tx * 4 + j;
       if (gm < M && gn < N) {
-        float v = acc[i][j];
-        if (beta != 0.f) v += beta * C[(long long)gm * ldc + gn];
-        if (bias) v += bias[gn];
-        C[(long long)gm * ldc + gn] = v;
-        if (H) H[(long long)gm * ldc + gn] = v / (1.f + expf(-v));
+        const long long at = (long long)gm * N + gn;
+        out[at] = gridDim.z == 1 ? gemm_epilogue(acc[i][j], bias, gn, Z, at, H) : acc[i][j];
       }
     }
+}
+
+// C = sum_z part[z], then the epilogue
+__global__ void k_gemm_finish(long long total, int N, int splits, const float* __restrict__ part, float* __restrict__ C,
+                              const float* __restrict__ bias, float* __restrict__ H, const float* __restrict__ Z) {
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
+    float v = part[i];
+    for (int z = 1; z < splits; ++z) v += part[z * total + i];
+    C[i] = gemm_epilogue(v, bias, (int)(i % N), Z, i, H);
+  }
+}
+
+// splits of K: enough for one CTA per SM, each with at least four K tiles
+static int gemm_splits(int M, int N, int K) {
+  const int tiles = ((N + GBN - 1) / GBN) * ((M + GBM - 1) / GBM);
+  return std::max(1, std::min((152 + tiles - 1) / tiles, K / (4 * GBK)));
+}
+static size_t gemm_part_floats(int M, int N, int K) {
+  const int sp = gemm_splits(M, N, K);
+  return sp > 1 ? (size_t)sp * M * N : 0;
 }
 
 template <bool TA, bool TB>
 static void gemm(cudaStream_t s, int M, int N, int K, const float* A, int lda, const float* B, int ldb, float* C,
-                 int ldc, float beta = 0.f, const float* bias = nullptr, float* H = nullptr) {
-  dim3 grid((N + GBN - 1) / GBN, (M + GBM - 1) / GBM);
-  k_gemm<TA, TB><<<grid, 256, 0, s>>>(M, N, K, A, lda, B, ldb, C, ldc, beta, bias, H);
+                 float* part, const float* bias = nullptr, float* H = nullptr, const float* Z = nullptr) {
+  const int sp = part ? gemm_splits(M, N, K) : 1;   // part: room for gemm_part_floats, or no split
+  const int kc = ((K + sp - 1) / sp + GBK - 1) / GBK * GBK;
+  const int nz = (K + kc - 1) / kc;
+  dim3 grid((N + GBN - 1) / GBN, (M + GBM - 1) / GBM, nz);
+  k_gemm<TA, TB><<<grid, 256, 0, s>>>(M, N, K, kc, A, lda, B, ldb, nz > 1 ? part : C, bias, H, Z);
+  const long long total = (long long)M * N;
+  if (nz > 1) k_gemm_finish<<<(unsigned)std::min((total + 255) / 256, 1216LL), 256, 0, s>>>(total, N, nz, part, C, bias, H, Z);
 }
 
-// dz = dh * silu'(z) in place on dh
-__global__ void k_silu_back(long long n, const float* __restrict__ z, float* __restrict__ dh) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const float s = 1.f / (1.f + expf(-z[i]));
-    dh[i] *= s * (1.f + z[i] * (1.f - s));
+// column sums of a [rows][cols] matrix (bias gradients), fixed order: 32 columns per CTA, rows over 16 warps
+__global__ void __launch_bounds__(512) k_colsum(int rows, int cols, const float* __restrict__ X, float* __restrict__ out) {
+  __shared__ float red[16][33];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, c = blockIdx.x * 32 + lane;
+  float s = 0.f;
+  if (c < cols)
+    for (int r = warp; r < rows; r += 16) s += X[(long long)r * cols + c];
+  red[warp][lane] = s;
+  __syncthreads();
+  if (warp == 0 && c < cols) {
+    for (int w = 1; w < 16; ++w) s += red[w][lane];
+    out[c] = s;
   }
 }
 
-// column sums of a [rows][cols] matrix (bias gradients), fixed order
-__global__ void k_colsum(int rows, int cols, const float* __restrict__ X, float* __restrict__ out) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= cols) return;
-  float s = 0.f;
-  for (int r = 0; r < rows; ++r) s += X[(long long)r * cols + c];
-  out[c] = s;
-}
-
 // ------------------------------------------------------------------------------------------
-// loss and output gradient, one CTA per sample, for P as a right inverse: R = Bs P - I (never
-// stored), P = diag(D) + U V^T, G = scale Bs^T R:
+// loss and output gradient, one CTA per sample, for P as a right inverse: R = Bs P - I, P = diag(D) + U V^T,
+// G = scale Bs^T R:
 //   W = Bs U (n x r);  R_ij = Bs_ij D_j + sum_k W_ik V_jk - delta_ij
 //   dD_j = scale sum_i Bs_ij R_ij;  dV = scale R^T W;  Z = R V;  dU = scale Bs^T Z
+// The block is read once, in strips of 16 rows held in shared memory: a strip gives its rows of W, R and Z
+// and its share of the two transposed products, which stay in registers (4 x 4 tiles, NT per thread).
+// 512 blocks of 135^2, rank 16: 1.15 ms with one row per thread and run-time indexed local arrays before.
 // ------------------------------------------------------------------------------------------
 constexpr int MLP_MAXR = 32;
+constexpr int LG_RB = 16;
 
-__global__ void k_loss_grad(int nb, int n, int r, const float* __restrict__ out, const float* __restrict__ Bs,
-                            float scale, float* __restrict__ dout, double* __restrict__ loss_part) {
-  extern __shared__ float sm[];
-  const int b = blockIdx.x;
+static size_t loss_smem(int n, int r) {
+  const size_t r4 = (r + 3) / 4 * 4, n4 = (n + 3) / 4 * 4;
+  return sizeof(float) * (2 * n4 * r4 + n4 + 2 * LG_RB * (n4 + 4) + LG_RB * 2 * r4 + 4096);
+}
+
+template <int NT>
+__global__ void __launch_bounds__(256) k_loss_grad(int n, int r, const float* __restrict__ out,
+                                                   const float* __restrict__ Bs, float scale, float* __restrict__ dout,
+                                                   double* __restrict__ loss_part) {
+  constexpr int RB = LG_RB;
+  extern __shared__ __align__(16) float sm[];
+  const int b = blockIdx.x, tid = threadIdx.x;
   const int no = n + 2 * n * r;
+  const int r4 = (r + 3) / 4 * 4, n4 = (n + 3) / 4 * 4, C = 2 * r4, ldb = n4 + 4;
   const float* o = out + (long long)b * no;
   const float* Bm = Bs + (long long)b * n * n;       // row-major
-  float* D = sm;                                     // [n]
-  float* U = D + n;                                  // [n][r]
-  float* V = U + n * r;                              // [n][r]
-  float* Wm = V + n * r;                             // [n][r]  Bs U
-  float* Z = Wm + n * r;                             // [n][r]  R V
-  __shared__ double red[256];
-  for (int i = threadIdx.x; i < n; i += blockDim.x) D[i] = 1.f + o[i];
-  for (int i = threadIdx.x; i < n * r; i += blockDim.x) {
-    U[i] = o[n + i];
-    V[i] = o[n + n * r + i];
+  float* U = sm;                                     // [n4][r4], zero padded
+  float* V = U + n4 * r4;                            // [n4][r4]
+  float* D = V + n4 * r4;                            // [n4]
+  float* Bb = D + n4;                                // [RB][ldb] rows of Bs
+  float* Rb = Bb + RB * ldb;                         // [RB][ldb] rows of R
+  float* Y = Rb + RB * ldb;                          // [RB][C]: W | Z
+  float* red = Y + RB * C;                           // [4096]
+  __shared__ double lred[256];
+  for (int i = tid; i < n4; i += 256) D[i] = i < n ? 1.f + o[i] : 0.f;
+  for (int i = tid; i < n4 * r4; i += 256) {
+    const int j = i / r4, k = i % r4;
+    const bool in = j < n && k < r;
+    U[i] = in ? o[n + j * r + k] : 0.f;
+    V[i] = in ? o[n + n * r + j * r + k] : 0.f;
   }
-  __syncthreads();
-  // W[i][k] = sum_j Bs_ij U_jk (threads over rows)
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    float acc[MLP_MAXR];
-    for (int k = 0; k < r; ++k) acc[k] = 0.f;
-    for (int j = 0; j < n; ++j) {
-      const float bij = Bm[(long long)i * n + j];
-      for (int k = 0; k < r; ++k) acc[k] = fmaf(bij, U[j * r + k], acc[k]);
+  // Y[:, c0 ...] = A (rows of a strip, n wide) times X [n][r4]: 4 x 4 tiles, n split over the other threads
+  auto strip_times = [&](const float* A, const float* X, int c_out) {
+    const int tiles = r4, KS = 256 / tiles;
+    const int tile = tid % tiles, ks = tid / tiles;
+    const int i0 = tile / (r4 / 4) * 4, c0 = tile % (r4 / 4) * 4;
+    if (ks < KS) {
+      float acc[4][4] = {};
+      for (int j = ks; j < n; j += KS) {
+        const float4 x = *reinterpret_cast<const float4*>(X + j * r4 + c0);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float a = A[(i0 + q) * ldb + j];
+          acc[q][0] = fmaf(a, x.x, acc[q][0]);
+          acc[q][1] = fmaf(a, x.y, acc[q][1]);
+          acc[q][2] = fmaf(a, x.z, acc[q][2]);
+          acc[q][3] = fmaf(a, x.w, acc[q][3]);
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) red[ks * (RB * r4) + (i0 + q) * r4 + c0 + c] = acc[q][c];
     }
-    for (int k = 0; k < r; ++k) Wm[i * r + k] = acc[k];
-  }
-  __syncthreads();
-  // rows: loss and Z = R V
-  double lsum = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    float z[MLP_MAXR];
-    for (int k = 0; k < r; ++k) z[k] = 0.f;
-    for (int j = 0; j < n; ++j) {
-      float rij = Bm[(long long)i * n + j] * D[j] - (i == j ? 1.f : 0.f);
-      for (int k = 0; k < r; ++k) rij = fmaf(Wm[i * r + k], V[j * r + k], rij);
-      lsum += (double)rij * rij;
-      for (int k = 0; k < r; ++k) z[k] = fmaf(rij, V[j * r + k], z[k]);
+    __syncthreads();
+    for (int i = tid; i < RB * r4; i += 256) {
+      float v = red[i];
+      for (int q = 1; q < KS; ++q) v += red[q * (RB * r4) + i];
+      Y[i / r4 * C + c_out + i % r4] = v;
     }
-    for (int k = 0; k < r; ++k) Z[i * r + k] = z[k];
-  }
-  __syncthreads();
-  // columns: dD_j, dV_j = sum_i R_ij W_i, dU_j = sum_i Bs_ij Z_i
-  float* g = dout + (long long)b * no;
-  for (int j = threadIdx.x; j < n; j += blockDim.x) {
-    float dv[MLP_MAXR], du[MLP_MAXR];
-    for (int k = 0; k < r; ++k) {
-      dv[k] = 0.f;
-      du[k] = 0.f;
+    __syncthreads();
+  };
+  float acc[NT][4][4] = {};
+  float dd[2] = {0.f, 0.f};                          // columns tid, tid + 256
+  float ls = 0.f, le = 0.f;                          // loss sum and its rounding error
+  const int tiles2 = (n4 / 4) * (C / 4);
+  for (int i0 = 0; i0 < n; i0 += RB) {
+    __syncthreads();
+    for (int i = tid; i < RB * n4; i += 256) {
+      const int q = i / n4, j = i % n4;
+      Bb[q * ldb + j] = (i0 + q < n && j < n) ? Bm[(long long)(i0 + q) * n + j] : 0.f;
     }
-    float dd = 0.f;
-    for (int i = 0; i < n; ++i) {
-      const float bij = Bm[(long long)i * n + j];
-      float rij = bij * D[j] - (i == j ? 1.f : 0.f);
-      for (int k = 0; k < r; ++k) rij = fmaf(Wm[i * r + k], V[j * r + k], rij);
-      dd = fmaf(bij, rij, dd);
-      for (int k = 0; k < r; ++k) {
-        dv[k] = fmaf(rij, Wm[i * r + k], dv[k]);
-        du[k] = fmaf(bij, Z[i * r + k], du[k]);
+    __syncthreads();
+    strip_times(Bb, U, 0);                           // W
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {                    // R, the loss and dD: one column per thread
+      const int j = tid + 256 * h;
+      if (j >= n4) continue;
+      float x[RB];
+#pragma unroll
+      for (int q = 0; q < RB; ++q) x[q] = Bb[q * ldb + j] * D[j] - (i0 + q == j ? 1.f : 0.f);
+      for (int k = 0; k < r4; k += 4) {
+        const float4 v = *reinterpret_cast<const float4*>(V + j * r4 + k);
+#pragma unroll
+        for (int q = 0; q < RB; ++q) {
+          const float4 w = *reinterpret_cast<const float4*>(Y + q * C + k);
+          x[q] = fmaf(w.x, v.x, fmaf(w.y, v.y, fmaf(w.z, v.z, fmaf(w.w, v.w, x[q]))));
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < RB; ++q) {
+        if (i0 + q >= n || j >= n) x[q] = 0.f;
+        Rb[q * ldb + j] = x[q];
+        dd[h] = fmaf(Bb[q * ldb + j], x[q], dd[h]);
+        const float sq = x[q] * x[q], se = fmaf(x[q], x[q], -sq);   // two-sum of the exact square
+        const float t = ls + sq, z = t - ls;
+        le += ((ls - (t - z)) + (sq - z)) + se;
+        ls = t;
       }
     }
-    g[j] = scale * dd;
-    for (int k = 0; k < r; ++k) {
-      g[n + j * r + k] = scale * du[k];
-      g[n + n * r + j * r + k] = scale * dv[k];
+    __syncthreads();
+    strip_times(Rb, V, r4);                          // Z
+#pragma unroll
+    for (int h = 0; h < NT; ++h) {                   // R^T W and Bs^T Z
+      const int tile = tid + 256 * h;
+      if (tile >= tiles2) continue;
+      const int j0 = tile % (n4 / 4) * 4, c0 = tile / (n4 / 4) * 4;
+      const float* A = c0 < r4 ? Rb : Bb;
+#pragma unroll 4
+      for (int q = 0; q < RB; ++q) {
+        const float4 a = *reinterpret_cast<const float4*>(A + q * ldb + j0);
+        const float4 y = *reinterpret_cast<const float4*>(Y + q * C + c0);
+        const float av[4] = {a.x, a.y, a.z, a.w}, yv[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+          for (int w = 0; w < 4; ++w) acc[h][u][w] = fmaf(av[u], yv[w], acc[h][u][w]);
+      }
     }
   }
-  red[threadIdx.x] = lsum;
+  float* g = dout + (long long)b * no;
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+    if (tid + 256 * h < n) g[tid + 256 * h] = scale * dd[h];
+#pragma unroll
+  for (int h = 0; h < NT; ++h) {
+    const int tile = tid + 256 * h;
+    if (tile >= tiles2) continue;
+    const int j0 = tile % (n4 / 4) * 4, c0 = tile / (n4 / 4) * 4;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int w = 0; w < 4; ++w) {
+        const int j = j0 + u, k = c0 < r4 ? c0 + w : c0 - r4 + w;
+        if (j < n && k < r) g[n + (c0 < r4 ? n * r : 0) + j * r + k] = scale * acc[h][u][w];
+      }
+  }
+  lred[tid] = (double)ls + (double)le;
   __syncthreads();
-  for (int st = blockDim.x / 2; st > 0; st >>= 1) {
-    if (threadIdx.x < st) red[threadIdx.x] += red[threadIdx.x + st];
+  for (int st = 128; st > 0; st >>= 1) {
+    if (tid < st) lred[tid] += lred[tid + st];
     __syncthreads();
   }
-  if (threadIdx.x == 0) loss_part[b] = red[0];
+  if (tid == 0) loss_part[b] = lred[0];
+}
+
+static int launch_loss(int nb, int n, int r, const float* out, const float* Bs, float scale, float* dout,
+                       double* loss_part, cudaStream_t s) {
+  const size_t smem = loss_smem(n, r);
+  const int r4 = (r + 3) / 4 * 4, n4 = (n + 3) / 4 * 4;
+  const int nt = ((n4 / 4) * (2 * r4 / 4) + 255) / 256;
+  if (smem > 227 * 1024 || n > 512 || nt > 5) return fail(DG_EINVAL, "MLP block too large for the loss kernel");
+  auto go = [&](auto kern) -> int {
+    DG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    kern<<<nb, 256, smem, s>>>(n, r, out, Bs, scale, dout, loss_part);
+    return DG_OK;
+  };
+  switch (nt) {
+    case 1: return go(k_loss_grad<1>);
+    case 2: return go(k_loss_grad<2>);
+    case 3: return go(k_loss_grad<3>);
+    case 4: return go(k_loss_grad<4>);
+    default: return go(k_loss_grad<5>);
+  }
 }
 
 __global__ void k_adam(long long n, float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
@@ -324,7 +465,8 @@ struct Mlp {
   float* Bs = nullptr;        // [cap][n][n]
   // scratch for a batch and for inference
   int batch_cap = 0;
-  float *z1 = nullptr, *h1 = nullptr, *z2 = nullptr, *h2 = nullptr, *o = nullptr, *dout = nullptr, *dh = nullptr;
+  float *z1 = nullptr, *h1 = nullptr, *z2 = nullptr, *h2 = nullptr, *o = nullptr, *dout = nullptr, *dh = nullptr,
+        *part = nullptr;
   double* loss_part = nullptr;
   // inference outputs for every element
   float* feat = nullptr;      // [E][n_in]
@@ -342,7 +484,7 @@ struct Mlp {
 static void mlp_free(Mlp* M) {
   if (!M) return;
   void* p[] = {M->params, M->grads, M->adam_m, M->adam_v, M->X, M->Bs, M->z1, M->h1, M->z2, M->h2, M->o, M->dout,
-               M->dh, M->loss_part, M->feat, M->sdiag, M->outE};
+               M->dh, M->part, M->loss_part, M->feat, M->sdiag, M->outE};
   for (void* q : p)
     if (q) cudaFree(q);
   delete M;
@@ -358,30 +500,38 @@ static inline uint64_t splitmix(uint64_t seed, uint64_t i) {
 
 static int ensure_batch(Mlp* M, int batch) {
   if (M->batch_cap >= batch) return DG_OK;
-  float** bufs[] = {&M->z1, &M->h1, &M->z2, &M->h2, &M->o, &M->dout, &M->dh};
+  float** bufs[] = {&M->z1, &M->h1, &M->z2, &M->h2, &M->o, &M->dout, &M->dh, &M->part};
   for (float** b : bufs)
     if (*b) { cudaFree(*b); *b = nullptr; }
   if (M->loss_part) cudaFree(M->loss_part);
-  const size_t H = (size_t)batch * M->hidden, O = (size_t)batch * M->n_out;
+  const size_t H = (size_t)batch * M->hidden, OB = (size_t)batch * M->n_out;
   cudaError_t err = cudaMalloc(&M->z1, H * 4);
   if (err == cudaSuccess) err = cudaMalloc(&M->h1, H * 4);
   if (err == cudaSuccess) err = cudaMalloc(&M->z2, H * 4);
   if (err == cudaSuccess) err = cudaMalloc(&M->h2, H * 4);
-  if (err == cudaSuccess) err = cudaMalloc(&M->o, O * 4);
-  if (err == cudaSuccess) err = cudaMalloc(&M->dout, O * 4);
+  if (err == cudaSuccess) err = cudaMalloc(&M->o, OB * 4);
+  if (err == cudaSuccess) err = cudaMalloc(&M->dout, OB * 4);
   if (err == cudaSuccess) err = cudaMalloc(&M->dh, (H > (size_t)batch * M->n_in ? H : (size_t)batch * M->n_in) * 4);
   if (err == cudaSuccess) err = cudaMalloc(&M->loss_part, sizeof(double) * batch);
+  // partial sums of the split products, for every batch up to this one (fewer rows may split more)
+  const int Hd = M->hidden, O = M->n_out, I = M->n_in;
+  size_t part = 1;
+  for (int nb = std::min(batch, GBM); ; nb = std::min(batch, nb + GBM)) {
+    part = std::max(part, std::max(gemm_part_floats(nb, Hd, Hd), gemm_part_floats(nb, Hd, O)));
+    if (nb == batch) break;
+  }
+  for (size_t p : {gemm_part_floats(O, Hd, batch), gemm_part_floats(Hd, Hd, batch), gemm_part_floats(Hd, I, batch)})
+    part = std::max(part, p);
+  if (err == cudaSuccess) err = cudaMalloc(&M->part, part * 4);
   if (err != cudaSuccess) return fail(DG_ENOMEM, std::string("MLP batch storage: ") + cudaGetErrorString(err));
   M->batch_cap = batch;
   return DG_OK;
 }
 
 static int forward(Mlp* M, const float* X, int nb, float* out, cudaStream_t s) {
-  gemm<false, true>(s, nb, M->hidden, M->n_in, X, M->n_in, M->W1(), M->n_in, M->z1, M->hidden, 0.f, M->b1(), M->h1);
-  gemm<false, true>(s, nb, M->hidden, M->hidden, M->h1, M->hidden, M->W2(), M->hidden, M->z2, M->hidden, 0.f, M->b2(),
-                    M->h2);
-  gemm<false, true>(s, nb, M->n_out, M->hidden, M->h2, M->hidden, M->W3(), M->hidden, out, M->n_out, 0.f, M->b3(),
-                    nullptr);
+  gemm<false, true>(s, nb, M->hidden, M->n_in, X, M->n_in, M->W1(), M->n_in, M->z1, nullptr, M->b1(), M->h1);
+  gemm<false, true>(s, nb, M->hidden, M->hidden, M->h1, M->hidden, M->W2(), M->hidden, M->z2, nullptr, M->b2(), M->h2);
+  gemm<false, true>(s, nb, M->n_out, M->hidden, M->h2, M->hidden, M->W3(), M->hidden, out, nullptr, M->b3());
   DG_LAUNCH_CHECK("mlp forward");
   return DG_OK;
 }
@@ -392,11 +542,9 @@ static int loss_grad(Mlp* M, const float* X, const float* Bs, int nb, double* lo
   if (rc) return rc;
   rc = forward(M, X, nb, M->o, s);
   if (rc) return rc;
-  const size_t smem = sizeof(float) * (M->n + 4 * M->n * M->rank);
-  if (smem > 200 * 1024) return fail(DG_EINVAL, "MLP block too large for the loss kernel");
-  cudaFuncSetAttribute(k_loss_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   const float scale = 2.f / ((float)nb * (float)M->n);
-  k_loss_grad<<<nb, 256, smem, s>>>(nb, M->n, M->rank, M->o, Bs, scale, M->dout, M->loss_part);
+  rc = launch_loss(nb, M->n, M->rank, M->o, Bs, scale, M->dout, M->loss_part, s);
+  if (rc) return rc;
   DG_LAUNCH_CHECK("k_loss_grad");
   const int H = M->hidden, I = M->n_in, O = M->n_out;
   float* gW1 = M->grads;
@@ -406,18 +554,16 @@ static int loss_grad(Mlp* M, const float* X, const float* Bs, int nb, double* lo
   float* gW3 = gb2 + H;
   float* gb3 = gW3 + (long long)O * H;
   // output layer
-  gemm<true, false>(s, O, H, nb, M->dout, O, M->h2, H, gW3, H);
-  k_colsum<<<(O + 255) / 256, 256, 0, s>>>(nb, O, M->dout, gb3);
-  // dh2 = dout W3, dz2 = dh2 * silu'(z2)
-  gemm<false, false>(s, nb, H, O, M->dout, O, M->W3(), H, M->dh, H);
-  k_silu_back<<<1024, 256, 0, s>>>((long long)nb * H, M->z2, M->dh);
-  gemm<true, false>(s, H, H, nb, M->dh, H, M->h1, H, gW2, H);
-  k_colsum<<<(H + 255) / 256, 256, 0, s>>>(nb, H, M->dh, gb2);
-  // dh1 = dz2 W2 (into z2's buffer, no longer needed), dz1 = dh1 * silu'(z1)
-  gemm<false, false>(s, nb, H, H, M->dh, H, M->W2(), H, M->z2, H);
-  k_silu_back<<<1024, 256, 0, s>>>((long long)nb * H, M->z1, M->z2);
-  gemm<true, false>(s, H, I, nb, M->z2, H, X, I, gW1, I);
-  k_colsum<<<(H + 255) / 256, 256, 0, s>>>(nb, H, M->z2, gb1);
+  gemm<true, false>(s, O, H, nb, M->dout, O, M->h2, H, gW3, M->part);
+  k_colsum<<<(O + 31) / 32, 512, 0, s>>>(nb, O, M->dout, gb3);
+  // dz2 = (dout W3) silu'(z2)
+  gemm<false, false>(s, nb, H, O, M->dout, O, M->W3(), H, M->dh, M->part, nullptr, nullptr, M->z2);
+  gemm<true, false>(s, H, H, nb, M->dh, H, M->h1, H, gW2, M->part);
+  k_colsum<<<(H + 31) / 32, 512, 0, s>>>(nb, H, M->dh, gb2);
+  // dz1 = (dz2 W2) silu'(z1), into z2's buffer, no longer needed
+  gemm<false, false>(s, nb, H, H, M->dh, H, M->W2(), H, M->z2, M->part, nullptr, nullptr, M->z1);
+  gemm<true, false>(s, H, I, nb, M->z2, H, X, I, gW1, M->part);
+  k_colsum<<<(H + 31) / 32, 512, 0, s>>>(nb, H, M->z2, gb1);
   DG_LAUNCH_CHECK("mlp backward");
   if (loss) {
     std::vector<double> part(nb);
