@@ -661,7 +661,7 @@ __global__ void __launch_bounds__(128, 3) k_faces64(long long E, long long F, Ph
 // --------------------------------------------------------------------------------------------
 // the state at Gauss point g and its fluxes and sources (volume64), with the stage operator's mass term
 template <int N, int NC, typename S>
-__device__ __forceinline__ void volume_load(long long e, long long E, int g, const PhysT<double>& P, double t,
+__device__ __forceinline__ void volume_load(long long e, long long E, int g, const PhysT<double>& P, const Sun64& sun,
                                             const double* __restrict__ gu, const double* __restrict__ accg,
                                             const double* __restrict__ xg, const double* __restrict__ ug,
                                             const double* __restrict__ qg, const double* __restrict__ mixg,
@@ -688,7 +688,7 @@ __device__ __forceinline__ void volume_load(long long e, long long E, int g, con
 #pragma unroll
     for (int k = 0; k < 8; ++k) mg[k] = mixg[(e * 8 + k) * NP + g];
   }
-  volume64<S>(P, u, q, det, a3, x3, t, mg, F, src);
+  volume64<S>(P, u, q, det, a3, x3, sun, mg, F, src);
   if constexpr (NC == 2)
     if (inv_stage_c != 0.0) {
       const double w = -det * inv_stage_c;
@@ -716,7 +716,7 @@ struct VolCells {
 // the FP64 twin of k_volume64 from the pointwise fluxes on
 template <int N, int NC>
 __device__ __noinline__ void volume_slow(const XOps<N>& so, long long e, long long E, int g, bool act, bool own,
-                                         const PhysT<double>& P, double t, const double* gu, const double* accg,
+                                         const PhysT<double>& P, const Sun64& sun, const double* gu, const double* accg,
                                          const double* xg, const double* ug, const double* qg, const double* fh,
                                          const double* mixg, double stage_c, double inv_stage_c, cell* cells, double* r,
                                          double* jv) {
@@ -726,7 +726,7 @@ __device__ __noinline__ void volume_slow(const XOps<N>& so, long long e, long lo
   cell *sF = cells, *sS = cells + C::S, *sH = cells + C::H;
   if (act) {
     S F[12], src[5];
-    volume_load<N, NC, S>(e, E, g, P, t, gu, accg, xg, ug, qg, mixg, inv_stage_c, F, src);
+    volume_load<N, NC, S>(e, E, g, P, sun, gu, accg, xg, ug, qg, mixg, inv_stage_c, F, src);
     for (int a = 0; a < 3; ++a)
 #pragma unroll
       for (int c = 0; c < 5; ++c) {
@@ -785,7 +785,7 @@ __device__ __noinline__ void volume_slow(const XOps<N>& so, long long e, long lo
 // formed as -stage_c (J_r v - M v / stage_c), with -|J| u_dot / stage_c added to the tangent's source.
 template <int N, int NC>
 __global__ void __launch_bounds__(128, NC == 2 ? 3 : 4)
-    k_volume64(long long E, const Ops* __restrict__ ops, PhysT<double> P, double t, const double* __restrict__ gu,
+    k_volume64(long long E, const Ops* __restrict__ ops, PhysT<double> P, Sun64 sun, const double* __restrict__ gu,
                const double* __restrict__ accg, const double* __restrict__ xg, const double* __restrict__ ug,
                const double* __restrict__ qg, const double* __restrict__ fh, double* __restrict__ r,
                double* __restrict__ jv, double stage_c, double inv_stage_c, const double* __restrict__ mixg) {
@@ -812,7 +812,7 @@ __global__ void __launch_bounds__(128, NC == 2 ? 3 : 4)
   int eG[3] = {0, 0, 0}, eF[NC][3];          // this point's exponents: geometry rows, flux groups
   if (live && act) {
     S F[12], src[5];
-    volume_load<N, NC, S>(e, E, g, P, t, gu, accg, xg, ug, qg, mixg, inv_stage_c, F, src);
+    volume_load<N, NC, S>(e, E, g, P, sun, gu, accg, xg, ug, qg, mixg, inv_stage_c, F, src);
     double Gd[9];
     const double* gp = gu + e * 11 * NP + g;
 #pragma unroll
@@ -889,7 +889,7 @@ __global__ void __launch_bounds__(128, NC == 2 ? 3 : 4)
     if (mx[k] == 0) mx[k] = 1023;
   }
   if (!grp_all<N>(ok)) {
-    volume_slow<N, NC>(so, e, E, g, act && live && !ok, live && !ok, P, t, gu, accg, xg, ug, qg, fh, mixg, stage_c, inv_stage_c, cells,
+    volume_slow<N, NC>(so, e, E, g, act && live && !ok, live && !ok, P, sun, gu, accg, xg, ug, qg, fh, mixg, stage_c, inv_stage_c, cells,
                        r, jv);
     if constexpr (T >= 32) return;
   }

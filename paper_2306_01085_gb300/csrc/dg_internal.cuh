@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "../../include/dg.h"
+#include "dg_euvac64.cuh"
 #include "dg_fx.cuh"
 
 namespace dg {
@@ -139,6 +140,7 @@ struct dg_mesh {
   dg::Phys phys;
   dg::Ops ops;
   dg::Ops* d_ops = nullptr;
+  dg::EuvFx* d_euv = nullptr;   // EUVAC band tables (euv = DG_EUV_EUVAC only)
   double* x = nullptr;     // [E][3][Np] node coordinates
   double* geo = nullptr;   // [E][10][Np]: G[a][d] = W detJ dxi_a/dx_d (9), W detJ (1)
   // the same without quadrature weights (FP64 kernels)

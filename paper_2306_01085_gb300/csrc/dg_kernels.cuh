@@ -30,6 +30,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <cmath>
 #include <string>
 #include <type_traits>
 
@@ -1249,9 +1250,19 @@ static int run_volume(dg_mesh* m, double t, double* r, double* jv, cudaStream_t 
     const size_t sm = sizeof(cell) * VolCells<N, NC>::size * per;
     int rc = set_smem(k_volume64<N, NC>, sm);
     if (rc) return rc;
+    Sun64 sun{{0.0, 0.0, 0.0}, m->d_euv};
+    const double wt = m->phys.euv_omega_t * t;
+    if (m->phys.euv == DG_EUV_GAUSS) {
+      sun.d[0] = std::cos(wt);
+      sun.d[1] = -std::sin(wt);
+    } else if (m->phys.euv == DG_EUV_EUVAC) {
+      sun.d[0] = -m->phys.sun_cd * std::cos(wt);
+      sun.d[1] = m->phys.sun_cd * std::sin(wt);
+      sun.d[2] = m->phys.sun_sd;
+    }
     prof_begin(m, s, KK_VOLUME);
     k_volume64<N, NC><<<(unsigned)((m->E + per - 1) / per), threads, sm, s>>>(
-        m->E, m->d_ops, phys_as<double>(m->phys), t, m->gu, m->acc, m->xg, m->ws.ug, m->ws.qg, m->ws.fh, r, jv, stage_c,
+        m->E, m->d_ops, phys_as<double>(m->phys), sun, m->gu, m->acc, m->xg, m->ws.ug, m->ws.qg, m->ws.fh, r, jv, stage_c,
         stage_c != 0.0 ? 1.0 / stage_c : 0.0, m->mixg);
     prof_end(m, s);
     DG_LAUNCH_CHECK("k_volume64");

@@ -324,7 +324,7 @@ static void free_mesh(dg_mesh* m) {
   dg_mlp_release(m);
   dg::interp_tc_release(m);
   if (m->w32_base) cudaFree(m->w32_base);
-  void* ptrs[] = {m->d_ops, m->x, m->geo, m->gu, m->fgu, m->kn, m->acc, m->xg, m->fgeo, m->mixg, m->mixf, m->nbr, m->nbr_fo, m->face_e,
+  void* ptrs[] = {m->d_ops, m->d_euv, m->x, m->geo, m->gu, m->fgu, m->kn, m->acc, m->xg, m->fgeo, m->mixg, m->mixf, m->nbr, m->nbr_fo, m->face_e,
                   m->face_f,
                   m->ws.ug, m->ws.uf, m->ws.qg, m->ws.qf, m->ws.fh, m->ws.tmp, m->ws.red, m->ws.qx};
   for (void* p : ptrs)
@@ -493,6 +493,7 @@ extern "C" int dg_mesh_create(const dg_mesh_desc* desc, const double* nodes, dg_
   X.shrink_to_fit();
 
   rc |= dalloc(&m->d_ops, 1);
+  if (d.euv == DG_EUV_EUVAC) rc |= dalloc(&m->d_euv, 1);
   rc |= dalloc(&m->geo, E * 10 * NP);
   rc |= dalloc(&m->gu, E * 11 * NP);
   rc |= dalloc(&m->fgu, E * 24 * NF);
@@ -517,6 +518,11 @@ extern "C" int dg_mesh_create(const dg_mesh_desc* desc, const double* nodes, dg_
   }
   cudaError_t err = cudaSuccess;
   err = cudaMemcpy(m->d_ops, &m->ops, sizeof(Ops), cudaMemcpyHostToDevice);
+  if (err == cudaSuccess && m->d_euv) {
+    EuvFx tables;
+    build_euv(P.n_euvac, P.euvac_B, P.euvac_phi, d.comp ? 4 : 1, &tables);
+    err = cudaMemcpy(m->d_euv, &tables, sizeof(tables), cudaMemcpyHostToDevice);
+  }
   if (err == cudaSuccess) err = cudaMemcpy(m->nbr, nbr.data(), sizeof(int32_t) * nbr.size(), cudaMemcpyHostToDevice);
   if (err == cudaSuccess) err = cudaMemcpy(m->nbr_fo, nbr_fo.data(), sizeof(int32_t) * nbr_fo.size(), cudaMemcpyHostToDevice);
   if (err == cudaSuccess && m->nfaces)

@@ -13,6 +13,7 @@
 // reference-space contraction (640 and 960 before, with CUDA's exp, log and divisions).
 #pragma once
 
+#include "dg_euvac64.cuh"
 #include "dg_internal.cuh"
 #include "dg_math64.cuh"
 
@@ -24,6 +25,12 @@ __device__ __forceinline__ D64 s_fma(D64 a, D64 b, D64 c) {
   return {fma(a.v, b.v, c.v), fma(a.v, b.d, fma(a.d, b.v, c.d))};
 }
 __device__ __forceinline__ D64 s_fma(double a, D64 b, D64 c) { return {fma(a, b.v, c.v), fma(a, b.d, c.d)}; }
+
+__device__ __forceinline__ double val64(double x) { return x; }
+__device__ __forceinline__ double val64(D64 x) { return x.v; }
+// f(k) of value f and derivative df
+__device__ __forceinline__ double tangent64(double f, double, double) { return f; }
+__device__ __forceinline__ D64 tangent64(double f, double df, D64 k) { return {f, df * k.d}; }
 
 // s = e^{-varrho/2}, sr = e^{varrho/2}
 __device__ __forceinline__ void s_rho(double u0, double& s, double& sr) { exp_pm_fast(0.5 * u0, sr, s); }
@@ -160,69 +167,60 @@ __device__ __forceinline__ void sigma64(const PhysT<double>& P, const S& uh0, co
   se = P.comp ? P.lam + ((P.c_k / mx.cv) * kappa) * s : P.lam + (P.c_k / (P.cv * P.c_mu)) * x;
 }
 
+// the Sun at the time of the call (host): unit direction for EUVAC, (cos, sin) of the rotation for the
+// Gaussian, and the band tables
+struct Sun64 {
+  double d[3];
+  const EuvFx* bands;
+};
+
 // EUVAC / Gaussian heating over c_v sqrt(rho), added to the energy source
 template <typename S>
-__device__ __forceinline__ S heating64(const PhysT<double>& P, const S& s, const S& sr, const S& T, double cvp,
-                                       const double* xg, double t, const double mg[8]) {
+__device__ __forceinline__ S heating64(const PhysT<double>& P, const Sun64& sun, const S& s, const S& sr, const S& T,
+                                       double cvp, const double* xg, const double mg[8]) {
   const double r2 = xg[0] * xg[0] + xg[1] * xg[1] + xg[2] * xg[2];
-  const double r = sqrt(r2);
+  const double r = sqrt(r2), ir = recip_fast(r), icv = recip_fast(cvp);
+  double cchi = (xg[0] * sun.d[0] + xg[1] * sun.d[1] + xg[2] * sun.d[2]) * ir;
+  cchi = fmin(1.0, fmax(-1.0, cchi));
   if (P.euv == DG_EUV_GAUSS) {
-    double sn, cs;
-    sincos(P.euv_omega_t * t, &sn, &cs);
-    double cchi = (xg[0] * cs - xg[1] * sn) / r;
-    cchi = fmin(1.0, fmax(-1.0, cchi));
     const double chi = acos(cchi);
     const double dz = (r - P.euv_r_peak) * P.euv_inv_w;
     const double Qh = P.euv_amp * exp_fast(fma(-chi * chi, P.euv_inv2s2, -0.6931471805599453 * dz * dz));
-    return (Qh / cvp) * s;
+    return (Qh * icv) * s;
   }
-  double sn, cs;
-  sincos(P.euv_omega_t * t, &sn, &cs);
-  double cchi = (xg[1] * (P.sun_cd * sn) - xg[0] * (P.sun_cd * cs) + xg[2] * P.sun_sd) / r;
-  cchi = fmin(1.0, fmax(-1.0, cchi));
   const double schi = sqrt(fmax(0.0, 1.0 - cchi * cchi));
   if (!(cchi > 0.0 || schi * r > P.g_r0)) return s_zero<S>();   // in the Earth's shadow
   const S er = sr * sr;                             // e^varrho
   const double minv = P.comp ? cvp : P.inv_m;       // 1/m*
   const S Hs = T * (r2 * minv / (P.g_r0 * P.g_r0));   // H* = T* r*^2 / (m* g_r0^2)
   const S rt = r * s_inv(Hs);                       // r~ = |r| / H
-  const S ex = s_erfcx(s_sqrt(0.5 * rt) * fabs(cchi));
-  const S base = s_sqrt(1.5707963267948966 * rt);
+  const S hr = s_sqrt(0.5 * rt);
+  const S ex = s_erfcx(hr * fabs(cchi));
+  const S base = 1.7724538509055160273 * hr;        // sqrt(pi r~ / 2)
   S ch;
   if (cchi > 0.0) ch = base * ex;
   else ch = base * (2.0 * s_exp(rt * (1.0 - schi)) - ex);
   // species weights w_s = chi_s / m_s* (O, N2, O2, He), or 1/m* on oxygen alone
-  double ws[4] = {P.inv_m, 0.0, 0.0, 0.0};
-  if (P.comp) {
-    ws[0] = 1.0 - mg[5] - mg[6] - mg[7];
-    ws[1] = mg[5] * (16.0 / 28.0);
-    ws[2] = mg[6] * (16.0 / 32.0);
-    ws[3] = mg[7] * (16.0 / 4.0);
-  }
   const S k = (P.euvac_cc * er) * Hs * ch;          // tau_j = Phi_j k
-  S qs = s_zero<S>();
-#pragma unroll 1
-  for (int j = 0; j < P.n_euvac; ++j) {
-    const double Phi = P.comp ? fma(ws[0], P.euvac_phi[0][j], fma(ws[1], P.euvac_phi[1][j],
-                                    fma(ws[2], P.euvac_phi[2][j], ws[3] * P.euvac_phi[3][j])))
-                              : ws[0] * P.euvac_phi[0][j];
-    if constexpr (std::is_same<S, double>::value) {
-      qs = fma(P.euvac_B[j] * Phi, exp_fast(-Phi * k), qs);
-    } else {   // d exp(-Phi k) = -Phi exp(-Phi k) dk; dk outside the sum
-      const double a = (P.euvac_B[j] * Phi) * exp_fast(-Phi * k.v);
-      qs.v += a;
-      qs.d = fma(-Phi, a, qs.d);
-    }
+  const double kv = val64(k);
+  double S0, S1;
+  if (P.comp) {
+    const double ws[4] = {1.0 - mg[5] - mg[6] - mg[7], mg[5] * (16.0 / 28.0), mg[6] * (16.0 / 32.0), mg[7] * (16.0 / 4.0)};
+    euvac_sums<4>(sun.bands, ws, kv, S0, S1);
+  } else {
+    const double ws[4] = {1.0, 0.0, 0.0, 0.0};
+    euvac_sums<1>(sun.bands, ws, P.inv_m * kv, S0, S1);
+    S0 *= P.inv_m;
+    S1 *= P.inv_m * P.inv_m;
   }
-  if constexpr (!std::is_same<S, double>::value) qs.d *= k.d;
-  return (er * qs) * (1.0 / cvp) * s;
+  return (er * tangent64(S0, -S1, k)) * icv * s;
 }
 
 // physical fluxes F[12]: momentum xx, yy, zz, xy, xz, yz (symmetric), varrho x, y, z, energy x, y, z; and
 // the sources, weighted with the Jacobian determinant
 template <typename S>
 __device__ __forceinline__ void volume64(const PhysT<double>& P, const S u[5], const S q[3][5], double det,
-                                         const double acc[3], const double* xg, double t, const double mg[8], S F[12],
+                                         const double acc[3], const double* xg, const Sun64& sun, const double mg[8], S F[12],
                                          S src[5]) {
   const Mix<double> mx{P.comp ? mg[0] : P.cv, P.comp ? mg[4] : 1.0};
   const double cvp = mx.cv;
@@ -287,7 +285,7 @@ __device__ __forceinline__ void volume64(const PhysT<double>& P, const S u[5], c
 #pragma unroll
     for (int d = 0; d < 3; ++d) x = s_fma(icv * mg[1 + d], F[9 + d], x);
   }
-  if (P.euv) x = x + heating64(P, s, sr, T, cvp, xg, t, mg);
+  if (P.euv) x = x + heating64(P, sun, s, sr, T, cvp, xg, mg);
   src[4] = det * x;
 }
 

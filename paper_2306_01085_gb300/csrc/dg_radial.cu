@@ -31,6 +31,7 @@
 
 #include "dg_internal.cuh"
 #include "dg_nvtx.h"
+#include "dg_phys64.cuh"
 
 struct dg_radial;
 
@@ -54,12 +55,15 @@ struct RPhys {
   int euv, bc_lo, bc_hi;
   int n_euvac;
   R B[40], phi[40], cc, sun_cd, sun_sd, omega_t, inv_m;   // EUVAC (oxygen), efficiency 1
+  double sun[3];          // FP64 path: the Sun direction at the time of the call and the band tables
+  const EuvFx* bands;
 };
 
-// per element geometry: [E] rL, rR; [E][N] rg, W = w J r^2, G = w r^2, T2 = 2 w J r
+// per element geometry: [E] rL, rR; [E][N] rg, W = w J r^2, G = w r^2, T2 = 2 w J r, ir = 1 / r, iW = 1 / W,
+// ar = -(g_r0 / r)^2 / gamma
 template <typename R>
 struct RGeo {
-  const R *rL, *rR, *rg, *W, *G, *T2;
+  const R *rL, *rR, *rg, *W, *G, *T2, *ir, *iW, *ar;
 };
 
 // per column parameters [5][n_col]: epsilon, alpha0, site unit vector
@@ -80,9 +84,18 @@ struct Prim1 {
   S isr, v, T, gvr, gvt, gT, div, er, et, mu, kap;
 };
 
+// T^visc_exp; the FP64 path forms it from varrho and sqrt(rho) T with few FP64 instructions (t_power)
+template <typename S, typename R>
+__device__ __forceinline__ S power1(const RPhys<R>& P, const S& u0, const S& u2, const S& T) {
+  if (P.visc_exp == R(0)) return s_const<S>(R(1));
+  if constexpr (std::is_same<R, double>::value) return t_power(P.visc_exp, u0, u2, t_dlog(u0, u2));
+  else return s_exp(P.visc_exp * s_log(T));
+}
+
 template <typename S, typename R>
 __device__ __forceinline__ void prim1(const RPhys<R>& P, const S u[3], const S q[4], R alpha, Prim1<S>& w) {
-  w.isr = s_exp(R(-0.5) * u[0]);
+  if constexpr (std::is_same<R, double>::value) w.isr = s_isr(u[0]);
+  else w.isr = s_exp(R(-0.5) * u[0]);
   w.v = u[1] * w.isr;
   w.T = u[2] * w.isr;
   w.gvr = w.isr * (q[1] - R(0.5) * (u[1] * q[0]));
@@ -91,7 +104,7 @@ __device__ __forceinline__ void prim1(const RPhys<R>& P, const S u[3], const S q
   w.div = w.gvr + R(2) * w.gvt;
   w.er = R(2) * w.gvr - R(2.0 / 3.0) * w.div;
   w.et = R(2) * w.gvt - R(2.0 / 3.0) * w.div;
-  w.mu = (P.visc_exp != R(0)) ? s_exp(P.visc_exp * s_log(w.T)) : s_const<S>(R(1));
+  w.mu = power1(P, u[0], u[2], w.T);
   w.kap = alpha * w.mu;
 }
 
@@ -103,7 +116,8 @@ __device__ __forceinline__ void flux1(const RPhys<R>& P, const S u[3], const S q
   if (viscous) {
     prim1(P, u, q, alpha, w);
   } else {
-    w.isr = s_exp(R(-0.5) * u[0]);
+    if constexpr (std::is_same<R, double>::value) w.isr = s_isr(u[0]);
+    else w.isr = s_exp(R(-0.5) * u[0]);
     w.v = u[1] * w.isr;
   }
   F[0] = u[0] * w.v;
@@ -121,9 +135,11 @@ __device__ __forceinline__ void flux1(const RPhys<R>& P, const S u[3], const S q
 
 template <typename S, typename R>
 __device__ __forceinline__ void sigma1(const RPhys<R>& P, const S uh[3], R alpha, S sg[3]) {
-  const S isr = s_exp(R(-0.5) * uh[0]);
+  S isr;
+  if constexpr (std::is_same<R, double>::value) isr = s_isr(uh[0]);
+  else isr = s_exp(R(-0.5) * uh[0]);
   const S T = uh[2] * isr;
-  const S mu = (P.visc_exp != R(0)) ? s_exp(P.visc_exp * s_log(T)) : s_const<S>(R(1));
+  const S mu = power1(P, uh[0], uh[2], T);
   sg[0] = s_const<S>(P.lam);
   sg[1] = P.lam + (P.c_mu * mu) * isr;
   sg[2] = P.lam + ((P.c_k / P.cv) * (alpha * mu)) * isr;
@@ -141,9 +157,31 @@ template <typename R> __device__ __forceinline__ R val_of(DualT<R> x) { return x
 
 // EUVAC heating q* (efficiency 1) at radius r above the site, Sec. 2.2 with Smith & Smith Chapman
 // depths for the single absorber (oxygen); zero in the Earth's shadow. Bands whose optical depth
-// exceeds 40 are skipped: their attenuated flux is below e^-40 (4e-18) of the band's own.
+// exceeds 40 are skipped in the FP32 probes: their attenuated flux is below e^-40 (4e-18) of the band's
+// own. The FP64 path sums the bands in fixed point (euvac_sums).
 template <typename S, typename R>
 __device__ __forceinline__ S heat1(const RPhys<R>& P, R r, const R site[3], R t, const S& isr, const S& T) {
+  if constexpr (std::is_same<R, double>::value) {
+    double cchi = site[0] * P.sun[0] + site[1] * P.sun[1] + site[2] * P.sun[2];
+    cchi = fmin(1.0, fmax(-1.0, cchi));
+    const double schi = sqrt(fmax(0.0, 1.0 - cchi * cchi));
+    if (!(cchi > 0.0 || schi * r > P.g_r0)) return s_zero<S>();
+    const S sr = s_inv(isr);
+    const S er = sr * sr;                                   // e^varrho
+    const S Hs = T * (r * r * P.inv_m / (P.g_r0 * P.g_r0)); // H* = T* r*^2 / (m* g_r0^2)
+    const S rt = r * s_inv(Hs);
+    const S hr = s_sqrt(0.5 * rt);
+    const S ex = s_erfcx(hr * fabs(cchi));
+    const S base = 1.7724538509055160273 * hr;              // sqrt(pi r~ / 2)
+    S ch;
+    if (cchi > 0.0) ch = base * ex;
+    else ch = base * (2.0 * s_exp(rt * (1.0 - schi)) - ex);
+    const S k = (P.cc * er) * Hs * ch;
+    const double one[4] = {1.0, 0.0, 0.0, 0.0};
+    double S0, S1;
+    euvac_sums<1>(P.bands, one, P.inv_m * val64(k), S0, S1);
+    return er * tangent64(P.inv_m * S0, -(P.inv_m * P.inv_m) * S1, k);
+  }
   const R wt = P.omega_t * t;
   R cchi = site[0] * (-P.sun_cd * cos(wt)) + site[1] * (P.sun_cd * sin(wt)) + site[2] * P.sun_sd;
   cchi = fmin(R(1), fmax(R(-1), cchi));
@@ -171,7 +209,7 @@ __device__ __forceinline__ S heat1(const RPhys<R>& P, R r, const R site[3], R t,
 
 // source (s_varrho, s_m + 2 F_tt / r, s_e) at a Gauss point
 template <typename S, typename R>
-__device__ __forceinline__ void source1(const RPhys<R>& P, const S u[3], const S q[4], R r, R alpha, R eps,
+__device__ __forceinline__ void source1(const RPhys<R>& P, const S u[3], const S q[4], R r, R ir, R ar, R alpha, R eps,
                                         const R site[3], R t, S F[3], S src[3]) {
   Prim1<S> w;
   prim1(P, u, q, alpha, w);
@@ -181,10 +219,11 @@ __device__ __forceinline__ void source1(const RPhys<R>& P, const S u[3], const S
   F[0] = u[0] * w.v;
   F[1] = u[1] * w.v + P.pc * u[2] - cm * w.er;
   F[2] = u[2] * w.v - ck * w.gT;
-  const R a_r = -(P.g_r0 / r) * (P.g_r0 / r) / P.gamma;
+  const bool f64 = std::is_same<R, double>::value;
+  const R a_r = f64 ? ar : -(P.g_r0 / r) * (P.g_r0 / r) / P.gamma;
   src[0] = (u[0] - R(1)) * w.div;
   src[1] = s_inv(w.isr) * a_r + R(0.5) * (w.div * u[1]) - (R(0.5) * P.pc) * (u[2] * q[0]) + R(0.5) * (cm * w.er * q[0]) +
-           (R(2) / r) * Ftt;
+           (f64 ? R(2) * ir : R(2) / r) * Ftt;
   S s2 = (R(1.5) - P.gamma) * (u[2] * w.div) + R(0.5) * (ck * w.gT * q[0]) +
          ((P.c_d / P.cv) * w.mu) * (w.isr * (w.er * w.gvr + R(2) * (w.et * w.gvt)));
   if (P.euv == DG_EUV_EUVAC) s2 = s2 + (eps * heat1<S, R>(P, r, site, t, w.isr, w.T)) * (R(1) / P.cv) * w.isr;
@@ -318,7 +357,7 @@ __global__ void k_rgrad(int E, long long nc, ROps<R> O, RPhys<R> P, RGeo<R> g, c
       S acc = (rR2 * O.eR[j]) * uhR[c] - (rL2 * O.eL[j]) * uhL[c] - T2[j] * U[c][j];
 #pragma unroll
       for (int gq = 0; gq < N; ++gq) acc = acc - (O.D[gq * N + j] * G[gq]) * U[c][gq];
-      const S qv = acc * (R(1) / W[j]);
+      const S qv = acc * (std::is_same<R, double>::value ? g.iW[k * N + j] : R(1) / W[j]);
       const long long o = (((long long)qmap[c] * E + k) * N + j) * nc + col;
       if constexpr (PROBE) {
         if (blockIdx.y == 0) qg[o] = qv.v;
@@ -330,7 +369,7 @@ __global__ void k_rgrad(int E, long long nc, ROps<R> O, RPhys<R> P, RGeo<R> g, c
   }
 #pragma unroll
   for (int j = 0; j < N; ++j) {
-    const S qv = U[1][j] * (R(1) / rg[j]);
+    const S qv = U[1][j] * (std::is_same<R, double>::value ? g.ir[k * N + j] : R(1) / rg[j]);
     const long long o = ((2LL * E + k) * N + j) * nc + col;
     if constexpr (PROBE) {
       if (blockIdx.y == 0) qg[o] = qv.v;
@@ -475,7 +514,7 @@ __global__ void k_rvol(int E, long long nc, ROps<R> O, RPhys<R> P, RGeo<R> g, RP
     }
     const R rg = g.rg[k * N + gq];
     S F[3], src[3];
-    source1<S, R>(P, ug, qq, rg, alpha, eps, site, t, F, src);
+    source1<S, R>(P, ug, qq, rg, g.ir[k * N + gq], g.ar[k * N + gq], alpha, eps, site, t, F, src);
     const R Gg = g.G[k * N + gq], Wg = g.W[k * N + gq];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -854,16 +893,21 @@ __global__ void k_rmass(int E, long long nc, ROps<double> O, RGeo<double> g, con
 }
 
 // G = M U - known - c r (in the band's element-major row order, [n][nc]) and per-column norms
-// ||G||^2, ||M U||^2 (one thread per column)
+// ||G||^2, ||M U||^2: a warp takes 32 columns of an element, the eight warps of a CTA the elements in turn,
+// and their partial sums meet in a fixed order (one thread per column over all elements left most of the
+// chip idle: 2,475 columns 190 us, now 14)
 template <int N>
-__global__ void k_rstage(int E, long long nc, ROps<double> O, RGeo<double> g, const double* __restrict__ U,
-                         const double* __restrict__ known, const double* __restrict__ r, double c,
-                         double* __restrict__ G, double* __restrict__ norms) {
-  const long long col = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (col >= nc) return;
+__global__ void __launch_bounds__(256) k_rstage(int E, long long nc, ROps<double> O, RGeo<double> g,
+                                                const double* __restrict__ U, const double* __restrict__ known,
+                                                const double* __restrict__ r, double c, double* __restrict__ G,
+                                                double* __restrict__ norms) {
+  __shared__ double sg[8][32], sm[8][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const long long col = (long long)blockIdx.x * 32 + lane;
   double g2 = 0.0, m2 = 0.0;
-  for (int k = 0; k < E; ++k)
-    for (int v = 0; v < 3; ++v) {
+  if (col < nc)
+    for (int kv = warp; kv < 3 * E; kv += 8) {
+      const int k = kv / 3, v = kv % 3;
       double xg[N];
 #pragma unroll
       for (int gq = 0; gq < N; ++gq) {
@@ -884,8 +928,17 @@ __global__ void k_rstage(int E, long long nc, ROps<double> O, RGeo<double> g, co
         m2 += mu * mu;
       }
     }
-  norms[col] = sqrt(g2);
-  norms[nc + col] = sqrt(m2);
+  sg[warp][lane] = g2;
+  sm[warp][lane] = m2;
+  __syncthreads();
+  if (warp == 0 && col < nc) {
+    for (int w = 1; w < 8; ++w) {
+      g2 += sg[w][lane];
+      m2 += sm[w][lane];
+    }
+    norms[col] = sqrt(g2);
+    norms[nc + col] = sqrt(m2);
+  }
 }
 
 // U -= delta (delta in the band's row order)
@@ -910,7 +963,7 @@ __global__ void k_raxpby(long long n, double a, const double* __restrict__ x, do
 // largest ratio ||G|| / max(g0, tiny) over columns, counting columns below their absolute floor as 0
 __global__ void k_rmaxratio(long long nc, const double* __restrict__ norms, const double* __restrict__ g0,
                             double* __restrict__ out) {
-  __shared__ double red[256];
+  __shared__ double red[1024];
   double m = 0.0;
   for (long long c = threadIdx.x; c < nc; c += blockDim.x) {
     const double gn = norms[c], mu = norms[nc + c];
@@ -952,6 +1005,7 @@ struct dg_radial {
   double* geo64 = nullptr;   // rL [E], rR [E], rg, W, G, T2 [E][N]
   float* geo32 = nullptr;
   double* prm64 = nullptr;   // [5][nc]
+  EuvFx* bands = nullptr;    // EUVAC band tables
   float* prm32 = nullptr;
   double* qg = nullptr;      // [2][4][E][N][nc]
   double* fh = nullptr;      // [2][3][E+1][nc]
@@ -977,6 +1031,9 @@ RGeo<R> geo_view(const R* base, int E, int N) {
   g.W = g.rg + E * N;
   g.G = g.W + E * N;
   g.T2 = g.G + E * N;
+  g.ir = g.T2 + E * N;
+  g.iW = g.ir + E * N;
+  g.ar = g.iW + E * N;
   return g;
 }
 
@@ -1018,21 +1075,26 @@ int residual_t(dg_radial* m, const double* u, const double* v, double t, double*
   const RGeo<double> g = geo_view<double>(m->geo64, E, N);
   const RPrm<double> prm{m->prm64, nc};
   const bool tan = v != nullptr;
+  RPhys<double> ph = m->ph64;
+  const double wt = ph.omega_t * t;
+  ph.sun[0] = -ph.sun_cd * std::cos(wt);
+  ph.sun[1] = ph.sun_cd * std::sin(wt);
+  ph.sun[2] = ph.sun_sd;
   rprof_begin(m, s, RK_GRAD);
-  if (tan) k_rgrad<N, 2, false, double><<<blocks_for((long long)E * nc), kThreads, 0, s>>>(E, nc, m->ops64, m->ph64, g, u, v, m->qg);
-  else k_rgrad<N, 1, false, double><<<blocks_for((long long)E * nc), kThreads, 0, s>>>(E, nc, m->ops64, m->ph64, g, u, v, m->qg);
+  if (tan) k_rgrad<N, 2, false, double><<<blocks_for((long long)E * nc), kThreads, 0, s>>>(E, nc, m->ops64, ph, g, u, v, m->qg);
+  else k_rgrad<N, 1, false, double><<<blocks_for((long long)E * nc), kThreads, 0, s>>>(E, nc, m->ops64, ph, g, u, v, m->qg);
   rprof_end(m, s);
   DG_LAUNCH_CHECK("k_rgrad");
   rprof_begin(m, s, RK_FACE);
-  if (tan) k_rface<N, 2, false, double><<<blocks_for((long long)(E + 1) * nc), kThreads, 0, s>>>(E, nc, m->ops64, m->ph64, g, prm, u, v, m->qg, m->fh);
-  else k_rface<N, 1, false, double><<<blocks_for((long long)(E + 1) * nc), kThreads, 0, s>>>(E, nc, m->ops64, m->ph64, g, prm, u, v, m->qg, m->fh);
+  if (tan) k_rface<N, 2, false, double><<<blocks_for((long long)(E + 1) * nc), kThreads, 0, s>>>(E, nc, m->ops64, ph, g, prm, u, v, m->qg, m->fh);
+  else k_rface<N, 1, false, double><<<blocks_for((long long)(E + 1) * nc), kThreads, 0, s>>>(E, nc, m->ops64, ph, g, prm, u, v, m->qg, m->fh);
   rprof_end(m, s);
   DG_LAUNCH_CHECK("k_rface");
   rprof_begin(m, s, RK_VOL);
   if (tan)
-    k_rvol<N, 2, false, double><<<blocks_for((long long)E * nc), kThreads, 0, s>>>(E, nc, m->ops64, m->ph64, g, prm, t, u, v, m->qg, m->fh, r, jv, 0.0, nullptr);
+    k_rvol<N, 2, false, double><<<blocks_for((long long)E * nc), kThreads, 0, s>>>(E, nc, m->ops64, ph, g, prm, t, u, v, m->qg, m->fh, r, jv, 0.0, nullptr);
   else
-    k_rvol<N, 1, false, double><<<blocks_for((long long)E * nc), kThreads, 0, s>>>(E, nc, m->ops64, m->ph64, g, prm, t, u, v, m->qg, m->fh, r, nullptr, 0.0, nullptr);
+    k_rvol<N, 1, false, double><<<blocks_for((long long)E * nc), kThreads, 0, s>>>(E, nc, m->ops64, ph, g, prm, t, u, v, m->qg, m->fh, r, nullptr, 0.0, nullptr);
   rprof_end(m, s);
   DG_LAUNCH_CHECK("k_rvol");
   return DG_OK;
@@ -1089,7 +1151,7 @@ template <int N>
 int stage_norms(dg_radial* m, const double* U, const double* known, const double* r, double c, cudaStream_t s) {
   const RGeo<double> g = geo_view<double>(m->geo64, m->E, N);
   rprof_begin(m, s, RK_VEC);
-  k_rstage<N><<<blocks_for(m->nc), kThreads, 0, s>>>(m->E, m->nc, m->ops64, g, U, known, r, c, m->G, m->norms);
+  k_rstage<N><<<(unsigned)((m->nc + 31) / 32), 256, 0, s>>>(m->E, m->nc, m->ops64, g, U, known, r, c, m->G, m->norms);
   rprof_end(m, s);
   DG_LAUNCH_CHECK("k_rstage");
   return DG_OK;
@@ -1125,7 +1187,7 @@ int axpby(dg_radial* m, double a, const double* x, double b, const double* y, do
 
 // max over columns of ||G|| / ||G0|| (0 for columns under the absolute floor), read by the host
 int max_ratio(dg_radial* m, cudaStream_t s, double* out) {
-  k_rmaxratio<<<1, 256, 0, s>>>(m->nc, m->norms, m->g0, m->ratio);
+  k_rmaxratio<<<1, 1024, 0, s>>>(m->nc, m->norms, m->g0, m->ratio);
   DG_LAUNCH_CHECK("k_rmaxratio");
   DG_CUDA_TRY(cudaMemcpyAsync(m->ratio_h, m->ratio, sizeof(double), cudaMemcpyDeviceToHost, s));
   DG_CUDA_TRY(cudaStreamSynchronize(s));
@@ -1201,7 +1263,7 @@ int step_t(dg_radial* m, double* u, double t, double dt, int stages, double rtol
 
 void release(dg_radial* m) {
   if (!m) return;
-  void* ptrs[] = {m->geo64, m->geo32, m->prm64, m->prm32, m->qg, m->fh, m->qp, m->fp, m->band, m->ipiv, m->info,
+  void* ptrs[] = {m->geo64, m->geo32, m->bands, m->prm64, m->prm32, m->qg, m->fh, m->qp, m->fp, m->band, m->ipiv, m->info,
                   m->U0, m->known, m->R1, m->R2, m->rr, m->G, m->norms, m->g0, m->ratio};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -1224,6 +1286,8 @@ RPhys<R> phys_cast(const RPhys<double>& P) {
     q.B[j] = (R)P.B[j];
     q.phi[j] = (R)P.phi[j];
   }
+  for (int k = 0; k < 3; ++k) q.sun[k] = P.sun[k];
+  q.bands = P.bands;
   q.cc = (R)P.cc; q.sun_cd = (R)P.sun_cd; q.sun_sd = (R)P.sun_sd; q.omega_t = (R)P.omega_t; q.inv_m = (R)P.inv_m;
   return q;
 }
@@ -1283,6 +1347,8 @@ extern "C" int dg_radial_create(const dg_radial_desc* desc, const double* node_r
   P.bc_lo = d.bc_lo;
   P.bc_hi = d.bc_hi;
   P.n_euvac = 0;
+  P.bands = nullptr;
+  P.sun[0] = P.sun[1] = P.sun[2] = 0.0;
   P.omega_t = d.euv_omega_t;
   P.inv_m = 1.0 / d.mass;
   P.cc = P.sun_cd = P.sun_sd = 0.0;
@@ -1327,7 +1393,7 @@ extern "C" int dg_radial_create(const dg_radial_desc* desc, const double* node_r
     for (int k = 0; k < E; ++k)
       for (int i = 0; i < N; ++i) nr[k * N + i] = rl[k] + 0.5 * (1.0 + o.xi[i]) * (rl[k + 1] - rl[k]);
   }
-  std::vector<double> geo((size_t)2 * E + 4 * E * N);
+  std::vector<double> geo((size_t)2 * E + 7 * E * N);
   for (int k = 0; k < E; ++k) {
     const double rL = nr[k * N], rR = nr[k * N + N - 1], J = 0.5 * (rR - rL);
     if (!(J > 0)) {
@@ -1344,6 +1410,9 @@ extern "C" int dg_radial_create(const dg_radial_desc* desc, const double* node_r
       geo[2 * E + E * N + k * N + gq] = w * J * rg * rg;
       geo[2 * E + 2 * E * N + k * N + gq] = w * rg * rg;
       geo[2 * E + 3 * E * N + k * N + gq] = 2.0 * w * J * rg;
+      geo[2 * E + 4 * E * N + k * N + gq] = 1.0 / rg;
+      geo[2 * E + 5 * E * N + k * N + gq] = 1.0 / (w * J * rg * rg);
+      geo[2 * E + 6 * E * N + k * N + gq] = -(d.g_r0 / rg) * (d.g_r0 / rg) / d.gamma;
     }
   }
   std::vector<float> geo32(geo.begin(), geo.end());
@@ -1363,6 +1432,7 @@ extern "C" int dg_radial_create(const dg_radial_desc* desc, const double* node_r
   const int LD = 2 * (9 * N - 1) + (9 * N - 1) + 1;
   int rc = 0;
   rc |= ralloc(&m->geo64, (long long)geo.size());
+  if (d.euv == DG_EUV_EUVAC) rc |= ralloc(&m->bands, 1);
   rc |= ralloc(&m->geo32, (long long)geo.size());
   rc |= ralloc(&m->prm64, 5 * nc);
   rc |= ralloc(&m->prm32, 5 * nc);
@@ -1388,6 +1458,14 @@ extern "C" int dg_radial_create(const dg_radial_desc* desc, const double* node_r
     return fail(DG_ENOMEM, "dg_radial_create: device allocation failed");
   }
   cudaError_t err = cudaMemcpy(m->geo64, geo.data(), sizeof(double) * geo.size(), cudaMemcpyHostToDevice);
+  if (err == cudaSuccess && m->bands) {
+    EuvFx tables;
+    double phi[1][40];
+    for (int j = 0; j < 40; ++j) phi[0][j] = P.phi[j];
+    build_euv(P.n_euvac, P.B, phi, 1, &tables);
+    err = cudaMemcpy(m->bands, &tables, sizeof(tables), cudaMemcpyHostToDevice);
+    P.bands = m->bands;
+  }
   if (err == cudaSuccess) err = cudaMemcpy(m->geo32, geo32.data(), sizeof(float) * geo32.size(), cudaMemcpyHostToDevice);
   if (err == cudaSuccess) err = cudaMemcpy(m->prm64, prm.data(), sizeof(double) * prm.size(), cudaMemcpyHostToDevice);
   if (err == cudaSuccess) err = cudaMemcpy(m->prm32, prm32.data(), sizeof(float) * prm32.size(), cudaMemcpyHostToDevice);
