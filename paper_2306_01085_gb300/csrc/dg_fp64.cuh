@@ -134,7 +134,7 @@ __device__ __forceinline__ void pass_b(const XOps<N>& so, const cell* in, cell* 
 // --------------------------------------------------------------------------------------------
 template <int N, bool FX>
 __device__ __forceinline__ void interp_body(const XOps<N>& so, const double (&x)[5], const int (&ex)[5], cell* b0,
-                                            cell* b1, int g, bool act, bool live, double* __restrict__ ug,
+                                            cell* b1, int g, bool act, bool live, int row, double* __restrict__ ug,
                                             double* __restrict__ uf) {
   constexpr int NP = Grp<N>::NP, NF = Grp<N>::NF, T = Grp<N>::T;
   if (act)
@@ -183,21 +183,23 @@ __device__ __forceinline__ void interp_body(const XOps<N>& so, const double (&x)
       }
     }
 #pragma unroll
-    for (int c = 0; c < 5; ++c) uf[(phi * 5 + c) * NF + f] = out[c];
+    for (int c = 0; c < 5; ++c) uf[(phi * row + c) * NF + f] = out[c];
   }
 }
 template <int N>
 __device__ __noinline__ void interp_slow(const XOps<N>& so, const double (&x)[5], const int (&ex)[5], cell* b0, cell* b1,
-                                         int g, bool act, bool live, double* ug, double* uf) {
-  interp_body<N, false>(so, x, ex, b0, b1, g, act, live, ug, uf);
+                                         int g, bool act, bool live, int row, double* ug, double* uf) {
+  interp_body<N, false>(so, x, ex, b0, b1, g, act, live, row, ug, uf);
 }
 
-// plane blockIdx.y: u -> value plane, v -> tangent plane of ug, uf (grid.y = 1: u alone)
-template <int N>
+// GRAD = false: plane blockIdx.y, u -> value plane, v -> tangent plane of ug, uf (grid.y = 1: u alone).
+// GRAD = true: a nodal gradient u [E][3][5][NP], direction blockIdx.y, to ug [E][3][5][NP], uf [E][6][15][NF].
+template <int N, bool GRAD>
 __global__ void __launch_bounds__(128) k_interp64(const double* __restrict__ u, const double* __restrict__ v,
                                                   long long E, const Ops* __restrict__ ops, double* __restrict__ ug,
                                                   double* __restrict__ uf) {
   constexpr int NP = Grp<N>::NP, NF = Grp<N>::NF, T = Grp<N>::T;
+  constexpr int ROW = GRAD ? 15 : 5;         // variables of an element's record
   __shared__ XOps<N> so;
   __shared__ int red[5 * 4];
   extern __shared__ __align__(16) cell cells[];
@@ -206,12 +208,13 @@ __global__ void __launch_bounds__(128) k_interp64(const double* __restrict__ u, 
   cell* b0 = cells + grp * 10 * NP;
   const long long e = (long long)blockIdx.x * (blockDim.x / T) + grp;
   const bool live = e < E, act = g < NP;
-  const double* in = blockIdx.y ? v : u;
+  const int c0 = GRAD ? 5 * blockIdx.y : 0;
+  const double* in = (!GRAD && blockIdx.y ? v : u) + (e * ROW + c0) * NP;
   double x[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
   int ex[5];
   if (live && act)
 #pragma unroll
-    for (int c = 0; c < 5; ++c) x[c] = in[(e * 5 + c) * NP + g];
+    for (int c = 0; c < 5; ++c) x[c] = in[c * NP + g];
 #pragma unroll
   for (int c = 0; c < 5; ++c) ex[c] = fx_mag(x[c]);
   grp_max<N, 5>(ex, red);
@@ -221,14 +224,185 @@ __global__ void __launch_bounds__(128) k_interp64(const double* __restrict__ u, 
     ok = ok && fx_ok(ex[c]);
     ex[c] = fx_exp(ex[c]);
   }
-  double* go = ug + (blockIdx.y ? E * 5 * NP : 0) + e * 5 * NP;
-  double* fo = uf + (blockIdx.y ? E * 30 * NF : 0) + e * 30 * NF;
+  const long long pl = !GRAD && blockIdx.y ? E : 0;
+  double* go = ug + ((pl + e) * ROW + c0) * NP;
+  double* fo = uf + ((pl + e) * 6 * ROW + c0) * NF;
   if (!grp_all<N>(ok)) {
-    interp_slow<N>(so, x, ex, b0, b0 + 5 * NP, g, act, live && !ok, go, fo);
+    interp_slow<N>(so, x, ex, b0, b0 + 5 * NP, g, act, live && !ok, ROW, go, fo);
     if constexpr (T >= 32) return;
     grp_sync<N>();                           // groups of this warp that passed take the fixed-point path
   }
-  interp_body<N, true>(so, x, ex, b0, b0 + 5 * NP, g, act, live && ok, go, fo);
+  interp_body<N, true>(so, x, ex, b0, b0 + 5 * NP, g, act, live && ok, ROW, go, fo);
+}
+
+// --------------------------------------------------------------------------------------------
+// products with the element mass matrix M = B^T W B and its inverse, and Gauss values -> nodal values
+// --------------------------------------------------------------------------------------------
+// Each is two or one sum-factorised transforms of the five variables (MODE 2: of one direction of the
+// gradient), bound by shared-memory loads and the integer pipe instead of the FP64 pipe (12,288 elements,
+// p = 2: mass 73 us, inverse 60 us with FP64 passes).
+enum { NODAL_MASS = 0, NODAL_MASS_INV = 1, NODAL_FROM_GAUSS = 2 };
+
+// one pass with an operator given by its fixed-point (cx) and FP64 (cd) coefficients
+template <int N, int DIR, bool TR, bool FX>
+__device__ __forceinline__ void pass_c(const cell* cx, const double* cd, const cell* in, cell* out, int g) {
+  constexpr int NP = N * N * N, ST = DIR == 0 ? 1 : DIR == 1 ? N : N * N;
+  const int i = (g / ST) % N, base = g - i * ST;
+  if constexpr (FX) {
+    fx a[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) a[k] = c_fx(cx[TR ? k * N + i : i * N + k]);
+#pragma unroll
+    for (int c = 0; c < 5; ++c) {
+      fxacc s = fx_zero<30>();
+#pragma unroll
+      for (int k = 0; k < N; ++k) fx_mac(s, a[k], c_fx(in[c * NP + base + k * ST]));
+      out[c * NP + g] = c_split<30>(fx_sum<30>(s));
+    }
+  } else {
+    for (int c = 0; c < 5; ++c) {
+      double s = 0.0;
+      for (int k = 0; k < N; ++k) s = fma(cd[TR ? k * N + i : i * N + k], c_d(in[c * NP + base + k * ST]), s);
+      out[c * NP + g] = c_of(s);
+    }
+  }
+}
+// three passes, from b0 into b1
+template <int N, bool TR, bool FX>
+__device__ __forceinline__ void transform(const cell* cx, const double* cd, cell* b0, cell* b1, int g, bool act) {
+  grp_sync<N>();
+  if (act) pass_c<N, 0, TR, FX>(cx, cd, b0, b1, g);
+  grp_sync<N>();
+  if (act) pass_c<N, 1, TR, FX>(cx, cd, b1, b0, g);
+  grp_sync<N>();
+  if (act) pass_c<N, 2, TR, FX>(cx, cd, b0, b1, g);
+  grp_sync<N>();
+}
+
+template <int N>
+struct NodalOps {
+  cell B[N * N], Bt[N * N], Binv[N * N];
+  double dB[N * N], dBt[N * N], dBinv[N * N], iw[N];
+};
+
+template <int N, int MODE>
+__device__ __noinline__ void nodal_slow(const NodalOps<N>& so, double (&x)[5], double factor, cell* b0, cell* b1, int g,
+                                        bool act) {
+  constexpr int NP = N * N * N;
+  auto put = [&](double f) {
+    if (act)
+      for (int c = 0; c < 5; ++c) b0[c * NP + g] = c_of(x[c] * f);
+  };
+  auto get = [&]() {
+    if (act)
+      for (int c = 0; c < 5; ++c) x[c] = c_d(b1[c * NP + g]);
+  };
+  put(1.0);
+  if constexpr (MODE == NODAL_MASS) transform<N, false, false>(nullptr, so.dB, b0, b1, g, act);
+  if constexpr (MODE == NODAL_MASS_INV) transform<N, true, false>(nullptr, so.dBinv, b0, b1, g, act);
+  if constexpr (MODE != NODAL_FROM_GAUSS) {
+    get();
+    put(factor);
+  }
+  if constexpr (MODE == NODAL_MASS) transform<N, true, false>(nullptr, so.dBt, b0, b1, g, act);
+  else transform<N, false, false>(nullptr, so.dBinv, b0, b1, g, act);
+  get();
+}
+
+// in and out [E][ROW][NP] (they may be the same array); NODAL_FROM_GAUSS: direction blockIdx.y of [E][3][5][NP]
+template <int N, int MODE>
+__global__ void __launch_bounds__(128) k_nodal64(long long E, const Ops* __restrict__ ops, const double* in_g,
+                                                 double* out_g, const double* __restrict__ gu) {
+  constexpr int NP = Grp<N>::NP, T = Grp<N>::T;
+  constexpr int ROW = MODE == NODAL_FROM_GAUSS ? 15 : 5;
+  __shared__ NodalOps<N> so;
+  __shared__ int red[6 * 4];
+  extern __shared__ __align__(16) cell cells[];
+  for (int i = threadIdx.x; i < N * N; i += blockDim.x) {
+    so.B[i] = c_of(fx{ops->xB[i].x, ops->xB[i].y});
+    so.Bt[i] = c_of(fx{ops->xBt[i].x, ops->xBt[i].y});
+    so.Binv[i] = c_of(fx{ops->xBinv[i].x, ops->xBinv[i].y});
+    so.dB[i] = ops->B[i];
+    so.dBt[i] = ops->Bt[i];
+    so.dBinv[i] = ops->Binv[i];
+  }
+  for (int i = threadIdx.x; i < N; i += blockDim.x) so.iw[i] = ops->iw[i];
+  __syncthreads();
+  const int grp = threadIdx.x / T, g = threadIdx.x % T;
+  cell *b0 = cells + grp * 10 * NP, *b1 = b0 + 5 * NP;
+  const long long e = (long long)blockIdx.x * (blockDim.x / T) + grp;
+  const bool live = e < E, act = g < NP;
+  const long long at = (e * ROW + (MODE == NODAL_FROM_GAUSS ? 5 * blockIdx.y : 0)) * NP + g;
+  double x[5] = {0.0, 0.0, 0.0, 0.0, 0.0}, factor = 1.0;
+  int mx[6] = {0, 0, 0, 0, 0, 0};
+  if (live && act) {
+#pragma unroll
+    for (int c = 0; c < 5; ++c) {
+      x[c] = in_g[at + c * NP];
+      mx[c] = fx_mag(x[c]);
+    }
+    if constexpr (MODE == NODAL_MASS) factor = gu[e * 11 * NP + 9 * NP + g];
+    if constexpr (MODE == NODAL_MASS_INV)
+      factor = gu[e * 11 * NP + 10 * NP + g] * (so.iw[g % N] * so.iw[(g / N) % N] * so.iw[g / (N * N)]);
+    mx[5] = fx_mag(factor);
+  }
+  grp_max<N, 6>(mx, red);
+  bool ok = true;
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+    ok = ok && fx_ok(mx[c]);
+    mx[c] = fx_exp(mx[c]);
+  }
+#pragma unroll
+  for (int c = 0; c < 5; ++c) ok = ok && mx[c] + mx[5] >= 1300 && mx[c] + mx[5] <= 2900;
+  const bool slow = live && !ok;
+  if (!grp_all<N>(ok)) {
+    nodal_slow<N, MODE>(so, x, factor, b0, b1, g, act && slow);
+    if (act && slow)
+#pragma unroll
+      for (int c = 0; c < 5; ++c) out_g[at + c * NP] = x[c];
+    if constexpr (T >= 32) return;
+    grp_sync<N>();
+  }
+  // data bits: the passes grow values by the operators' sums (B 2.7, Bt 2.4, Binv^T 16.1, Binv 36.7 for
+  // three passes), and the splits hold 61 bits
+  constexpr int BITS = MODE == NODAL_MASS ? 57 : MODE == NODAL_MASS_INV ? 56 : 55;
+  int sh[5];                                 // exponent of a unit
+#pragma unroll
+  for (int c = 0; c < 5; ++c) {
+    sh[c] = mx[c] - BITS - 1022;
+    if (act) b0[c * NP + g] = c_split<30>(fx_from<BITS>(x[c], mx[c]));
+  }
+  if constexpr (MODE == NODAL_MASS) transform<N, false, true>(so.B, nullptr, b0, b1, g, act);
+  if constexpr (MODE == NODAL_MASS_INV) transform<N, true, true>(so.Binv, nullptr, b0, b1, g, act);
+  if constexpr (MODE != NODAL_FROM_GAUSS) {
+    const fx f = fx_split<27>(fx_from<57>(factor, mx[5]));
+    long long y[5] = {0, 0, 0, 0, 0};
+    int up[5] = {0, 0, 0, 0, 0};
+#pragma unroll
+    for (int c = 0; c < 5; ++c) {
+      if (act) y[c] = fx_mul<30>(f, c_fx(b1[c * NP + g]));
+      sh[c] += mx[5] - 1022;
+      if constexpr (MODE == NODAL_MASS_INV) up[c] = 64 - __clzll(y[c] < 0 ? -y[c] : y[c]);
+    }
+    if constexpr (MODE == NODAL_MASS_INV) {
+      grp_max<N, 5>(up, red);
+#pragma unroll
+      for (int c = 0; c < 5; ++c) {          // to 55 bits
+        const int d = up[c] ? up[c] - 55 : 0;
+        sh[c] += d;
+        y[c] = d >= 0 ? (y[c] + (d ? 1LL << (d - 1) : 0LL)) >> d : y[c] << -d;
+      }
+    }
+    if (act)
+#pragma unroll
+      for (int c = 0; c < 5; ++c) b0[c * NP + g] = c_split<30>(y[c]);
+  }
+  if constexpr (MODE == NODAL_MASS) transform<N, true, true>(so.Bt, nullptr, b0, b1, g, act);
+  else transform<N, false, true>(so.Binv, nullptr, b0, b1, g, act);
+  if (act && live && ok)
+#pragma unroll
+    for (int c = 0; c < 5; ++c) out_g[at + c * NP] = fx_to_double(fx_join<30>(c_fx(b1[c * NP + g])), sh[c]);
 }
 
 // --------------------------------------------------------------------------------------------
@@ -809,7 +983,7 @@ __global__ void __launch_bounds__(128, NC == 2 ? 3 : 4)
 #pragma unroll
   for (int k = 0; k < NC * 5; ++k) mx[k] = 0;
   auto expo = [](int mag) { return mag == 0 ? 0 : fx_ok(mag) ? mag >> 20 : BAD; };
-  int eG[3] = {0, 0, 0}, eF[NC][3];          // this point's exponents: geometry rows, flux groups
+  int eG[3] = {0, 0, 0}, eF[NC][3] = {};          // this point's exponents: geometry rows, flux groups
   if (live && act) {
     S F[12], src[5];
     volume_load<N, NC, S>(e, E, g, P, sun, gu, accg, xg, ug, qg, mixg, inv_stage_c, F, src);
@@ -861,13 +1035,14 @@ __global__ void __launch_bounds__(128, NC == 2 ? 3 : 4)
         mx[PL * 5 + c] = ec;
       }
     };
-    contract(std::integral_constant<int, 0>{});
+    if (NC == 1 || r) contract(std::integral_constant<int, 0>{});
     if constexpr (NC == 2) contract(std::integral_constant<int, 1>{});
     if (bad) mx[0] = BAD;
   }
   const double* fhe = fh + e * 30 * NF;
+  const int pl0 = NC == 2 && !r ? 1 : 0;     // the tangent alone when r is not wanted
   if (live)
-    for (int pl = 0; pl < NC; ++pl)
+    for (int pl = pl0; pl < NC; ++pl)
       for (int idx = g; idx < 6 * NF; idx += T) {
         const int phi = idx / NF, f = idx % NF;
 #pragma unroll
@@ -896,7 +1071,7 @@ __global__ void __launch_bounds__(128, NC == 2 ? 3 : 4)
   live = live && ok;
   const int ig[3] = {g % N, (g / N) % N, g / (N * N)};
 #pragma unroll 1
-  for (int pl = 0; pl < NC; ++pl) {
+  for (int pl = pl0; pl < NC; ++pl) {
     int ef[5];
 #pragma unroll
     for (int c = 0; c < 5; ++c) ef[c] = pl == 0 ? mx[c] : mx[NC * 5 - 5 + c];

@@ -46,9 +46,9 @@ struct Ops {
   double xi[MAXN];           // GLL nodes
   // with the weights folded in (dg_fx.cuh): Dh[k][i] = D[k][i] w_k / w_i, eh[side][i] = e[i] / w_i,
   // Bt[q][a] = B[q][a] w_q
-  double Dh[MAXN * MAXN], eh[2][MAXN], Bt[MAXN * MAXN];
-  // fixed-point coefficients: B and Bt with exponent FX_T_B, -Dh and eh with FX_T_D, eL / eR with FX_T_E
-  int2 xB[MAXN * MAXN], xBt[MAXN * MAXN], xDn[MAXN * MAXN], xlift[2][MAXN], xend[2][MAXN];
+  double Dh[MAXN * MAXN], eh[2][MAXN], Bt[MAXN * MAXN], iw[MAXN];   // iw = 1 / w
+  // fixed-point coefficients: B, Bt and Binv with exponent FX_T_B, -Dh and eh with FX_T_D, eL / eR with FX_T_E
+  int2 xB[MAXN * MAXN], xBt[MAXN * MAXN], xBinv[MAXN * MAXN], xDn[MAXN * MAXN], xlift[2][MAXN], xend[2][MAXN];
 };
 void build_ops(int n, Ops* ops);   // host, defined in dg_ops.cu
 // the operators before rounding (end-point rows e[0] at -1, e[1] at +1)

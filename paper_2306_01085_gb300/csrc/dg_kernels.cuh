@@ -787,71 +787,54 @@ k_volume(long long E, const Ops* __restrict__ ops, PhysT<R> P, R t,
 namespace dg {
 
 // --------------------------------------------------------------------------------------------
-// tensor transforms of nodal q and the mass matrix
+// FP32 mass product
 // --------------------------------------------------------------------------------------------
-// out = A x A x A in (T: A^T) for C components of EPB elements per CTA (one thread per point of
-// each element), optional W-weighting and back-transform (mass matrix), optional face traces.
-// Arithmetic in R (FP32 for the mass columns of FP32-assembled blocks); input and output FP64.
-template <int N, bool T, int C, typename R = double>
-__global__ void k_tensor(long long E, const Ops* __restrict__ ops, int which, const double* __restrict__ in_g,
-                         double* __restrict__ out_g, const R* __restrict__ weight,
-                         double* __restrict__ traces) {
-  constexpr int NP = Shape<N>::NP, NF = Shape<N>::NF, EPB = Epb<N, 1>::value;
-  __shared__ SmemOpsT<R> so;
+// FP32 mass product of EPB elements per CTA (one thread per point of each element): out = B^T W B in for the
+// five variables, FP32 arithmetic, input and output FP64 (the mass columns of FP32-assembled blocks)
+template <int N>
+__global__ void k_mass32(long long E, const Ops* __restrict__ ops, const double* __restrict__ in_g,
+                         double* __restrict__ out_g, const float* __restrict__ weight) {
+  constexpr int NP = Shape<N>::NP, EPB = Epb<N, 1>::value, C = 5;
+  __shared__ SmemOpsT<float> so;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  R* b0 = reinterpret_cast<R*>(smem_raw);   // [EPB][C][NP]
-  R* b1 = b0 + EPB * C * NP;                // [EPB][C][NP]
-  load_ops<N, R>(ops, so);
+  float* b0 = reinterpret_cast<float*>(smem_raw);   // [EPB][C][NP]
+  float* b1 = b0 + EPB * C * NP;                    // [EPB][C][NP]
+  load_ops<N, float>(ops, so);
   const long long e0 = (long long)blockIdx.x * EPB;
   for (int idx = threadIdx.x; idx < EPB * C * NP; idx += blockDim.x) {
     const long long e = e0 + idx / (C * NP);
-    if (e < E) b0[idx] = (R)in_g[e0 * C * NP + idx];
+    if (e < E) b0[idx] = (float)in_g[e0 * C * NP + idx];
   }
   __syncthreads();
   const int el = threadIdx.x / NP, g = threadIdx.x % NP;
   const bool active = el < EPB && (e0 + el) < E;
-  const R* A = (which == 0) ? so.B : so.Binv;
-  R* in = b0;
-  R* out = b1;
+  float* in = b0;
+  float* out = b1;
   for (int dir = 0; dir < 3; ++dir) {
     if (active)
-      for (int c = 0; c < C; ++c) out[(el * C + c) * NP + g] = line<N, T>(A, in + (el * C + c) * NP, g, dir);
+      for (int c = 0; c < C; ++c) out[(el * C + c) * NP + g] = line<N, false>(so.B, in + (el * C + c) * NP, g, dir);
     __syncthreads();
-    R* tt = in;
+    float* tt = in;
     in = out;
     out = tt;
   }
-  if (weight) {
-    // mass matrix: W-weighted Gauss values, then back with B^T
-    if (active) {
-      const R wd = weight[(e0 + el) * 10 * NP + 9 * NP + g];
-      for (int c = 0; c < C; ++c) in[(el * C + c) * NP + g] *= wd;
-    }
+  // W-weighted Gauss values, then back with B^T
+  if (active) {
+    const float wd = weight[(e0 + el) * 10 * NP + 9 * NP + g];
+    for (int c = 0; c < C; ++c) in[(el * C + c) * NP + g] *= wd;
+  }
+  __syncthreads();
+  for (int dir = 0; dir < 3; ++dir) {
+    if (active)
+      for (int c = 0; c < C; ++c) out[(el * C + c) * NP + g] = line<N, true>(so.B, in + (el * C + c) * NP, g, dir);
     __syncthreads();
-    for (int dir = 0; dir < 3; ++dir) {
-      if (active)
-        for (int c = 0; c < C; ++c) out[(el * C + c) * NP + g] = line<N, true>(A, in + (el * C + c) * NP, g, dir);
-      __syncthreads();
-      R* tt = in;
-      in = out;
-      out = tt;
-    }
+    float* tt = in;
+    in = out;
+    out = tt;
   }
   for (int idx = threadIdx.x; idx < EPB * C * NP; idx += blockDim.x) {
     const long long e = e0 + idx / (C * NP);
     if (e < E) out_g[e0 * C * NP + idx] = (double)in[idx];
-  }
-  if (traces) {
-    for (int idx = threadIdx.x; idx < EPB * 6 * C * NF; idx += blockDim.x) {
-      const int l = idx / (6 * C * NF), rem = idx % (6 * C * NF);
-      const long long e = e0 + l;
-      if (e >= E) continue;
-      const int phi = rem / (C * NF), c = (rem / NF) % C, f = rem % NF;
-      const R* ev = (phi & 1) ? so.eR : so.eL;
-      R acc = R(0);
-      for (int k = 0; k < N; ++k) acc = fma(ev[k], in[(l * C + c) * NP + face_vol_point<N>(phi, f, k)], acc);
-      traces[e * 6 * C * NF + rem] = (double)acc;
-    }
   }
 }
 
@@ -914,54 +897,6 @@ __global__ void k_mixture(long long E, const Ops* __restrict__ ops, Phys P, cons
     mixture_at(P, x, o);
     mixf[((e * 6 + phi) * 2) * NF + f] = o[0];
     mixf[((e * 6 + phi) * 2 + 1) * NF + f] = o[4];
-  }
-}
-
-// M^{-1} v = B^{-1} (w |J|)^{-1} B^{-T} v for the 5 variables of EPB elements per CTA (the nodal
-// mass matrix is B^T W B with B the square GLL-to-Gauss interpolation); in place allowed
-template <int N>
-__global__ void k_mass_inv(long long E, const Ops* __restrict__ ops, const double* in_g, double* out_g,
-                           const double* __restrict__ geo) {
-  constexpr int NP = Shape<N>::NP, EPB = Epb<N, 1>::value, C = 5;
-  __shared__ SmemOps so;
-  extern __shared__ double smem[];
-  double* b0 = smem;                 // [EPB][C][NP]
-  double* b1 = smem + EPB * C * NP;  // [EPB][C][NP]
-  load_ops<N, double>(ops, so);
-  const long long e0 = (long long)blockIdx.x * EPB;
-  for (int idx = threadIdx.x; idx < EPB * C * NP; idx += blockDim.x) {
-    const long long e = e0 + idx / (C * NP);
-    if (e < E) b0[idx] = in_g[e0 * C * NP + idx];
-  }
-  __syncthreads();
-  const int el = threadIdx.x / NP, g = threadIdx.x % NP;
-  const bool active = el < EPB && (e0 + el) < E;
-  double* in = b0;
-  double* out = b1;
-  for (int dir = 0; dir < 3; ++dir) {   // B^{-T}
-    if (active)
-      for (int c = 0; c < C; ++c) out[(el * C + c) * NP + g] = line<N, true>(so.Binv, in + (el * C + c) * NP, g, dir);
-    __syncthreads();
-    double* tt = in;
-    in = out;
-    out = tt;
-  }
-  if (active) {
-    const double iw = 1.0 / geo[(e0 + el) * 10 * NP + 9 * NP + g];
-    for (int c = 0; c < C; ++c) in[(el * C + c) * NP + g] *= iw;
-  }
-  __syncthreads();
-  for (int dir = 0; dir < 3; ++dir) {   // B^{-1}
-    if (active)
-      for (int c = 0; c < C; ++c) out[(el * C + c) * NP + g] = line<N, false>(so.Binv, in + (el * C + c) * NP, g, dir);
-    __syncthreads();
-    double* tt = in;
-    in = out;
-    out = tt;
-  }
-  for (int idx = threadIdx.x; idx < EPB * C * NP; idx += blockDim.x) {
-    const long long e = e0 + idx / (C * NP);
-    if (e < E) out_g[e0 * C * NP + idx] = in[idx];
   }
 }
 
@@ -1116,10 +1051,10 @@ static int launch_interp64(dg_mesh* m, const double* u, const double* v, int fir
   using G = Grp<N>;
   const int threads = threads64<N>(m->E * (v ? 2 : 1)), per = threads / G::T;
   const size_t sm = sizeof(cell) * 10 * G::NP * per;
-  int rc = set_smem(k_interp64<N>, sm);
+  int rc = set_smem(k_interp64<N, false>, sm);
   if (rc) return rc;
   prof_begin(m, s, KK_INTERP);
-  k_interp64<N><<<dim3((unsigned)((m->E + per - 1) / per), v ? 2 : 1), threads, sm, s>>>(
+  k_interp64<N, false><<<dim3((unsigned)((m->E + per - 1) / per), v ? 2 : 1), threads, sm, s>>>(
       u, v, m->E, m->d_ops, m->ws.ug + first * m->E * 5 * G::NP, m->ws.uf + first * m->E * 30 * G::NF);
   prof_end(m, s);
   DG_LAUNCH_CHECK("k_interp64");
@@ -1399,33 +1334,38 @@ int Driver<N>::eval_cm(dg_mesh* m, const double* u, const double* v, double t, d
   }
 }
 
-template <int N>
-int Driver<N>::q_to_nodal(dg_mesh* m, double* q, cudaStream_t s) {
-  constexpr int NP = Shape<N>::NP;
-  constexpr int EPB = Epb<N, 1>::value;
-  const size_t sm = sizeof(double) * 2 * EPB * 15 * NP;
-  int rc = set_smem(k_tensor<N, false, 15, double>, sm);
+template <int N, int MODE>
+static int run_nodal(dg_mesh* m, const double* in, double* out, cudaStream_t s) {
+  using G = Grp<N>;
+  constexpr int planes = MODE == NODAL_FROM_GAUSS ? 3 : 1;
+  const int threads = threads64<N>(m->E * planes), per = threads / G::T;
+  const size_t sm = sizeof(cell) * 10 * G::NP * per;
+  int rc = set_smem(k_nodal64<N, MODE>, sm);
   if (rc) return rc;
   prof_begin(m, s, KK_TENSOR);
-  k_tensor<N, false, 15, double><<<(unsigned)((m->E + EPB - 1) / EPB), EPB * NP, sm, s>>>(m->E, m->d_ops, 1, m->ws.qg, q,
-                                                                                   nullptr, nullptr);
+  k_nodal64<N, MODE><<<dim3((unsigned)((m->E + per - 1) / per), planes), threads, sm, s>>>(m->E, m->d_ops, in, out, m->gu);
   prof_end(m, s);
-  DG_LAUNCH_CHECK("k_tensor(q nodal)");
+  DG_LAUNCH_CHECK("k_nodal64");
   return DG_OK;
 }
 
 template <int N>
+int Driver<N>::q_to_nodal(dg_mesh* m, double* q, cudaStream_t s) {
+  return run_nodal<N, NODAL_FROM_GAUSS>(m, m->ws.qg, q, s);
+}
+
+template <int N>
 int Driver<N>::q_from_nodal(dg_mesh* m, const double* q, cudaStream_t s) {
-  constexpr int NP = Shape<N>::NP;
-  constexpr int EPB = Epb<N, 1>::value;
-  const size_t sm = sizeof(double) * 2 * EPB * 15 * NP;
-  int rc = set_smem(k_tensor<N, false, 15, double>, sm);
+  using G = Grp<N>;
+  const int threads = threads64<N>(m->E * 3), per = threads / G::T;
+  const size_t sm = sizeof(cell) * 10 * G::NP * per;
+  int rc = set_smem(k_interp64<N, true>, sm);
   if (rc) return rc;
   prof_begin(m, s, KK_TENSOR);
-  k_tensor<N, false, 15, double><<<(unsigned)((m->E + EPB - 1) / EPB), EPB * NP, sm, s>>>(m->E, m->d_ops, 0, q, m->ws.qg,
-                                                                                   nullptr, m->ws.qf);
+  k_interp64<N, true><<<dim3((unsigned)((m->E + per - 1) / per), 3), threads, sm, s>>>(q, nullptr, m->E, m->d_ops,
+                                                                                     m->ws.qg, m->ws.qf);
   prof_end(m, s);
-  DG_LAUNCH_CHECK("k_tensor(q gauss)");
+  DG_LAUNCH_CHECK("k_interp64(q)");
   return DG_OK;
 }
 
@@ -1438,40 +1378,23 @@ int Driver<N>::mixture(dg_mesh* m) {
 
 template <int N>
 int Driver<N>::mass_inv(dg_mesh* m, const double* v, double* mv, cudaStream_t s) {
-  constexpr int NP = Shape<N>::NP;
-  constexpr int EPB = Epb<N, 1>::value;
-  const size_t sm = sizeof(double) * 2 * EPB * 5 * NP;
-  int rc = set_smem(k_mass_inv<N>, sm);
-  if (rc) return rc;
-  prof_begin(m, s, KK_TENSOR);
-  k_mass_inv<N><<<(unsigned)((m->E + EPB - 1) / EPB), EPB * NP, sm, s>>>(m->E, m->d_ops, v, mv, m->geo);
-  prof_end(m, s);
-  DG_LAUNCH_CHECK("k_mass_inv");
-  return DG_OK;
+  return run_nodal<N, NODAL_MASS_INV>(m, v, mv, s);
 }
 
 template <int N>
 int Driver<N>::mass(dg_mesh* m, const double* v, double* mv, cudaStream_t s, bool f32) {
+  if (!f32) return run_nodal<N, NODAL_MASS>(m, v, mv, s);
   constexpr int NP = Shape<N>::NP;
   constexpr int EPB = Epb<N, 1>::value;
-  const unsigned grid = (unsigned)((m->E + EPB - 1) / EPB);
-  int rc;
-  if (f32) {   // FP32 arithmetic on the FP32 geometry (ensure_f32 has run)
-    if (!m->w32.geo) return fail(DG_EINVAL, "FP32 mass apply without the FP32 geometry");
-    const size_t sm = sizeof(float) * 2 * EPB * 5 * NP;
-    rc = set_smem(k_tensor<N, false, 5, float>, sm);
-    if (rc) return rc;
-    prof_begin(m, s, KK_TENSOR);
-    k_tensor<N, false, 5, float><<<grid, EPB * NP, sm, s>>>(m->E, m->d_ops, 0, v, mv, m->w32.geo, nullptr);
-  } else {
-    const size_t sm = sizeof(double) * 2 * EPB * 5 * NP;
-    rc = set_smem(k_tensor<N, false, 5, double>, sm);
-    if (rc) return rc;
-    prof_begin(m, s, KK_TENSOR);
-    k_tensor<N, false, 5, double><<<grid, EPB * NP, sm, s>>>(m->E, m->d_ops, 0, v, mv, m->geo, nullptr);
-  }
+  // FP32 arithmetic on the FP32 geometry (ensure_f32 has run)
+  if (!m->w32.geo) return fail(DG_EINVAL, "FP32 mass apply without the FP32 geometry");
+  const size_t sm = sizeof(float) * 2 * EPB * 5 * NP;
+  int rc = set_smem(k_mass32<N>, sm);
+  if (rc) return rc;
+  prof_begin(m, s, KK_TENSOR);
+  k_mass32<N><<<(unsigned)((m->E + EPB - 1) / EPB), EPB * NP, sm, s>>>(m->E, m->d_ops, v, mv, m->w32.geo);
   prof_end(m, s);
-  DG_LAUNCH_CHECK("k_tensor(mass)");
+  DG_LAUNCH_CHECK("k_mass32");
   return DG_OK;
 }
 

@@ -124,6 +124,7 @@ void build_ops(int n, Ops* o) {
   for (int k = 0; k < n; ++k) {
     o->eta[k] = (double)L.eta[k];
     o->w[k] = (double)L.w[k];
+    o->iw[k] = (double)(1.0L / L.w[k]);
     o->xi[k] = (double)L.xi[k];
     o->eL[k] = (double)L.e[0][k];
     o->eR[k] = (double)L.e[1][k];
@@ -139,6 +140,7 @@ void build_ops(int n, Ops* o) {
       o->Bt[i] = (double)Bt;
       o->xB[i] = fx_coef(L.B[i], FX_T_B, 27);
       o->xBt[i] = fx_coef(Bt, FX_T_B, 27);
+      o->xBinv[i] = fx_coef(L.Binv[i], FX_T_B, 27);
       o->xDn[i] = fx_coef(-Dh, FX_T_D, 29);
     }
   for (int side = 0; side < 2; ++side)

@@ -80,3 +80,33 @@ def test_range_check_hands_an_element_to_the_fp64_twin(torch_cuda, p):
     for got, want in ((r, r_ref), (jv, jv_ref)):
         err = np.abs(got - want).max(axis=(0, 2)) / np.abs(want).max(axis=(0, 2))
         assert np.all(err <= 1e-12), err
+
+
+@pytest.mark.parametrize("p", [1, 2, 3, 4])
+def test_mass_products_scale_exactly_and_invert(torch_cuda, p):
+    """M v and M^-1 v on a shell (an odd number of elements): exact under powers of two inside the
+    fixed-point range, equal to FP64 rounding outside it (the FP64 twin), a NaN node confined to its
+    element, and M^-1 M v = v to 1e-12 of the largest entry."""
+    torch = torch_cuda
+    from paper_2306_01085_gb300.dg import Mesh
+    m = Mesh(W.shell_desc(n=1, nr=7, p=p))
+    v = torch.from_numpy(W.normal(8, m.n_dof).reshape(m.u_shape)).cuda()
+    v[3, 1] = 0.0
+    for op in (m.mass, m.mass_inverse):
+        ref = op(v)
+        for k in (-200, 9, 200):
+            assert torch.equal(op(v * 2.0 ** k), ref * 2.0 ** k), k
+        far = op(v * 2.0 ** 900) * 2.0 ** -900
+        assert float(((far - ref).abs().amax((1, 2)) / ref.abs().amax((1, 2))).max()) < 1e-13
+        w = v.clone()
+        w[5, 2, 0] = float("nan")
+        got = op(w)
+        assert bool(torch.isnan(got[5, 2]).all())
+        keep = torch.arange(m.n_elem, device="cuda") != 5
+        assert torch.equal(got[keep], ref[keep])
+    back = m.mass_inverse(m.mass(v))
+    assert float((back - v).abs().max() / v.abs().max()) < 1e-12
+    alias = m.mass(v)
+    m.mass_inverse(alias, out=alias)
+    assert torch.equal(alias, back)
+    m.close()
