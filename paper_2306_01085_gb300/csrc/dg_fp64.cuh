@@ -466,17 +466,12 @@ __device__ __noinline__ void grad_slow(const XOps<N>& so, const double* gu, cell
 
 // plane plane0 + blockIdx.y of qg, qf from the same plane of ug, uf (0: value, 1: tangent). The wall
 // trace of the tangent reads the value plane's varrho trace.
-// BLK (the tangent of block-diagonal probes): the tangent's u_hat keeps only the element's own half on
-// interior faces, and qx receives per face the trace of the gradient tangent this element would get
-// from its neighbour's perturbation across that face: kn(f) u_dot_nb(f), kn = kappa (w n dS) / 2 with
-// kappa(f) = sum_k e_face[k]^2 / (w |J|)(g(f, k)), a property of the mesh (k_cross_kappa).
-template <int N, bool BLK>
+template <int N>
 __global__ void __launch_bounds__(128, 5) k_grad64(long long E, const Ops* __restrict__ ops, double t_wall, int plane0,
                                                 const double* __restrict__ gu, const double* __restrict__ fgu,
-                                                const double* __restrict__ kn, const int* __restrict__ nbr,
-                                                const int* __restrict__ nbr_fo, const double* __restrict__ ug,
-                                                const double* __restrict__ uf, double* __restrict__ qg,
-                                                double* __restrict__ qf, double* __restrict__ qx) {
+                                                const int* __restrict__ nbr, const int* __restrict__ nbr_fo,
+                                                const double* __restrict__ ug, const double* __restrict__ uf,
+                                                double* __restrict__ qg, double* __restrict__ qf) {
   using C = GradCells<N>;
   constexpr int NP = Grp<N>::NP, NF = Grp<N>::NF, T = Grp<N>::T, NI = Grp<N>::NI, SH = C::SH;
   __shared__ XOps<N> so;
@@ -530,31 +525,12 @@ __global__ void __launch_bounds__(128, 5) k_grad64(long long E, const Ops* __res
       double oth[5];
 #pragma unroll
       for (int c = 0; c < 5; ++c) oth[c] = ufp[nbase + c * NF];
-      if (BLK && plane == 1) {
 #pragma unroll
-        for (int c = 0; c < 5; ++c) uh[c] = 0.5 * uh[c];
-        double* xo = qx + (e * 6 + phi) * 15 * NF + f;
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-          const double k = kn[((e * 6 + phi) * 3 + d) * NF + f];
-#pragma unroll
-          for (int c = 0; c < 5; ++c) xo[(d * 5 + c) * NF] = k * oth[c];
-        }
-      } else {
-#pragma unroll
-        for (int c = 0; c < 5; ++c) uh[c] = 0.5 * (uh[c] + oth[c]);
-      }
-    } else {
-      if (nb == -DG_BC_WALL) {
-        const double sr = exp_fast(0.5 * uf[fbase]);   // the value plane's varrho trace
-        uh[1] = uh[2] = uh[3] = 0.0;
-        uh[4] = plane == 0 ? sr * t_wall : 0.5 * sr * t_wall * uh[0];
-      }
-      if (BLK && plane == 1) {
-        double* xo = qx + (e * 6 + phi) * 15 * NF + f;
-#pragma unroll
-        for (int k = 0; k < 15; ++k) xo[k * NF] = 0.0;
-      }
+      for (int c = 0; c < 5; ++c) uh[c] = 0.5 * (uh[c] + oth[c]);
+    } else if (nb == -DG_BC_WALL) {
+      const double sr = exp_fast(0.5 * uf[fbase]);   // the value plane's varrho trace
+      uh[1] = uh[2] = uh[3] = 0.0;
+      uh[4] = plane == 0 ? sr * t_wall : 0.5 * sr * t_wall * uh[0];
     }
 #pragma unroll
     for (int c = 0; c < 5; ++c) {
@@ -673,7 +649,8 @@ __global__ void __launch_bounds__(128, 5) k_grad64(long long E, const Ops* __res
   }
 }
 
-// kn[e][phi][d][f] = kappa(f) (w n_d dS)(f) / 2 (see k_grad64)
+// The gradient trace that an element gets at a face from its neighbour's perturbation alone is
+// kn(f) u_dot_nb(f): kn = kappa (w n dS) / 2 with kappa(f) = sum_k e_face[k]^2 / (w |J|)(g(f, k)).
 template <int N>
 __global__ void k_cross_kappa(long long E, const Ops* __restrict__ ops, const double* __restrict__ geo,
                               const double* __restrict__ fgeo, double* __restrict__ kn) {
@@ -694,16 +671,13 @@ __global__ void k_cross_kappa(long long E, const Ops* __restrict__ ops, const do
 // --------------------------------------------------------------------------------------------
 // F_hat . n = (F(u, q) + F(u2, q2)) . n / 2 + sigma(u_hat) (u - u_hat) |n| inside,
 // F(u_b, q) . n + sigma(u_b) (u - u_b) |n| at a wall, F_inviscid(u) . n at an outflow face.
-// BLK (NC = 2): the tangent is evaluated for each side's diagonal block: one side carries its
-// perturbation, the other only the gradient tangent it receives from it across this face (qx of the other
-// element). The flux is linear in the gradient, so that part needs no second evaluation of the state.
-template <int N, int NC, bool BLK>
+template <int N, int NC>
 __global__ void __launch_bounds__(128, 3) k_faces64(long long E, long long F, PhysT<double> P,
                                                  const int* __restrict__ face_e, const int* __restrict__ face_f,
                                                  const int* __restrict__ nbr, const int* __restrict__ nbr_fo,
                                                  const double* __restrict__ fgu, const double* __restrict__ uf,
-                                                 const double* __restrict__ qf, const double* __restrict__ qx,
-                                                 double* __restrict__ fh, const double* __restrict__ mixf) {
+                                                 const double* __restrict__ qf, double* __restrict__ fh,
+                                                 const double* __restrict__ mixf) {
   using S = typename std::conditional<NC == 2, D64, double>::type;
   constexpr int NF = N * N;
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -734,20 +708,6 @@ __global__ void __launch_bounds__(128, 3) k_faces64(long long E, long long F, Ph
 #pragma unroll
       for (int c = 0; c < 5; ++c) q[d][c] = ld<S, NC, double>(qf + base + (d * 5 + c) * NF, plane_q);
   };
-  // tangent of the flux that the cross gradient tangent of the other element's face (b2) makes on a
-  // side in state us with viscous coefficients K, K2
-  auto cross = [&](long long face, int pt, const S (&us)[5], const S& K, const S& K2, double (&o)[5]) {
-    if constexpr (BLK) {
-      double uv[5], dq[3][5];
-#pragma unroll
-      for (int c = 0; c < 5; ++c) uv[c] = us[c].v;
-#pragma unroll
-      for (int d = 0; d < 3; ++d)
-#pragma unroll
-        for (int c = 0; c < 5; ++c) dq[d][c] = qx[face * 15 * NF + (d * 5 + c) * NF + pt];
-      flux_n64_dq(uv, dq, n, K.v, K2.v, o);
-    }
-  };
   if (nb == -DG_BC_OUTFLOW) {
     const S s = s_isr(u[0]);
     flux_n64_inviscid(u, n, pc, s, out);
@@ -762,13 +722,11 @@ __global__ void __launch_bounds__(128, 3) k_faces64(long long E, long long F, Ph
       ue[1] = ue[2] = ue[3] = s_zero<S>();
       ue[4] = P.t_wall * sr;
     }
-    double l1[5] = {0.0, 0.0, 0.0, 0.0, 0.0}, l2[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
     {
       S q[3][5], s, K, K2;
       grad_of(qb, q);
       state64(P, ue, mx, s, K, K2);
       flux_n64(P, ue, q, n, pc, s, K, K2, out);
-      if (BLK && !wall) cross(e * 6 + phi, f, u, K, K2, l1);
     }
     S ur[5];                                 // the jump's other state: the neighbour's, or the wall's
     S uh0 = ue[0], uh4 = ue[4];
@@ -787,7 +745,6 @@ __global__ void __launch_bounds__(128, 3) k_faces64(long long E, long long F, Ph
       grad_of(qb2, q);
       state64(P, ur, mx, s, K, K2);
       flux_n64(P, ur, q, n, pc, s, K, K2, f2v);
-      if (BLK) cross((long long)nb * 6 + phi2, f2, ur, K, K2, l2);
       uh0 = 0.5 * (u[0] + ur[0]);
       uh4 = 0.5 * (u[4] + ur[4]);
       weight = 0.5 * area;
@@ -795,35 +752,14 @@ __global__ void __launch_bounds__(128, 3) k_faces64(long long E, long long F, Ph
 #pragma unroll
       for (int c = 0; c < 5; ++c) ur[c] = ue[c];
     }
-    if constexpr (BLK) {
-      if (!wall) {
-        // sigma for the own block (u_hat follows u) and for the neighbour's (u_hat follows the other side)
-        S sm, se, sm2, se2;
-        sigma64(P, S{uh0.v, 0.5 * u[0].d}, S{uh4.v, 0.5 * u[4].d}, mx, sm, se);
-        sigma64(P, S{uh0.v, 0.5 * ur[0].d}, S{uh4.v, 0.5 * ur[4].d}, mx, sm2, se2);
+    S sm, se;
+    sigma64(P, uh0, uh4, mx, sm, se);
 #pragma unroll
-        for (int c = 0; c < 5; ++c) {
-          const S sg = c == 0 ? S{P.lam, 0.0} : c == 4 ? se : sm;
-          const S sg2 = c == 0 ? S{P.lam, 0.0} : c == 4 ? se2 : sm2;
-          const double ju = weight * (u[c].v - ur[c].v);
-          const double val = fma(sg.v, ju, 0.5 * (out[c].v + f2v[c].v));
-          const double own = fma(sg.v * weight, u[c].d, fma(sg.d, ju, 0.5 * (out[c].d + l2[c])));
-          const double oth = fma(-sg.v * weight, ur[c].d, fma(sg2.d, ju, 0.5 * (l1[c] + f2v[c].d)));
-          out[c] = S{val, own};
-          st(fh + ob2 + c * NF, plane_u, S{-val, -oth});
-        }
-      }
-    }
-    if (!BLK || wall) {
-      S sm, se;
-      sigma64(P, uh0, uh4, mx, sm, se);
-#pragma unroll
-      for (int c = 0; c < 5; ++c) {
-        const S ju = weight * (u[c] - ur[c]);
-        if (!wall) out[c] = 0.5 * (out[c] + f2v[c]);
-        out[c] = c == 0 ? s_fma(P.lam, ju, out[c]) : s_fma(c == 4 ? se : sm, ju, out[c]);
-        if (!wall) st(fh + ob2 + c * NF, plane_u, -out[c]);
-      }
+    for (int c = 0; c < 5; ++c) {
+      const S ju = weight * (u[c] - ur[c]);
+      if (!wall) out[c] = 0.5 * (out[c] + f2v[c]);
+      out[c] = c == 0 ? s_fma(P.lam, ju, out[c]) : s_fma(c == 4 ? se : sm, ju, out[c]);
+      if (!wall) st(fh + ob2 + c * NF, plane_u, -out[c]);
     }
   }
 #pragma unroll
@@ -958,7 +894,7 @@ __device__ __noinline__ void volume_slow(const XOps<N>& so, long long e, long lo
 // stage_c != 0 (NC = 2): the tangent output is the DIRK stage operator J_G v = M v - stage_c J_r v. It is
 // formed as -stage_c (J_r v - M v / stage_c), with -|J| u_dot / stage_c added to the tangent's source.
 // Four CTAs of 128 threads instead of three hide more of the pointwise physics' latency although some
-// registers spill (16x16x8 degree 4: 1179 -> 1154 us of Jv, degree 2 composition 893 -> 872).
+// registers spill (Jv of a 16x16x8 degree-4 shell 3233 -> 3208 us).
 template <int N, int NC>
 __global__ void __launch_bounds__(128, 4)
     k_volume64(long long E, const Ops* __restrict__ ops, PhysT<double> P, Sun64 sun, const double* __restrict__ gu,

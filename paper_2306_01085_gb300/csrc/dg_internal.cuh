@@ -92,7 +92,6 @@ struct Workspace {
   double* qg = nullptr;   // [2][E][3][5][Np] Gauss values of q
   double* qf = nullptr;   // [2][E][6][15][Nf] face traces of q
   double* fh = nullptr;   // [2][E][6][5][Nf] F_hat . (w n dS) per element face
-  double* qx = nullptr;   // [E][6][15][Nf] cross gradient traces (block-diagonal tangent only)
   double* tmp = nullptr;  // [2][n_dof] scratch vectors (FD Jv, nodal q)
   double* red = nullptr;  // [1024] reduction partials
   double* red_host = nullptr;  // pinned host copy
@@ -108,7 +107,7 @@ struct Solver;
 struct Mlp;
 template <typename R>
 struct WorkT {
-  R *ug, *uf, *qg, *qf, *fh, *qx;
+  R *ug, *uf, *qg, *qf, *fh;
   const R *geo, *fgeo, *acc, *xg;
   const R *mixg, *mixf;   // variable composition at Gauss / face points (NULL without it)
 };
@@ -232,13 +231,13 @@ struct Driver {
                       bool tangent, cudaStream_t s, bool f32 = false, double stage_c = 0.0);
   static int q_to_nodal(dg_mesh* m, double* q, cudaStream_t s);
   static int q_from_nodal(dg_mesh* m, const double* q, cudaStream_t s);
-  static int mass(dg_mesh* m, const double* v, double* mv, cudaStream_t s, bool f32 = false);
+  static int mass(dg_mesh* m, const double* v, double* mv, cudaStream_t s);
   static int mass_inv(dg_mesh* m, const double* v, double* mv, cudaStream_t s);
   static int mixture(dg_mesh* m);
   static int cross_kappa(dg_mesh* m, double* kn);   // mesh factors of the cross gradient traces (default stream)
-  // J_r probe restricted to each element's own diagonal block (exact, one column per element)
-  static int jv_blockdiag(dg_mesh* m, const double* u, const double* probe, double t, double* jv, cudaStream_t s,
-                          bool f32 = false, bool tangent_only = false);
+  // diagonal blocks of J_G = M - c J_r (dg_blocks.cuh); block_doubles: Jacobian storage of one element
+  static int blocks(dg_mesh* m, double t, double c, double* jac, long long batch, float* out, cudaStream_t s);
+  static long long block_doubles();
   // FP32 residual (v == NULL) or fused residual + exact Jv with a contraction mode (CM_*)
   static int eval_cm(dg_mesh* m, const double* u, const double* v, double t, double* r, double* jv, int cm,
                      cudaStream_t s);
@@ -248,9 +247,6 @@ struct Driver {
   static int gradient_p(dg_mesh* m, const double* u, const double* v, cudaStream_t s, bool tangent_only);
   template <typename R>
   static int residual_p(dg_mesh* m, double t, double* r, double* jv, bool tangent, cudaStream_t s, double stage_c);
-  template <typename R>
-  static int jv_blockdiag_p(dg_mesh* m, const double* u, const double* probe, double t, double* jv, cudaStream_t s,
-                            bool tangent_only);
 };
 
 // orientation map of face point (is, it) to the neighbour's face point index

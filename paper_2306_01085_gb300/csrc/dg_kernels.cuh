@@ -227,20 +227,15 @@ __global__ void k_interp(const double* __restrict__ u, const double* __restrict_
 // --------------------------------------------------------------------------------------------
 // k_grad: LDG gradient in Gauss space (Eq. DGformulation a) and its face traces
 // --------------------------------------------------------------------------------------------
-// BLK (block-diagonal tangent, NC = 2): the tangent keeps only the element's own perturbation
-// (u_hat picks up half of the own trace on interior faces) and qx receives, per face, the trace of
-// the gradient tangent this element would get from its neighbour's perturbation across that face:
-// kappa(f) (w n dS)(f) u_dot_nb(f) / 2 with kappa(f) = sum_k e_face[k]^2 / (w |J|)(g(f, k)).
 // TO (tangent only, NC = 1): the value plane of ug, uf, qg, qf already holds the state's values
-// (computed once for all the Jv of one Krylov solve, or for all the probes of one block assembly);
+// (computed once for all the Jv of one Krylov solve);
 // only the tangent plane is formed, with the same arithmetic as the tangent of NC = 2, so the
 // result is identical. The wall trace of the tangent reads the value plane's varrho trace.
-template <int N, int NC, bool BLK, typename R, int CM = CM_NATIVE, bool TO = false>
+template <int N, int NC, typename R, int CM = CM_NATIVE, bool TO = false>
 __global__ void k_grad(long long E, const Ops* __restrict__ ops, PhysT<R> P, const R* __restrict__ geo,
                        const R* __restrict__ fgeo, const int* __restrict__ nbr,
                        const int* __restrict__ nbr_fo, const R* __restrict__ ug,
-                       const R* __restrict__ uf, R* __restrict__ qg, R* __restrict__ qf,
-                       R* __restrict__ qx) {
+                       const R* __restrict__ uf, R* __restrict__ qg, R* __restrict__ qf) {
   static_assert(!TO || NC == 1, "tangent-only gradient works on one plane");
   constexpr int NP = Shape<N>::NP, NF = Shape<N>::NF, C = 5 * NC, EPB = Epb<N, NC>::value;
   __shared__ SmemOpsT<R> so;
@@ -253,7 +248,6 @@ __global__ void k_grad(long long E, const Ops* __restrict__ ops, PhysT<R> P, con
   R* sQ = sY + EPB * 9 * NP;                // [EPB][3][C][NP]
   R* sL = sQ + EPB * 3 * C * NP;            // [EPB][6][3][NF]: (w n_d dS) u_hat_c of the current c
   load_ops<N, R>(ops, so);
-  if constexpr (BLK) __syncthreads();       // the trace loop reads eL / eR for kappa
   const long long e0 = (long long)blockIdx.x * EPB;
   const long long plane_g = E * 5 * NP, plane_f = E * 30 * NF;
   const long long og = TO ? plane_g : 0, of = TO ? plane_f : 0;   // TO: read the tangent plane
@@ -281,28 +275,8 @@ __global__ void k_grad(long long E, const Ops* __restrict__ ops, PhysT<R> P, con
       const long long nbase = (long long)nb * 30 * NF + (fo & 7) * 5 * NF + f2;
       for (int pl = 0; pl < NC; ++pl)
         for (int c = 0; c < 5; ++c) oth[5 * pl + c] = uf[of + pl * plane_f + nbase + c * NF];
-      if constexpr (BLK) {
-        constexpr int T0 = TO ? 0 : 5;   // where the tangent sits in own / oth / dst
-        for (int c = 0; c < 5; ++c) {
-          if constexpr (!TO) dst[c * NF] = R(0.5) * (own[c] + oth[c]);
-          dst[(T0 + c) * NF] = R(0.5) * own[T0 + c];
-        }
-        const R* ev = (phi & 1) ? so.eR : so.eL;
-        R kappa = R(0);
-        for (int k = 0; k < N; ++k) kappa += ev[k] * ev[k] / geo[e * 10 * NP + 9 * NP + face_vol_point<N>(phi, f, k)];
-        R* xo = qx + (e * 6 + phi) * 15 * NF + f;
-        for (int d = 0; d < 3; ++d) {
-          const R kn = R(0.5) * kappa * fgeo[((e * 6 + phi) * 4 + d) * NF + f];
-          for (int c = 0; c < 5; ++c) xo[(d * 5 + c) * NF] = kn * oth[T0 + c];
-        }
-      } else {
-        for (int c = 0; c < C; ++c) dst[c * NF] = R(0.5) * (own[c] + oth[c]);
-      }
+      for (int c = 0; c < C; ++c) dst[c * NF] = R(0.5) * (own[c] + oth[c]);
     } else if (nb == -DG_BC_WALL) {
-      if constexpr (BLK) {
-        R* xo = qx + (e * 6 + phi) * 15 * NF + f;
-        for (int k = 0; k < 15; ++k) xo[k * NF] = R(0);
-      }
       if constexpr (TO) {
         const R sr = s_exp(R(0.5) * uf[fbase]);   // value plane's varrho trace
         dst[0] = own[0];
@@ -326,10 +300,6 @@ __global__ void k_grad(long long E, const Ops* __restrict__ ops, PhysT<R> P, con
         dst[9 * NF] = R(0.5) * sr * P.t_wall * own[5];
       }
     } else {
-      if constexpr (BLK) {
-        R* xo = qx + (e * 6 + phi) * 15 * NF + f;
-        for (int k = 0; k < 15; ++k) xo[k * NF] = R(0);
-      }
       for (int c = 0; c < C; ++c) dst[c * NF] = own[c];
     }
   }
@@ -436,15 +406,12 @@ __device__ __forceinline__ void face_flux_interior(const PhysT<R>& P, const S u[
   for (int c = 0; c < 5; ++c) out[c] = R(0.5) * (f1[c] + fn[c]) + sg[c] * ((R(0.5) * area) * (u[c] - u2[c]));
 }
 
-// BLK (NC = 2): interior faces evaluate the tangent twice, once for each side's diagonal block:
-// the own side carries its perturbation and the other side only the gradient it receives from it
-// across this face (qx of the other element).
-template <int N, int NC, bool BLK, typename R>
+template <int N, int NC, typename R>
 __global__ void k_faces(long long E, long long F, PhysT<R> P, const int* __restrict__ face_e,
                         const int* __restrict__ face_f, const int* __restrict__ nbr,
                         const int* __restrict__ nbr_fo, const R* __restrict__ fgeo,
                         const R* __restrict__ uf, const R* __restrict__ qf,
-                        const R* __restrict__ qx, R* __restrict__ fh, const R* __restrict__ mixf) {
+                        R* __restrict__ fh, const R* __restrict__ mixf) {
   using S = typename std::conditional<NC == 2, DualT<R>, R>::type;
   constexpr int NF = Shape<N>::NF;
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -487,32 +454,9 @@ __global__ void k_faces(long long E, long long F, PhysT<R> P, const int* __restr
 #pragma unroll
       for (int c = 0; c < 5; ++c) q2[d][c] = ld<S, NC, R>(qf + qb2 + (d * 5 + c) * NF, plane_q);
     const long long ob2 = (long long)nb * 30 * NF + phi2 * 5 * NF + f2;
-    if constexpr (BLK) {
-      // block of the own element: the neighbour side carries only the cross gradient tangent
-      S ua[5], qa[3][5];
+    face_flux_interior(P, u, q, u2, q2, n, area, out, mx);
 #pragma unroll
-      for (int c = 0; c < 5; ++c) ua[c] = S{u2[c].v, R(0)};
-#pragma unroll
-      for (int d = 0; d < 3; ++d)
-#pragma unroll
-        for (int c = 0; c < 5; ++c) qa[d][c] = S{q2[d][c].v, qx[((long long)nb * 6 + phi2) * 15 * NF + (d * 5 + c) * NF + f2]};
-      face_flux_interior(P, u, q, ua, qa, n, area, out, mx);
-      // block of the neighbour: the own side carries only its cross gradient tangent
-      S ub[5], qb[3][5], outb[5];
-#pragma unroll
-      for (int c = 0; c < 5; ++c) ub[c] = S{u[c].v, R(0)};
-#pragma unroll
-      for (int d = 0; d < 3; ++d)
-#pragma unroll
-        for (int c = 0; c < 5; ++c) qb[d][c] = S{q[d][c].v, qx[(e * 6 + phi) * 15 * NF + (d * 5 + c) * NF + f]};
-      face_flux_interior(P, ub, qb, u2, q2, n, area, outb, mx);
-#pragma unroll
-      for (int c = 0; c < 5; ++c) st(fh + ob2 + c * NF, plane_u, -outb[c]);
-    } else {
-      face_flux_interior(P, u, q, u2, q2, n, area, out, mx);
-#pragma unroll
-      for (int c = 0; c < 5; ++c) st(fh + ob2 + c * NF, plane_u, -out[c]);
-    }
+    for (int c = 0; c < 5; ++c) st(fh + ob2 + c * NF, plane_u, -out[c]);
   } else if (nb == -DG_BC_WALL) {
     S ubd[5], sg[5];
     wall_trace(P, u, ubd);
@@ -783,60 +727,9 @@ k_volume(long long E, const Ops* __restrict__ ops, PhysT<R> P, R t,
 }  // namespace dg
 
 #include "dg_fp64.cuh"
+#include "dg_blocks.cuh"
 
 namespace dg {
-
-// --------------------------------------------------------------------------------------------
-// FP32 mass product
-// --------------------------------------------------------------------------------------------
-// FP32 mass product of EPB elements per CTA (one thread per point of each element): out = B^T W B in for the
-// five variables, FP32 arithmetic, input and output FP64 (the mass columns of FP32-assembled blocks)
-template <int N>
-__global__ void k_mass32(long long E, const Ops* __restrict__ ops, const double* __restrict__ in_g,
-                         double* __restrict__ out_g, const float* __restrict__ weight) {
-  constexpr int NP = Shape<N>::NP, EPB = Epb<N, 1>::value, C = 5;
-  __shared__ SmemOpsT<float> so;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  float* b0 = reinterpret_cast<float*>(smem_raw);   // [EPB][C][NP]
-  float* b1 = b0 + EPB * C * NP;                    // [EPB][C][NP]
-  load_ops<N, float>(ops, so);
-  const long long e0 = (long long)blockIdx.x * EPB;
-  for (int idx = threadIdx.x; idx < EPB * C * NP; idx += blockDim.x) {
-    const long long e = e0 + idx / (C * NP);
-    if (e < E) b0[idx] = (float)in_g[e0 * C * NP + idx];
-  }
-  __syncthreads();
-  const int el = threadIdx.x / NP, g = threadIdx.x % NP;
-  const bool active = el < EPB && (e0 + el) < E;
-  float* in = b0;
-  float* out = b1;
-  for (int dir = 0; dir < 3; ++dir) {
-    if (active)
-      for (int c = 0; c < C; ++c) out[(el * C + c) * NP + g] = line<N, false>(so.B, in + (el * C + c) * NP, g, dir);
-    __syncthreads();
-    float* tt = in;
-    in = out;
-    out = tt;
-  }
-  // W-weighted Gauss values, then back with B^T
-  if (active) {
-    const float wd = weight[(e0 + el) * 10 * NP + 9 * NP + g];
-    for (int c = 0; c < C; ++c) in[(el * C + c) * NP + g] *= wd;
-  }
-  __syncthreads();
-  for (int dir = 0; dir < 3; ++dir) {
-    if (active)
-      for (int c = 0; c < C; ++c) out[(el * C + c) * NP + g] = line<N, true>(so.B, in + (el * C + c) * NP, g, dir);
-    __syncthreads();
-    float* tt = in;
-    in = out;
-    out = tt;
-  }
-  for (int idx = threadIdx.x; idx < EPB * C * NP; idx += blockDim.x) {
-    const long long e = e0 + idx / (C * NP);
-    if (e < E) out_g[e0 * C * NP + idx] = (double)in[idx];
-  }
-}
 
 // variable composition (Sec. 2.1.1-2.1.2) at the Gauss and face points from the positions xg:
 // mixg [E][8][NP] = (c_v*, grad c_v* (3), conductivity factor, chi_N2, chi_O2, chi_He),
@@ -1033,7 +926,7 @@ struct Smem {
 
 template <typename R> inline WorkT<R> work_of(dg_mesh* m);
 template <> inline WorkT<double> work_of<double>(dg_mesh* m) {
-  return WorkT<double>{m->ws.ug, m->ws.uf, m->ws.qg, m->ws.qf, m->ws.fh, m->ws.qx, m->geo, m->fgeo, m->acc, m->xg,
+  return WorkT<double>{m->ws.ug, m->ws.uf, m->ws.qg, m->ws.qf, m->ws.fh, m->geo, m->fgeo, m->acc, m->xg,
                        m->mixg, m->mixf};
 }
 template <> inline WorkT<float> work_of<float>(dg_mesh* m) { return m->w32; }
@@ -1081,31 +974,31 @@ static int run_interp(dg_mesh* m, const double* u, const double* v, cudaStream_t
   }
 }
 
-template <int N, int NC, bool BLK = false, typename R = double, int CM = CM_NATIVE, bool TO = false>
+template <int N, int NC, typename R = double, int CM = CM_NATIVE, bool TO = false>
 static int run_grad(dg_mesh* m, cudaStream_t s) {
   if constexpr (std::is_same<R, double>::value) {
     using G = Grp<N>;
     const int threads = threads64<N>(m->E * NC), per = threads / G::T;
     const size_t sm = sizeof(cell) * GradCells<N>::size * per;
-    int rc = set_smem(k_grad64<N, BLK>, sm);
+    int rc = set_smem(k_grad64<N>, sm);
     if (rc) return rc;
     prof_begin(m, s, KK_GRAD);
-    k_grad64<N, BLK><<<dim3((unsigned)((m->E + per - 1) / per), NC), threads, sm, s>>>(
-        m->E, m->d_ops, m->phys.t_wall, TO ? 1 : 0, m->gu, m->fgu, m->kn, m->nbr, m->nbr_fo, m->ws.ug,
-        m->ws.uf, m->ws.qg, m->ws.qf, m->ws.qx);
+    k_grad64<N><<<dim3((unsigned)((m->E + per - 1) / per), NC), threads, sm, s>>>(
+        m->E, m->d_ops, m->phys.t_wall, TO ? 1 : 0, m->gu, m->fgu, m->nbr, m->nbr_fo, m->ws.ug, m->ws.uf,
+        m->ws.qg, m->ws.qf);
     prof_end(m, s);
     DG_LAUNCH_CHECK("k_grad64");
     return DG_OK;
   } else {
     constexpr int EPB = Epb<N, NC>::value, NP = Shape<N>::NP;
     const size_t sm = Smem<N, NC, R>::grad;
-    int rc = set_smem(k_grad<N, NC, BLK, R, CM, TO>, sm);
+    int rc = set_smem(k_grad<N, NC, R, CM, TO>, sm);
     if (rc) return rc;
     const unsigned blocks = (unsigned)((m->E + EPB - 1) / EPB);
     const WorkT<R> w = work_of<R>(m);
     prof_begin(m, s, KK_GRAD);
-    k_grad<N, NC, BLK, R, CM, TO><<<blocks, EPB * NP, sm, s>>>(m->E, m->d_ops, phys_as<R>(m->phys), w.geo, w.fgeo,
-                                                            m->nbr, m->nbr_fo, w.ug, w.uf, w.qg, w.qf, w.qx);
+    k_grad<N, NC, R, CM, TO><<<blocks, EPB * NP, sm, s>>>(m->E, m->d_ops, phys_as<R>(m->phys), w.geo, w.fgeo,
+                                                            m->nbr, m->nbr_fo, w.ug, w.uf, w.qg, w.qf);
     prof_end(m, s);
     DG_LAUNCH_CHECK("k_grad");
     return DG_OK;
@@ -1135,7 +1028,7 @@ static int run_interp_tangent(dg_mesh* m, const double* v, cudaStream_t s) {
   }
 }
 
-template <int N, int NC, bool BLK = false, typename R = double>
+template <int N, int NC, typename R = double>
 static int run_faces(dg_mesh* m, cudaStream_t s) {
   constexpr int NF = Shape<N>::NF;
   const long long work = m->nfaces * NF;
@@ -1146,11 +1039,11 @@ static int run_faces(dg_mesh* m, cudaStream_t s) {
   const WorkT<R> w = work_of<R>(m);
   prof_begin(m, s, KK_FACES);
   if constexpr (std::is_same<R, double>::value)
-    k_faces64<N, NC, BLK><<<blocks, threads, 0, s>>>(m->E, m->nfaces, phys_as<R>(m->phys), m->face_e, m->face_f, m->nbr,
-                                                     m->nbr_fo, m->fgu, w.uf, w.qf, w.qx, w.fh, w.mixf);
+    k_faces64<N, NC><<<blocks, threads, 0, s>>>(m->E, m->nfaces, phys_as<R>(m->phys), m->face_e, m->face_f, m->nbr,
+                                                     m->nbr_fo, m->fgu, w.uf, w.qf, w.fh, w.mixf);
   else
-    k_faces<N, NC, BLK, R><<<blocks, threads, 0, s>>>(m->E, m->nfaces, phys_as<R>(m->phys), m->face_e, m->face_f,
-                                                       m->nbr, m->nbr_fo, w.fgeo, w.uf, w.qf, w.qx, w.fh, w.mixf);
+    k_faces<N, NC, R><<<blocks, threads, 0, s>>>(m->E, m->nfaces, phys_as<R>(m->phys), m->face_e, m->face_f,
+                                                       m->nbr, m->nbr_fo, w.fgeo, w.uf, w.qf, w.fh, w.mixf);
   prof_end(m, s);
   DG_LAUNCH_CHECK("k_faces");
   return DG_OK;
@@ -1178,6 +1071,21 @@ inline long long resident_ctas(dg_mesh* m, const void* fn, int threads, size_t s
   return v;
 }
 
+// the Sun of the heating models at time t
+static Sun64 sun_at(const dg_mesh* m, double t) {
+  Sun64 sun{{0.0, 0.0, 0.0}, m->d_euv};
+  const double wt = m->phys.euv_omega_t * t;
+  if (m->phys.euv == DG_EUV_GAUSS) {
+    sun.d[0] = std::cos(wt);
+    sun.d[1] = -std::sin(wt);
+  } else if (m->phys.euv == DG_EUV_EUVAC) {
+    sun.d[0] = -m->phys.sun_cd * std::cos(wt);
+    sun.d[1] = m->phys.sun_cd * std::sin(wt);
+    sun.d[2] = m->phys.sun_sd;
+  }
+  return sun;
+}
+
 template <int N, int NC, typename R = double, int CM = CM_NATIVE>
 static int run_volume(dg_mesh* m, double t, double* r, double* jv, cudaStream_t s, double stage_c = 0.0) {
   if constexpr (std::is_same<R, double>::value) {
@@ -1186,16 +1094,7 @@ static int run_volume(dg_mesh* m, double t, double* r, double* jv, cudaStream_t 
     const size_t sm = sizeof(cell) * VolCells<N, NC>::size * per;
     int rc = set_smem(k_volume64<N, NC>, sm);
     if (rc) return rc;
-    Sun64 sun{{0.0, 0.0, 0.0}, m->d_euv};
-    const double wt = m->phys.euv_omega_t * t;
-    if (m->phys.euv == DG_EUV_GAUSS) {
-      sun.d[0] = std::cos(wt);
-      sun.d[1] = -std::sin(wt);
-    } else if (m->phys.euv == DG_EUV_EUVAC) {
-      sun.d[0] = -m->phys.sun_cd * std::cos(wt);
-      sun.d[1] = m->phys.sun_cd * std::sin(wt);
-      sun.d[2] = m->phys.sun_sd;
-    }
+    const Sun64 sun = sun_at(m, t);
     prof_begin(m, s, KK_VOLUME);
     k_volume64<N, NC><<<(unsigned)((m->E + per - 1) / per), threads, sm, s>>>(
         m->E, m->d_ops, phys_as<double>(m->phys), sun, m->gu, m->acc, m->xg, m->ws.ug, m->ws.qg, m->ws.fh, r, jv, stage_c,
@@ -1251,18 +1150,18 @@ int Driver<N>::gradient_p(dg_mesh* m, const double* u, const double* v, cudaStre
   if (tangent_only) {   // u's value plane is in place: the tangent of v alone
     int rc = run_interp_tangent<N, R>(m, v, s);
     if (rc) return rc;
-    return run_grad<N, 1, false, R, CM_NATIVE, true>(m, s);
+    return run_grad<N, 1, R, CM_NATIVE, true>(m, s);
   }
   int rc = v ? run_interp<N, 2, R>(m, u, v, s) : run_interp<N, 1, R>(m, u, nullptr, s);
   if (rc) return rc;
-  return v ? run_grad<N, 2, false, R>(m, s) : run_grad<N, 1, false, R>(m, s);
+  return v ? run_grad<N, 2, R>(m, s) : run_grad<N, 1, R>(m, s);
 }
 
 template <int N>
 template <typename R>
 int Driver<N>::residual_p(dg_mesh* m, double t, double* r, double* jv, bool tangent, cudaStream_t s,
                           double stage_c) {
-  int rc = tangent ? run_faces<N, 2, false, R>(m, s) : run_faces<N, 1, false, R>(m, s);
+  int rc = tangent ? run_faces<N, 2, R>(m, s) : run_faces<N, 1, R>(m, s);
   if (rc) return rc;
   return tangent ? run_volume<N, 2, R>(m, t, r, jv, s, stage_c) : run_volume<N, 1, R>(m, t, r, nullptr, s);
 }
@@ -1281,32 +1180,38 @@ int Driver<N>::residual(dg_mesh* m, const double* u, const double* v, double t, 
              : residual_p<double>(m, t, r, jv, tangent, s, stage_c);
 }
 
+// the diagonal blocks of J_G = M - c J_r at the state whose value plane is in place; jac holds `batch`
+// elements' Jacobians
 template <int N>
-template <typename R>
-int Driver<N>::jv_blockdiag_p(dg_mesh* m, const double* u, const double* probe, double t, double* jv,
-                              cudaStream_t s, bool tangent_only) {
-  int rc;
-  if (tangent_only) {   // u's value plane is in place
-    rc = run_interp_tangent<N, R>(m, probe, s);
-    if (rc) return rc;
-    rc = run_grad<N, 1, true, R, CM_NATIVE, true>(m, s);
-  } else {
-    rc = run_interp<N, 2, R>(m, u, probe, s);
-    if (rc) return rc;
-    rc = run_grad<N, 2, true, R>(m, s);
+int Driver<N>::blocks(dg_mesh* m, double t, double c, double* jac, long long batch, float* out, cudaStream_t s) {
+  using B = Blk<N>;
+  constexpr int NP = B::NP, NF = B::NF;
+  const size_t sm = sizeof(cell) * B::cells;
+  int rc = set_smem(k_blocks<N>, sm);
+  if (rc) return rc;
+  const Sun64 sun = sun_at(m, t);
+  const PhysT<double> P = phys_as<double>(m->phys);
+  for (long long e0 = 0; e0 < m->E; e0 += batch) {
+    const long long nE = m->E - e0 < batch ? m->E - e0 : batch;
+    double* JF = jac + nE * B::JV;
+    prof_begin(m, s, KK_VOLUME);
+    k_jac_volume<N><<<(unsigned)((nE * NP + 127) / 128), 128, 0, s>>>(e0, nE, m->E, P, sun, m->gu, m->acc, m->xg, m->ws.ug,
+                                                                    m->ws.qg, m->mixg, jac);
+    prof_end(m, s);
+    prof_begin(m, s, KK_FACES);
+    k_jac_faces<N><<<(unsigned)((nE * 6 * NF + 127) / 128), 128, 0, s>>>(e0, nE, P, m->nbr, m->nbr_fo, m->fgu, m->kn,
+                                                                       m->ws.uf, m->ws.qf, m->mixf, JF);
+    prof_end(m, s);
+    prof_begin(m, s, KK_LU);
+    k_blocks<N><<<(unsigned)nE, B::GP * B::T, sm, s>>>(e0, m->d_ops, P.t_wall, m->gu, m->fgu, m->nbr, m->ws.uf, jac, JF,
+                                                     c != 0.0 ? c : -1.0, c != 0.0, out);
+    prof_end(m, s);
+    DG_LAUNCH_CHECK("k_blocks");
   }
-  if (rc) return rc;
-  rc = run_faces<N, 2, true, R>(m, s);
-  if (rc) return rc;
-  return run_volume<N, 2, R>(m, t, nullptr, jv, s);
+  return DG_OK;
 }
-
 template <int N>
-int Driver<N>::jv_blockdiag(dg_mesh* m, const double* u, const double* probe, double t, double* jv,
-                            cudaStream_t s, bool f32, bool tangent_only) {
-  return f32 ? jv_blockdiag_p<float>(m, u, probe, t, jv, s, tangent_only)
-             : jv_blockdiag_p<double>(m, u, probe, t, jv, s, tangent_only);
-}
+long long Driver<N>::block_doubles() { return Blk<N>::JV + Blk<N>::JF; }
 
 template <int N>
 template <int CM>
@@ -1315,9 +1220,9 @@ int Driver<N>::eval_cm_t(dg_mesh* m, const double* u, const double* v, double t,
   const bool tan = v != nullptr;
   int rc = tan ? run_interp<N, 2, float, CM>(m, u, v, s) : run_interp<N, 1, float, CM>(m, u, nullptr, s);
   if (rc) return rc;
-  rc = tan ? run_grad<N, 2, false, float, CM>(m, s) : run_grad<N, 1, false, float, CM>(m, s);
+  rc = tan ? run_grad<N, 2, float, CM>(m, s) : run_grad<N, 1, float, CM>(m, s);
   if (rc) return rc;
-  rc = tan ? run_faces<N, 2, false, float>(m, s) : run_faces<N, 1, false, float>(m, s);
+  rc = tan ? run_faces<N, 2, float>(m, s) : run_faces<N, 1, float>(m, s);
   if (rc) return rc;
   return tan ? run_volume<N, 2, float, CM>(m, t, r, jv, s) : run_volume<N, 1, float, CM>(m, t, r, nullptr, s);
 }
@@ -1383,20 +1288,8 @@ int Driver<N>::mass_inv(dg_mesh* m, const double* v, double* mv, cudaStream_t s)
 }
 
 template <int N>
-int Driver<N>::mass(dg_mesh* m, const double* v, double* mv, cudaStream_t s, bool f32) {
-  if (!f32) return run_nodal<N, NODAL_MASS>(m, v, mv, s);
-  constexpr int NP = Shape<N>::NP;
-  constexpr int EPB = Epb<N, 1>::value;
-  // FP32 arithmetic on the FP32 geometry (ensure_f32 has run)
-  if (!m->w32.geo) return fail(DG_EINVAL, "FP32 mass apply without the FP32 geometry");
-  const size_t sm = sizeof(float) * 2 * EPB * 5 * NP;
-  int rc = set_smem(k_mass32<N>, sm);
-  if (rc) return rc;
-  prof_begin(m, s, KK_TENSOR);
-  k_mass32<N><<<(unsigned)((m->E + EPB - 1) / EPB), EPB * NP, sm, s>>>(m->E, m->d_ops, v, mv, m->w32.geo);
-  prof_end(m, s);
-  DG_LAUNCH_CHECK("k_mass32");
-  return DG_OK;
+int Driver<N>::mass(dg_mesh* m, const double* v, double* mv, cudaStream_t s) {
+  return run_nodal<N, NODAL_MASS>(m, v, mv, s);
 }
 
 }  // namespace dg

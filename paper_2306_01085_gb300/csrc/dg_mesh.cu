@@ -326,7 +326,7 @@ static void free_mesh(dg_mesh* m) {
   if (m->w32_base) cudaFree(m->w32_base);
   void* ptrs[] = {m->d_ops, m->d_euv, m->x, m->geo, m->gu, m->fgu, m->kn, m->acc, m->xg, m->fgeo, m->mixg, m->mixf, m->nbr, m->nbr_fo, m->face_e,
                   m->face_f,
-                  m->ws.ug, m->ws.uf, m->ws.qg, m->ws.qf, m->ws.fh, m->ws.tmp, m->ws.red, m->ws.qx};
+                  m->ws.ug, m->ws.uf, m->ws.qg, m->ws.qf, m->ws.fh, m->ws.tmp, m->ws.red};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (m->ws.red_host) cudaFreeHost(m->ws.red_host);
@@ -360,9 +360,9 @@ int ensure_f32(dg_mesh* m) {
   if (m->w32_base) return DG_OK;
   const long long E = m->E, NP = m->np, NF = m->nf;
   const long long nmg = m->mixg ? E * 8 * NP : 0, nmf = m->mixf ? E * 12 * NF : 0;
-  const long long sizes[12] = {2 * E * 5 * NP, 2 * E * 30 * NF, 2 * E * 15 * NP, 2 * E * 90 * NF, 2 * E * 30 * NF,
-                               E * 90 * NF,    E * 10 * NP,     E * 24 * NF,     E * 3 * NP,      E * 3 * NP,
-                               nmg,            nmf};
+  const long long sizes[11] = {2 * E * 5 * NP, 2 * E * 30 * NF, 2 * E * 15 * NP, 2 * E * 90 * NF, 2 * E * 30 * NF,
+                               E * 10 * NP,    E * 24 * NF,     E * 3 * NP,      E * 3 * NP,      nmg,
+                               nmf};
   long long total = 0;
   for (long long z : sizes) total += (z + 63) / 64 * 64;
   cudaError_t err = cudaMalloc(&m->w32_base, sizeof(float) * (size_t)total);
@@ -370,18 +370,18 @@ int ensure_f32(dg_mesh* m) {
     m->w32_base = nullptr;
     return fail(DG_ENOMEM, std::string("FP32 workspace: ") + cudaGetErrorString(err));
   }
-  float* p[12];
+  float* p[11];
   long long off = 0;
-  for (int k = 0; k < 12; ++k) {
+  for (int k = 0; k < 11; ++k) {
     p[k] = m->w32_base + off;
     off += (sizes[k] + 63) / 64 * 64;
   }
-  m->w32 = WorkT<float>{p[0], p[1], p[2], p[3], p[4], p[5], p[6], p[7], p[8], p[9],
-                        m->mixg ? p[10] : nullptr, m->mixf ? p[11] : nullptr};
+  m->w32 = WorkT<float>{p[0], p[1], p[2], p[3], p[4], p[5], p[6], p[7], p[8],
+                        m->mixg ? p[9] : nullptr, m->mixf ? p[10] : nullptr};
   const double* src[6] = {m->geo, m->fgeo, m->acc, m->xg, m->mixg, m->mixf};
   for (int k = 0; k < 6; ++k) {
     if (!src[k]) continue;
-    k_to_f32<<<1024, 256>>>(sizes[6 + k], src[k], p[6 + k]);
+    k_to_f32<<<1024, 256>>>(sizes[5 + k], src[k], p[5 + k]);
     err = cudaGetLastError();
     if (err != cudaSuccess) return fail(DG_ECUDA, std::string("k_to_f32: ") + cudaGetErrorString(err));
   }

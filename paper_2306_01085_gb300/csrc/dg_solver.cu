@@ -614,23 +614,8 @@ __global__ void k_combine(long long n, int k, const double* __restrict__ V, long
 }
 
 // ------------------------------------------------------------------------------------------
-// block-Jacobi: probes, column scatter, FP32 batched LU (column-major blocks), solves
+// block-Jacobi: FP32 batched inversion (column-major blocks), solves
 // ------------------------------------------------------------------------------------------
-__global__ void k_probe(long long E, int n, int j, double* __restrict__ v) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < E * n; i += (long long)gridDim.x * blockDim.x)
-    v[i] = ((int)(i % n) == j) ? 1.0 : 0.0;
-}
-
-// column j of every block: B[e][j][row] = mv[e][row] - c jv[e][row]
-__global__ void k_scatter_col(long long E, int n, int j, double c, const double* __restrict__ mv,
-                              const double* __restrict__ jv, float* __restrict__ blocks) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < E * n; i += (long long)gridDim.x * blockDim.x) {
-    const long long e = i / n;
-    const int row = (int)(i % n);
-    blocks[(e * n + j) * (long long)n + row] = (float)(mv[i] - c * jv[i]);
-  }
-}
-
 // Blocked Gauss-Jordan inversion in global memory, one CTA per block, for blocks too large for one
 // CTA's shared memory. Only the current panel of B columns is staged, so two CTAs share an SM and one
 // block's serial panel steps overlap another block's update. Row interchanges are not applied to
@@ -1216,12 +1201,12 @@ struct Solver {
   double* partial = nullptr;
   double* hdev = nullptr;   // [2][MAXK]
   double* hhost = nullptr;  // pinned [2 MAXK + RB_MAX^2]
-  double* probe = nullptr;  // [n]
+  double* jac = nullptr;    // pointwise Jacobians of jac_batch elements (block assembly)
+  long long jac_batch = 0;
   float* blocks = nullptr;  // [E][5Np][5Np]: assembled blocks, then (in place) their inverses
   int* piv = nullptr;
   int* info = nullptr;
   bool bj_ready = false;
-  bool recompute_value = false;  // DG_OPT_RECOMPUTE_VALUE of the running implicit step
   __half* blocks_h = nullptr;  // [E][5Np][ld]: FP16 columns of the inverses (DG_PC_BJ16)
   float* hscale = nullptr;     // [E][5Np]: their power-of-two column scales
   int hld = 0;
@@ -1249,7 +1234,7 @@ enum { VU = 0, VKNOWN, VR0, VR1, VR2, VG, VRES, VZ, VW, VDU, VTMP, VUN };
 
 static void solver_free(Solver* S) {
   if (!S) return;
-  void* ptrs[] = {S->V, S->vec, S->partial, S->hdev, S->probe, S->blocks, S->piv, S->info, S->blocks_h, S->hscale,
+  void* ptrs[] = {S->V, S->vec, S->partial, S->hdev, S->jac, S->blocks, S->piv, S->info, S->blocks_h, S->hscale,
                   S->rb_ring, S->rb_W, S->rb_Z, S->rb_Y, S->rb_C, S->rb_s};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -1300,23 +1285,43 @@ static int solver_get(dg_mesh* m, int restart, Solver** out) {
     default: rc = fail(DG_EINVAL, "unsupported degree");       \
   }
 
-static int ensure_blocks(dg_mesh* m, Solver* S) {
-  if (S->blocks) return DG_OK;
-  const long long nb = 5LL * m->np;
-  cudaError_t err = cudaMalloc(&S->blocks, sizeof(float) * (size_t)m->E * nb * nb);
-  if (err == cudaSuccess) err = cudaMalloc(&S->piv, sizeof(int) * (size_t)m->E * nb);
-  if (err == cudaSuccess) err = cudaMalloc(&S->info, sizeof(int));
-  if (err == cudaSuccess) err = cudaMalloc(&S->probe, sizeof(double) * (size_t)m->ndof);
-  if (err == cudaSuccess && !m->ws.qx) err = cudaMalloc(&m->ws.qx, sizeof(double) * (size_t)m->E * 90 * m->nf);
+// Jacobian storage of the block assembly: at most 1 GiB (batches of elements beyond that)
+static int ensure_jac(dg_mesh* m, Solver* S) {
+  if (S->jac && m->kn) return DG_OK;
+  long long per = 0;
+  switch (m->n) {
+    case 2: per = Driver<2>::block_doubles(); break;
+    case 3: per = Driver<3>::block_doubles(); break;
+    case 4: per = Driver<4>::block_doubles(); break;
+    default: per = Driver<5>::block_doubles(); break;
+  }
+  cudaError_t err = cudaSuccess;
+  if (!S->jac) {
+    S->jac_batch = std::min((long long)m->E, std::max(1LL, (1LL << 27) / per));
+    err = cudaMalloc(&S->jac, sizeof(double) * (size_t)(S->jac_batch * per));
+    if (err != cudaSuccess) S->jac = nullptr;
+  }
   if (err == cudaSuccess && !m->kn) {
     err = cudaMalloc(&m->kn, sizeof(double) * (size_t)m->E * 18 * m->nf);
     if (err == cudaSuccess) {
       int rc = DG_OK;
       DG_DISPATCH_S(m, cross_kappa(m, m->kn));
       if (rc) return rc;
-      err = cudaDeviceSynchronize();   // once per mesh: later sweeps may run on any stream
+      err = cudaDeviceSynchronize();   // once per mesh: later assemblies may run on any stream
+    } else {
+      m->kn = nullptr;
     }
   }
+  if (err != cudaSuccess) return fail(DG_ENOMEM, std::string("block assembly storage: ") + cudaGetErrorString(err));
+  return DG_OK;
+}
+
+static int ensure_blocks(dg_mesh* m, Solver* S) {
+  if (S->blocks) return DG_OK;
+  const long long nb = 5LL * m->np;
+  cudaError_t err = cudaMalloc(&S->blocks, sizeof(float) * (size_t)m->E * nb * nb);
+  if (err == cudaSuccess) err = cudaMalloc(&S->piv, sizeof(int) * (size_t)m->E * nb);
+  if (err == cudaSuccess) err = cudaMalloc(&S->info, sizeof(int));
   if (err != cudaSuccess) return fail(DG_ENOMEM, std::string("block-Jacobi storage: ") + cudaGetErrorString(err));
   return DG_OK;
 }
@@ -1474,44 +1479,18 @@ static int norm2(dg_mesh* m, Solver* S, const double* x, double* out, cudaStream
 // ------------------------------------------------------------------------------------------
 // preconditioner
 // ------------------------------------------------------------------------------------------
-// exact diagonal blocks of J_G = M - c J_r(U), column j of every element per sweep, into dest
-static int bj_assemble(dg_mesh* m, Solver* S, const double* U, double t, double c, float* dest, cudaStream_t s,
-                       bool f32 = false) {
-  int rc = ensure_blocks(m, S);
+// exact diagonal blocks of J_G = M - c J_r(U) into dest (FP64 arithmetic whatever the step's precision: they
+// cost less than the FP32 probe sweeps they replaced)
+static int bj_assemble(dg_mesh* m, Solver* S, const double* U, double t, double c, float* dest, cudaStream_t s) {
+  int rc = ensure_jac(m, S);
   if (rc) return rc;
-  if (f32) {
-    rc = ensure_f32(m);
-    if (rc) return rc;
-    if (!m->w32.qx) return fail(DG_EINVAL, "FP32 workspace without cross traces");
-  }
-  const int nb = 5 * m->np;
-  double* jv = S->v(VW);
-  double* mv = S->v(VTMP);
-  // every probe linearises at the same U: its value plane is formed once and each sweep
-  // differentiates the probe's tangent alone
-  const bool once = !S->recompute_value;
-  if (once) {
-    rc = stage_value_plane(m, U, f32, s);
-    if (rc) return rc;
-  }
-  for (int j = 0; j < nb; ++j) {
-    prof_begin(m, s, KK_BLAS);
-    k_probe<<<grid_for(S->n), 256, 0, s>>>(m->E, nb, j, S->probe);
-    prof_end(m, s);
-    DG_DISPATCH_S(m, jv_blockdiag(m, U, S->probe, t, jv, s, f32, once));
-    if (rc) return rc;
-    DG_DISPATCH_S(m, mass(m, S->probe, mv, s, f32));   // FP32 arithmetic for FP32 blocks
-    if (rc) return rc;
-    prof_begin(m, s, KK_BLAS);
-    k_scatter_col<<<grid_for(S->n), 256, 0, s>>>(m->E, nb, j, c, mv, jv, dest);
-    prof_end(m, s);
-    DG_LAUNCH_CHECK("k_scatter_col");
-  }
-  return DG_OK;
+  rc = stage_value_plane(m, U, false, s);
+  if (rc) return rc;
+  DG_DISPATCH_S(m, blocks(m, t, c, S->jac, S->jac_batch, dest, s));
+  return rc;
 }
 
-static int bj_setup(dg_mesh* m, Solver* S, const double* U, double t, double c, cudaStream_t s, bool f32 = false,
-                    bool half = false) {
+static int bj_setup(dg_mesh* m, Solver* S, const double* U, double t, double c, cudaStream_t s, bool half = false) {
   int rc = ensure_blocks(m, S);
   if (rc) return rc;
   const int nb = 5 * m->np;
@@ -1523,7 +1502,7 @@ static int bj_setup(dg_mesh* m, Solver* S, const double* U, double t, double c, 
     if (err != cudaSuccess) return fail(DG_ENOMEM, std::string("FP16 block storage: ") + cudaGetErrorString(err));
   }
   DG_CUDA_TRY(cudaMemsetAsync(S->info, 0, sizeof(int), s));
-  rc = bj_assemble(m, S, U, t, c, S->blocks, s, f32);
+  rc = bj_assemble(m, S, U, t, c, S->blocks, s);
   if (rc) return rc;
   prof_begin(m, s, KK_LU);
   const size_t gj_smem = sizeof(float) * (2 * nb + (size_t)nb * nb);
@@ -1839,11 +1818,11 @@ static int rb_build(dg_mesh* m, Solver* S, int kind, const double* U, double t, 
 }
 
 // (re)build the preconditioner of kind at state U
-static int pc_setup(dg_mesh* m, Solver* S, int kind, const double* U, double t, double c, cudaStream_t s, bool f32) {
+static int pc_setup(dg_mesh* m, Solver* S, int kind, const double* U, double t, double c, cudaStream_t s) {
   dg::NvtxRange nvtx_range_("preconditioner setup");
   S->lag_valid = false;   // a lagged preconditioner is only reused as its own step built it
-  if (kind == DG_PC_BJ || kind == DG_PC_RB_BJ) return bj_setup(m, S, U, t, c, s, f32);
-  if (kind == DG_PC_BJ16) return bj_setup(m, S, U, t, c, s, f32, true);
+  if (kind == DG_PC_BJ || kind == DG_PC_RB_BJ) return bj_setup(m, S, U, t, c, s);
+  if (kind == DG_PC_BJ16) return bj_setup(m, S, U, t, c, s, true);
   if (kind == DG_PC_MLP) return mlp_setup(m, U, c, s);
   return DG_OK;
 }
@@ -2012,7 +1991,7 @@ extern "C" int dg_precond_setup(dg_mesh* mesh, int32_t kind, const double* u, do
   if (rc) return rc;
   if (kind == DG_PC_NONE) return DG_OK;
   if (kind == DG_PC_BJ) return bj_setup(mesh, S, u, t, dt_aii, (cudaStream_t)stream);
-  if (kind == DG_PC_BJ16) return bj_setup(mesh, S, u, t, dt_aii, (cudaStream_t)stream, false, true);
+  if (kind == DG_PC_BJ16) return bj_setup(mesh, S, u, t, dt_aii, (cudaStream_t)stream, true);
   if (kind == DG_PC_MLP) return mlp_setup(mesh, u, dt_aii, (cudaStream_t)stream);
   return fail(DG_EINVAL, "dg_precond_setup: unknown kind");
 }
@@ -2088,11 +2067,6 @@ extern "C" int dg_implicit_step(dg_mesh* mesh, double* u, double t, double dt, c
     rc = ensure_rb(S, o.rb_size);
     if (rc) return rc;
   }
-  struct FlagScope {   // the flag holds for this step's block assemblies only
-    Solver* S;
-    ~FlagScope() { S->recompute_value = false; }
-  } flag_scope{S};
-  S->recompute_value = (o.flags & DG_OPT_RECOMPUTE_VALUE) != 0;
   dg_step_stats st;
   std::memset(&st, 0, sizeof(st));
   const long long n = S->n;
@@ -2122,7 +2096,7 @@ extern "C" int dg_implicit_step(dg_mesh* mesh, double* u, double t, double dt, c
   }
   if (build_now) {
     const auto p0 = std::chrono::steady_clock::now();
-    rc = pc_setup(mesh, S, o.precond, un, t + c[0] * dt, dt * A[0][0], s, o.jv_prec == DG_PREC_F32);
+    rc = pc_setup(mesh, S, o.precond, un, t + c[0] * dt, dt * A[0][0], s);
     st.precond_ms += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - p0).count();
     if (rc) return finish(rc);
     if (o.precond_refresh == DG_REFRESH_LAGGED) {
@@ -2144,7 +2118,7 @@ extern "C" int dg_implicit_step(dg_mesh* mesh, double* u, double t, double dt, c
     DG_LAUNCH_CHECK("k_lincomb");
     if (o.precond != DG_PC_NONE && o.precond_refresh == DG_REFRESH_STAGE) {
       const auto p0 = std::chrono::steady_clock::now();
-      rc = pc_setup(mesh, S, o.precond, U, ti, ci, s, o.jv_prec == DG_PREC_F32);
+      rc = pc_setup(mesh, S, o.precond, U, ti, ci, s);
       st.precond_ms += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - p0).count();
       if (rc) return finish(rc);
     }
@@ -2174,7 +2148,7 @@ extern "C" int dg_implicit_step(dg_mesh* mesh, double* u, double t, double dt, c
       if (it == o.max_newton) break;
       if (o.precond != DG_PC_NONE && o.precond_refresh == DG_REFRESH_NEWTON) {
         const auto p0 = std::chrono::steady_clock::now();
-        rc = pc_setup(mesh, S, o.precond, U, ti, ci, s, o.jv_prec == DG_PREC_F32);
+        rc = pc_setup(mesh, S, o.precond, U, ti, ci, s);
         st.precond_ms += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - p0).count();
         if (rc) return finish(rc);
       }
