@@ -568,13 +568,20 @@ __global__ void k_combine_f32v(long long n, int k, const float* __restrict__ V, 
   }
 }
 
-// out[j] = sum_b partial[j][b] (+= into out when accumulate); also out_sq = partial[k] sum
-__global__ void k_mdot_finish(int k, const double* __restrict__ partial, double* __restrict__ out, int accumulate) {
-  const int j = threadIdx.x;
-  if (j > k) return;
-  double s = 0.0;
-  for (int b = 0; b < RED_BLOCKS; ++b) s += partial[j * RED_BLOCKS + b];
-  out[j] = accumulate ? out[j] + s : s;
+// out[j] = sum_b partial[j][b], one warp per row j: ten partials per lane, then a shuffle tree. (One thread
+// per row spent 304 dependent FP64 additions on it, 17.5 us against about 3, three times per Arnoldi step.)
+__global__ void __launch_bounds__(32) k_mdot_finish(const double* __restrict__ partial, double* __restrict__ out) {
+  const double* p = partial + (size_t)blockIdx.x * RED_BLOCKS;
+  double v[(RED_BLOCKS + 31) / 32], s = 0.0;
+#pragma unroll
+  for (int q = 0; q < (RED_BLOCKS + 31) / 32; ++q) {
+    const int b = threadIdx.x + 32 * q;
+    v[q] = b < RED_BLOCKS ? p[b] : 0.0;
+  }
+#pragma unroll
+  for (int q = 0; q < (RED_BLOCKS + 31) / 32; ++q) s += v[q];
+  for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
+  if (threadIdx.x == 0) out[blockIdx.x] = s;
 }
 
 // w -= sum_j h[j] V_j for j < k
@@ -1096,27 +1103,76 @@ __global__ void k_gj_inverse(long long E, int n, float* __restrict__ blocks, int
     for (int t = threadIdx.x; t < n * n; t += blockDim.x) Ag[t] = A[t];
 }
 
-// y = B^{-1} x per element with the explicit FP32 inverse (column-major): coalesced over rows
-__global__ void k_inv_apply(long long E, int n, const float* __restrict__ inv, const double* __restrict__ x,
-                            double* __restrict__ y) {
-  extern __shared__ float sx[];
+// y = B^{-1} x per element with the explicit FP32 inverse (column-major), one thread per row (MR rows above
+// 320). Bound by HBM: the inverse streams through a ring of INV_S column chunks in shared memory, filled by
+// 16-byte asynchronous copies, so that a CTA keeps about 45 KB in flight whatever its row sums wait for (loads
+// by the rows' threads: 2,304 blocks of 135^2 68.6 -> 49.5 us, 864 of 320^2 137 -> 76, 162 of 625^2 350 -> 100,
+// 24,576 of 40^2 64 -> 49, about 15 us of each outside the kernel; unrolling those loads 32 deep made the
+// first case 92). An
+// element's inverse starts at a multiple of 4 bytes only: copies start at the 16-byte boundary below and the
+// rows index from the remainder; the storage is padded by 16 bytes. Row sums run over the columns
+// j = q mod 4, the last n mod 4 columns with q = 0.
+constexpr int INV_S = 4;
+// columns per chunk: about 16 KB or a quarter of the block, a multiple of 4 (so that every chunk starts at
+// the element's own remainder); and a chunk's bytes
+__host__ __device__ inline int inv_cols(int n) {
+  const int most = 16384 / (4 * n) & ~3, quarter = ((n + 3) / 4 + 3) & ~3;
+  return most < 4 ? 4 : most < quarter ? most : quarter;
+}
+__host__ __device__ inline int inv_chunk(int n) { return (inv_cols(n) * n * 4 + 31) & ~15; }
+
+template <int MR>
+__global__ void k_inv_apply(int n, const float* __restrict__ inv, const double* __restrict__ x, double* __restrict__ y) {
+  extern __shared__ __align__(16) unsigned char inv_sm[];
+  const int cols = inv_cols(n), chunk = inv_chunk(n), nch = (n + cols - 1) / cols;
+  float* sx = reinterpret_cast<float*>(inv_sm + INV_S * chunk);   // [n rounded up to 4]
   const long long e = blockIdx.x;
-  const float* A = inv + e * (long long)n * n;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) sx[i] = (float)x[e * n + i];
-  __syncthreads();
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    float acc0 = 0.f, acc1 = 0.f, acc2 = 0.f, acc3 = 0.f;
-    const float* a = A + i;
-    int j = 0;
-#pragma unroll 2
-    for (; j + 3 < n; j += 4) {
-      acc0 = fmaf(a[(long long)j * n], sx[j], acc0);
-      acc1 = fmaf(a[(long long)(j + 1) * n], sx[j + 1], acc1);
-      acc2 = fmaf(a[(long long)(j + 2) * n], sx[j + 2], acc2);
-      acc3 = fmaf(a[(long long)(j + 3) * n], sx[j + 3], acc3);
+  const long long byte0 = e * (long long)n * n * 4;
+  const int rem = (int)(byte0 & 15);
+  const char* src = reinterpret_cast<const char*>(inv) + (byte0 - rem);
+  const int total = (rem + n * n * 4 + 15) & ~15;              // bytes of the element from src
+  auto fill = [&](int t) {
+    if (t < nch) {
+      const int b0 = t * cols * n * 4, b1 = min(b0 + cols * n * 4 + 16, total);
+      const unsigned dst = (unsigned)__cvta_generic_to_shared(inv_sm + (t % INV_S) * chunk);
+      for (int b = b0 + 16 * threadIdx.x; b < b1; b += 16 * blockDim.x)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + b - b0), "l"(src + b) : "memory");
     }
-    for (; j < n; ++j) acc0 = fmaf(a[(long long)j * n], sx[j], acc0);
-    y[e * n + i] = (double)((acc0 + acc1) + (acc2 + acc3));
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+#pragma unroll
+  for (int t = 0; t < INV_S - 1; ++t) fill(t);
+  for (int i = threadIdx.x; i < (n + 3) / 4 * 4; i += blockDim.x) sx[i] = i < n ? (float)x[e * n + i] : 0.0f;
+  float acc[MR][4];
+#pragma unroll
+  for (int m = 0; m < MR; ++m)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc[m][q] = 0.0f;
+  for (int t = 0; t < nch; ++t) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(INV_S - 2) : "memory");
+    __syncthreads();                          // chunk t has arrived, chunk t - 1 has been read
+    fill(t + INV_S - 1);
+    const float* a = reinterpret_cast<const float*>(inv_sm + (t % INV_S) * chunk + rem);
+    const int j0 = t * cols, jn = min(cols, n - j0), j4 = jn & ~3;
+#pragma unroll
+    for (int m = 0; m < MR; ++m) {
+      const int i = threadIdx.x + m * blockDim.x;
+      if (i >= n) continue;
+#pragma unroll 4
+      for (int j = 0; j < j4; j += 4) {
+        const float4 w = *reinterpret_cast<const float4*>(sx + j0 + j);
+        acc[m][0] = fmaf(a[j * n + i], w.x, acc[m][0]);
+        acc[m][1] = fmaf(a[(j + 1) * n + i], w.y, acc[m][1]);
+        acc[m][2] = fmaf(a[(j + 2) * n + i], w.z, acc[m][2]);
+        acc[m][3] = fmaf(a[(j + 3) * n + i], w.w, acc[m][3]);
+      }
+      for (int j = j4; j < jn; ++j) acc[m][0] = fmaf(a[j * n + i], sx[j0 + j], acc[m][0]);
+    }
+  }
+#pragma unroll
+  for (int m = 0; m < MR; ++m) {
+    const int i = threadIdx.x + m * blockDim.x;
+    if (i < n) y[e * n + i] = (double)((acc[m][0] + acc[m][1]) + (acc[m][2] + acc[m][3]));
   }
 }
 
@@ -1319,7 +1375,7 @@ static int ensure_jac(dg_mesh* m, Solver* S) {
 static int ensure_blocks(dg_mesh* m, Solver* S) {
   if (S->blocks) return DG_OK;
   const long long nb = 5LL * m->np;
-  cudaError_t err = cudaMalloc(&S->blocks, sizeof(float) * (size_t)m->E * nb * nb);
+  cudaError_t err = cudaMalloc(&S->blocks, sizeof(float) * (size_t)m->E * nb * nb + 16);   // + 16: k_inv_apply
   if (err == cudaSuccess) err = cudaMalloc(&S->piv, sizeof(int) * (size_t)m->E * nb);
   if (err == cudaSuccess) err = cudaMalloc(&S->info, sizeof(int));
   if (err != cudaSuccess) return fail(DG_ENOMEM, std::string("block-Jacobi storage: ") + cudaGetErrorString(err));
@@ -1467,7 +1523,7 @@ static int stage_matvec(dg_mesh* m, Solver* S, const double* U, double t, double
 static int norm2(dg_mesh* m, Solver* S, const double* x, double* out, cudaStream_t s) {
   prof_begin(m, s, KK_BLAS);
   mdot(S->n, 0, S->V, x, S->partial, s);
-  k_mdot_finish<<<1, MAXK, 0, s>>>(0, S->partial, S->hdev, 0);
+  k_mdot_finish<<<1, 32, 0, s>>>(S->partial, S->hdev);
   prof_end(m, s);
   DG_LAUNCH_CHECK("k_mdot");
   DG_CUDA_TRY(cudaMemcpyAsync(S->hhost, S->hdev, sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -1587,7 +1643,7 @@ static void rb_push(Solver* S, const double* du, cudaStream_t s) {
 static int host_dots(dg_mesh* m, Solver* S, const double* V, int k, const double* x, double* out, cudaStream_t s) {
   prof_begin(m, s, KK_BLAS);
   mdot(S->n, k, V, x, S->partial, s);
-  k_mdot_finish<<<1, MAXK, 0, s>>>(k, S->partial, S->hdev, 0);
+  k_mdot_finish<<<k + 1, 32, 0, s>>>(S->partial, S->hdev);
   prof_end(m, s);
   DG_LAUNCH_CHECK("k_mdot");
   DG_CUDA_TRY(cudaMemcpyAsync(S->hhost, S->hdev, sizeof(double) * (k + 1), cudaMemcpyDeviceToHost, s));
@@ -1648,9 +1704,9 @@ static int rb_orthonormalise(dg_mesh* m, Solver* S, cudaStream_t s) {
     if (r > 0) {   // h1 is in hdev[0..r-1]
       prof_begin(m, s, KK_BLAS);
       update_dot(n, r, S->rb_W, S->hdev, w, S->partial, true, s);
-      k_mdot_finish<<<1, MAXK, 0, s>>>(r - 1, S->partial, S->hdev + MAXK, 0);
+      k_mdot_finish<<<r, 32, 0, s>>>(S->partial, S->hdev + MAXK);
       update_dot(n, r, S->rb_W, S->hdev + MAXK, w, S->partial, false, s);
-      k_mdot_finish<<<1, MAXK, 0, s>>>(0, S->partial, S->hdev + 2 * MAXK - 1, 0);
+      k_mdot_finish<<<1, 32, 0, s>>>(S->partial, S->hdev + 2 * MAXK - 1);
       prof_end(m, s);
       DG_LAUNCH_CHECK("rb orthonormalise");
       DG_CUDA_TRY(cudaMemcpyAsync(S->hhost, S->hdev + 2 * MAXK - 1, sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -1685,7 +1741,7 @@ static int rb_apply(dg_mesh* m, Solver* S, const double* x, double* y, cudaStrea
   const long long n = S->n;
   prof_begin(m, s, KK_PRECOND);
   mdot(n, r, S->rb_W, y, S->partial, s);
-  k_mdot_finish<<<1, MAXK, 0, s>>>(r - 1, S->partial, S->rb_s, 0);
+  k_mdot_finish<<<r, 32, 0, s>>>(S->partial, S->rb_s);
   k_small_matvec<<<1, 32, 0, s>>>(r, S->rb_C, S->rb_s, S->rb_s + RB_MAX);
   k_maxpy<<<grid_for(n), 256, 0, s>>>(n, r, S->rb_Y, n, S->rb_s + RB_MAX, y);
   prof_end(m, s);
@@ -1740,7 +1796,10 @@ static int precond_apply(dg_mesh* m, Solver* S, int kind, const double* x, doubl
     if (!S->bj_ready) return fail(DG_EINVAL, "block-Jacobi preconditioner used before dg_precond_setup");
     const int nb = 5 * m->np;
     prof_begin(m, s, KK_PRECOND);
-    k_inv_apply<<<(unsigned)m->E, nb <= 256 ? (nb + 31) / 32 * 32 : 256, sizeof(float) * nb, s>>>(m->E, nb, S->blocks, x, y);
+    const size_t sm = (size_t)INV_S * inv_chunk(nb) + sizeof(float) * ((nb + 3) / 4 * 4);
+    auto kern = nb <= 320 ? k_inv_apply<1> : k_inv_apply<2>;
+    DG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    kern<<<(unsigned)m->E, nb <= 320 ? (nb + 31) / 32 * 32 : ((nb + 1) / 2 + 31) / 32 * 32, sm, s>>>(nb, S->blocks, x, y);
     prof_end(m, s);
     DG_LAUNCH_CHECK("k_inv_apply");
     return DG_OK;
@@ -1901,19 +1960,19 @@ static int gmres(dg_mesh* m, Solver* S, const dg_solver_opts& o, const double* U
       // h1 = V^T w; w -= V h1 fused with h2 = V^T w; w -= V h2 fused with |w|^2
       if (f32basis) {
         mdot_f32v(n, k + 1, Vf, w, S->partial, s);
-        k_mdot_finish<<<1, MAXK, 0, s>>>(k, S->partial, S->hdev, 0);
+        k_mdot_finish<<<k + 1, 32, 0, s>>>(S->partial, S->hdev);
         update_dot_f32v(n, k + 1, Vf, S->hdev, w, S->partial, true, s);
-        k_mdot_finish<<<1, MAXK, 0, s>>>(k, S->partial, S->hdev + MAXK, 0);
+        k_mdot_finish<<<k + 1, 32, 0, s>>>(S->partial, S->hdev + MAXK);
         update_dot_f32v(n, k + 1, Vf, S->hdev + MAXK, w, S->partial, false, s);
-        k_mdot_finish<<<1, MAXK, 0, s>>>(0, S->partial, S->hdev + MAXK + k + 1, 0);
+        k_mdot_finish<<<1, 32, 0, s>>>(S->partial, S->hdev + MAXK + k + 1);
         k_scale_to_f32<<<grid_for(n), 256, 0, s>>>(n, w, 0.0, S->hdev + MAXK + k + 1, Vf + (long long)(k + 1) * n);
       } else {
         mdot(n, k + 1, V, w, S->partial, s, f32gs);
-        k_mdot_finish<<<1, MAXK, 0, s>>>(k, S->partial, S->hdev, 0);
+        k_mdot_finish<<<k + 1, 32, 0, s>>>(S->partial, S->hdev);
         update_dot(n, k + 1, V, S->hdev, w, S->partial, true, s, f32gs);
-        k_mdot_finish<<<1, MAXK, 0, s>>>(k, S->partial, S->hdev + MAXK, 0);
+        k_mdot_finish<<<k + 1, 32, 0, s>>>(S->partial, S->hdev + MAXK);
         update_dot(n, k + 1, V, S->hdev + MAXK, w, S->partial, false, s, f32gs);
-        k_mdot_finish<<<1, MAXK, 0, s>>>(0, S->partial, S->hdev + MAXK + k + 1, 0);
+        k_mdot_finish<<<1, 32, 0, s>>>(S->partial, S->hdev + MAXK + k + 1);
         k_scale_dev<<<grid_for(n), 256, 0, s>>>(n, w, S->hdev + MAXK + k + 1, V + (long long)(k + 1) * n);
       }
       prof_end(m, s);
