@@ -34,6 +34,7 @@
 #include <string>
 #include <type_traits>
 
+#include "dg_bits.cuh"
 #include "dg_internal.cuh"
 #include "dg_phys64.cuh"
 
@@ -156,221 +157,338 @@ __device__ __forceinline__ void load_ops(const Ops* __restrict__ o, SmemOpsT<R>&
 }
 
 
+// NC values of one entry (value and tangent planes), moved through shared memory by one access
+template <int V, typename R>
+struct alignas(V * sizeof(R)) Pack { R v[V]; };
+
+// the 1D operator entries of this thread's point, held in registers: along each axis the column i of A
+// (T: sum over k of A[k][i] x_k), else its row
+template <int N, bool T, typename R>
+__device__ __forceinline__ void axis_coefs(const R* A, const int (&ig)[3], R (&out)[3][N]) {
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int k = 0; k < N; ++k) out[a][k] = T ? A[k * N + ig[a]] : A[ig[a] * N + k];
+}
+// the two end-point coefficients of this thread's point along each axis, in face order
+template <typename R>
+__device__ __forceinline__ void end_coefs(const SmemOpsT<R>& so, const int (&ig)[3], R (&out)[6]) {
+#pragma unroll
+  for (int phi = 0; phi < 6; ++phi) out[phi] = ((phi & 1) ? so.eR : so.eL)[ig[phi >> 1]];
+}
+
+// the extrapolations of a line of N entries to its two ends
+template <int N, int CM, int V, typename R>
+__device__ __forceinline__ void line_ends(const SmemOpsT<R>& so, const Pack<V, R>* in, int st, Pack<V, R> (&end)[2]) {
+#pragma unroll
+  for (int p = 0; p < V; ++p) end[0].v[p] = end[1].v[p] = R(0);
+#pragma unroll
+  for (int k = 0; k < N; ++k) {
+    const Pack<V, R> x = in[k * st];
+#pragma unroll
+    for (int p = 0; p < V; ++p) {
+      end[0].v[p] = cm_fma<CM>(so.eL[k], x.v[p], end[0].v[p]);
+      end[1].v[p] = cm_fma<CM>(so.eR[k], x.v[p], end[1].v[p]);
+    }
+  }
+}
+
+// FP64 <-> FP32 at the nodal ends of the FP32 path: the integer conversions, since a cvt issues on the FP64
+// pipe (2 per cycle and SM)
+// (one branch for K values, after all of them have been loaded)
+static __device__ __noinline__ float cvt_any(double x) { return (float)x; }
+template <int K, typename R>
+__device__ __forceinline__ void from_f64(const double (&x)[K], R (&y)[K]) {
+  if constexpr (std::is_same<R, float>::value) {
+    bool plain = true;
+#pragma unroll
+    for (int k = 0; k < K; ++k) plain = plain && to_f32_plain(x[k]);
+    if (plain) {
+#pragma unroll
+      for (int k = 0; k < K; ++k) y[k] = to_f32_rn(x[k]);
+    } else {
+#pragma unroll
+      for (int k = 0; k < K; ++k) y[k] = cvt_any(x[k]);
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < K; ++k) y[k] = (R)x[k];
+  }
+}
+template <typename R>
+__device__ __forceinline__ double as_f64(R x) {
+  if constexpr (std::is_same<R, float>::value) return to_f64_exact(x);
+  else return (double)x;
+}
+
+// The element kernels below give each thread one Gauss point and pass lines through shared memory. They were
+// bound by instruction issue and the load/store unit, most of it not the contraction: operator entries read
+// again for every variable, index arithmetic, FP64 conversions. Operator entries and line addresses now stay
+// in registers, value and tangent go through shared memory as one 8-byte entry, results leave from registers,
+// and conversions run on the integer pipe; every sum keeps its order. Jv and r of 27,648 degree-3 elements:
+//   k_interp 81 -> 74 us (shared-memory bandwidth), k_grad 321 -> 232, k_volume 268 -> 188; k_faces 101
+//   (DRAM); HBM traffic alone 47, 135, 81 and 85.
+
 // --------------------------------------------------------------------------------------------
 // k_interp: nodal -> Gauss values and face traces. NC = 1 (u) or 2 (u and tangent v).
 // --------------------------------------------------------------------------------------------
 template <int N, int NC, typename R, int CM = CM_NATIVE>
-__global__ void k_interp(const double* __restrict__ u, const double* __restrict__ v, long long E,
-                         const Ops* __restrict__ ops, R* __restrict__ ug, R* __restrict__ uf) {
-  constexpr int NP = Shape<N>::NP, NF = Shape<N>::NF, C = 5 * NC, EPB = Epb<N, NC>::value;
+__global__ void __launch_bounds__(Epb<N, NC>::value * Shape<N>::NP)
+    k_interp(const double* __restrict__ u, const double* __restrict__ v, long long E,
+             const Ops* __restrict__ ops, R* __restrict__ ug, R* __restrict__ uf) {
+  constexpr int NP = Shape<N>::NP, NF = Shape<N>::NF, EPB = Epb<N, NC>::value, NT = EPB * NP;
+  using V = Pack<NC, R>;
   __shared__ SmemOpsT<R> so;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  R* smem = reinterpret_cast<R*>(smem_raw);
-  R* b0 = smem;                            // [EPB][C][NP]
-  R* b1 = smem + EPB * C * NP;             // [EPB][C][NP]
+  V* b0 = reinterpret_cast<V*>(smem_raw);   // [5][NT]
+  V* b1 = b0 + 5 * NT;                      // [5][NT]
   load_ops<N, R>(ops, so);
-  const long long e0 = (long long)blockIdx.x * EPB;
-  for (int idx = threadIdx.x; idx < EPB * 5 * NP; idx += blockDim.x) {
-    const int el = idx / (5 * NP), rem = idx % (5 * NP);
-    const long long e = e0 + el;
-    if (e < E) {
-      b0[(el * C) * NP + rem] = (R)u[e * 5 * NP + rem];
-      if (NC == 2) b0[(el * C + 5) * NP + rem] = (R)v[e * 5 * NP + rem];
+  const int tid = threadIdx.x, g = tid % NP;
+  const long long e0 = (long long)blockIdx.x * EPB, e = e0 + tid / NP;
+  const bool active = e < E;
+  if (active) {
+    double x[5 * NC];
+#pragma unroll
+    for (int c = 0; c < 5 * NC; ++c) x[c] = (c < 5 ? u : v)[e * 5 * NP + c % 5 * NP + g];
+    R y[5 * NC];
+    from_f64<5 * NC>(x, y);
+#pragma unroll
+    for (int c = 0; c < 5; ++c) {
+      V z;
+#pragma unroll
+      for (int p = 0; p < NC; ++p) z.v[p] = y[p * 5 + c];
+      b0[c * NT + tid] = z;
     }
   }
   __syncthreads();
-  const int el = threadIdx.x / NP, g = threadIdx.x % NP;
-  const bool active = el < EPB;
-  R* in = b0;
-  R* out = b1;
+  const long long plane_g = E * 5 * NP;
+  const int ig[3] = {g % N, (g / N) % N, g / (N * N)};
+  V *in = b0, *out = b1;
 #pragma unroll
   for (int dir = 0; dir < 3; ++dir) {
+    const int st = pt_stride<N>(dir), base = tid - ig[dir] * st;
+    R B[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) B[k] = so.B[ig[dir] * N + k];
     if (active)
-      for (int c = 0; c < C; ++c) out[(el * C + c) * NP + g] = line<N, false, R, CM>(so.B, in + (el * C + c) * NP, g, dir);
+#pragma unroll
+      for (int c = 0; c < 5; ++c) {
+        V acc;
+#pragma unroll
+        for (int p = 0; p < NC; ++p) acc.v[p] = R(0);
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+          const V x = in[c * NT + base + k * st];
+#pragma unroll
+          for (int p = 0; p < NC; ++p) acc.v[p] = cm_fma<CM>(B[k], x.v[p], acc.v[p]);
+        }
+        out[c * NT + tid] = acc;
+        if (dir == 2)
+#pragma unroll
+          for (int p = 0; p < NC; ++p) ug[p * plane_g + e * 5 * NP + c * NP + g] = acc.v[p];
+      }
     __syncthreads();
-    R* t = in;
+    V* t = in;
     in = out;
     out = t;
   }
-  // `in` holds Gauss values
-  const long long plane_g = E * 5 * NP;
-  for (int idx = threadIdx.x; idx < EPB * 5 * NP; idx += blockDim.x) {
-    const int l = idx / (5 * NP), rem = idx % (5 * NP);
-    const long long e = e0 + l;
-    if (e < E) {
-      ug[e * 5 * NP + rem] = in[(l * C) * NP + rem];
-      if (NC == 2) ug[plane_g + e * 5 * NP + rem] = in[(l * C + 5) * NP + rem];
-    }
-  }
-  // face traces, one face point per iteration, its N volume points found once (less index arithmetic)
+  // `in` holds Gauss values; face traces, both ends of a line per iteration
   const long long plane_f = E * 6 * 5 * NF;
-  for (int idx = threadIdx.x; idx < EPB * 6 * NF; idx += blockDim.x) {
-    const int l = idx / (6 * NF), phi = (idx / NF) % 6, f = idx % NF;
-    const long long e = e0 + l;
-    if (e >= E) continue;
-    const R* ev = (phi & 1) ? so.eR : so.eL;
-    int vp[N];
+  for (int idx = tid; idx < EPB * 3 * NF; idx += NT) {
+    const int l = idx / (3 * NF), a = (idx / NF) % 3, f = idx % NF;
+    if (e0 + l >= E) continue;
+    const int base = l * NP + face_vol_point<N>(2 * a, f, 0), st = pt_stride<N>(a);
+    R* dst = uf + (e0 + l) * 30 * NF + a * 10 * NF + f;
 #pragma unroll
-    for (int k = 0; k < N; ++k) vp[k] = face_vol_point<N>(phi, f, k);
-    for (int pl = 0; pl < NC; ++pl)
+    for (int c = 0; c < 5; ++c) {
+      V end[2];
+      line_ends<N, CM>(so, in + c * NT + base, st, end);
 #pragma unroll
-      for (int c = 0; c < 5; ++c) {
-        const R* src = in + (l * C + 5 * pl + c) * NP;
-        R acc = R(0);
+      for (int side = 0; side < 2; ++side)
 #pragma unroll
-        for (int k = 0; k < N; ++k) acc = cm_fma<CM>(ev[k], src[vp[k]], acc);
-        uf[pl * plane_f + e * 30 * NF + (phi * 5 + c) * NF + f] = acc;
-      }
+        for (int p = 0; p < NC; ++p) dst[p * plane_f + (side * 5 + c) * NF] = end[side].v[p];
+    }
   }
 }
 
 // --------------------------------------------------------------------------------------------
 // k_grad: LDG gradient in Gauss space (Eq. DGformulation a) and its face traces
 // --------------------------------------------------------------------------------------------
+// Shared memory holds the field and its traces alone: a line's products G u and a face's n u_hat are formed
+// again by every point that adds them, from geometry that stays in registers for all variables (N + 2 entries
+// per axis). That takes 3 FP32 multiplications for each shared load it saves; storing the products made shared-
+// memory bandwidth the bound (289 us). 4 CTAs per SM at 128 registers; more CTAs with fewer registers are
+// slower (236, 252).
 // TO (tangent only, NC = 1): the value plane of ug, uf, qg, qf already holds the state's values
 // (computed once for all the Jv of one Krylov solve);
 // only the tangent plane is formed, with the same arithmetic as the tangent of NC = 2, so the
 // result is identical. The wall trace of the tangent reads the value plane's varrho trace.
 template <int N, int NC, typename R, int CM = CM_NATIVE, bool TO = false>
-__global__ void k_grad(long long E, const Ops* __restrict__ ops, PhysT<R> P, const R* __restrict__ geo,
-                       const R* __restrict__ fgeo, const int* __restrict__ nbr,
-                       const int* __restrict__ nbr_fo, const R* __restrict__ ug,
-                       const R* __restrict__ uf, R* __restrict__ qg, R* __restrict__ qf) {
+__global__ void __launch_bounds__(Epb<N, NC>::value * Shape<N>::NP)
+    k_grad(long long E, const Ops* __restrict__ ops, PhysT<R> P, const R* __restrict__ geo,
+           const R* __restrict__ fgeo, const int* __restrict__ nbr, const int* __restrict__ nbr_fo,
+           const R* __restrict__ ug, const R* __restrict__ uf, R* __restrict__ qg, R* __restrict__ qf) {
   static_assert(!TO || NC == 1, "tangent-only gradient works on one plane");
-  constexpr int NP = Shape<N>::NP, NF = Shape<N>::NF, C = 5 * NC, EPB = Epb<N, NC>::value;
+  constexpr int NP = Shape<N>::NP, NF = Shape<N>::NF, EPB = Epb<N, NC>::value, NT = EPB * NP, FT = EPB * 6 * NF;
+  constexpr int NI = (FT + NT - 1) / NT;    // face points of a thread
+  using V = Pack<NC, R>;
   __shared__ SmemOpsT<R> so;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  R* smem = reinterpret_cast<R*>(smem_raw);
-  R* sU = smem;                             // [EPB][C][NP]
-  R* sUh = sU + EPB * C * NP;               // [EPB][6][C][NF]   U_hat
-  R* sN = sUh + EPB * 6 * C * NF;           // [EPB][6][3][NF]   w n dS
-  R* sY = sN + EPB * 6 * 3 * NF;            // [EPB][9][NP]
-  R* sQ = sY + EPB * 9 * NP;                // [EPB][3][C][NP]
-  R* sL = sQ + EPB * 3 * C * NP;            // [EPB][6][3][NF]: (w n_d dS) u_hat_c of the current c
+  V* sU = reinterpret_cast<V*>(smem_raw);   // [5][NT]
+  V* sUh = sU + 5 * NT;                     // [5][FT]
+  V* sQ = sUh + 5 * FT;                     // [2][3][NT] gradient of the current variable and the last
   load_ops<N, R>(ops, so);
-  const long long e0 = (long long)blockIdx.x * EPB;
+  const int tid = threadIdx.x, el = tid / NP, g = tid % NP;
+  const long long e0 = (long long)blockIdx.x * EPB, e = e0 + el;
+  const bool active = e < E;
   const long long plane_g = E * 5 * NP, plane_f = E * 30 * NF;
-  const long long og = TO ? plane_g : 0, of = TO ? plane_f : 0;   // TO: read the tangent plane
-  for (int idx = threadIdx.x; idx < EPB * 5 * NP; idx += blockDim.x) {
-    const int l = idx / (5 * NP), rem = idx % (5 * NP);
-    const long long e = e0 + l;
-    if (e < E)
-      for (int pl = 0; pl < NC; ++pl) sU[(l * C + 5 * pl) * NP + rem] = ug[og + pl * plane_g + e * 5 * NP + rem];
+  const long long og = TO ? plane_g : 0, of = TO ? plane_f : 0;   // TO: the tangent plane
+  // all loads are issued before the first is needed: neighbours, values (asynchronous copies), geometry of the
+  // point's lines and of the face points at their ends (kept for all variables), traces
+  int nb[NI], fo[NI];
+#pragma unroll
+  for (int it = 0; it < NI; ++it) {
+    const int idx = tid + it * NT;
+    const long long face = (e0 + idx / (6 * NF)) * 6 + (idx / NF) % 6;
+    const bool ok = idx < FT && face < E * 6;
+    nb[it] = ok ? nbr[face] : 0;
+    fo[it] = ok ? nbr_fo[face] : 0;
   }
-  // traces: u_hat on every face point (Eq. LDG2), and the face geometry
-  for (int idx = threadIdx.x; idx < EPB * 6 * NF; idx += blockDim.x) {
-    const int l = idx / (6 * NF), phi = (idx / NF) % 6, f = idx % NF;
-    const long long e = e0 + l;
-    if (e >= E) continue;
-    const long long fbase = e * 30 * NF + phi * 5 * NF + f;
-    for (int d = 0; d < 3; ++d) sN[((l * 6 + phi) * 3 + d) * NF + f] = fgeo[((e * 6 + phi) * 4 + d) * NF + f];
-    const int nb = nbr[e * 6 + phi];
-    R own[10], oth[10];
-    for (int pl = 0; pl < NC; ++pl)
-      for (int c = 0; c < 5; ++c) own[5 * pl + c] = uf[of + pl * plane_f + fbase + c * NF];
-    R* dst = sUh + ((l * 6 + phi) * C) * NF + f;
-    if (nb >= 0) {
-      const int fo = nbr_fo[e * 6 + phi];
-      const int f2 = orient_map(fo >> 3, f % N, f / N, N);
-      const long long nbase = (long long)nb * 30 * NF + (fo & 7) * 5 * NF + f2;
-      for (int pl = 0; pl < NC; ++pl)
-        for (int c = 0; c < 5; ++c) oth[5 * pl + c] = uf[of + pl * plane_f + nbase + c * NF];
-      for (int c = 0; c < C; ++c) dst[c * NF] = R(0.5) * (own[c] + oth[c]);
-    } else if (nb == -DG_BC_WALL) {
-      if constexpr (TO) {
-        const R sr = s_exp(R(0.5) * uf[fbase]);   // value plane's varrho trace
-        dst[0] = own[0];
-        dst[NF] = R(0);
-        dst[2 * NF] = R(0);
-        dst[3 * NF] = R(0);
-        dst[4 * NF] = R(0.5) * sr * P.t_wall * own[0];
-        continue;
-      }
-      const R sr = s_exp(R(0.5) * own[0]);
-      dst[0] = own[0];
-      dst[NF] = R(0);
-      dst[2 * NF] = R(0);
-      dst[3 * NF] = R(0);
-      dst[4 * NF] = sr * P.t_wall;
-      if (NC == 2) {
-        dst[5 * NF] = own[5];
-        dst[6 * NF] = R(0);
-        dst[7 * NF] = R(0);
-        dst[8 * NF] = R(0);
-        dst[9 * NF] = R(0.5) * sr * P.t_wall * own[5];
-      }
-    } else {
-      for (int c = 0; c < C; ++c) dst[c * NF] = own[c];
-    }
+  if (active)
+#pragma unroll
+    for (int c = 0; c < 5; ++c)
+#pragma unroll
+      for (int p = 0; p < NC; ++p)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(
+                         (unsigned)__cvta_generic_to_shared(sU + c * NT + tid) + p * (unsigned)sizeof(R)),
+                     "l"(ug + og + p * plane_g + e * 5 * NP + c * NP + g), "n"(sizeof(R)) : "memory");
+  const int ig[3] = {g % N, (g / N) % N, g / (N * N)};
+  int lb[3], fp[3];
+  R G[3][N][3], n[6][3], invW = R(0);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    lb[a] = g - ig[a] * pt_stride<N>(a);
+    fp[a] = vol_face_point<N>(g, a);
   }
-  __syncthreads();
-  const int el = threadIdx.x / NP, g = threadIdx.x % NP;
-  const bool active = el < EPB && (e0 + el) < E;
-  R G[9], invW = R(0);
   if (active) {
-    const R* gp = geo + (e0 + el) * 10 * NP + g;
-    for (int k = 0; k < 9; ++k) G[k] = gp[k * NP];
-    invW = R(1) / gp[9 * NP];
+    const R* gp = geo + e * 10 * NP;
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+#pragma unroll
+        for (int k = 0; k < N; ++k) G[a][k][d] = gp[(a * 3 + d) * NP + lb[a] + k * pt_stride<N>(a)];
+#pragma unroll
+        for (int side = 0; side < 2; ++side) n[2 * a + side][d] = fgeo[((e * 6 + 2 * a + side) * 4 + d) * NF + fp[a]];
+      }
+    invW = R(1) / gp[9 * NP + g];
   }
-  for (int c = 0; c < C; ++c) {
-    if (active) {
-      const R uc = sU[(el * C + c) * NP + g];
-      for (int k = 0; k < 9; ++k) sY[(el * 9 + k) * NP + g] = G[k] * uc;
-    }
-    // (w n_d dS) u_hat_c once per face point, shared by the N volume points behind it
-    for (int idx = threadIdx.x; idx < EPB * 6 * NF; idx += blockDim.x) {
-      const int l = idx / (6 * NF), phi = (idx / NF) % 6, f = idx % NF;
-      if (e0 + l < E) {
-        const R uh = sUh[((l * 6 + phi) * C + c) * NF + f];
-        for (int d = 0; d < 3; ++d) sL[((l * 6 + phi) * 3 + d) * NF + f] = sN[((l * 6 + phi) * 3 + d) * NF + f] * uh;
+  // traces: u_hat on every face point (Eq. LDG2)
+#pragma unroll
+  for (int it = 0; it < NI; ++it) {
+    const int idx = tid + it * NT;
+    const int l = idx / (6 * NF), phi = (idx / NF) % 6, f = idx % NF;
+    const long long ee = e0 + l;
+    if (idx >= FT || ee >= E) continue;
+    const long long fbase = ee * 30 * NF + phi * 5 * NF + f;
+    const int f2 = orient_map((fo[it] >> 3) & 7, f % N, f / N, N);
+    const long long nbase = nb[it] >= 0 ? (long long)nb[it] * 30 * NF + (fo[it] & 7) * 5 * NF + f2 : fbase;
+    V own[5], oth[5];
+#pragma unroll
+    for (int c = 0; c < 5; ++c)
+#pragma unroll
+      for (int p = 0; p < NC; ++p) {
+        own[c].v[p] = uf[of + p * plane_f + fbase + c * NF];
+        oth[c].v[p] = uf[of + p * plane_f + nbase + c * NF];
+      }
+    V* dst = sUh + idx;
+    if (nb[it] == -DG_BC_WALL) {
+      const R sr = s_exp(R(0.5) * (TO ? uf[fbase] : own[0].v[0]));   // TO: the value plane's varrho trace
+      V zero, last;
+#pragma unroll
+      for (int p = 0; p < NC; ++p) zero.v[p] = R(0);
+      if constexpr (TO) {
+        last.v[0] = R(0.5) * sr * P.t_wall * own[0].v[0];
+      } else {
+        last.v[0] = sr * P.t_wall;
+        if constexpr (NC == 2) last.v[1] = R(0.5) * sr * P.t_wall * own[0].v[1];
+      }
+      dst[0] = own[0];
+      dst[FT] = dst[2 * FT] = dst[3 * FT] = zero;
+      dst[4 * FT] = last;
+    } else {
+#pragma unroll
+      for (int c = 0; c < 5; ++c) {
+        V x;
+#pragma unroll
+        for (int p = 0; p < NC; ++p) x.v[p] = nb[it] >= 0 ? R(0.5) * (own[c].v[p] + oth[c].v[p]) : own[c].v[p];
+        dst[c * FT] = x;
       }
     }
-    __syncthreads();
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();
+  R D[3][N], ec[6];
+  axis_coefs<N, true>(so.D, ig, D);
+  end_coefs(so, ig, ec);
+  R* qge = qg + (TO ? E * 15 * NP : 0) + e * 15 * NP + g;
+#pragma unroll 1
+  for (int c = 0; c < 5; ++c) {
+    V* q = sQ + (c & 1) * 3 * NT;           // the other half is still being read for the traces
     if (active) {
       // q_d = (sum over the 6 faces of e_face[i_axis] (w n_d dS) u_hat_c - D^T (G u_c)) / (w |J|)
-      for (int d = 0; d < 3; ++d) {
-        R acc = R(0);
+      V acc[3];
 #pragma unroll
-        for (int phi = 0; phi < 6; ++phi) {
-          const int axis = phi >> 1;
-          const R coef = ((phi & 1) ? so.eR : so.eL)[axis_index<N>(g, axis)];
-          acc = cm_fma<CM>(coef, sL[((el * 6 + phi) * 3 + d) * NF + vol_face_point<N>(g, axis)], acc);
+      for (int d = 0; d < 3; ++d)
+#pragma unroll
+        for (int p = 0; p < NC; ++p) acc[d].v[p] = R(0);
+#pragma unroll
+      for (int phi = 0; phi < 6; ++phi) {
+        const V uh = sUh[c * FT + (el * 6 + phi) * NF + fp[phi >> 1]];
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+#pragma unroll
+          for (int p = 0; p < NC; ++p) acc[d].v[p] = cm_fma<CM>(ec[phi], n[phi][d] * uh.v[p], acc[d].v[p]);
+      }
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+          const V x = sU[c * NT + el * NP + lb[a] + k * pt_stride<N>(a)];
+#pragma unroll
+          for (int d = 0; d < 3; ++d)
+#pragma unroll
+            for (int p = 0; p < NC; ++p) acc[d].v[p] = cm_fma<CM>(-D[a][k], G[a][k][d] * x.v[p], acc[d].v[p]);
         }
 #pragma unroll
-        for (int a = 0; a < 3; ++a) acc = line_fma<N, true, true, R, CM>(so.D, sY + (el * 9 + a * 3 + d) * NP, g, a, acc);
-        sQ[((el * 3 + d) * C + c) * NP + g] = acc * invW;
+      for (int d = 0; d < 3; ++d) {
+#pragma unroll
+        for (int p = 0; p < NC; ++p) {
+          acc[d].v[p] = acc[d].v[p] * invW;
+          qge[p * E * 15 * NP + (d * 5 + c) * NP] = acc[d].v[p];
+        }
+        q[d * NT + tid] = acc[d];
       }
     }
     __syncthreads();
-  }
-  // write Q (Gauss space): each thread its own point, the 15 (d, c) entries unrolled; the face traces go
-  // one face point per iteration with its N volume points found once (the kernel is bound by
-  // instruction issue, much of it index arithmetic)
-  if (active) {
-    const long long e = e0 + el;
-    for (int pl = 0; pl < NC; ++pl)
+    // both ends of a line per iteration
 #pragma unroll
-      for (int dc = 0; dc < 15; ++dc)
-        qg[(TO ? E * 15 * NP : 0) + pl * E * 15 * NP + e * 15 * NP + dc * NP + g] =
-            sQ[((el * 3 + dc / 5) * C + 5 * pl + dc % 5) * NP + g];
-  }
-  for (int idx = threadIdx.x; idx < EPB * 6 * NF; idx += blockDim.x) {
-    const int l = idx / (6 * NF), phi = (idx / NF) % 6, f = idx % NF;
-    const long long e = e0 + l;
-    if (e >= E) continue;
-    const R* ev = (phi & 1) ? so.eR : so.eL;
-    int vp[N];
+    for (int it = 0; it < (EPB * 3 * NF + NT - 1) / NT; ++it) {
+      const int idx = tid + it * NT;
+      const int l = idx / (3 * NF), a = (idx / NF) % 3, f = idx % NF;
+      if (idx >= EPB * 3 * NF || e0 + l >= E) continue;
+      const int base = l * NP + face_vol_point<N>(2 * a, f, 0);
+      R* dst = qf + (TO ? E * 90 * NF : 0) + (e0 + l) * 90 * NF + a * 30 * NF + f;
 #pragma unroll
-    for (int k = 0; k < N; ++k) vp[k] = face_vol_point<N>(phi, f, k);
-    for (int pl = 0; pl < NC; ++pl)
+      for (int d = 0; d < 3; ++d) {
+        V end[2];
+        line_ends<N, CM>(so, q + d * NT + base, pt_stride<N>(a), end);
 #pragma unroll
-      for (int dc = 0; dc < 15; ++dc) {
-        const R* src = sQ + ((l * 3 + dc / 5) * C + 5 * pl + dc % 5) * NP;
-        R acc = R(0);
+        for (int side = 0; side < 2; ++side)
 #pragma unroll
-        for (int k = 0; k < N; ++k) acc = cm_fma<CM>(ev[k], src[vp[k]], acc);
-        qf[(TO ? E * 90 * NF : 0) + pl * E * 90 * NF + e * 90 * NF + (phi * 15 + dc) * NF + f] = acc;
+          for (int p = 0; p < NC; ++p) dst[p * E * 90 * NF + (side * 15 + d * 5 + c) * NF] = end[side].v[p];
       }
+    }
   }
 }
 
@@ -406,12 +524,21 @@ __device__ __forceinline__ void face_flux_interior(const PhysT<R>& P, const S u[
   for (int c = 0; c < 5; ++c) out[c] = R(0.5) * (f1[c] + fn[c]) + sg[c] * ((R(0.5) * area) * (u[c] - u2[c]));
 }
 
+// vout false (NC = 2): only the flux's tangent is written, r being unwanted
 template <int N, int NC, typename R>
 __global__ void k_faces(long long E, long long F, PhysT<R> P, const int* __restrict__ face_e,
                         const int* __restrict__ face_f, const int* __restrict__ nbr,
                         const int* __restrict__ nbr_fo, const R* __restrict__ fgeo,
                         const R* __restrict__ uf, const R* __restrict__ qf,
-                        R* __restrict__ fh, const R* __restrict__ mixf) {
+                        R* __restrict__ fh, const R* __restrict__ mixf, bool vout) {
+  auto put = [&](R* p, long long plane, const auto& x) {
+    if constexpr (NC == 1) {
+      p[0] = x;
+    } else {
+      if (vout) p[0] = x.v;
+      p[plane] = x.d;
+    }
+  };
   using S = typename std::conditional<NC == 2, DualT<R>, R>::type;
   constexpr int NF = Shape<N>::NF;
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -456,7 +583,7 @@ __global__ void k_faces(long long E, long long F, PhysT<R> P, const int* __restr
     const long long ob2 = (long long)nb * 30 * NF + phi2 * 5 * NF + f2;
     face_flux_interior(P, u, q, u2, q2, n, area, out, mx);
 #pragma unroll
-    for (int c = 0; c < 5; ++c) st(fh + ob2 + c * NF, plane_u, -out[c]);
+    for (int c = 0; c < 5; ++c) put(fh + ob2 + c * NF, plane_u, -out[c]);
   } else if (nb == -DG_BC_WALL) {
     S ubd[5], sg[5];
     wall_trace(P, u, ubd);
@@ -468,7 +595,7 @@ __global__ void k_faces(long long E, long long F, PhysT<R> P, const int* __restr
     flux_dot_n(P, u, q, n, false, out, mx);
   }
 #pragma unroll
-  for (int c = 0; c < 5; ++c) st(fh + ub + c * NF, plane_u, out[c]);
+  for (int c = 0; c < 5; ++c) put(fh + ub + c * NF, plane_u, out[c]);
 }
 
 // --------------------------------------------------------------------------------------------
@@ -589,7 +716,18 @@ __device__ __forceinline__ void prefetch_l2(const R* p, long long n) {
 // FP32: at least two CTAs per SM (four for the p = 3 Jv, where 128 registers suffice without spills), since
 // the value + tangent physics would otherwise take enough registers to halve the resident warps of
 // this latency-bound kernel (FP64 is bound by its pipe instead)
-template <int N, int NC, typename R, int CM = CM_NATIVE>
+template <int OUT, typename R>
+__device__ __forceinline__ Pack<OUT, R> planes_of(R x) { return {x}; }
+template <int OUT, typename R>
+__device__ __forceinline__ Pack<OUT, R> planes_of(DualT<R> x) {
+  Pack<OUT, R> y;
+  if constexpr (OUT == 2) y.v[0] = x.v;
+  y.v[OUT - 1] = x.d;
+  return y;
+}
+
+// OUT planes leave the kernel: NC, or 1 of the 2 (r not wanted: the tangent alone is contracted)
+template <int N, int NC, int OUT, typename R, int CM = CM_NATIVE>
 __global__ void __launch_bounds__(Epb<N, NC>::value * Shape<N>::NP, N == 4 && NC == 2 ? 4 : 2)
 k_volume(long long E, const Ops* __restrict__ ops, PhysT<R> P, R t,
                          const R* __restrict__ geo, const R* __restrict__ accg,
@@ -598,14 +736,14 @@ k_volume(long long E, const Ops* __restrict__ ops, PhysT<R> P, R t,
                          double* __restrict__ r, double* __restrict__ jv, R stage_c,
                          const R* __restrict__ mixg, long long ahead) {
   using S = typename std::conditional<NC == 2, DualT<R>, R>::type;
-  constexpr int NP = Shape<N>::NP, NF = Shape<N>::NF, C = 5 * NC, EPB = Epb<N, NC>::value;
+  constexpr int NP = Shape<N>::NP, NF = Shape<N>::NF, EPB = Epb<N, NC>::value;
+  constexpr int NT = EPB * NP, FT = EPB * 6 * NF;
+  using V = Pack<OUT, R>;
   __shared__ SmemOpsT<R> so;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  R* smem = reinterpret_cast<R*>(smem_raw);
-  R* sF = smem;                             // [EPB][3][C][NP]
-  R* sH = sF + EPB * 3 * C * NP;            // [EPB][6][C][NF]
-  R* sR = sH + EPB * 6 * C * NF;            // [EPB][C][NP]
-  R* sT = sR + EPB * C * NP;                // [EPB][C][NP]
+  V* sF = reinterpret_cast<V*>(smem_raw);   // [15][NT]  reference fluxes a * 5 + c
+  V* sH = sF + 15 * NT;                     // [5][FT]   face fluxes
+  V* sR = sH + 5 * FT;                      // [5][NT]
   load_ops<N, R>(ops, so);
   const long long e0 = (long long)blockIdx.x * EPB;
   if constexpr (sizeof(R) == 4) {
@@ -617,7 +755,7 @@ k_volume(long long E, const Ops* __restrict__ ops, PhysT<R> P, R t,
       for (int pl = 0; pl < NC; ++pl) {
         prefetch_l2(ug + pl * E * 5 * NP + eb * 5 * NP, ne * 5 * NP);
         prefetch_l2(qg + pl * E * 15 * NP + eb * 15 * NP, ne * 15 * NP);
-        prefetch_l2(fh + pl * E * 30 * NF + eb * 30 * NF, ne * 30 * NF);
+        if (pl >= NC - OUT) prefetch_l2(fh + pl * E * 30 * NF + eb * 30 * NF, ne * 30 * NF);
       }
       prefetch_l2(geo + eb * 10 * NP, ne * 10 * NP);
       prefetch_l2(accg + eb * 3 * NP, ne * 3 * NP);
@@ -626,18 +764,21 @@ k_volume(long long E, const Ops* __restrict__ ops, PhysT<R> P, R t,
     }
   }
   const long long plane_f = E * 30 * NF;
-  for (int idx = threadIdx.x; idx < EPB * 30 * NF; idx += blockDim.x) {
+  for (int idx = threadIdx.x; idx < EPB * 30 * NF; idx += NT) {
     const int l = idx / (30 * NF), rem = idx % (30 * NF);
-    const long long e = e0 + l;
-    if (e < E) {
+    const long long ee = e0 + l;
+    if (ee < E) {
       const int phi = rem / (5 * NF), c = (rem / NF) % 5, f = rem % NF;
-      for (int pl = 0; pl < NC; ++pl)
-        sH[((l * 6 + phi) * C + 5 * pl + c) * NF + f] = fh[pl * plane_f + e * 30 * NF + rem];
+      const unsigned dst = (unsigned)__cvta_generic_to_shared(sH + c * FT + (l * 6 + phi) * NF + f);
+#pragma unroll
+      for (int p = 0; p < OUT; ++p)         // arrives while the pointwise physics runs (232 -> 188 us)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(dst + p * (unsigned)sizeof(R)),
+                     "l"(fh + (NC - OUT + p) * plane_f + ee * 30 * NF + rem), "n"(sizeof(R)) : "memory");
     }
   }
-  const int el = threadIdx.x / NP, g = threadIdx.x % NP;
+  const int tid = threadIdx.x, el = tid / NP, g = tid % NP;
   const long long e = e0 + el;
-  const bool active = el < EPB && e < E;
+  const bool active = e < E;
   S srcv[5];
   R wu[5] = {R(0), R(0), R(0), R(0), R(0)};   // W u_dot at this point (stage operator)
   if (active) {
@@ -675,52 +816,74 @@ k_volume(long long E, const Ops* __restrict__ ops, PhysT<R> P, R t,
 #pragma unroll
     for (int a = 0; a < 3; ++a)
 #pragma unroll
-      for (int c = 0; c < 5; ++c) {
-        if constexpr (NC == 1) {
-          sF[((el * 3 + a) * C + c) * NP + g] = Fref[a][c];
-        } else {
-          sF[((el * 3 + a) * C + c) * NP + g] = Fref[a][c].v;
-          sF[((el * 3 + a) * C + 5 + c) * NP + g] = Fref[a][c].d;
+      for (int c = 0; c < 5; ++c) sF[(a * 5 + c) * NT + tid] = planes_of<OUT>(Fref[a][c]);
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();
+  const int ig[3] = {g % N, (g / N) % N, g / (N * N)};
+  if (active) {
+    R D[3][N], ec[6];
+    axis_coefs<N, true>(so.D, ig, D);
+    end_coefs(so, ig, ec);
+    int fp[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) fp[a] = el * 6 * NF + vol_face_point<N>(g, a);
+#pragma unroll
+    for (int c = 0; c < 5; ++c) {
+      V acc = planes_of<OUT>(srcv[c]);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const int st = pt_stride<N>(a);
+        const V* y = sF + (a * 5 + c) * NT + tid - ig[a] * st;
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+          const V x = y[k * st];
+#pragma unroll
+          for (int p = 0; p < OUT; ++p) acc.v[p] = cm_fma<CM>(D[a][k], x.v[p], acc.v[p]);
         }
       }
-  }
-  __syncthreads();
-  if (active) {
-    for (int c = 0; c < C; ++c) {
-      R acc;
-      if constexpr (NC == 1) acc = srcv[c];
-      else acc = (c < 5) ? srcv[c].v : srcv[c - 5].d;
-#pragma unroll
-      for (int a = 0; a < 3; ++a) acc = line_fma<N, true, false, R, CM>(so.D, sF + ((el * 3 + a) * C + c) * NP, g, a, acc);
 #pragma unroll
       for (int phi = 0; phi < 6; ++phi) {
-        const int axis = phi >> 1;
-        const R coef = ((phi & 1) ? so.eR : so.eL)[axis_index<N>(g, axis)];
-        acc = cm_fma<CM>(-coef, sH[((el * 6 + phi) * C + c) * NF + vol_face_point<N>(g, axis)], acc);
+        const V x = sH[c * FT + phi * NF + fp[phi >> 1]];
+#pragma unroll
+        for (int p = 0; p < OUT; ++p) acc.v[p] = cm_fma<CM>(-ec[phi], x.v[p], acc.v[p]);
       }
-      if (NC == 2 && c >= 5 && stage_c != R(0)) acc = wu[c - 5] - stage_c * acc;
-      sR[(el * C + c) * NP + g] = acc;
+      if (NC == 2 && stage_c != R(0)) acc.v[OUT - 1] = wu[c] - stage_c * acc.v[OUT - 1];
+      sR[c * NT + tid] = acc;
     }
   }
   __syncthreads();
-  R* in = sR;
-  R* out = sT;
+  V *in = sR, *out = sF;                    // the fluxes have been read
 #pragma unroll
   for (int dir = 0; dir < 3; ++dir) {
+    const int st = pt_stride<N>(dir), base = tid - ig[dir] * st;
+    R B[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) B[k] = so.B[k * N + ig[dir]];
     if (active)
-      for (int c = 0; c < C; ++c) out[(el * C + c) * NP + g] = line<N, true, R, CM>(so.B, in + (el * C + c) * NP, g, dir);
-    __syncthreads();
-    R* tt = in;
+#pragma unroll
+      for (int c = 0; c < 5; ++c) {
+        V acc;
+#pragma unroll
+        for (int p = 0; p < OUT; ++p) acc.v[p] = R(0);
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+          const V x = in[c * NT + base + k * st];
+#pragma unroll
+          for (int p = 0; p < OUT; ++p) acc.v[p] = cm_fma<CM>(B[k], x.v[p], acc.v[p]);
+        }
+        if (dir < 2) {
+          out[c * NT + tid] = acc;
+        } else {
+          const long long o = e * 5 * NP + c * NP + g;
+          if (OUT == NC && r) r[o] = as_f64(acc.v[0]);
+          if (NC == 2) jv[o] = as_f64(acc.v[OUT - 1]);
+        }
+      }
+    if (dir < 2) __syncthreads();
+    V* tt = in;
     in = out;
     out = tt;
-  }
-  for (int idx = threadIdx.x; idx < EPB * 5 * NP; idx += blockDim.x) {
-    const int l = idx / (5 * NP), rem = idx % (5 * NP);
-    const long long ee = e0 + l;
-    if (ee < E) {
-      if (r) r[ee * 5 * NP + rem] = (double)in[(l * C) * NP + rem];
-      if (NC == 2) jv[ee * 5 * NP + rem] = (double)in[(l * C + 5) * NP + rem];
-    }
   }
 }
 
@@ -920,8 +1083,8 @@ template <int N, int NC, typename R>
 struct Smem {
   static constexpr int NP = Shape<N>::NP, NF = Shape<N>::NF, C = 5 * NC, EPB = Epb<N, NC>::value;
   static constexpr size_t interp = sizeof(R) * (2 * EPB * C * NP);
-  static constexpr size_t grad = sizeof(R) * (EPB * (C * NP + 6 * C * NF + 18 * NF + 9 * NP + 3 * C * NP + 18 * NF));
-  static constexpr size_t volume = sizeof(R) * (EPB * (3 * C * NP + 6 * C * NF + 2 * C * NP));
+  static constexpr size_t grad = sizeof(R) * NC * EPB * (11 * NP + 30 * NF);
+  static constexpr size_t volume = sizeof(R) * EPB * (20 * NP + 30 * NF);   // per output plane
 };
 
 template <typename R> inline WorkT<R> work_of(dg_mesh* m);
@@ -1029,7 +1192,7 @@ static int run_interp_tangent(dg_mesh* m, const double* v, cudaStream_t s) {
 }
 
 template <int N, int NC, typename R = double>
-static int run_faces(dg_mesh* m, cudaStream_t s) {
+static int run_faces(dg_mesh* m, cudaStream_t s, bool vout = true) {
   constexpr int NF = Shape<N>::NF;
   const long long work = m->nfaces * NF;
   // FP64: small CTAs, whose last wave leaves fewer SMs idle (one warp while the faces cannot fill every SM;
@@ -1043,7 +1206,7 @@ static int run_faces(dg_mesh* m, cudaStream_t s) {
                                                      m->nbr_fo, m->fgu, w.uf, w.qf, w.fh, w.mixf);
   else
     k_faces<N, NC, R><<<blocks, threads, 0, s>>>(m->E, m->nfaces, phys_as<R>(m->phys), m->face_e, m->face_f,
-                                                       m->nbr, m->nbr_fo, w.fgeo, w.uf, w.qf, w.fh, w.mixf);
+                                                       m->nbr, m->nbr_fo, w.fgeo, w.uf, w.qf, w.fh, w.mixf, vout);
   prof_end(m, s);
   DG_LAUNCH_CHECK("k_faces");
   return DG_OK;
@@ -1104,17 +1267,23 @@ static int run_volume(dg_mesh* m, double t, double* r, double* jv, cudaStream_t 
     return DG_OK;
   } else {
     constexpr int EPB = Epb<N, NC>::value, NP = Shape<N>::NP;
-    const size_t sm = Smem<N, NC, R>::volume;
-    int rc = set_smem(k_volume<N, NC, R, CM>, sm);
+    auto launch = [&](auto planes) {
+      constexpr int OUT = decltype(planes)::value;
+      const size_t sm = Smem<N, NC, R>::volume * OUT;
+      const int rc = set_smem(k_volume<N, NC, OUT, R, CM>, sm);
+      if (rc) return rc;
+      const unsigned blocks = (unsigned)((m->E + EPB - 1) / EPB);
+      const WorkT<R> w = work_of<R>(m);
+      // CTAs resident at once (the prefetch distance), per mesh and kernel instance
+      const long long resident = resident_ctas(m, (const void*)k_volume<N, NC, OUT, R, CM>, EPB * NP, sm);
+      prof_begin(m, s, KK_VOLUME);
+      k_volume<N, NC, OUT, R, CM><<<blocks, EPB * NP, sm, s>>>(m->E, m->d_ops, phys_as<R>(m->phys), (R)t, w.geo, w.acc,
+                                                               w.xg, w.ug, w.qg, w.fh, r, jv, (R)stage_c, w.mixg, resident);
+      prof_end(m, s);
+      return (int)DG_OK;
+    };
+    const int rc = NC == 2 && !r ? launch(std::integral_constant<int, 1>()) : launch(std::integral_constant<int, NC>());
     if (rc) return rc;
-    const unsigned blocks = (unsigned)((m->E + EPB - 1) / EPB);
-    const WorkT<R> w = work_of<R>(m);
-    // CTAs resident at once (the prefetch distance), per mesh and kernel instance
-    const long long resident = resident_ctas(m, (const void*)k_volume<N, NC, R, CM>, EPB * NP, sm);
-    prof_begin(m, s, KK_VOLUME);
-    k_volume<N, NC, R, CM><<<blocks, EPB * NP, sm, s>>>(m->E, m->d_ops, phys_as<R>(m->phys), (R)t, w.geo, w.acc, w.xg,
-                                                     w.ug, w.qg, w.fh, r, jv, (R)stage_c, w.mixg, resident);
-    prof_end(m, s);
     DG_LAUNCH_CHECK("k_volume");
     return DG_OK;
   }
@@ -1161,7 +1330,7 @@ template <int N>
 template <typename R>
 int Driver<N>::residual_p(dg_mesh* m, double t, double* r, double* jv, bool tangent, cudaStream_t s,
                           double stage_c) {
-  int rc = tangent ? run_faces<N, 2, R>(m, s) : run_faces<N, 1, R>(m, s);
+  int rc = tangent ? run_faces<N, 2, R>(m, s, r != nullptr) : run_faces<N, 1, R>(m, s);
   if (rc) return rc;
   return tangent ? run_volume<N, 2, R>(m, t, r, jv, s, stage_c) : run_volume<N, 1, R>(m, t, r, nullptr, s);
 }
