@@ -134,6 +134,38 @@ __global__ void k_scale_dev(long long n, const double* x, const double* __restri
     out[i] = x[i] * s;
 }
 
+// The threads' sums acc[0..K-1] of a block to rows row0.. of partial: through shared memory, eight rows at a
+// time, a warp adding one row's RED_THREADS values, eight per lane and then a shuffle tree. FP64 additions cost
+// 16 cycles of the SM's pipe per warp: 13 of them per row, where a tree in every warp took 48. (With
+// k_scale_to_f32 below: vector kernels of a reduced-basis step on 1.66 M entries 13.4 -> 10.6 ms, of a
+// block-Jacobi step on 0.31 M entries 6.8 -> 6.0.)
+constexpr int RED_ROWS = RED_THREADS / 32;
+__device__ __forceinline__ double sum_f64(double x) { return x; }
+__device__ __forceinline__ double sum_f64(float x) { return to_f64(x); }
+template <typename T>
+__device__ __forceinline__ void row_to_partial(const T* row, double* out) {
+  const int lane = threadIdx.x & 31;
+  double v = 0.0;
+#pragma unroll
+  for (int q = 0; q < RED_ROWS; ++q) v += sum_f64(row[lane + 32 * q]);
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+  if (lane == 0) out[blockIdx.x] = v;
+}
+template <int K, typename T>
+__device__ __forceinline__ void rows_to_partials(const T (&acc)[K], int row0, double* __restrict__ partial) {
+  __shared__ T buf[(K < RED_ROWS ? K : RED_ROWS) * RED_THREADS];
+  const int warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int r0 = 0; r0 < K; r0 += RED_ROWS) {
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < RED_ROWS; ++j)
+      if (r0 + j < K) buf[j * RED_THREADS + threadIdx.x] = acc[r0 + j < K ? r0 + j : 0];
+    __syncthreads();
+    if (r0 + warp < K) row_to_partial(buf + warp * RED_THREADS, partial + (size_t)(row0 + r0 + warp) * RED_BLOCKS);
+  }
+}
+
 // partial[j][block] = sum_i V_j[i] w[i] for j < k; partial[k][block] = sum_i w[i]^2.
 // Vectors are taken 16 at a time (one pass over w per group) so the accumulators stay in
 // registers; warp-shuffle and cross-warp reductions, fixed order.
@@ -245,20 +277,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_mdot_k(long long n2, const doub
     }
     acc[K] = fma(x.x, x.x, fma(x.y, x.y, acc[K]));
   }
-  __shared__ double red[RED_THREADS / 32][K + 1];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int j = 0; j <= K; ++j) {
-    double v = acc[j];
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-    if (lane == 0) red[warp][j] = v;
-  }
-  __syncthreads();
-  for (int j = threadIdx.x; j <= K; j += blockDim.x) {
-    double v = 0.0;
-    for (int q = 0; q < RED_THREADS / 32; ++q) v += red[q][j];
-    partial[j * RED_BLOCKS + blockIdx.x] = v;
-  }
+  rows_to_partials(acc, 0, partial);
 }
 
 template <int K, bool DOTS>
@@ -315,21 +334,13 @@ __global__ void __launch_bounds__(RED_THREADS, 2) k_update_dot_k(long long n2, c
     }
     acc[NR - 1] = fma(x.x, x.x, fma(x.y, x.y, acc[NR - 1]));
   }
-  constexpr int NA = DOTS ? K + 1 : 1;
-  __shared__ double red[RED_THREADS / 32][NA];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int j = 0; j < NA; ++j) {
-    double a;
-    if constexpr (SACC) a = (j < K) ? sacc[j * RED_THREADS + threadIdx.x] : acc[0];
-    else a = (NR == 1) ? acc[0] : acc[j < NR ? j : NR - 1];
-    for (int off = 16; off > 0; off >>= 1) a += __shfl_down_sync(0xffffffffu, a, off);
-    if (lane == 0) red[warp][j] = a;
-  }
-  __syncthreads();
-  for (int j = threadIdx.x; j < NA; j += blockDim.x) {
-    double a = 0.0;
-    for (int q = 0; q < RED_THREADS / 32; ++q) a += red[q][j];
-    partial[j * RED_BLOCKS + blockIdx.x] = a;
+  if constexpr (SACC) {                             // (row K: |w|^2)
+    __syncthreads();
+    for (int j = threadIdx.x >> 5; j < K; j += RED_ROWS)
+      row_to_partial(sacc + j * RED_THREADS, partial + (size_t)j * RED_BLOCKS);
+    rows_to_partials(acc, K, partial);
+  } else {
+    rows_to_partials(acc, 0, partial);
   }
 }
 
@@ -355,22 +366,9 @@ __global__ void __launch_bounds__(RED_THREADS, 2) k_mdot_f32(long long n2, const
     }
     nrm = fma(x.x, x.x, fma(x.y, x.y, nrm));
   }
-  __shared__ double red[RED_THREADS / 32][K + 1];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int j = 0; j < K; ++j) {
-    double v = to_f64(acc[j]);
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-    if (lane == 0) red[warp][j] = v;
-  }
-  for (int off = 16; off > 0; off >>= 1) nrm += __shfl_down_sync(0xffffffffu, nrm, off);
-  if (lane == 0) red[warp][K] = nrm;
-  __syncthreads();
-  for (int j = threadIdx.x; j <= K; j += blockDim.x) {
-    double v = 0.0;
-    for (int q = 0; q < RED_THREADS / 32; ++q) v += red[q][j];
-    partial[j * RED_BLOCKS + blockIdx.x] = v;
-  }
+  rows_to_partials(acc, 0, partial);
+  const double sq[1] = {nrm};
+  rows_to_partials(sq, K, partial);
 }
 
 // k_update_dot_k with the correction sum_j h_j V_j formed in FP32 and subtracted from w in FP64
@@ -420,26 +418,10 @@ __global__ void __launch_bounds__(RED_THREADS, 2) k_update_dot_f32(long long n2,
     }
     nrm = fma(x.x, x.x, fma(x.y, x.y, nrm));
   }
-  __shared__ double red[RED_THREADS / 32][NA + 1];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if constexpr (DOTS) {
-#pragma unroll
-    for (int j = 0; j < K; ++j) {
-      double a = to_f64(acc[j]);
-      for (int off = 16; off > 0; off >>= 1) a += __shfl_down_sync(0xffffffffu, a, off);
-      if (lane == 0) red[warp][j] = a;
-    }
-  }
-  for (int off = 16; off > 0; off >>= 1) nrm += __shfl_down_sync(0xffffffffu, nrm, off);
-  if (lane == 0) red[warp][NA] = nrm;
-  __syncthreads();
   // DOTS: rows 0..K-1 the dots, row K |w|^2; otherwise row 0 |w|^2
-  for (int j = threadIdx.x; j < (DOTS ? K + 1 : 1); j += blockDim.x) {
-    const int src = DOTS ? j : NA;
-    double a = 0.0;
-    for (int q = 0; q < RED_THREADS / 32; ++q) a += red[q][src];
-    partial[j * RED_BLOCKS + blockIdx.x] = a;
-  }
+  if constexpr (DOTS) rows_to_partials(acc, 0, partial);
+  const double sq[1] = {nrm};
+  rows_to_partials(sq, DOTS ? K : 0, partial);
 }
 
 // The same two sweeps on an FP32-stored basis (the mixed-precision solve keeps its Krylov vectors
@@ -461,22 +443,9 @@ __global__ void __launch_bounds__(RED_THREADS, 2) k_mdot_f32v(long long n2, cons
     }
     nrm = fma(x.x, x.x, fma(x.y, x.y, nrm));
   }
-  __shared__ double red[RED_THREADS / 32][K + 1];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int j = 0; j < K; ++j) {
-    double v = to_f64(acc[j]);
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-    if (lane == 0) red[warp][j] = v;
-  }
-  for (int off = 16; off > 0; off >>= 1) nrm += __shfl_down_sync(0xffffffffu, nrm, off);
-  if (lane == 0) red[warp][K] = nrm;
-  __syncthreads();
-  for (int j = threadIdx.x; j <= K; j += blockDim.x) {
-    double v = 0.0;
-    for (int q = 0; q < RED_THREADS / 32; ++q) v += red[q][j];
-    partial[j * RED_BLOCKS + blockIdx.x] = v;
-  }
+  rows_to_partials(acc, 0, partial);
+  const double sq[1] = {nrm};
+  rows_to_partials(sq, K, partial);
 }
 
 template <int K, bool DOTS>
@@ -518,41 +487,28 @@ __global__ void __launch_bounds__(RED_THREADS, 2) k_update_dot_f32v(long long n2
     }
     nrm = fma(x.x, x.x, fma(x.y, x.y, nrm));
   }
-  __shared__ double red[RED_THREADS / 32][NA + 1];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if constexpr (DOTS) {
-#pragma unroll
-    for (int j = 0; j < K; ++j) {
-      double a = to_f64(acc[j]);
-      for (int off = 16; off > 0; off >>= 1) a += __shfl_down_sync(0xffffffffu, a, off);
-      if (lane == 0) red[warp][j] = a;
-    }
-  }
-  for (int off = 16; off > 0; off >>= 1) nrm += __shfl_down_sync(0xffffffffu, nrm, off);
-  if (lane == 0) red[warp][NA] = nrm;
-  __syncthreads();
-  for (int j = threadIdx.x; j < (DOTS ? K + 1 : 1); j += blockDim.x) {
-    const int src = DOTS ? j : NA;
-    double a = 0.0;
-    for (int q = 0; q < RED_THREADS / 32; ++q) a += red[q][src];
-    partial[j * RED_BLOCKS + blockIdx.x] = a;
-  }
+  // DOTS: rows 0..K-1 the dots, row K |w|^2; otherwise row 0 |w|^2
+  if constexpr (DOTS) rows_to_partials(acc, 0, partial);
+  const double sq[1] = {nrm};
+  rows_to_partials(sq, DOTS ? K : 0, partial);
 }
 
-// out = a x in FP32 (a new basis vector), and the FP32 vector widened back to FP64
-__global__ void k_scale_to_f32(long long n, const double* __restrict__ x, double a, const double* __restrict__ den,
-                               float* __restrict__ out) {
-  __shared__ float sf_sh;   // the scale formed once per block
+// A new FP32 basis vector out = a x (a = 1 / sqrt(*den) if given) and the same widened to FP64, which the
+// preconditioner reads; n even. A few blocks per SM loop over the entries: each forms the scale once, an FP64
+// square root and division in sequence.
+__global__ void __launch_bounds__(256) k_scale_to_f32(long long n2, const double2* __restrict__ x, double a,
+                                                      const double* __restrict__ den, float2* __restrict__ out,
+                                                      double2* __restrict__ wide) {
+  __shared__ float sf_sh;
   if (threadIdx.x == 0) sf_sh = den ? (float)(1.0 / sqrt(*den)) : (float)a;
   __syncthreads();
   const float sf = sf_sh;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    out[i] = to_f32(x[i]) * sf;
-}
-
-__global__ void k_widen(long long n, const float* __restrict__ x, double* __restrict__ out) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    out[i] = to_f64(x[i]);
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n2; i += (long long)gridDim.x * blockDim.x) {
+    const double2 v = x[i];
+    const float2 f = make_float2(to_f32(v.x) * sf, to_f32(v.y) * sf);
+    out[i] = f;
+    wide[i] = make_double2(to_f64(f.x), to_f64(f.y));
+  }
 }
 
 // out = sum_j y[j] V_j (j < k) on the FP32 basis, FP32 sums widened to FP64
@@ -1502,6 +1458,12 @@ static void update_dot_f32v(long long n, int k, const float* V, const double* h,
   }
 }
 
+static void scale_to_f32(long long n, const double* x, double a, const double* den, float* out, double* wide,
+                         cudaStream_t s) {
+  k_scale_to_f32<<<std::min(grid_for(n / 2), 4u * 152u), 256, 0, s>>>(
+      n / 2, reinterpret_cast<const double2*>(x), a, den, reinterpret_cast<float2*>(out), reinterpret_cast<double2*>(wide));
+}
+
 // J_G v = M v - c J_r(U) v
 static int stage_matvec(dg_mesh* m, Solver* S, const double* U, double t, double c, int jv_mode, int jv_prec,
                         const double* v, double* out, cudaStream_t s, bool value_ready = false) {
@@ -1719,7 +1681,7 @@ static int rb_orthonormalise(dg_mesh* m, Solver* S, cudaStream_t s) {
     if (!std::isfinite(n0) || !std::isfinite(nf)) return fail(DG_ENAN, "reduced basis: non-finite Newton update");
     if (!(n0 > 0.0) || !(nf > 1e-20 * n0)) continue;
     prof_begin(m, s, KK_BLAS);
-    k_scale_dev<<<grid_for(n), 256, 0, s>>>(n, w, S->hdev + 2 * MAXK - 1, w);
+    k_scale_dev<<<std::min(grid_for(n), 4u * 152u), 256, 0, s>>>(n, w, S->hdev + 2 * MAXK - 1, w);
     prof_end(m, s);
     DG_LAUNCH_CHECK("k_scale_dev");
     ++r;
@@ -1933,7 +1895,7 @@ static int gmres(dg_mesh* m, Solver* S, const dg_solver_opts& o, const double* U
     if (rc) return rc;
     if (!std::isfinite(beta)) return fail(DG_ENAN, "GMRES: non-finite residual");
     if (beta <= o.gmres_rtol * bnorm) return DG_OK;
-    if (f32basis) k_scale_to_f32<<<grid_for(n), 256, 0, s>>>(n, r, 1.0 / beta, nullptr, Vf);
+    if (f32basis) scale_to_f32(n, r, 1.0 / beta, nullptr, Vf, S->v(VTMP), s);
     else k_lincomb<<<grid_for(n), 256, 0, s>>>(n, 1.0 / beta, r, 0.0, nullptr, 0.0, nullptr, V);
     DG_LAUNCH_CHECK("k_lincomb");
     std::fill(g.begin(), g.end(), 0.0);
@@ -1941,11 +1903,7 @@ static int gmres(dg_mesh* m, Solver* S, const dg_solver_opts& o, const double* U
     int kdone = 0;
     bool converged = false;
     for (int k = 0; k < R; ++k) {
-      if (f32basis) {
-        prof_begin(m, s, KK_BLAS);
-        k_widen<<<grid_for(n), 256, 0, s>>>(n, Vf + (long long)k * n, S->v(VTMP));
-        prof_end(m, s);
-        DG_LAUNCH_CHECK("k_widen");
+      if (f32basis) {                         // VTMP: the widened vector
         rc = precond_apply(m, S, o.precond, S->v(VTMP), z, s);
       } else {
         rc = precond_apply(m, S, o.precond, V + (long long)k * n, z, s);
@@ -1965,7 +1923,7 @@ static int gmres(dg_mesh* m, Solver* S, const dg_solver_opts& o, const double* U
         k_mdot_finish<<<k + 1, 32, 0, s>>>(S->partial, S->hdev + MAXK);
         update_dot_f32v(n, k + 1, Vf, S->hdev + MAXK, w, S->partial, false, s);
         k_mdot_finish<<<1, 32, 0, s>>>(S->partial, S->hdev + MAXK + k + 1);
-        k_scale_to_f32<<<grid_for(n), 256, 0, s>>>(n, w, 0.0, S->hdev + MAXK + k + 1, Vf + (long long)(k + 1) * n);
+        scale_to_f32(n, w, 0.0, S->hdev + MAXK + k + 1, Vf + (long long)(k + 1) * n, S->v(VTMP), s);
       } else {
         mdot(n, k + 1, V, w, S->partial, s, f32gs);
         k_mdot_finish<<<k + 1, 32, 0, s>>>(S->partial, S->hdev);
@@ -1973,7 +1931,7 @@ static int gmres(dg_mesh* m, Solver* S, const dg_solver_opts& o, const double* U
         k_mdot_finish<<<k + 1, 32, 0, s>>>(S->partial, S->hdev + MAXK);
         update_dot(n, k + 1, V, S->hdev + MAXK, w, S->partial, false, s, f32gs);
         k_mdot_finish<<<1, 32, 0, s>>>(S->partial, S->hdev + MAXK + k + 1);
-        k_scale_dev<<<grid_for(n), 256, 0, s>>>(n, w, S->hdev + MAXK + k + 1, V + (long long)(k + 1) * n);
+        k_scale_dev<<<std::min(grid_for(n), 4u * 152u), 256, 0, s>>>(n, w, S->hdev + MAXK + k + 1, V + (long long)(k + 1) * n);
       }
       prof_end(m, s);
       DG_LAUNCH_CHECK("arnoldi");
