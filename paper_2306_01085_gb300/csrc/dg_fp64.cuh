@@ -893,10 +893,10 @@ __device__ __noinline__ void volume_slow(const XOps<N>& so, long long e, long lo
 
 // stage_c != 0 (NC = 2): the tangent output is the DIRK stage operator J_G v = M v - stage_c J_r v. It is
 // formed as -stage_c (J_r v - M v / stage_c), with -|J| u_dot / stage_c added to the tangent's source.
-// Four CTAs of 128 threads instead of three hide more of the pointwise physics' latency although some
-// registers spill (Jv of a 16x16x8 degree-4 shell 3233 -> 3208 us).
+// CTAs per SM: latency of the pointwise physics against spills (Jv of a 16x16x8 degree-4 shell: 3 CTAs 1135 us, 4
+// 1066, 5 1160; r of a 21x21x9 degree-3 shell: 3 CTAs 748, 4 685, 5 651).
 template <int N, int NC>
-__global__ void __launch_bounds__(128, 4)
+__global__ void __launch_bounds__(128, NC == 2 ? 4 : 5)
     k_volume64(long long E, const Ops* __restrict__ ops, PhysT<double> P, Sun64 sun, const double* __restrict__ gu,
                const double* __restrict__ accg, const double* __restrict__ xg, const double* __restrict__ ug,
                const double* __restrict__ qg, const double* __restrict__ fh, double* __restrict__ r,

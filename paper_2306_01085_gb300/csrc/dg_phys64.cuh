@@ -49,8 +49,7 @@ __device__ __forceinline__ D64 s_isr(D64 u0) {
 // T^a with T = u4 e^{-varrho/2}: exp(a (log u4 - varrho/2)); dl is d(log T) of the tangent
 __device__ __forceinline__ double t_power(double a, double u0, double u4, double dl) {
   (void)dl;
-  if (!positive_normal(u4)) return exp(a * log(u4 * exp(-0.5 * u0)));
-  return exp_fast(a * fma(-0.5, u0, log_fast(u4)));
+  return power_fast(a, u4, u0);
 }
 __device__ __forceinline__ D64 t_power(double a, D64 u0, D64 u4, double dl) {
   const double p = t_power(a, u0.v, u4.v, 0.0);
