@@ -728,6 +728,142 @@ __global__ void __launch_bounds__(128) k_rband_lu(int n, long long nc, float* __
   if (bad && lane == 0) atomicOr(info, 1);
 }
 
+// The same factorisation for KL + 1 <= 32 (degrees 1 and 2) with the active window in registers: a lane holds one
+// row, entry q of it in column j + q at step j, and knows which logical row it is, so that a row interchange
+// only changes a number. Per step the pivot's lane writes its row to shared memory, every lane reads it back
+// as broadcasts and updates its own row, one entry further left (the window moves by one column), and the
+// pivot's lane takes the next row. The kernel above spends about eleven instructions per column and step and
+// waits for its stores in global memory; here it is one FMA and a fraction of a shared-memory access (252
+// rows: 25 systems 481 -> 119 us, 2,475 systems 763 -> 404; at 9 warps per SM, 25 KB each, it waits for its own
+// chain of pivot, reciprocal and broadcast). Rows to come are gathered from the band's columns by asynchronous
+// copies into row order; U's rows wait in a ring until their column is complete, so that all global accesses
+// run along columns. Stored factors are those of the kernel above.
+template <int N>
+struct LuWin {
+  static constexpr int KL = Band<N>::KL, KV = 2 * KL, NC = KV + 1, XW = (NC + 3) / 4 * 4;   // window width, padded
+  static constexpr int PF = 4, SR = NC + PF + 1, UR = NC;      // columns copied ahead; rows to come; U's rows
+  static constexpr size_t smem = sizeof(float) * XW * (SR + UR);
+};
+template <int N>
+__global__ void __launch_bounds__(32) k_rband_lu_reg(int n, float* __restrict__ ab, int* __restrict__ ipiv,
+                                                     int* __restrict__ info) {
+  using L = LuWin<N>;
+  constexpr int KL = L::KL, KV = L::KV, LD = Band<N>::LD, NC = L::NC, XW = L::XW, SR = L::SR, UR = L::UR, PF = L::PF;
+  constexpr int GONE = 1 << 30;                 // logical row of a lane without one
+  extern __shared__ __align__(16) float lu_sm[];
+  float *stage = lu_sm, *ur = lu_sm + SR * XW;  // [SR][XW] rows i in slot i mod SR; [UR][XW] U's rows j mod UR
+  const int lane = threadIdx.x;
+  float* A0 = ab + (long long)blockIdx.x * n * LD;
+  int* pv = ipiv + (long long)blockIdx.x * n;
+  constexpr int NK = (NC + 31) / 32;
+  // column c = 0, 1, .. of the band into the rows below the first KL + 1, one group per call: entry k of this
+  // lane is row c - KL + k, its place in the ring advances by a row
+  const float* fsrc[NK];
+  int frow[NK], fdst[NK];
+#pragma unroll
+  for (int t = 0; t < NK; ++t) {
+    const int k = lane + 32 * t;
+    frow[t] = k < NC ? k - KL : GONE;
+    fdst[t] = (k - KL + 2 * SR) % SR * XW + KV - k;
+    fsrc[t] = A0 + KL + k;
+  }
+  auto fetch = [&](bool in) {
+#pragma unroll
+    for (int t = 0; t < NK; ++t) {
+      if (in && frow[t] > KL && frow[t] < n)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(stage + fdst[t])),
+                     "l"(fsrc[t]) : "memory");
+      if (frow[t] < GONE) ++frow[t];
+      fdst[t] += XW;
+      if (fdst[t] >= SR * XW) fdst[t] -= SR * XW;
+      fsrc[t] += LD;
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  for (int c = 0; c < NC + PF; ++c) fetch(c < n);
+  int row = lane <= KL && lane < n ? lane : GONE;
+  float x[XW];
+#pragma unroll
+  for (int q = 0; q < XW; ++q) x[q] = row < GONE && q < NC && q < n && q <= row + KL ? A0[(long long)q * LD + KV + row - q] : 0.0f;
+  int bad = 0, us = 0, ns = (KL + 1) % SR;      // j mod UR, (j + KL + 1) mod SR
+  int uoff[NK];                                 // entry k of row j - k of U
+#pragma unroll
+  for (int t = 0; t < NK; ++t) uoff[t] = (2 * UR - (lane + 32 * t)) % UR * XW + lane + 32 * t;
+  for (int j = 0; j < n; ++j) {
+    // the largest magnitude by its bits (NaN above Inf), then the smallest row that has it
+    const unsigned mag = row < GONE ? __float_as_uint(x[0]) & 0x7fffffffu : 0u;
+    const unsigned best = __reduce_max_sync(0xffffffffu, mag);
+    unsigned who = __ballot_sync(0xffffffffu, mag == best && row < GONE);
+    if (best == 0u || best >= 0x7f800000u) {        // no elimination with this column: row j leaves as it is
+      bad = 1;
+      who = __ballot_sync(0xffffffffu, row == j);
+    } else if (who & (who - 1)) {
+      const int first = __reduce_min_sync(0xffffffffu, mag == best ? row : GONE);
+      who = __ballot_sync(0xffffffffu, row == first);
+    }
+    const int bl = __ffs(who) - 1, bi = __shfl_sync(0xffffffffu, row, bl);
+    const bool pivot = lane == bl;
+    if (pivot) {
+      pv[j] = bi;
+#pragma unroll
+      for (int q = 0; q < XW; q += 4) *reinterpret_cast<float4*>(ur + us * XW + q) = make_float4(x[q], x[q + 1], x[q + 2], x[q + 3]);
+    }
+    const float inv = 1.0f / __shfl_sync(0xffffffffu, x[0], bl);
+    if (row == j) row = bi;                     // the interchange (the pivot's lane takes another row below)
+    const float l = pivot || row == GONE || bad ? 0.0f : x[0] * inv;
+    if (!pivot && row < GONE) A0[(long long)j * LD + KV + row - j] = l;
+    const bool plain = __all_sync(0xffffffffu, isfinite(l));
+    __syncwarp();
+    // x - l p, shifted by one column
+    const float* p = ur + us * XW;
+    if (plain) {
+#pragma unroll
+      for (int q = 0; q < XW; q += 4) {
+        const float4 v = *reinterpret_cast<const float4*>(p + q);
+        if (q > 0) x[q - 1] = x[q] - l * v.x;
+        x[q] = x[q + 1] - l * v.y;
+        x[q + 1] = x[q + 2] - l * v.z;
+        x[q + 2] = x[q + 3] - l * v.w;
+      }
+    } else {                                    // a column in which the pivot's row is zero is left alone
+#pragma unroll
+      for (int q = 1; q < XW; ++q) x[q - 1] = p[q] != 0.0f ? x[q] - l * p[q] : x[q];
+    }
+    x[XW - 1] = 0.0f;
+    // column j of U is complete
+#pragma unroll
+    for (int t = 0; t < NK; ++t) {
+      const int k = lane + 32 * t;
+      if (k < NC && k <= j) A0[(long long)j * LD + KV - k] = ur[uoff[t]];
+      uoff[t] += XW;
+      if (uoff[t] >= UR * XW) uoff[t] -= UR * XW;
+    }
+    // the next row
+    asm volatile("cp.async.wait_group %0;" ::"n"(PF - 1) : "memory");   // column j + NC has arrived
+    __syncwarp();
+    if (pivot) {
+      const int i = j + KL + 1;
+      row = i < n ? i : GONE;
+      const float* src = stage + ns * XW;
+#pragma unroll
+      for (int q = 0; q < XW; q += 4) {
+        const float4 v = *reinterpret_cast<const float4*>(src + q);
+        x[q] = v.x;
+        x[q + 1] = v.y;
+        x[q + 2] = v.z;
+        x[q + 3] = v.w;
+      }
+#pragma unroll
+      for (int q = NC; q < XW; ++q) x[q] = 0.0f;
+    }
+    __syncwarp();
+    fetch(j + NC + PF < n);
+    us = us + 1 == UR ? 0 : us + 1;
+    ns = ns + 1 == SR ? 0 : ns + 1;
+  }
+  if (bad && lane == 0) atomicOr(info, 1);
+}
+
 // solve L U x = b in place on b (FP64 [n][nc] rows of the element-major ordering), FP32 products
 // accumulated in float-float pairs (hi + lo, about 48 bits: the accuracy of the former FP64
 // accumulation without the FP64 pipe, which issues 2 lanes per SM per cycle on this GPU); one warp
@@ -1132,7 +1268,14 @@ int jacobian_lu(dg_radial* m, const double* U, double t, double c, cudaStream_t 
   DG_LAUNCH_CHECK("k_rprobe");
   DG_CUDA_TRY(cudaMemsetAsync(m->info, 0, sizeof(int), s));
   rprof_begin(m, s, RK_LU);
-  k_rband_lu<N><<<blocks_for(32 * nc), kThreads, 0, s>>>(n, nc, m->band, m->ipiv, m->info);
+  if constexpr (Band<N>::KL < 32) {
+    const size_t smem = LuWin<N>::smem;
+    DG_CUDA_TRY(cudaFuncSetAttribute(k_rband_lu_reg<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    DG_CUDA_TRY(cudaFuncSetAttribute(k_rband_lu_reg<N>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
+    k_rband_lu_reg<N><<<(unsigned)nc, 32, smem, s>>>(n, m->band, m->ipiv, m->info);
+  } else {
+    k_rband_lu<N><<<blocks_for(32 * nc), kThreads, 0, s>>>(n, nc, m->band, m->ipiv, m->info);
+  }
   rprof_end(m, s);
   DG_LAUNCH_CHECK("k_rband_lu");
   return DG_OK;
