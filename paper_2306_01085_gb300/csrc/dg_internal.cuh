@@ -56,6 +56,9 @@ struct OpsLd {
   long double B[MAXN * MAXN], Binv[MAXN * MAXN], D[MAXN * MAXN], e[2][MAXN], w[MAXN], eta[MAXN], xi[MAXN];
 };
 void build_ops_ld(int n, OpsLd* ops);
+// B, Binv, D, eL, eR, w, eta, xi alone, evaluated in double: the node positions and the geometry that the FP32
+// path rounds come from these (a geometry that differs in its last FP64 bits rounds to another float here and there)
+void build_ops_geo(int n, Ops* ops);
 
 // --------------------------------------------------------------------------------------------
 // physics parameters (nondimensional, Sec. 2.4), passed by value to kernels
@@ -138,7 +141,7 @@ struct dg_mesh {
   int device;
   dg::Phys phys;
   dg::Ops ops;
-  dg::Ops* d_ops = nullptr;
+  dg::Ops *d_ops = nullptr, *d_ops_geo = nullptr;
   dg::EuvFx* d_euv = nullptr;   // EUVAC band tables (euv = DG_EUV_EUVAC only)
   double* x = nullptr;     // [E][3][Np] node coordinates
   double* geo = nullptr;   // [E][10][Np]: G[a][d] = W detJ dxi_a/dx_d (9), W detJ (1)

@@ -959,7 +959,8 @@ __global__ void k_mixture(long long E, const Ops* __restrict__ ops, Phys P, cons
 // --------------------------------------------------------------------------------------------
 // geometry at Gauss points and face points (isoparametric map of the node coordinates)
 // --------------------------------------------------------------------------------------------
-template <int N>
+// UNW: gu and fgu, without weights, for the FP64 kernels; else geo, acc, xg and fgeo
+template <int N, bool UNW>
 __global__ void k_geometry(long long E, const Ops* __restrict__ ops, Phys P, int gravity_kind,
                            double g0, double g1, double g2, double g_r0,
                            const double* __restrict__ x, double* __restrict__ geo,
@@ -1017,30 +1018,33 @@ __global__ void k_geometry(long long E, const Ops* __restrict__ ops, Phys P, int
     const double det = j[0][0] * cof[0][0] + j[0][1] * cof[0][1] + j[0][2] * cof[0][2];
     const int i0 = g % N, i1 = (g / N) % N, i2 = g / (N * N);
     const double wq = w1[i0] * w1[i1] * w1[i2];
-    double* gp = geo + e * 10 * NP + g;
-    for (int a = 0; a < 3; ++a)
-      for (int d = 0; d < 3; ++d) gp[(a * 3 + d) * NP] = wq * cof[d][a];
-    gp[9 * NP] = wq * det;
-    double* gq = gu + e * 11 * NP + g;
-    for (int a = 0; a < 3; ++a)
-      for (int d = 0; d < 3; ++d) gq[(a * 3 + d) * NP] = cof[d][a];
-    gq[9 * NP] = det;
-    gq[10 * NP] = 1.0 / det;
-    const double X[3] = {x[e * 3 * NP] + in[g], x[e * 3 * NP + NP] + in[NP + g], x[e * 3 * NP + 2 * NP] + in[2 * NP + g]};
-    for (int d = 0; d < 3; ++d) xg[e * 3 * NP + d * NP + g] = X[d];
-    double gv[3];
-    if (gravity_kind == 0) {
-      gv[0] = g0; gv[1] = g1; gv[2] = g2;
+    if constexpr (UNW) {
+      double* gq = gu + e * 11 * NP + g;
+      for (int a = 0; a < 3; ++a)
+        for (int d = 0; d < 3; ++d) gq[(a * 3 + d) * NP] = cof[d][a];
+      gq[9 * NP] = det;
+      gq[10 * NP] = 1.0 / det;
     } else {
-      const double rr = sqrt(X[0] * X[0] + X[1] * X[1] + X[2] * X[2]);
-      const double fac = -(g_r0 / rr) * (g_r0 / rr) / rr;
-      for (int d = 0; d < 3; ++d) gv[d] = fac * X[d];
+      double* gp = geo + e * 10 * NP + g;
+      for (int a = 0; a < 3; ++a)
+        for (int d = 0; d < 3; ++d) gp[(a * 3 + d) * NP] = wq * cof[d][a];
+      gp[9 * NP] = wq * det;
+      const double X[3] = {x[e * 3 * NP] + in[g], x[e * 3 * NP + NP] + in[NP + g], x[e * 3 * NP + 2 * NP] + in[2 * NP + g]};
+      for (int d = 0; d < 3; ++d) xg[e * 3 * NP + d * NP + g] = X[d];
+      double gv[3];
+      if (gravity_kind == 0) {
+        gv[0] = g0; gv[1] = g1; gv[2] = g2;
+      } else {
+        const double rr = sqrt(X[0] * X[0] + X[1] * X[1] + X[2] * X[2]);
+        const double fac = -(g_r0 / rr) * (g_r0 / rr) / rr;
+        for (int d = 0; d < 3; ++d) gv[d] = fac * X[d];
+      }
+      const double* w = P.omega;
+      const double wx[3] = {w[1] * X[2] - w[2] * X[1], w[2] * X[0] - w[0] * X[2], w[0] * X[1] - w[1] * X[0]};
+      const double wwx[3] = {w[1] * wx[2] - w[2] * wx[1], w[2] * wx[0] - w[0] * wx[2], w[0] * wx[1] - w[1] * wx[0]};
+      const double cen = (P.cor * P.cor * 0.25);   // Fr^2 (cor = 2 Fr / sqrt(gamma))
+      for (int d = 0; d < 3; ++d) accg[e * 3 * NP + d * NP + g] = gv[d] / P.gamma - cen * wwx[d];
     }
-    const double* w = P.omega;
-    const double wx[3] = {w[1] * X[2] - w[2] * X[1], w[2] * X[0] - w[0] * X[2], w[0] * X[1] - w[1] * X[0]};
-    const double wwx[3] = {w[1] * wx[2] - w[2] * wx[1], w[2] * wx[0] - w[0] * wx[2], w[0] * wx[1] - w[1] * wx[0]};
-    const double cen = (P.cor * P.cor * 0.25);   // Fr^2 (cor = 2 Fr / sqrt(gamma))
-    for (int d = 0; d < 3; ++d) accg[e * 3 * NP + d * NP + g] = gv[d] / P.gamma - cen * wwx[d];
   }
   // faces: extrapolate the tangential Jacobian columns, n dS = side * (J_{a+1} x J_{a+2})
   for (int idx = threadIdx.x; idx < 6 * NF; idx += blockDim.x) {
@@ -1063,16 +1067,22 @@ __global__ void k_geometry(long long E, const Ops* __restrict__ ops, Phys P, int
     double nv[3] = {t1[1] * t2[2] - t1[2] * t2[1], t1[2] * t2[0] - t1[0] * t2[2], t1[0] * t2[1] - t1[1] * t2[0]};
     const int is = f % N, it = f / N;
     const double wf = w1[is] * w1[it];
-    double* fp = fgeo + ((e * 6 + phi) * 4) * NF + f;
     double a2n = 0.0;
-    for (int d = 0; d < 3; ++d) {
-      fp[d * NF] = wf * side * nv[d];
-      a2n += nv[d] * nv[d];
+    if constexpr (UNW) {
+      double* fq = fgu + ((e * 6 + phi) * 4) * NF + f;
+      for (int d = 0; d < 3; ++d) {
+        fq[d * NF] = side * nv[d];
+        a2n += nv[d] * nv[d];
+      }
+      fq[3 * NF] = sqrt(a2n);
+    } else {
+      double* fp = fgeo + ((e * 6 + phi) * 4) * NF + f;
+      for (int d = 0; d < 3; ++d) {
+        fp[d * NF] = wf * side * nv[d];
+        a2n += nv[d] * nv[d];
+      }
+      fp[3 * NF] = wf * sqrt(a2n);
     }
-    fp[3 * NF] = wf * sqrt(a2n);
-    double* fq = fgu + ((e * 6 + phi) * 4) * NF + f;
-    for (int d = 0; d < 3; ++d) fq[d * NF] = side * nv[d];
-    fq[3 * NF] = sqrt(a2n);
   }
 }
 
@@ -1301,13 +1311,17 @@ template <int N>
 int Driver<N>::geometry(dg_mesh* m, cudaStream_t s) {
   constexpr int NP = Shape<N>::NP;
   const size_t sm = sizeof(double) * 15 * NP;
-  int rc = set_smem(k_geometry<N>, sm);
+  int rc = set_smem(k_geometry<N, false>, sm);
+  if (rc == DG_OK) rc = set_smem(k_geometry<N, true>, sm);
   if (rc) return rc;
   const dg_mesh_desc& d = m->desc;
   prof_begin(m, s, KK_GEOMETRY);
-  k_geometry<N><<<(unsigned)m->E, NP < 32 ? 32 : NP, sm, s>>>(m->E, m->d_ops, m->phys, d.gravity_kind, d.gvec[0],
-                                                            d.gvec[1], d.gvec[2], d.g_r0, m->x, m->geo, m->acc,
-                                                            m->xg, m->fgeo, m->gu, m->fgu);
+  for (int unw = 0; unw < 2; ++unw) {
+    auto kern = unw ? k_geometry<N, true> : k_geometry<N, false>;
+    kern<<<(unsigned)m->E, NP < 32 ? 32 : NP, sm, s>>>(m->E, unw ? m->d_ops : m->d_ops_geo, m->phys, d.gravity_kind,
+                                                      d.gvec[0], d.gvec[1], d.gvec[2], d.g_r0, m->x, m->geo, m->acc,
+                                                      m->xg, m->fgeo, m->gu, m->fgu);
+  }
   prof_end(m, s);
   DG_LAUNCH_CHECK("k_geometry");
   return DG_OK;
@@ -1446,7 +1460,7 @@ int Driver<N>::q_from_nodal(dg_mesh* m, const double* q, cudaStream_t s) {
 
 template <int N>
 int Driver<N>::mixture(dg_mesh* m) {
-  k_mixture<N><<<(unsigned)m->E, 128>>>(m->E, m->d_ops, m->phys, m->xg, m->mixg, m->mixf);
+  k_mixture<N><<<(unsigned)m->E, 128>>>(m->E, m->d_ops_geo, m->phys, m->xg, m->mixg, m->mixf);
   DG_LAUNCH_CHECK("k_mixture");
   return DG_OK;
 }

@@ -324,7 +324,7 @@ static void free_mesh(dg_mesh* m) {
   dg_mlp_release(m);
   dg::interp_tc_release(m);
   if (m->w32_base) cudaFree(m->w32_base);
-  void* ptrs[] = {m->d_ops, m->d_euv, m->x, m->geo, m->gu, m->fgu, m->kn, m->acc, m->xg, m->fgeo, m->mixg, m->mixf, m->nbr, m->nbr_fo, m->face_e,
+  void* ptrs[] = {m->d_ops, m->d_ops_geo, m->d_euv, m->x, m->geo, m->gu, m->fgu, m->kn, m->acc, m->xg, m->fgeo, m->mixg, m->mixf, m->nbr, m->nbr_fo, m->face_e,
                   m->face_f,
                   m->ws.ug, m->ws.uf, m->ws.qg, m->ws.qf, m->ws.fh, m->ws.tmp, m->ws.red};
   for (void* p : ptrs)
@@ -418,6 +418,8 @@ extern "C" int dg_mesh_create(const dg_mesh_desc* desc, const double* nodes, dg_
   m->ndof = 5 * m->E * m->np;
   cudaGetDevice(&m->device);
   build_ops(m->n, &m->ops);
+  Ops ops_geo;
+  build_ops_geo(m->n, &ops_geo);
   // physics coefficients of Eq. fluxSWNondimensional
   Phys& P = m->phys;
   P.gamma = d.gamma;
@@ -473,7 +475,7 @@ extern "C" int dg_mesh_create(const dg_mesh_desc* desc, const double* nodes, dg_
       return DG_ENOMEM;
     }
     cudaError_t e1 = cudaMemcpy(d_layers, layers.data(), sizeof(double) * layers.size(), cudaMemcpyHostToDevice);
-    if (e1 == cudaSuccess) e1 = cudaMemcpy(d_xi, m->ops.xi, sizeof(double) * MAXN, cudaMemcpyHostToDevice);
+    if (e1 == cudaSuccess) e1 = cudaMemcpy(d_xi, ops_geo.xi, sizeof(double) * MAXN, cudaMemcpyHostToDevice);
     MapParams mpd = mp;
     mpd.r_layers = d_layers;
     if (e1 == cudaSuccess) {
@@ -492,7 +494,7 @@ extern "C" int dg_mesh_create(const dg_mesh_desc* desc, const double* nodes, dg_
   X.clear();
   X.shrink_to_fit();
 
-  rc |= dalloc(&m->d_ops, 1);
+  rc |= dalloc(&m->d_ops, 1) | dalloc(&m->d_ops_geo, 1);
   if (d.euv == DG_EUV_EUVAC) rc |= dalloc(&m->d_euv, 1);
   rc |= dalloc(&m->geo, E * 10 * NP);
   rc |= dalloc(&m->gu, E * 11 * NP);
@@ -518,6 +520,7 @@ extern "C" int dg_mesh_create(const dg_mesh_desc* desc, const double* nodes, dg_
   }
   cudaError_t err = cudaSuccess;
   err = cudaMemcpy(m->d_ops, &m->ops, sizeof(Ops), cudaMemcpyHostToDevice);
+  if (err == cudaSuccess) err = cudaMemcpy(m->d_ops_geo, &ops_geo, sizeof(Ops), cudaMemcpyHostToDevice);
   if (err == cudaSuccess && m->d_euv) {
     EuvFx tables;
     build_euv(P.n_euvac, P.euvac_B, P.euvac_phi, d.comp ? 4 : 1, &tables);

@@ -15,80 +15,105 @@ namespace {
 
 // The operators are formed in extended precision and rounded once: their errors act on every element
 // alike (a row of B that sums to 1 + 1e-16 turns a large constant into a gradient), so they are worth
-// more than the rounding of the data.
+// more than the rounding of the data. The same code in double serves the geometry (build_ops_geo).
 using ld = long double;
 
 // Legendre P_n(x) and its derivative by the three-term recurrence
-void legendre(int n, ld x, ld* p, ld* dp) {
-  ld p0 = 1.0L, p1 = x;
-  if (n == 0) { *p = 1.0L; *dp = 0.0L; return; }
+template <typename T>
+void legendre(int n, T x, T* p, T* dp) {
+  T p0 = T(1.0), p1 = x;
+  if (n == 0) { *p = T(1.0); *dp = T(0.0); return; }
   for (int k = 2; k <= n; ++k) {
-    ld p2 = ((2.0L * k - 1.0L) * x * p1 - (k - 1.0L) * p0) / k;
+    T p2 = ((T(2.0) * k - T(1.0)) * x * p1 - (k - T(1.0)) * p0) / k;
     p0 = p1;
     p1 = p2;
   }
   *p = p1;
-  *dp = (std::fabs(x) < 1.0L) ? n * (p0 - x * p1) / (1.0L - x * x) : 0.5L * n * (n + 1) * std::pow(x, n + 1);
+  *dp = (std::fabs(x) < T(1.0)) ? n * (p0 - x * p1) / (T(1.0) - x * x) : T(0.5) * n * (n + 1) * std::pow(x, n + 1);
 }
 
 // Gauss-Legendre: roots of P_n by Newton from Chebyshev-like guesses, weights 2/((1-x^2) P_n'^2)
-void gauss_rule(int n, ld* x, ld* w) {
+template <typename T>
+void gauss_rule(int n, T* x, T* w) {
   for (int i = 0; i < n; ++i) {
-    ld z = -std::cos((ld)M_PI * (i + 0.75L) / (n + 0.5L));
-    if (2 * i + 1 == n) z = 0.0L;
+    T z = -std::cos(T(M_PI) * (i + T(0.75)) / (n + T(0.5)));
+    if (sizeof(T) > sizeof(double) && 2 * i + 1 == n) z = T(0.0);
+    const T tol = sizeof(T) > sizeof(double) ? T(1e-19L) : T(1e-16);
     for (int it = 0; it < 100; ++it) {
-      ld p, dp;
+      T p, dp;
       legendre(n, z, &p, &dp);
-      ld dz = p / dp;
+      T dz = p / dp;
       z -= dz;
-      if (std::fabs(dz) < 1e-19L) break;
+      if (std::fabs(dz) < tol) break;
     }
-    ld p, dp;
+    T p, dp;
     legendre(n, z, &p, &dp);
     x[i] = z;
-    w[i] = 2.0L / ((1.0L - z * z) * dp * dp);
+    w[i] = T(2.0) / ((T(1.0) - z * z) * dp * dp);
   }
 }
 
 // GLL nodes: -1, roots of P'_{n-1}, +1. Newton on q(x) = (1 - x^2) P'_{n-1}(x), whose
 // derivative is -(n-1) n P_{n-1}(x) (Legendre's equation).
-void gll_nodes(int n, ld* x) {
+template <typename T>
+void gll_nodes(int n, T* x) {
   int N = n - 1;
-  x[0] = -1.0L;
-  x[N] = 1.0L;
+  x[0] = -T(1.0);
+  x[N] = T(1.0);
   for (int i = 1; i < N; ++i) {
-    ld z = -std::cos((ld)M_PI * i / N);
-    if (2 * i == N) z = 0.0L;
+    T z = -std::cos(T(M_PI) * i / N);
+    if (sizeof(T) > sizeof(double) && 2 * i == N) z = T(0.0);
+    const T tol = sizeof(T) > sizeof(double) ? T(1e-19L) : T(1e-16);
     for (int it = 0; it < 100; ++it) {
-      ld p, dp;
+      T p, dp;
       legendre(N, z, &p, &dp);
-      ld qv = (1.0L - z * z) * dp;
-      ld dq = -ld(N) * (N + 1) * p;
-      ld dz = qv / dq;
+      T qv = (T(1.0) - z * z) * dp;
+      T dq = -T(N) * (N + 1) * p;
+      T dz = qv / dq;
       z -= dz;
-      if (std::fabs(dz) < 1e-19L) break;
+      if (std::fabs(dz) < tol) break;
     }
     x[i] = z;
   }
 }
 
 // barycentric weights of a node set
-void bary(int n, const ld* x, ld* lam) {
+template <typename T>
+void bary(int n, const T* x, T* lam) {
   for (int k = 0; k < n; ++k) {
-    ld prod = 1.0L;
+    T prod = T(1.0);
     for (int m = 0; m < n; ++m)
       if (m != k) prod *= (x[k] - x[m]);
-    lam[k] = 1.0L / prod;
+    lam[k] = T(1.0) / prod;
   }
 }
 
 // Lagrange basis of node set x evaluated at point t: out[k] = l_k(t) (product form)
-void lagrange_at(int n, const ld* x, ld t, ld* out) {
+template <typename T>
+void lagrange_at(int n, const T* x, T t, T* out) {
   for (int k = 0; k < n; ++k) {
-    ld v = 1.0L;
+    T v = T(1.0);
     for (int m = 0; m < n; ++m)
       if (m != k) v *= (t - x[m]) / (x[k] - x[m]);
     out[k] = v;
+  }
+}
+
+// derivative matrix on the Gauss points: D[q][k] = lam_k / lam_q / (eta_q - eta_k), q != k;
+// the diagonal makes every row sum to zero (derivative of a constant)
+template <typename T>
+void derivative(int n, const T* eta, T* D) {
+  T lam[MAXN];
+  bary(n, eta, lam);
+  for (int q = 0; q < n; ++q) {
+    T diag = T(0.0);
+    for (int k = 0; k < n; ++k) {
+      if (k == q) continue;
+      T v = lam[k] / lam[q] / (eta[q] - eta[k]);
+      D[q * n + k] = v;
+      diag -= v;
+    }
+    D[q * n + q] = diag;
   }
 }
 
@@ -101,20 +126,18 @@ void build_ops_ld(int n, OpsLd* o) {
   for (int a = 0; a < n; ++a) lagrange_at(n, o->eta, o->xi[a], o->Binv + a * n);
   lagrange_at(n, o->eta, -1.0L, o->e[0]);
   lagrange_at(n, o->eta, 1.0L, o->e[1]);
-  // derivative matrix on the Gauss points: D[q][k] = lam_k / lam_q / (eta_q - eta_k), q != k;
-  // the diagonal makes every row sum to zero (derivative of a constant)
-  ld lam[MAXN];
-  bary(n, o->eta, lam);
-  for (int q = 0; q < n; ++q) {
-    ld diag = 0.0L;
-    for (int k = 0; k < n; ++k) {
-      if (k == q) continue;
-      ld v = lam[k] / lam[q] / (o->eta[q] - o->eta[k]);
-      o->D[q * n + k] = v;
-      diag -= v;
-    }
-    o->D[q * n + q] = diag;
-  }
+  derivative(n, o->eta, o->D);
+}
+
+void build_ops_geo(int n, Ops* o) {
+  std::memset(o, 0, sizeof(Ops));
+  gauss_rule(n, o->eta, o->w);
+  gll_nodes(n, o->xi);
+  for (int q = 0; q < n; ++q) lagrange_at(n, o->xi, o->eta[q], o->B + q * n);
+  for (int a = 0; a < n; ++a) lagrange_at(n, o->eta, o->xi[a], o->Binv + a * n);
+  lagrange_at(n, o->eta, -1.0, o->eL);
+  lagrange_at(n, o->eta, 1.0, o->eR);
+  derivative(n, o->eta, o->D);
 }
 
 void build_ops(int n, Ops* o) {
