@@ -277,8 +277,8 @@ typedef struct dg_solver_opts {
     int32_t precond;         /* DG_PC_* */
     int32_t precond_refresh; /* DG_REFRESH_* */
     int32_t jv_mode;         /* DG_JV_EXACT or DG_JV_FD for the GMRES operator */
-    int32_t jv_prec;         /* DG_PREC_F64, or DG_PREC_F32 (mixed): FP32 inner Jv, block assembly and
-                                Gram-Schmidt arithmetic; the Krylov basis is stored in FP32 when
+    int32_t jv_prec;         /* DG_PREC_F64, or DG_PREC_F32 (mixed): FP32 inner Jv and Gram-Schmidt
+                                arithmetic (blocks are assembled in FP64 either way); the Krylov basis is stored in FP32 when
                                 gmres_restart <= 31 and gmres_rtol >= 1e-6 (FP64 otherwise) */
     double newton_rtol;      /* stop when ||G||_2 <= newton_rtol ||G(U^0)||_2 (1e-8) */
     double gmres_rtol;       /* each Newton system to ||b - J x|| <= gmres_rtol ||b|| (1e-3) */
@@ -290,8 +290,7 @@ typedef struct dg_solver_opts {
 } dg_solver_opts;
 
 /* dg_solver_opts.flags: recompute the state's Gauss values, traces and LDG gradient in every
- * operator application and every block-assembly sweep, instead of once per Krylov solve and once
- * per assembly (same results; for checking). */
+ * operator application, instead of once per Krylov solve (same results; for checking). */
 #define DG_OPT_RECOMPUTE_VALUE 1
 
 typedef struct dg_step_stats {
@@ -329,7 +328,7 @@ int dg_implicit_step(dg_mesh* mesh, double* u, double t, double dt, const dg_sol
  * Build a preconditioner of J_G = M - dt_aii J_r(u) at state u and time t (DG_PC_MLP: network
  * inference for every element; see dg_mlp_init).
  * DG_PC_BJ: the exact diagonal block of every element (including the path through the
- * neighbours' LDG gradients) is computed column by column by block-diagonal tangent sweeps and
+ * neighbours' LDG gradients) is computed from the pointwise Jacobians of fluxes and sources and
  * inverted in place in FP32 by Gauss-Jordan elimination with partial pivoting (one CTA per block in
  * shared memory when it fits; otherwise blocked by panels of 16 to 32 columns in global memory,
  * each panel's transform applied to the other columns as one product of that rank), so that applying the

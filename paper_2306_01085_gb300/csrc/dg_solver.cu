@@ -1497,8 +1497,8 @@ static int norm2(dg_mesh* m, Solver* S, const double* x, double* out, cudaStream
 // ------------------------------------------------------------------------------------------
 // preconditioner
 // ------------------------------------------------------------------------------------------
-// exact diagonal blocks of J_G = M - c J_r(U) into dest (FP64 arithmetic whatever the step's precision: they
-// cost less than the FP32 probe sweeps they replaced)
+// exact diagonal blocks of J_G = M - c J_r(U) into dest (FP64 arithmetic whatever the step's precision: with
+// inversion 0.31 s for 98,304 degree-2 blocks; probing the tangent took 2.33 s in FP64 and 0.26 s in FP32)
 static int bj_assemble(dg_mesh* m, Solver* S, const double* U, double t, double c, float* dest, cudaStream_t s) {
   int rc = ensure_jac(m, S);
   if (rc) return rc;
