@@ -1310,7 +1310,12 @@ static int ensure_jac(dg_mesh* m, Solver* S) {
   cudaError_t err = cudaSuccess;
   if (!S->jac) {
     S->jac_batch = std::min((long long)m->E, std::max(1LL, (1LL << 27) / per));
-    err = cudaMalloc(&S->jac, sizeof(double) * (size_t)(S->jac_batch * per));
+    // (on a nearly full device: fewer elements at a time)
+    while ((err = cudaMalloc(&S->jac, sizeof(double) * (size_t)(S->jac_batch * per))) == cudaErrorMemoryAllocation &&
+           S->jac_batch > 1) {
+      cudaGetLastError();
+      S->jac_batch = (S->jac_batch + 1) / 2;
+    }
     if (err != cudaSuccess) S->jac = nullptr;
   }
   if (err == cudaSuccess && !m->kn) {
@@ -1318,7 +1323,11 @@ static int ensure_jac(dg_mesh* m, Solver* S) {
     if (err == cudaSuccess) {
       int rc = DG_OK;
       DG_DISPATCH_S(m, cross_kappa(m, m->kn));
-      if (rc) return rc;
+      if (rc) {
+        cudaFree(m->kn);
+        m->kn = nullptr;
+        return rc;
+      }
       err = cudaDeviceSynchronize();   // once per mesh: later assemblies may run on any stream
     } else {
       m->kn = nullptr;
