@@ -1464,7 +1464,7 @@ extern "C" int dg_radial_create(const dg_radial_desc* desc, const double* node_r
   cudaGetDevice(&m->device);
   const int N = m->N, E = m->E;
   Ops o;
-  build_ops(N, &o);
+  build_ops_geo(N, &o);   // the operators of the 3D geometry: no fixed-point coefficients here
   for (int i = 0; i < N * N; ++i) {
     m->ops64.B[i] = o.B[i];
     m->ops64.D[i] = o.D[i];
