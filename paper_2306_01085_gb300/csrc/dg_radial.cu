@@ -40,7 +40,7 @@ namespace rad {
 
 constexpr int MAXN = 5;
 
-// 1D operators (from build_ops) passed by value
+// 1D operators (from build_ops_geo) passed by value
 template <typename R>
 struct ROps {
   R B[MAXN * MAXN];   // B[g][i] = l^GLL_i(xi_g)
