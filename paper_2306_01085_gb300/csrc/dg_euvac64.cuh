@@ -2,65 +2,62 @@
 // dS0/dk) on the integer pipe.
 //
 // 37 exponentials per point are most of the heating's cost in FP64 (16 FP64 instructions per band, 64 issue
-// cycles of a warp each). Here a band takes about 75 integer instructions: with t = 128 Phi k / ln2 = n + f,
+// cycles of a warp each). Here a band takes about 110 integer instructions: with t = 128 Phi k / ln2 = n + f,
 // |f| <= 1/2, e^{-Phi k} = 2^-(n >> 7) W[n & 127] 2^{-f/128}, where W[i] = 2^{-i/128} is a table and
-// 1 - 2^{-f/128} a Taylor polynomial of degree 5, all in 57-bit fixed point (absolute error of the
-// exponential below 2^-56, checked against 60-digit arithmetic). t keeps 57 bits, as many as the FP64 product
-// Phi k. The terms are positive and summed exactly; they share the exponent of the least attenuated band, so
-// a strongly attenuated sum keeps its relative accuracy. Arguments outside the checked range (negative,
-// NaN, larger than 2^27) take the FP64 loop.
+// 1 - 2^{-f/128} a Taylor polynomial of degree 5, in 57-bit fixed point (absolute error of the exponential
+// below 2^-56). Bands differ by orders of magnitude in Phi, and at depth the weakest absorption carries the
+// whole sum, so every band has its own exponents: Phi, B Phi, B Phi^2 and t are 58-bit mantissas with a
+// binary exponent each (relative error a few 2^-57; four absorbers: their weighted sum likewise), and the
+// sums' exponents follow the largest term met so far. Terms are positive. In units of 2^-53 (2 + tau), tau the
+// mean optical depth of the bands that carry the sum, the relative errors stay below 0.46 (one absorber) and
+// 0.64 (four) over 13 decades of k and fractions down to 1e-12; those of the FP64 loop reach 4 and 5.7. One
+// exponent for all bands (that of the largest Phi) takes about 75 instructions and loses up to 1e-9 of S1 at depth.
+// Negative or non-finite arguments, weights and fluxes, and zero or subnormal k, take the FP64 loop.
 #pragma once
 
+#include "dg_bits.cuh"
 #include "dg_fx.cuh"
-#include "dg_math64.cuh"
 
 namespace dg {
 
+// m 2^(e - 58) with 2^57 <= m < 2^58 (or m = 0), m = hi 2^29 + lo
+struct alignas(16) EuvNum { int hi, lo, e, pad; };   // read by 16-byte loads
+constexpr int EUV_NONE = -(1 << 20);   // exponent of zero
+
 struct EuvFx {
   int n;
-  double tscale;             // max phi * 128 / ln2
-  double s0, s1;             // one absorber: max(B phi), max(B phi^2); four: max B max phi, max B max phi^2
+  int fixed;                 // every B and phi is finite and not negative
   double B[40], phi[4][40];  // the bands themselves (FP64 loop)
-  int2 xphi[4][40], xlow[4]; // phi / max phi, and each species' smallest
-  int2 xb[40], xc[40];       // B phi and B phi^2 of the first species over their maxima
-  int2 xB[40];               // B / max B
+  EuvNum xphi[4][40];
+  EuvNum xb[40], xc[40];     // one absorber: B phi and B phi^2; four: B and unused
 };
-// host: tables of n bands (coefficients with exponent 57, split at 29)
-inline void build_euv(int n, const double* B, const double (*phi)[40], int species, EuvFx* x) {
-  auto top = [](double m) { return m > 0.0 ? m : 1.0; };
-  double pm = 0.0, bm = 0.0, b0 = 0.0, c0 = 0.0;
-  for (int j = 0; j < n; ++j) {
-    bm = B[j] > bm ? B[j] : bm;
-    for (int s = 0; s < species; ++s) pm = phi[s][j] > pm ? phi[s][j] : pm;
-    b0 = B[j] * phi[0][j] > b0 ? B[j] * phi[0][j] : b0;
-    c0 = B[j] * phi[0][j] * phi[0][j] > c0 ? B[j] * phi[0][j] * phi[0][j] : c0;
+static_assert(sizeof(EuvNum) == 16 && alignof(EuvFx) == 16, "band tables: one aligned 16-byte load per number");
+inline EuvNum euv_num(long double v) {
+  if (!(v > 0.0L)) return {0, 0, EUV_NONE, 0};
+  int e;
+  long long m = __builtin_llrintl(__builtin_ldexpl(__builtin_frexpl(v, &e), 58));
+  if (m >> 58) {
+    m >>= 1;
+    ++e;
   }
-  pm = top(pm);
-  bm = top(bm);
-  b0 = top(b0);
-  c0 = top(c0);
-  auto coef = [](long double v) { return fx_coef(v < 1.0L ? v : 1.0L - 0x1p-57L, 57, 29); };
+  return {(int)(m >> 29), (int)(m & ((1 << 29) - 1)), e, 0};
+}
+// host: tables of n bands
+inline void build_euv(int n, const double* B, const double (*phi)[40], int species, EuvFx* x) {
   *x = EuvFx();
   x->n = n;
-  x->tscale = (double)((long double)pm * 128.0L / 0.693147180559945309417232121458176568L);
-  x->s0 = species == 1 ? b0 : bm * pm;
-  x->s1 = species == 1 ? c0 : bm * pm * pm;
-  for (int s = 0; s < 4; ++s) {
-    double low = s < species && n > 0 ? phi[s][0] : 0.0;
-    for (int j = 0; j < n; ++j) {
-      x->phi[s][j] = s < species ? phi[s][j] : 0.0;
-      x->xphi[s][j] = coef((long double)x->phi[s][j] / pm);
-      // one absorber: bands it does not absorb do not count
-      if (s < species && (species > 1 || phi[s][j] > 0.0) && (phi[s][j] < low || (species == 1 && low == 0.0)))
-        low = phi[s][j];
-    }
-    x->xlow[s] = coef((long double)low / pm);
-  }
+  x->fixed = 1;
   for (int j = 0; j < n; ++j) {
+    const long double b = B[j], f = phi[0][j];
     x->B[j] = B[j];
-    x->xB[j] = coef((long double)B[j] / bm);
-    x->xb[j] = coef((long double)B[j] * phi[0][j] / b0);
-    x->xc[j] = coef((long double)B[j] * phi[0][j] * phi[0][j] / c0);
+    if (!(B[j] >= 0.0 && B[j] < 1e100)) x->fixed = 0;
+    for (int s = 0; s < species; ++s) {
+      x->phi[s][j] = phi[s][j];
+      x->xphi[s][j] = euv_num(phi[s][j]);
+      if (!(phi[s][j] >= 0.0 && phi[s][j] < 1e100)) x->fixed = 0;
+    }
+    x->xb[j] = euv_num(species == 1 ? b * f : b);
+    x->xc[j] = euv_num(b * f * f);
   }
 }
 
@@ -99,41 +96,47 @@ static __device__ const long long kExp2Neg[128] = {
     0x10b5586cf9890f6LL, 0x109e3ecac6f3834LL, 0x10874518759bc81LL, 0x10706b29ddf6ddcLL,
     0x1059b0d31585744LL, 0x104315e86e7f84cLL, 0x102c9a3e778060fLL, 0x10163da9fb33357LL};
 
-__device__ __forceinline__ fx fx_ld(const int2* p) {
-  const int2 v = __ldg(p);
-  return {v.x, v.y};
+__device__ __forceinline__ EuvNum euv_ld(const EuvNum* p) {
+#ifdef __CUDA_ARCH__
+  const int4 v = __ldg(reinterpret_cast<const int4*>(p));
+  return {v.x, v.y, v.z, 0};
+#else
+  return *p;
+#endif
 }
-
-// t = A K 2^-s (A of exponent 57): n = rint(t), f57 = (t - n) 2^57
-__device__ __forceinline__ int euv_split(fx A, fx K, int s, long long& f57) {
-  const long long R = fx_mul<28>(A, K);
-  const int sn = min(s, 62);
-  const long long n = (R + (1LL << (sn - 1))) >> sn;
-  f57 = ((R - (n << sn)) << max(57 - s, 0)) >> max(s - 57, 0);
-  return (int)n;
+// mantissa and exponent of a positive normal double
+__device__ __forceinline__ long long euv_mantissa(double x, int& e) {
+  const uint64_t b = bits_of(x);
+  e = (int)(b >> 52) - 1022;
+  return (long long)((b & 0xfffffffffffffull) | 0x10000000000000ull) << 5;
+}
+// a mantissa of up to 59 bits back to 58
+__device__ __forceinline__ void euv_norm(long long& m, int& e) {
+  const int up = (int)(m >> 58);             // 0 or 1
+  m >>= up;
+  e += up;
+}
+// a 2^e += m 2^me, to 2^-56 of the larger; the sum holds 40 terms below 2^58 at half their unit
+__device__ __forceinline__ void euv_add(long long& a, int& e, long long m, int me) {
+  if (me > e) {
+    a = ((a >> (min(me - e, 63) - 1)) + 1) >> 1;
+    e = me;
+  }
+  a += ((m >> min(e - me, 62)) + 1) >> 1;
+}
+// x 2^e
+__device__ __forceinline__ double euv_scale(double x, int e) {
+  return e > -960 && e < 900 ? x * double_of((uint32_t)(e + 1023) << 20, 0u) : ldexp(x, e);
 }
 
 // NS = 1: Phi_j = phi_j of the first species; NS = 4: Phi_j = sum_s w[s] phi_sj
 template <int NS>
 __device__ __forceinline__ void euvac_sums(const EuvFx* __restrict__ X, const double w[4], double k, double& S0,
                                            double& S1) {
-  double kk = k * X->tscale;
-  bool ok = kk >= 0.0;
-  fx ws[4];
-  int ew = 1020;
-  if constexpr (NS == 4) {
-    int m = 0;
-    for (int s = 0; s < 4; ++s) {
-      ok = ok && w[s] >= 0.0;
-      m = max(m, fx_mag(w[s]));
-    }
-    ok = ok && (m >> 20) >= 900 && (m >> 20) <= 1100;
-    ew = m >> 20;
-    for (int s = 0; s < 4; ++s) ws[s] = fx_split<28>(fx_from<55>(w[s], ew));
-    kk *= __hiloint2double((ew + 3) << 20, 0);   // 2^(ew - 1020)
-  }
-  const int hk = __double2hiint(kk);
-  ok = ok && hk < (1050 << 20);
+  auto usable = [](double x) { const int h = (int)(bits_of(x) >> 32); return h >= (200 << 20) && h < (1846 << 20); };
+  bool ok = X->fixed != 0 && usable(k);
+  if constexpr (NS == 4)
+    for (int s = 0; s < 4; ++s) ok = ok && (w[s] == 0.0 || usable(w[s]));
   if (!ok) {
     S0 = S1 = 0.0;
 #pragma unroll 1
@@ -146,55 +149,86 @@ __device__ __forceinline__ void euvac_sums(const EuvFx* __restrict__ X, const do
     }
     return;
   }
-  const int ek = max(hk >> 20, 963), s = 1079 - ek;
-  const fx K = fx_split<28>(fx_from<57>(kk, ek));
-  fx low = fx_ld(&X->xlow[0]);
-  if constexpr (NS == 4) {
-    fxacc a = fx_zero<28>();
-    for (int q = 0; q < 4; ++q) fx_mac(a, fx_ld(&X->xlow[q]), ws[q]);
-    low = fx_split<29>(fx_sum<28>(a));
-  }
-  long long f57;
-  const int emin = euv_split(low, K, s, f57) >> 7;
-  fxacc a0 = fx_zero<28>(), a1 = fx_zero<28>();
+  fx ws[4];
+  int ew[4];
+  if constexpr (NS == 4)
+    for (int s = 0; s < 4; ++s) {
+      const long long m = euv_mantissa(w[s], ew[s]);
+      ws[s] = fx_split<28>(w[s] == 0.0 ? 0LL : m);
+    }
+  // K = k 128 / ln2
+  int eK;
+  long long Km = euv_mantissa(k, eK);
+  Km = fx_mul<28>(fx_split<29>(207914267153817539LL), fx_split<28>(Km));
+  eK += 7;
+  euv_norm(Km, eK);
+  const fx K = fx_split<28>(Km);
+  long long a0 = 0, a1 = 0;
+  int e0 = EUV_NONE, e1 = EUV_NONE;
 #pragma unroll 1
   for (int j = 0; j < X->n; ++j) {
-    fx A = fx_ld(&X->xphi[0][j]), b, c;
+    EuvNum q = euv_ld(&X->xphi[0][j]);
+    fx A{q.hi, q.lo}, b, c;
+    int eA = q.e, eb, ec;
     if constexpr (NS == 4) {
-      fxacc a = fx_zero<28>();
-      fx_mac(a, A, ws[0]);
+      long long m[4];
+      int em[4];
 #pragma unroll
-      for (int q = 1; q < 4; ++q) fx_mac(a, fx_ld(&X->xphi[q][j]), ws[q]);
-      const long long Ai = fx_sum<28>(a);
-      A = fx_split<29>(Ai);
-      const fx Ah = fx_split<28>(Ai);
-      const long long bi = fx_mul<28>(fx_ld(&X->xB[j]), Ah);
-      b = fx_split<29>(bi);
-      c = fx_split<29>(fx_mul<28>(b, Ah));
+      for (int s = 0; s < 4; ++s) {
+        if (s) q = euv_ld(&X->xphi[s][j]);
+        m[s] = fx_mul<28>(fx{q.hi, q.lo}, ws[s]);
+        em[s] = m[s] ? q.e + ew[s] - 1 : EUV_NONE;
+      }
+      eA = max(max(em[0], em[1]), max(em[2], em[3]));
+      long long Am = 0;                      // below 2^61
+#pragma unroll
+      for (int s = 0; s < 4; ++s) Am += m[s] >> min(eA - em[s], 63);
+      if (Am == 0) continue;
+      const int up = max(6 - __clzll(Am), 0);
+      Am >>= up;
+      eA += up;
+      A = fx_split<29>(Am);
+      const fx Ah = fx_split<28>(Am);
+      const EuvNum B = euv_ld(&X->xb[j]);
+      long long x = fx_mul<28>(fx{B.hi, B.lo}, Ah);
+      eb = B.e + eA - 1;
+      euv_norm(x, eb);
+      b = fx_split<29>(x);
+      x = fx_mul<28>(b, Ah);
+      ec = eb + eA - 1;
+      euv_norm(x, ec);
+      c = fx_split<29>(x);
     } else {
-      b = fx_ld(&X->xb[j]);
-      c = fx_ld(&X->xc[j]);
+      q = euv_ld(&X->xb[j]);
+      b = fx{q.hi, q.lo};
+      eb = q.e;
+      q = euv_ld(&X->xc[j]);
+      c = fx{q.hi, q.lo};
+      ec = q.e;
     }
-    const int n = euv_split(A, K, s, f57);
+    // t = R 2^-s = n + f57 2^-57
+    const int s = 59 - eA - eK;
+    if (s < 31 || b.hi == 0) continue;       // t of 2^26 and more: the attenuation is below the FP64 range
+    const long long R = fx_mul<28>(A, K);
+    const int sn = min(s, 62);
+    const int n = (int)((R + (1LL << (sn - 1))) >> sn);
+    const long long f57 = ((R - ((long long)n << sn)) << max(57 - s, 0)) >> min(max(s - 57, 0), 63);
     // g = 1 - 2^{-f/128}, Horner with 2^31 f; the leading terms with all 57 bits of f
     const int u = (int)(f57 >> 26);
     const int p = 2581847 - (int)(((long long)u * 2796) >> 31);
-    const int q = 1907106652 - (int)(((long long)u * p) >> 31);
-    const long long h = 69240576462433397LL - (((long long)u * q) >> 15);
+    const int r = 1907106652 - (int)(((long long)u * p) >> 31);
+    const long long h = 69240576462433397LL - (((long long)u * r) >> 15);
     const fx f = fx_split<29>(f57);
     const long long y = 99893036290645747LL - (fx_mul<28>(f, fx_split<28>(h)) >> 8);
     const long long g = fx_mul<28>(f, fx_split<28>(y));
     const long long W = kExp2Neg[n & 127];
-    long long E = W - ((fx_mul<28>(fx_split<29>(W), fx_split<28>(g)) + 64) >> 7);
-    E >>= min(max((n >> 7) - emin, 0), 63);
-    const fx e = fx_split<28>(E);
-    fx_mac(a0, b, e);
-    fx_mac(a1, c, e);
+    const fx E = fx_split<28>(W - ((fx_mul<28>(fx_split<29>(W), fx_split<28>(g)) + 64) >> 7));
+    const int d = n >> 7;
+    euv_add(a0, e0, fx_mul<28>(b, E), eb - d);
+    euv_add(a1, e1, fx_mul<28>(c, E), ec - d);
   }
-  const double z = emin > 900 ? 0.0 : __hiloint2double((1023 - 57 - emin) << 20, 0);
-  const double sw = NS == 4 ? __hiloint2double((ew + 3) << 20, 0) : 1.0;
-  S0 = (double)fx_sum<28>(a0) * (X->s0 * sw) * z;
-  S1 = (double)fx_sum<28>(a1) * (X->s1 * sw * sw) * z;
+  S0 = a0 ? euv_scale((double)a0, e0 - 57) : 0.0;
+  S1 = a1 ? euv_scale((double)a1, e1 - 57) : 0.0;
 }
 
 }  // namespace dg

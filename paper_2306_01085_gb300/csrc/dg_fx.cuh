@@ -65,9 +65,15 @@ struct fxacc { long long H, M, L; };
 template <int LH>
 __device__ __forceinline__ fxacc fx_zero() { return {0, 1LL << (LH - 1), 0}; }
 __device__ __forceinline__ void fx_mac(fxacc& s, fx a, fx x) {
+#ifdef __CUDA_ARCH__
   asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(s.H) : "r"(a.hi), "r"(x.hi));
   asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(s.M) : "r"(a.hi), "r"(x.lo));
   asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(s.L) : "r"(a.lo), "r"(x.hi));
+#else
+  s.H += (long long)a.hi * x.hi;
+  s.M += (long long)a.hi * x.lo;
+  s.L += (long long)a.lo * x.hi;
+#endif
 }
 template <int LH>
 __device__ __forceinline__ long long fx_sum(const fxacc& s) { return s.H + (s.M >> LH) + (s.L >> (57 - LH)); }
