@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(256) k_loss_grad(int n, int r, const float* __
   };
   float acc[NT][4][4] = {};
   float dd[2] = {0.f, 0.f};                          // columns tid, tid + 256
-  float ls = 0.f, le = 0.f;                          // loss sum and its rounding error
+  double ls = 0.0;                                   // in FP64: squares beyond the FP32 range stay finite
   const int tiles2 = (n4 / 4) * (C / 4);
   for (int i0 = 0; i0 < n; i0 += RB) {
     __syncthreads();
@@ -259,10 +259,8 @@ __global__ void __launch_bounds__(256) k_loss_grad(int n, int r, const float* __
         if (i0 + q >= n || j >= n) x[q] = 0.f;
         Rb[q * ldb + j] = x[q];
         dd[h] = fmaf(Bb[q * ldb + j], x[q], dd[h]);
-        const float sq = x[q] * x[q], se = fmaf(x[q], x[q], -sq);   // two-sum of the exact square
-        const float t = ls + sq, z = t - ls;
-        le += ((ls - (t - z)) + (sq - z)) + se;
-        ls = t;
+        const double xd = to_f64_exact(x[q]);
+        ls = fma(xd, xd, ls);
       }
     }
     __syncthreads();
@@ -302,7 +300,7 @@ __global__ void __launch_bounds__(256) k_loss_grad(int n, int r, const float* __
         if (j < n && k < r) g[n + (c0 < r4 ? n * r : 0) + j * r + k] = scale * acc[h][u][w];
       }
   }
-  lred[tid] = (double)ls + (double)le;
+  lred[tid] = ls;
   __syncthreads();
   for (int st = 128; st > 0; st >>= 1) {
     if (tid < st) lred[tid] += lred[tid + st];
