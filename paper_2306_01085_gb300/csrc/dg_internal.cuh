@@ -252,6 +252,9 @@ struct Driver {
   static int residual_p(dg_mesh* m, double t, double* r, double* jv, bool tangent, cudaStream_t s, double stage_c);
 };
 
+// smallest |c| of J_G = M - c J_r that the FP64 kernels take together with M (they hold M / c)
+constexpr double STAGE_C_MIN = 1e-200;
+
 // orientation map of face point (is, it) to the neighbour's face point index
 __host__ __device__ inline int orient_map(int o, int is, int it, int n) {
   int a = (o & 1) ? it : is;

@@ -1476,8 +1476,11 @@ static void scale_to_f32(long long n, const double* x, double a, const double* d
 // J_G v = M v - c J_r(U) v
 static int stage_matvec(dg_mesh* m, Solver* S, const double* U, double t, double c, int jv_mode, int jv_prec,
                         const double* v, double* out, cudaStream_t s, bool value_ready = false) {
-  // exact tangent: one fused pass forms M v - c J_r v
-  if (jv_mode == DG_JV_EXACT) return stage_jvp(m, U, v, t, c, out, jv_prec == DG_PREC_F32, s, value_ready);
+  // exact tangent: one fused pass forms M v - c J_r v. It holds M v / c (FP64) or c as a float, so a c too small for
+  // either, zero among them, takes the two products apart
+  const double least = jv_prec == DG_PREC_F32 ? 1e-37 : STAGE_C_MIN;
+  if (jv_mode == DG_JV_EXACT && !(std::fabs(c) < least))
+    return stage_jvp(m, U, v, t, c, out, jv_prec == DG_PREC_F32, s, value_ready);
   double* mv = S->v(VTMP);
   int rc = dg_mass_apply(m, v, mv, s);
   if (rc) return rc;
