@@ -1107,6 +1107,8 @@ __global__ void __launch_bounds__(128, NC == 2 ? 4 : 5)
 // threads per CTA: groups of a warp or less share a CTA of four warps once that still gives every SM
 // several CTAs; with fewer elements one warp per CTA spreads them over all SMs
 template <int N>
+constexpr int groups64_max() { return Grp<N>::T > 32 ? 1 : 128 / Grp<N>::T; }   // groups of the largest CTA
+template <int N>
 inline int threads64(long long groups) {
   if constexpr (Grp<N>::T > 32) return Grp<N>::T;
   const long long warps = (groups * Grp<N>::T + 31) / 32;

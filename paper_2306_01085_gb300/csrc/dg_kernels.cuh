@@ -1104,6 +1104,9 @@ template <> inline WorkT<double> work_of<double>(dg_mesh* m) {
 }
 template <> inline WorkT<float> work_of<float>(dg_mesh* m) { return m->w32; }
 
+// The limit is a property of the kernel in the whole process, so every caller sets the same value, the size of the
+// instance's largest launch: with each call's own size, a thread working on a small mesh could lower it between
+// another thread's call and its launch, which was then refused.
 template <typename K>
 static int set_smem(K kernel, size_t bytes) {
   cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
@@ -1117,7 +1120,7 @@ static int launch_interp64(dg_mesh* m, const double* u, const double* v, int fir
   using G = Grp<N>;
   const int threads = threads64<N>(m->E * (v ? 2 : 1)), per = threads / G::T;
   const size_t sm = sizeof(cell) * 10 * G::NP * per;
-  int rc = set_smem(k_interp64<N, false>, sm);
+  int rc = set_smem(k_interp64<N, false>, sizeof(cell) * 10 * G::NP * groups64_max<N>());
   if (rc) return rc;
   prof_begin(m, s, KK_INTERP);
   k_interp64<N, false><<<dim3((unsigned)((m->E + per - 1) / per), v ? 2 : 1), threads, sm, s>>>(
@@ -1153,7 +1156,7 @@ static int run_grad(dg_mesh* m, cudaStream_t s) {
     using G = Grp<N>;
     const int threads = threads64<N>(m->E * NC), per = threads / G::T;
     const size_t sm = sizeof(cell) * GradCells<N>::size * per;
-    int rc = set_smem(k_grad64<N>, sm);
+    int rc = set_smem(k_grad64<N>, sizeof(cell) * GradCells<N>::size * groups64_max<N>());
     if (rc) return rc;
     prof_begin(m, s, KK_GRAD);
     k_grad64<N><<<dim3((unsigned)((m->E + per - 1) / per), NC), threads, sm, s>>>(
@@ -1265,7 +1268,7 @@ static int run_volume(dg_mesh* m, double t, double* r, double* jv, cudaStream_t 
     using G = Grp<N>;
     const int threads = threads64<N>(m->E), per = threads / G::T;
     const size_t sm = sizeof(cell) * VolCells<N, NC>::size * per;
-    int rc = set_smem(k_volume64<N, NC>, sm);
+    int rc = set_smem(k_volume64<N, NC>, sizeof(cell) * VolCells<N, NC>::size * groups64_max<N>());
     if (rc) return rc;
     const Sun64 sun = sun_at(m, t);
     prof_begin(m, s, KK_VOLUME);
@@ -1430,7 +1433,7 @@ static int run_nodal(dg_mesh* m, const double* in, double* out, cudaStream_t s) 
   constexpr int planes = MODE == NODAL_FROM_GAUSS ? 3 : 1;
   const int threads = threads64<N>(m->E * planes), per = threads / G::T;
   const size_t sm = sizeof(cell) * 10 * G::NP * per;
-  int rc = set_smem(k_nodal64<N, MODE>, sm);
+  int rc = set_smem(k_nodal64<N, MODE>, sizeof(cell) * 10 * G::NP * groups64_max<N>());
   if (rc) return rc;
   prof_begin(m, s, KK_TENSOR);
   k_nodal64<N, MODE><<<dim3((unsigned)((m->E + per - 1) / per), planes), threads, sm, s>>>(m->E, m->d_ops, in, out, m->gu);
@@ -1449,7 +1452,7 @@ int Driver<N>::q_from_nodal(dg_mesh* m, const double* q, cudaStream_t s) {
   using G = Grp<N>;
   const int threads = threads64<N>(m->E * 3), per = threads / G::T;
   const size_t sm = sizeof(cell) * 10 * G::NP * per;
-  int rc = set_smem(k_interp64<N, true>, sm);
+  int rc = set_smem(k_interp64<N, true>, sizeof(cell) * 10 * G::NP * groups64_max<N>());
   if (rc) return rc;
   prof_begin(m, s, KK_TENSOR);
   k_interp64<N, true><<<dim3((unsigned)((m->E + per - 1) / per), 3), threads, sm, s>>>(q, nullptr, m->E, m->d_ops,

@@ -164,6 +164,7 @@ __global__ void __launch_bounds__(512) k_colsum(int rows, int cols, const float*
 // ------------------------------------------------------------------------------------------
 constexpr int MLP_MAXR = 32;
 constexpr int LG_RB = 16;
+constexpr int LG_SMEM = 224 * 1024;
 
 static size_t loss_smem(int n, int r) {
   const size_t r4 = (r + 3) / 4 * 4, n4 = (n + 3) / 4 * 4;
@@ -314,9 +315,10 @@ static int launch_loss(int nb, int n, int r, const float* out, const float* Bs, 
   const size_t smem = loss_smem(n, r);
   const int r4 = (r + 3) / 4 * 4, n4 = (n + 3) / 4 * 4;
   const int nt = ((n4 / 4) * (2 * r4 / 4) + 255) / 256;
-  if (smem > 227 * 1024 || n > 512 || nt > 5) return fail(DG_EINVAL, "MLP block too large for the loss kernel");
+  if (smem > LG_SMEM || n > 512 || nt > 5) return fail(DG_EINVAL, "MLP block too large for the loss kernel");
   auto go = [&](auto kern) -> int {
-    DG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // the same limit for every network (threads may train others), beside the kernel's static 2 KB
+    DG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, LG_SMEM));
     kern<<<nb, 256, smem, s>>>(n, r, out, Bs, scale, dout, loss_part);
     return DG_OK;
   };

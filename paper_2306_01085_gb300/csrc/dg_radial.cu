@@ -1285,7 +1285,8 @@ template <int N>
 int solve_t(dg_radial* m, double* b, cudaStream_t s) {
   rprof_begin(m, s, RK_SOLVE);
   const size_t smem = sizeof(float2) * (size_t)(kThreads / 32) * m->n;
-  DG_CUDA_TRY(cudaFuncSetAttribute(k_rband_solve<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  // (one limit for all ensembles: it belongs to the kernel, and threads may step ensembles of other sizes)
+  DG_CUDA_TRY(cudaFuncSetAttribute(k_rband_solve<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
   k_rband_solve<N><<<blocks_for(32 * m->nc), kThreads, smem, s>>>(m->n, m->nc, m->band, m->ipiv, b);
   rprof_end(m, s);
   DG_LAUNCH_CHECK("k_rband_solve");

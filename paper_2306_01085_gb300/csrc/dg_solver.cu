@@ -1076,6 +1076,7 @@ __host__ __device__ inline int inv_cols(int n) {
   return most < 4 ? 4 : most < quarter ? most : quarter;
 }
 __host__ __device__ inline int inv_chunk(int n) { return (inv_cols(n) * n * 4 + 31) & ~15; }
+inline int inv_smem(int n) { return INV_S * inv_chunk(n) + 4 * ((n + 3) / 4 * 4); }
 
 template <int MR>
 __global__ void k_inv_apply(int n, const float* __restrict__ inv, const double* __restrict__ x, double* __restrict__ y) {
@@ -1770,9 +1771,11 @@ static int precond_apply(dg_mesh* m, Solver* S, int kind, const double* x, doubl
     if (!S->bj_ready) return fail(DG_EINVAL, "block-Jacobi preconditioner used before dg_precond_setup");
     const int nb = 5 * m->np;
     prof_begin(m, s, KK_PRECOND);
-    const size_t sm = (size_t)INV_S * inv_chunk(nb) + sizeof(float) * ((nb + 3) / 4 * 4);
+    const int sm = inv_smem(nb);
     auto kern = nb <= 320 ? k_inv_apply<1> : k_inv_apply<2>;
-    DG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    // one limit per kernel, whatever the degree of this mesh (see set_smem)
+    const int limit = nb <= 320 ? std::max(inv_smem(40), std::max(inv_smem(135), inv_smem(320))) : inv_smem(625);
+    DG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, limit));
     kern<<<(unsigned)m->E, nb <= 320 ? (nb + 31) / 32 * 32 : ((nb + 1) / 2 + 31) / 32 * 32, sm, s>>>(nb, S->blocks, x, y);
     prof_end(m, s);
     DG_LAUNCH_CHECK("k_inv_apply");
