@@ -19,6 +19,7 @@ static thread_local std::string g_last_error;
 void set_error(const std::string& msg) { g_last_error = msg; }
 int fail(int code, const std::string& msg) {
   g_last_error = msg;
+  if (code == DG_ENOMEM) cudaGetLastError();   // reported here, not by the next call's launch check
   return code;
 }
 

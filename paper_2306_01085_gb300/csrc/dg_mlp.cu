@@ -500,10 +500,15 @@ static inline uint64_t splitmix(uint64_t seed, uint64_t i) {
 
 static int ensure_batch(Mlp* M, int batch) {
   if (M->batch_cap >= batch) return DG_OK;
-  float** bufs[] = {&M->z1, &M->h1, &M->z2, &M->h2, &M->o, &M->dout, &M->dh, &M->part};
-  for (float** b : bufs)
-    if (*b) { cudaFree(*b); *b = nullptr; }
-  if (M->loss_part) cudaFree(M->loss_part);
+  auto release = [&]() {                     // and no batch fits: a failed call leaves nothing half allocated
+    float** bufs[] = {&M->z1, &M->h1, &M->z2, &M->h2, &M->o, &M->dout, &M->dh, &M->part};
+    for (float** b : bufs)
+      if (*b) { cudaFree(*b); *b = nullptr; }
+    if (M->loss_part) cudaFree(M->loss_part);
+    M->loss_part = nullptr;
+    M->batch_cap = 0;
+  };
+  release();
   const size_t H = (size_t)batch * M->hidden, OB = (size_t)batch * M->n_out;
   cudaError_t err = cudaMalloc(&M->z1, H * 4);
   if (err == cudaSuccess) err = cudaMalloc(&M->h1, H * 4);
@@ -513,17 +518,21 @@ static int ensure_batch(Mlp* M, int batch) {
   if (err == cudaSuccess) err = cudaMalloc(&M->dout, OB * 4);
   if (err == cudaSuccess) err = cudaMalloc(&M->dh, (H > (size_t)batch * M->n_in ? H : (size_t)batch * M->n_in) * 4);
   if (err == cudaSuccess) err = cudaMalloc(&M->loss_part, sizeof(double) * batch);
-  // partial sums of the split products, for every batch up to this one (fewer rows may split more)
+  // partial sums of the split products, for every batch up to this one: fewer rows may split more, no more than
+  // 152 tiles of 64 rows at all
   const int Hd = M->hidden, O = M->n_out, I = M->n_in;
   size_t part = 1;
-  for (int nb = std::min(batch, GBM); ; nb = std::min(batch, nb + GBM)) {
+  for (long long rows = GBM; rows < (long long)batch + GBM && rows <= 153 * GBM; rows += GBM) {
+    const int nb = (int)std::min(rows, (long long)batch);
     part = std::max(part, std::max(gemm_part_floats(nb, Hd, Hd), gemm_part_floats(nb, Hd, O)));
-    if (nb == batch) break;
   }
   for (size_t p : {gemm_part_floats(O, Hd, batch), gemm_part_floats(Hd, Hd, batch), gemm_part_floats(Hd, I, batch)})
     part = std::max(part, p);
   if (err == cudaSuccess) err = cudaMalloc(&M->part, part * 4);
-  if (err != cudaSuccess) return fail(DG_ENOMEM, std::string("MLP batch storage: ") + cudaGetErrorString(err));
+  if (err != cudaSuccess) {
+    release();
+    return fail(DG_ENOMEM, std::string("MLP batch storage: ") + cudaGetErrorString(err));
+  }
   M->batch_cap = batch;
   return DG_OK;
 }

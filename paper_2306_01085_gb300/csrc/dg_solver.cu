@@ -1298,6 +1298,12 @@ static int solver_get(dg_mesh* m, int restart, Solver** out) {
     default: rc = fail(DG_EINVAL, "unsupported degree");       \
   }
 
+template <typename T>
+static void drop(T*& p) {
+  if (p) cudaFree(p);
+  p = nullptr;
+}
+
 // Jacobian storage of the block assembly: at most 1 GiB (batches of elements beyond that)
 static int ensure_jac(dg_mesh* m, Solver* S) {
   if (S->jac && m->kn) return DG_OK;
@@ -1311,7 +1317,7 @@ static int ensure_jac(dg_mesh* m, Solver* S) {
   cudaError_t err = cudaSuccess;
   if (!S->jac) {
     S->jac_batch = std::min((long long)m->E, std::max(1LL, (1LL << 27) / per));
-    // (on a nearly full device: fewer elements at a time)
+    // (on a nearly full device: fewer elements at a time, for the mesh's life, since captured assemblies hold the address)
     while ((err = cudaMalloc(&S->jac, sizeof(double) * (size_t)(S->jac_batch * per))) == cudaErrorMemoryAllocation &&
            S->jac_batch > 1) {
       cudaGetLastError();
@@ -1344,7 +1350,12 @@ static int ensure_blocks(dg_mesh* m, Solver* S) {
   cudaError_t err = cudaMalloc(&S->blocks, sizeof(float) * (size_t)m->E * nb * nb + 16);   // + 16: k_inv_apply
   if (err == cudaSuccess) err = cudaMalloc(&S->piv, sizeof(int) * (size_t)m->E * nb);
   if (err == cudaSuccess) err = cudaMalloc(&S->info, sizeof(int));
-  if (err != cudaSuccess) return fail(DG_ENOMEM, std::string("block-Jacobi storage: ") + cudaGetErrorString(err));
+  if (err != cudaSuccess) {                  // all or none: the next call looks at blocks alone
+    drop(S->blocks);
+    drop(S->piv);
+    drop(S->info);
+    return fail(DG_ENOMEM, std::string("block-Jacobi storage: ") + cudaGetErrorString(err));
+  }
   return DG_OK;
 }
 
@@ -1530,7 +1541,11 @@ static int bj_setup(dg_mesh* m, Solver* S, const double* U, double t, double c, 
     S->hld = (nb + 7) / 8 * 8;
     cudaError_t err = cudaMalloc(&S->blocks_h, sizeof(__half) * (size_t)m->E * nb * S->hld);
     if (err == cudaSuccess) err = cudaMalloc(&S->hscale, sizeof(float) * (size_t)m->E * nb);
-    if (err != cudaSuccess) return fail(DG_ENOMEM, std::string("FP16 block storage: ") + cudaGetErrorString(err));
+    if (err != cudaSuccess) {
+      drop(S->blocks_h);
+      drop(S->hscale);
+      return fail(DG_ENOMEM, std::string("FP16 block storage: ") + cudaGetErrorString(err));
+    }
   }
   DG_CUDA_TRY(cudaMemsetAsync(S->info, 0, sizeof(int), s));
   rc = bj_assemble(m, S, U, t, c, S->blocks, s);

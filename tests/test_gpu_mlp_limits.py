@@ -1,4 +1,6 @@
-"""Training loss beyond the FP32 range."""
+"""Training loss beyond the FP32 range, and the network's batch storage after a batch that does not fit."""
+import ctypes
+
 import pytest
 
 from paper_2306_01085_gb300 import workloads as W
@@ -40,3 +42,19 @@ def test_loss_is_summed_in_fp64(p, scale):
     R = Bs.double() @ (torch.diag_embed(1.0 + o[:, :n]) + U @ V.transpose(1, 2)) - torch.eye(n, device="cuda")
     ref = float(R.square().sum() / (X.shape[0] * n))
     assert abs(loss - ref) <= 1e-6 * ref
+
+
+def test_a_batch_that_does_not_fit_leaves_the_network_usable():
+    """2^31 - 1 samples (550 GB for the first layer alone) are refused with DG_ENOMEM; the next batch is computed
+    as before, and the refused allocation is not reported by its launches."""
+    import torch
+    from paper_2306_01085_gb300 import dg
+    m, n, r, X, Bs = _batch()
+    loss, grad = m.mlp_loss_grad(X, Bs)
+    out = ctypes.c_double()
+    rc = dg.lib().dg_mlp_loss_grad(m._h, ctypes.c_void_p(X.data_ptr()), ctypes.c_void_p(Bs.data_ptr()), 2 ** 31 - 1,
+                                   ctypes.byref(out), None, None)
+    assert rc == -3, rc
+    again, grad2 = m.mlp_loss_grad(X, Bs)
+    m.close()
+    assert again == loss and torch.equal(grad, grad2)
