@@ -823,37 +823,15 @@ struct VolCells {
   static constexpr int S = NC * 15 * NP, H = S + NC * 5 * NP, size = H + 30 * NF;
 };
 
-// the FP64 twin of k_volume64 from the pointwise fluxes on
+// the FP64 twin of k_volume64 from the reference fluxes on: sF and sS hold doubles
 template <int N, int NC>
 __device__ __noinline__ void volume_slow(const XOps<N>& so, long long e, long long E, int g, bool act, bool own,
-                                         const PhysT<double>& P, const Sun64& sun, const double* gu, const double* accg,
-                                         const double* xg, const double* ug, const double* qg, const double* fh,
-                                         const double* mixg, double stage_c, double inv_stage_c, cell* cells, double* r,
-                                         double* jv) {
-  using S = typename std::conditional<NC == 2, D64, double>::type;
+                                         const double* fh, double stage_c, int pl0, cell* cells, double* r, double* jv) {
   using C = VolCells<N, NC>;
   constexpr int NP = C::NP, NF = C::NF, T = Grp<N>::T;
   cell *sF = cells, *sS = cells + C::S, *sH = cells + C::H;
-  if (act) {
-    S F[12], src[5];
-    volume_load<N, NC, S>(e, E, g, P, sun, gu, accg, xg, ug, qg, mixg, inv_stage_c, F, src);
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-      for (int c = 0; c < 5; ++c) {
-        S x = s_zero<S>();
-#pragma unroll
-        for (int d = 0; d < 3; ++d) x = s_fma(gu[e * 11 * NP + (a * 3 + d) * NP + g], F[flux_index(c, d)], x);
-        sF[(a * 5 + c) * NP + g] = c_of(plane_of<NC, 0>(x));
-        if (NC == 2) sF[(15 + a * 5 + c) * NP + g] = c_of(plane_of<NC, NC - 1>(x));
-      }
-#pragma unroll
-    for (int c = 0; c < 5; ++c) {
-      sS[c * NP + g] = c_of(plane_of<NC, 0>(src[c]));
-      if (NC == 2) sS[(5 + c) * NP + g] = c_of(plane_of<NC, NC - 1>(src[c]));
-    }
-  }
   const int ig[3] = {g % N, (g / N) % N, g / (N * N)};
-  for (int pl = 0; pl < NC; ++pl) {
+  for (int pl = pl0; pl < NC; ++pl) {
     grp_sync<N>();
     if (own)
       for (int idx = g; idx < 6 * NF; idx += T)
@@ -921,7 +899,9 @@ __global__ void __launch_bounds__(128, NC == 2 ? 4 : 5)
 #pragma unroll
   for (int k = 0; k < NC * 5; ++k) mx[k] = 0;
   auto expo = [](int mag) { return mag == 0 ? 0 : fx_ok(mag) ? mag >> 20 : BAD; };
+  const int pl0 = NC == 2 && !r ? 1 : 0;     // the tangent alone when r is not wanted
   int eG[3] = {0, 0, 0}, eF[NC][3] = {};          // this point's exponents: geometry rows, flux groups
+  bool bad = false;                               // this point's reference fluxes are doubles
   if (live && act) {
     S F[12], src[5];
     volume_load<N, NC, S>(e, E, g, P, sun, gu, accg, xg, ug, qg, mixg, inv_stage_c, F, src);
@@ -932,19 +912,14 @@ __global__ void __launch_bounds__(128, NC == 2 ? 4 : 5)
       Gd[k] = gp[k * NP];
       eG[k / 3] = max(eG[k / 3], fx_mag(Gd[k]));
     }
-    bool bad = false;
-    fx G[9];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       bad = bad || !fx_ok(eG[a]);
       eG[a] = fx_exp(eG[a]);
-#pragma unroll
-      for (int d = 0; d < 3; ++d) G[a * 3 + d] = fx_split<29>(fx_from<58>(Gd[a * 3 + d], eG[a]));
     }
-    // Fref[a][c] = sum_d G[a][d] F[c][d], exact to 2^-58 of this point's largest term of the row and group
-    auto contract = [&](auto plc) {
+    auto flux_exps = [&](auto plc) {              // momentum, varrho, energy
       constexpr int PL = decltype(plc)::value;
-      int m[3] = {0, 0, 0};                  // momentum, varrho, energy
+      int m[3] = {0, 0, 0};
 #pragma unroll
       for (int k = 0; k < 12; ++k) m[k < 6 ? 0 : k < 9 ? 1 : 2] = max(m[k < 6 ? 0 : k < 9 ? 1 : 2], fx_mag(plane_of<NC, PL>(F[k])));
 #pragma unroll
@@ -952,33 +927,58 @@ __global__ void __launch_bounds__(128, NC == 2 ? 4 : 5)
         bad = bad || !fx_ok(m[k]);
         eF[PL][k] = fx_exp(m[k]);
       }
-      fx X[12];
-#pragma unroll
-      for (int k = 0; k < 12; ++k) X[k] = fx_split<28>(fx_from<58>(plane_of<NC, PL>(F[k]), eF[PL][k < 6 ? 0 : k < 9 ? 1 : 2]));
-#pragma unroll
-      for (int c = 0; c < 5; ++c) {
-        const int grp_c = c == 0 ? 1 : c == 4 ? 2 : 0;
-        int ec = expo(fx_mag(plane_of<NC, PL>(src[c])));
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-          fxacc s = fx_zero<28>();
-#pragma unroll
-          for (int d = 0; d < 3; ++d) fx_mac(s, G[a * 3 + d], X[flux_index(c, d)]);
-          const long long R = fx_sum<28>(s);  // scale 2^(2103 - eG - eF)
-          sF[(PL * 15 + a * 5 + c) * NP + g] = R;
-          const int bits = 64 - __clzll(R < 0 ? -R : R);
-          if (bits > 0) ec = max(ec, bits + eG[a] + eF[PL][grp_c] - 1081);
-        }
-        sS[(PL * 5 + c) * NP + g] = c_of(plane_of<NC, PL>(src[c]));
-        mx[PL * 5 + c] = ec;
-      }
     };
-    if (NC == 1 || r) contract(std::integral_constant<int, 0>{});
-    if constexpr (NC == 2) contract(std::integral_constant<int, 1>{});
-    if (bad) mx[0] = BAD;
+    if (NC == 1 || r) flux_exps(std::integral_constant<int, 0>{});
+    if constexpr (NC == 2) flux_exps(std::integral_constant<int, 1>{});
+#pragma unroll
+    for (int c = 0; c < 5; ++c) {
+      sS[c * NP + g] = c_of(plane_of<NC, 0>(src[c]));
+      if (NC == 2) sS[(5 + c) * NP + g] = c_of(plane_of<NC, NC - 1>(src[c]));
+    }
+    if (bad) {
+      mx[0] = BAD;
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int c = 0; c < 5; ++c) {
+          S x = s_zero<S>();
+#pragma unroll
+          for (int d = 0; d < 3; ++d) x = s_fma(Gd[a * 3 + d], F[flux_index(c, d)], x);
+          sF[(a * 5 + c) * NP + g] = c_of(plane_of<NC, 0>(x));
+          if (NC == 2) sF[(15 + a * 5 + c) * NP + g] = c_of(plane_of<NC, NC - 1>(x));
+        }
+    } else {
+      fx G[9];
+#pragma unroll
+      for (int k = 0; k < 9; ++k) G[k] = fx_split<29>(fx_from<58>(Gd[k], eG[k / 3]));
+      // Fref[a][c] = sum_d G[a][d] F[c][d], exact to 2^-58 of this point's largest term of the row and group
+      auto contract = [&](auto plc) {
+        constexpr int PL = decltype(plc)::value;
+        fx X[12];
+#pragma unroll
+        for (int k = 0; k < 12; ++k) X[k] = fx_split<28>(fx_from<58>(plane_of<NC, PL>(F[k]), eF[PL][k < 6 ? 0 : k < 9 ? 1 : 2]));
+#pragma unroll
+        for (int c = 0; c < 5; ++c) {
+          const int grp_c = c == 0 ? 1 : c == 4 ? 2 : 0;
+          int ec = expo(fx_mag(plane_of<NC, PL>(src[c])));
+#pragma unroll
+          for (int a = 0; a < 3; ++a) {
+            fxacc s = fx_zero<28>();
+#pragma unroll
+            for (int d = 0; d < 3; ++d) fx_mac(s, G[a * 3 + d], X[flux_index(c, d)]);
+            const long long R = fx_sum<28>(s);  // scale 2^(2103 - eG - eF)
+            sF[(PL * 15 + a * 5 + c) * NP + g] = R;
+            const int bits = 64 - __clzll(R < 0 ? -R : R);
+            if (bits > 0) ec = max(ec, bits + eG[a] + eF[PL][grp_c] - 1081);
+          }
+          mx[PL * 5 + c] = ec;
+        }
+      };
+      if (NC == 1 || r) contract(std::integral_constant<int, 0>{});
+      if constexpr (NC == 2) contract(std::integral_constant<int, 1>{});
+    }
   }
   const double* fhe = fh + e * 30 * NF;
-  const int pl0 = NC == 2 && !r ? 1 : 0;     // the tangent alone when r is not wanted
   if (live)
     for (int pl = pl0; pl < NC; ++pl)
       for (int idx = g; idx < 6 * NF; idx += T) {
@@ -1002,8 +1002,16 @@ __global__ void __launch_bounds__(128, NC == 2 ? 4 : 5)
     if (mx[k] == 0) mx[k] = 1023;
   }
   if (!grp_all<N>(ok)) {
-    volume_slow<N, NC>(so, e, E, g, act && live && !ok, live && !ok, P, sun, gu, accg, xg, ug, qg, fh, mixg, stage_c, inv_stage_c, cells,
-                       r, jv);
+    // the reference fluxes of the points that passed leave the fixed point (own entries)
+    if (act && live && !ok && !bad)
+      for (int pl = pl0; pl < NC; ++pl)
+        for (int a = 0; a < 3; ++a)
+          for (int c = 0; c < 5; ++c) {
+            cell& x = sF[(pl * 15 + a * 5 + c) * NP + g];
+            const int eFc = NC == 2 && pl == 1 ? eF[NC - 1][c == 0 ? 1 : c == 4 ? 2 : 0] : eF[0][c == 0 ? 1 : c == 4 ? 2 : 0];
+            x = c_of(ldexp((double)x, eG[a] + eFc - 2103));
+          }
+    volume_slow<N, NC>(so, e, E, g, act && live && !ok, live && !ok, fh, stage_c, pl0, cells, r, jv);
     if constexpr (T >= 32) return;
   }
   live = live && ok;
