@@ -574,4 +574,321 @@ __global__ void __launch_bounds__(Blk<N>::GP * Blk<N>::T, N == 3 ? 2 : 1)
   }
 }
 
+// --------------------------------------------------------------------------------------------
+// FP32 assembly, for steps whose inner operator is the FP32 one (jv_prec f32)
+// --------------------------------------------------------------------------------------------
+// The same columns from FP32 Jacobians, geometry and sums (the weighted geometry of the FP32 kernels). The
+// gradient of a unit value needs no contraction through shared memory: its line values are products of entries
+// of B, so a thread keeps D G / (w |J|) of its lines and e n / (w |J|) of its faces in registers for all columns.
+// In FP64 the assembly is bound by the FP64 pipe and by the fixed point's issue; here by issue and shared-memory loads.
+// Set-up (assembly, inversion, FP16 copies) of 98,304 degree-2 blocks 309 ms in FP64, 245 with FP32 probing of the
+// tangent, 99 now (43 of it assembly); of 24,576 degree-3 blocks 365 in FP64, 322 with probing, 147 now.
+template <int N>
+struct Blk32 {
+  static constexpr int NP = N * N * N, NF = N * N;
+  static constexpr int T = Blk<N>::T, GP = Blk<N>::GP;
+  // floats of a column: gradient [3][NP], then reference fluxes [15][NP], then the passes; face fluxes [5][6 NF];
+  // traces of the column's variable [6 NF]
+  static constexpr int W = 15 * NP + 36 * NF;
+  static constexpr int floats = 80 * NP + 120 * NF + GP * W;
+};
+
+template <int N>
+__global__ void __launch_bounds__(128) k_jac_volume32(long long e0, long long nE, PhysT<float> P, float t,
+                                                      const float* __restrict__ geo, const float* __restrict__ accg,
+                                                      const float* __restrict__ xg, const float* __restrict__ ug,
+                                                      const float* __restrict__ qg, const float* __restrict__ mixg,
+                                                      float* __restrict__ JV) {
+  using D32 = DualT<float>;
+  constexpr int NP = Blk32<N>::NP;
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= nE * NP) return;
+  const long long eb = i / NP, e = e0 + eb;
+  const int g = (int)(i % NP);
+  float x3[3] = {0.f, 0.f, 0.f}, mg[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, G[9];
+  const float a3[3] = {accg[e * 3 * NP + g], accg[e * 3 * NP + NP + g], accg[e * 3 * NP + 2 * NP + g]};
+  if (P.euv)
+    for (int d = 0; d < 3; ++d) x3[d] = xg[e * 3 * NP + d * NP + g];
+  if (P.comp)
+    for (int k = 0; k < 8; ++k) mg[k] = mixg[(e * 8 + k) * NP + g];
+  const float* gp = geo + e * 10 * NP + g;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) G[k] = gp[k * NP];
+  const float Wd = gp[9 * NP];
+#pragma unroll 1
+  for (int dir = 0; dir < 20; ++dir) {
+    D32 u[5], q[3][5], F[3][5], src[5];
+#pragma unroll
+    for (int c = 0; c < 5; ++c) u[c] = D32{ug[(e * 5 + c) * NP + g], dir == c ? 1.f : 0.f};
+#pragma unroll
+    for (int k = 0; k < 15; ++k) q[k / 5][k % 5] = D32{qg[(e * 15 + k) * NP + g], dir == 5 + k ? 1.f : 0.f};
+    volume_point<D32>(P, u, q, G, Wd, a3, x3, t, F, src, mg);
+    float* out = JV + (eb * 20 + dir) * 20 * NP + g;
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+      for (int c = 0; c < 5; ++c) out[(a * 5 + c) * NP] = F[a][c].d;
+#pragma unroll
+    for (int c = 0; c < 5; ++c) out[(15 + c) * NP] = src[c].d;
+  }
+}
+
+template <int N>
+__global__ void __launch_bounds__(128) k_jac_faces32(long long e0, long long nE, PhysT<float> P,
+                                                     const int* __restrict__ nbr, const int* __restrict__ nbr_fo,
+                                                     const float* __restrict__ fgeo, const double* __restrict__ kn,
+                                                     const float* __restrict__ uf, const float* __restrict__ qf,
+                                                     const float* __restrict__ mixf, float* __restrict__ JF) {
+  using D32 = DualT<float>;
+  constexpr int NF = Blk32<N>::NF;
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= nE * 6 * NF) return;
+  const long long eb = i / (6 * NF), e = e0 + eb;
+  const int phi = (int)(i / NF % 6), f = (int)(i % NF);
+  const long long face = e * 6 + phi;
+  const int nb = nbr[face];
+  Mix<float> mx{P.cv, 1.f};
+  if (P.comp) {
+    mx.cv = mixf[(face * 2) * NF + f];
+    mx.kfac = mixf[(face * 2 + 1) * NF + f];
+  }
+  const float* gp = fgeo + face * 4 * NF + f;
+  const float n[3] = {gp[0], gp[NF], gp[2 * NF]}, area = gp[3 * NF];
+  long long face2 = face;
+  int f2 = f;
+  if (nb >= 0) {
+    const int fo = nbr_fo[face];
+    face2 = (long long)nb * 6 + (fo & 7);
+    f2 = orient_map(fo >> 3, f % N, f / N, N);
+  }
+  const float kn2[3] = {(float)kn[face2 * 3 * NF + f2], (float)kn[(face2 * 3 + 1) * NF + f2],
+                        (float)kn[(face2 * 3 + 2) * NF + f2]};
+  float* out = JF + eb * 600 * NF + phi * NF + f;
+#pragma unroll 1
+  for (int dir = 0; dir < 20; ++dir) {
+    D32 u[5], q[3][5], res[5];
+#pragma unroll
+    for (int c = 0; c < 5; ++c) u[c] = D32{uf[(face * 5 + c) * NF + f], dir == c ? 1.f : 0.f};
+#pragma unroll
+    for (int k = 0; k < 15; ++k) q[k / 5][k % 5] = D32{qf[(face * 15 + k) * NF + f], dir == 5 + k ? 1.f : 0.f};
+    if (nb >= 0) {
+      // the other side answers through its gradient alone
+      D32 u2[5], q2[3][5];
+#pragma unroll
+      for (int c = 0; c < 5; ++c) u2[c] = D32{uf[(face2 * 5 + c) * NF + f2], 0.f};
+#pragma unroll
+      for (int k = 0; k < 15; ++k) q2[k / 5][k % 5] = D32{qf[(face2 * 15 + k) * NF + f2], k % 5 == dir ? kn2[k / 5] : 0.f};
+      face_flux_interior(P, u, q, u2, q2, n, area, res, mx);
+    } else if (nb == -DG_BC_WALL) {
+      D32 ub[5], sg[5];
+      wall_trace(P, u, ub);
+      flux_dot_n(P, ub, q, n, true, res, mx);
+      sigma_diag(P, ub, sg, mx);
+#pragma unroll
+      for (int c = 0; c < 5; ++c) res[c] = res[c] + sg[c] * (area * (u[c] - ub[c]));
+    } else {
+      flux_dot_n(P, u, q, n, false, res, mx);
+    }
+#pragma unroll
+    for (int k = 0; k < 5; ++k) out[(dir * 5 + k) * 6 * NF] = res[k].d;
+  }
+}
+
+template <int N>
+__global__ void __launch_bounds__(Blk32<N>::GP * Blk32<N>::T, 2)
+    k_blocks32(long long e0, const Ops* __restrict__ ops, float t_wall, const float* __restrict__ geo,
+               const float* __restrict__ fgeo, const int* __restrict__ nbr, const float* __restrict__ uf,
+               const float* __restrict__ JV, const float* __restrict__ JF, float stage_c, float* __restrict__ out) {
+  using B = Blk32<N>;
+  constexpr int NP = B::NP, NF = B::NF, T = B::T, GP = B::GP, NI = Grp<N>::NI, n = 5 * NP;
+  __shared__ SmemOpsT<float> so;
+  __shared__ float uw[6 * NF];               // d u_hat_4 / d varrho at wall face points, else 0
+  extern __shared__ __align__(16) float sm32[];
+  load_ops<N, float>(ops, so);
+  const int grp = threadIdx.x / T, g = threadIdx.x % T;
+  const bool act = g < NP;
+  const long long eb = blockIdx.x, e = e0 + eb;
+  float* VA = sm32;                          // [4][20][NP] Jacobian columns u_c, q_0c, q_1c, q_2c
+  float* FA = VA + 80 * NP;                  // [4][5][6 NF]
+  float* sF = FA + 120 * NF + grp * B::W;    // [15][NP]
+  float* sH = sF + 15 * NP;                  // [5][6 NF]
+  float* sT = sH + 30 * NF;                  // [6 NF]
+  bool has_wall = false;
+  for (int phi = 0; phi < 6; ++phi) has_wall = has_wall || nbr[e * 6 + phi] == -DG_BC_WALL;
+  for (int i = threadIdx.x; i < 6 * NF; i += blockDim.x)
+    uw[i] = nbr[e * 6 + i / NF] == -DG_BC_WALL ? 0.5f * t_wall * expf(0.5f * uf[(e * 6 + i / NF) * 5 * NF + i % NF]) : 0.f;
+  __syncthreads();
+  const int ig[3] = {g % N, (g / N) % N, g / (N * N) % N};
+  int fp[3], lb[3];
+  float DG[3][N][3], en[6][3], D[3][N], ec[6], Wd = 0.f;
+  axis_coefs<N, true>(so.D, ig, D);
+  end_coefs(so, ig, ec);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    lb[a] = g - ig[a] * pt_stride<N>(a);
+    fp[a] = vol_face_point<N>(g, a);
+  }
+  if (act) {
+    const float* gp = geo + e * 10 * NP;
+    Wd = gp[9 * NP + g];
+    const float iW = 1.f / Wd;
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+#pragma unroll
+        for (int k = 0; k < N; ++k) DG[a][k][d] = -D[a][k] * gp[(a * 3 + d) * NP + lb[a] + k * pt_stride<N>(a)] * iW;
+#pragma unroll
+        for (int side = 0; side < 2; ++side)
+          en[2 * a + side][d] = ec[2 * a + side] * fgeo[((e * 6 + 2 * a + side) * 4 + d) * NF + fp[a]] * iW;
+      }
+  }
+  int tb[NI], ts[NI];
+#pragma unroll
+  for (int it = 0; it < NI; ++it) face_line<N>((g + it * T) / NF, (g + it * T) % NF, tb[it], ts[it]);
+#pragma unroll 1
+  for (int c = 0; c < 5; ++c) {
+    __syncthreads();
+    for (int i = threadIdx.x; i < 80 * NP; i += blockDim.x) {
+      const int k = i / (20 * NP);
+      VA[i] = JV[(eb * 20 + (k ? 5 * k + c : c)) * 20 * NP + i % (20 * NP)];
+    }
+    for (int i = threadIdx.x; i < 120 * NF; i += blockDim.x) {
+      const int k = i / (30 * NF);
+      FA[i] = JF[(eb * 20 + (k ? 5 * k + c : c)) * 30 * NF + i % (30 * NF)];
+    }
+    __syncthreads();
+    for (int b = grp; b < (NP + GP - 1) / GP * GP; b += GP) {
+      // (every group runs the same number of columns; those beyond the last one write nothing)
+      const int ib[3] = {b % N, (b / N) % N, b / (N * N) % N};
+      const float Bo[3] = {so.B[ig[0] * N + ib[0]], so.B[ig[1] * N + ib[1]], so.B[ig[2] * N + ib[2]]};
+      const float ud = Bo[0] * Bo[1] * Bo[2];
+      float uft[NI], qt[NI][3], qw[3] = {0.f, 0.f, 0.f}, qwt[NI][3];
+      // gradient of the traces in sT and, when vol, of the unit value; and its face traces
+      auto gradient = [&](bool vol, float (&q)[3], float (&qtr)[NI][3]) {
+        col_sync<N>(grp);
+        if (act) {
+#pragma unroll
+          for (int d = 0; d < 3; ++d) q[d] = 0.f;
+#pragma unroll
+          for (int phi = 0; phi < 6; ++phi) {
+            const float x = sT[phi * NF + fp[phi >> 1]];
+#pragma unroll
+            for (int d = 0; d < 3; ++d) q[d] = fmaf(en[phi][d], x, q[d]);
+          }
+          if (vol)
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+              const float rest = Bo[(a + 1) % 3] * Bo[(a + 2) % 3];
+#pragma unroll
+              for (int k = 0; k < N; ++k) {
+                const float x = so.B[k * N + ib[a]] * rest;
+#pragma unroll
+                for (int d = 0; d < 3; ++d) q[d] = fmaf(DG[a][k][d], x, q[d]);
+              }
+            }
+#pragma unroll
+          for (int d = 0; d < 3; ++d) sF[d * NP + g] = q[d];
+        }
+        col_sync<N>(grp);
+#pragma unroll
+        for (int it = 0; it < NI; ++it) {
+          const int idx = g + it * T;
+          if (idx >= 6 * NF) continue;
+          const float* ev = ((idx / NF) & 1) ? so.eR : so.eL;
+#pragma unroll
+          for (int d = 0; d < 3; ++d) {
+            qtr[it][d] = 0.f;
+#pragma unroll
+            for (int k = 0; k < N; ++k) qtr[it][d] = fmaf(ev[k], sF[d * NP + tb[it] + k * ts[it]], qtr[it][d]);
+          }
+        }
+        col_sync<N>(grp);
+      };
+      // its traces: l_b(-1), l_b(1) are 1 at the end nodes, else 0
+#pragma unroll
+      for (int it = 0; it < NI; ++it) {
+        const int idx = g + it * T, phi = idx / NF, f = idx % NF, axis = phi >> 1;
+        uft[it] = 0.f;
+        if (idx >= 6 * NF) continue;
+        const int s_ax = axis == 0 ? 1 : 0, t_ax = axis == 2 ? 1 : 2;
+        if (ib[axis] == ((phi & 1) ? N - 1 : 0)) uft[it] = so.B[f % N * N + ib[s_ax]] * so.B[f / N * N + ib[t_ax]];
+        const int nb = nbr[e * 6 + phi];
+        sT[idx] = nb >= 0 ? 0.5f * uft[it] : nb == -DG_BC_OUTFLOW ? uft[it] : c == 0 ? uft[it] : 0.f;
+      }
+      float qd[3] = {0.f, 0.f, 0.f};
+      gradient(true, qd, qt);
+      if (c == 0 && has_wall) {              // varrho moves the wall's energy trace
+#pragma unroll
+        for (int it = 0; it < NI; ++it)
+          if (g + it * T < 6 * NF) sT[g + it * T] = uw[g + it * T] * uft[it];
+        gradient(false, qw, qwt);
+      }
+      float src[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+      if (act)
+#pragma unroll
+        for (int r = 0; r < 20; ++r) {
+          const float* A = VA + r * NP + g;
+          float x = fmaf(A[0], ud, fmaf(A[20 * NP], qd[0], fmaf(A[40 * NP], qd[1], A[60 * NP] * qd[2])));
+          if (c == 0 && has_wall)
+#pragma unroll
+            for (int d = 0; d < 3; ++d) x = fmaf(JV[((eb * 20 + 9 + 5 * d) * 20 + r) * NP + g], qw[d], x);
+          if (r < 15) sF[r * NP + g] = x;
+          else src[r - 15] = x;
+        }
+#pragma unroll
+      for (int it = 0; it < NI; ++it) {
+        const int idx = g + it * T;
+        if (idx >= 6 * NF) continue;
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+          const float* A = FA + k * 6 * NF + idx;
+          float h = fmaf(A[0], uft[it], fmaf(A[30 * NF], qt[it][0], fmaf(A[60 * NF], qt[it][1], A[90 * NF] * qt[it][2])));
+          if (c == 0 && has_wall)
+#pragma unroll
+            for (int d = 0; d < 3; ++d) h = fmaf(JF[((eb * 20 + 9 + 5 * d) * 5 + k) * 6 * NF + idx], qwt[it][d], h);
+          sH[k * 6 * NF + idx] = h;
+        }
+      }
+      col_sync<N>(grp);
+      float R[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+      if (act)
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+          float x = src[k];
+#pragma unroll
+          for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int q = 0; q < N; ++q) x = fmaf(D[a][q], sF[(a * 5 + k) * NP + lb[a] + q * pt_stride<N>(a)], x);
+#pragma unroll
+          for (int phi = 0; phi < 6; ++phi) x = fmaf(-ec[phi], sH[k * 6 * NF + phi * NF + fp[phi >> 1]], x);
+          R[k] = (k == c ? Wd * ud : 0.f) - stage_c * x;
+        }
+      col_sync<N>(grp);
+      // B^T along each direction
+      float *in = sF, *to = sF + 5 * NP;
+      if (act)
+#pragma unroll
+        for (int k = 0; k < 5; ++k) in[k * NP + g] = R[k];
+      col_sync<N>(grp);
+#pragma unroll
+      for (int dir = 0; dir < 3; ++dir) {
+        if (act)
+#pragma unroll
+          for (int k = 0; k < 5; ++k) {
+            float x = 0.f;
+#pragma unroll
+            for (int q = 0; q < N; ++q) x = fmaf(so.B[q * N + ig[dir]], in[k * NP + lb[dir] + q * pt_stride<N>(dir)], x);
+            if (dir < 2) to[k * NP + g] = x;
+            else if (b < NP) out[(e * n + c * NP + b) * (long long)n + k * NP + g] = x;
+          }
+        col_sync<N>(grp);
+        float* z = in;
+        in = to;
+        to = z;
+      }
+    }
+  }
+}
+
 }  // namespace dg

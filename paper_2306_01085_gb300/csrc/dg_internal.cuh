@@ -240,6 +240,7 @@ struct Driver {
   static int cross_kappa(dg_mesh* m, double* kn);   // mesh factors of the cross gradient traces (default stream)
   // diagonal blocks of J_G = M - c J_r (dg_blocks.cuh); block_doubles: Jacobian storage of one element
   static int blocks(dg_mesh* m, double t, double c, double* jac, long long batch, float* out, cudaStream_t s);
+  static int blocks_f32(dg_mesh* m, double t, double c, float* jac, long long batch, float* out, cudaStream_t s);
   static long long block_doubles();
   // FP32 residual (v == NULL) or fused residual + exact Jv with a contraction mode (CM_*)
   static int eval_cm(dg_mesh* m, const double* u, const double* v, double t, double* r, double* jv, int cm,

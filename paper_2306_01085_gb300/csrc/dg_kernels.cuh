@@ -1397,6 +1397,35 @@ int Driver<N>::blocks(dg_mesh* m, double t, double c, double* jac, long long bat
   }
   return DG_OK;
 }
+// the same in FP32 at the state whose FP32 value plane is in place; jac holds `batch` elements' FP32 Jacobians
+template <int N>
+int Driver<N>::blocks_f32(dg_mesh* m, double t, double c, float* jac, long long batch, float* out, cudaStream_t s) {
+  using B = Blk32<N>;
+  constexpr int NP = B::NP, NF = B::NF;
+  const size_t sm = sizeof(float) * B::floats;
+  int rc = set_smem(k_blocks32<N>, sm);
+  if (rc) return rc;
+  const PhysT<float> P = phys_as<float>(m->phys);
+  const WorkT<float> w = m->w32;
+  for (long long e0 = 0; e0 < m->E; e0 += batch) {
+    const long long nE = m->E - e0 < batch ? m->E - e0 : batch;
+    float* JF = jac + nE * Blk<N>::JV;
+    prof_begin(m, s, KK_VOLUME);
+    k_jac_volume32<N><<<(unsigned)((nE * NP + 127) / 128), 128, 0, s>>>(e0, nE, P, (float)t, w.geo, w.acc, w.xg, w.ug, w.qg,
+                                                                      w.mixg, jac);
+    prof_end(m, s);
+    prof_begin(m, s, KK_FACES);
+    k_jac_faces32<N><<<(unsigned)((nE * 6 * NF + 127) / 128), 128, 0, s>>>(e0, nE, P, m->nbr, m->nbr_fo, w.fgeo, m->kn, w.uf,
+                                                                         w.qf, w.mixf, JF);
+    prof_end(m, s);
+    prof_begin(m, s, KK_LU);
+    k_blocks32<N><<<(unsigned)nE, B::GP * B::T, sm, s>>>(e0, m->d_ops, P.t_wall, w.geo, w.fgeo, m->nbr, w.uf, jac, JF,
+                                                       (float)c, out);
+    prof_end(m, s);
+    DG_LAUNCH_CHECK("k_blocks32");
+  }
+  return DG_OK;
+}
 template <int N>
 long long Driver<N>::block_doubles() { return Blk<N>::JV + Blk<N>::JF; }
 

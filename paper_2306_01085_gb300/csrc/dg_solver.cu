@@ -1521,18 +1521,23 @@ static int norm2(dg_mesh* m, Solver* S, const double* x, double* out, cudaStream
 // ------------------------------------------------------------------------------------------
 // preconditioner
 // ------------------------------------------------------------------------------------------
-// exact diagonal blocks of J_G = M - c J_r(U) into dest (FP64 arithmetic whatever the step's precision: with
-// inversion 0.31 s for 98,304 degree-2 blocks; probing the tangent took 2.33 s in FP64 and 0.26 s in FP32)
-static int bj_assemble(dg_mesh* m, Solver* S, const double* U, double t, double c, float* dest, cudaStream_t s) {
+// exact diagonal blocks of J_G = M - c J_r(U) into dest, in FP64 or, for steps whose inner operator is the FP32 one
+// (f32), in FP32 arithmetic: with inversion 0.31 and 0.10 s for 98,304 degree-2 blocks
+static int bj_assemble(dg_mesh* m, Solver* S, const double* U, double t, double c, float* dest, cudaStream_t s,
+                       bool f32 = false) {
   int rc = ensure_jac(m, S);
+  if (rc == DG_OK) rc = stage_value_plane(m, U, f32, s);
   if (rc) return rc;
-  rc = stage_value_plane(m, U, false, s);
-  if (rc) return rc;
-  DG_DISPATCH_S(m, blocks(m, t, c, S->jac, S->jac_batch, dest, s));
+  if (f32) {                                 // twice as many elements at a time in the same storage
+    DG_DISPATCH_S(m, blocks_f32(m, t, c, reinterpret_cast<float*>(S->jac), 2 * S->jac_batch, dest, s));
+  } else {
+    DG_DISPATCH_S(m, blocks(m, t, c, S->jac, S->jac_batch, dest, s));
+  }
   return rc;
 }
 
-static int bj_setup(dg_mesh* m, Solver* S, const double* U, double t, double c, cudaStream_t s, bool half = false) {
+static int bj_setup(dg_mesh* m, Solver* S, const double* U, double t, double c, cudaStream_t s, bool f32 = false,
+                    bool half = false) {
   int rc = ensure_blocks(m, S);
   if (rc) return rc;
   const int nb = 5 * m->np;
@@ -1548,7 +1553,7 @@ static int bj_setup(dg_mesh* m, Solver* S, const double* U, double t, double c, 
     }
   }
   DG_CUDA_TRY(cudaMemsetAsync(S->info, 0, sizeof(int), s));
-  rc = bj_assemble(m, S, U, t, c, S->blocks, s);
+  rc = bj_assemble(m, S, U, t, c, S->blocks, s, f32);
   if (rc) return rc;
   prof_begin(m, s, KK_LU);
   const size_t gj_smem = sizeof(float) * (2 * nb + (size_t)nb * nb);
@@ -1869,11 +1874,11 @@ static int rb_build(dg_mesh* m, Solver* S, int kind, const double* U, double t, 
 }
 
 // (re)build the preconditioner of kind at state U
-static int pc_setup(dg_mesh* m, Solver* S, int kind, const double* U, double t, double c, cudaStream_t s) {
+static int pc_setup(dg_mesh* m, Solver* S, int kind, const double* U, double t, double c, cudaStream_t s, bool f32) {
   dg::NvtxRange nvtx_range_("preconditioner setup");
   S->lag_valid = false;   // a lagged preconditioner is only reused as its own step built it
-  if (kind == DG_PC_BJ || kind == DG_PC_RB_BJ) return bj_setup(m, S, U, t, c, s);
-  if (kind == DG_PC_BJ16) return bj_setup(m, S, U, t, c, s, true);
+  if (kind == DG_PC_BJ || kind == DG_PC_RB_BJ) return bj_setup(m, S, U, t, c, s, f32);
+  if (kind == DG_PC_BJ16) return bj_setup(m, S, U, t, c, s, f32, true);
   if (kind == DG_PC_MLP) return mlp_setup(m, U, c, s);
   return DG_OK;
 }
@@ -2038,7 +2043,7 @@ extern "C" int dg_precond_setup(dg_mesh* mesh, int32_t kind, const double* u, do
   if (rc) return rc;
   if (kind == DG_PC_NONE) return DG_OK;
   if (kind == DG_PC_BJ) return bj_setup(mesh, S, u, t, dt_aii, (cudaStream_t)stream);
-  if (kind == DG_PC_BJ16) return bj_setup(mesh, S, u, t, dt_aii, (cudaStream_t)stream, true);
+  if (kind == DG_PC_BJ16) return bj_setup(mesh, S, u, t, dt_aii, (cudaStream_t)stream, false, true);
   if (kind == DG_PC_MLP) return mlp_setup(mesh, u, dt_aii, (cudaStream_t)stream);
   return fail(DG_EINVAL, "dg_precond_setup: unknown kind");
 }
@@ -2143,7 +2148,7 @@ extern "C" int dg_implicit_step(dg_mesh* mesh, double* u, double t, double dt, c
   }
   if (build_now) {
     const auto p0 = std::chrono::steady_clock::now();
-    rc = pc_setup(mesh, S, o.precond, un, t + c[0] * dt, dt * A[0][0], s);
+    rc = pc_setup(mesh, S, o.precond, un, t + c[0] * dt, dt * A[0][0], s, o.jv_prec == DG_PREC_F32);
     st.precond_ms += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - p0).count();
     if (rc) return finish(rc);
     if (o.precond_refresh == DG_REFRESH_LAGGED) {
@@ -2165,7 +2170,7 @@ extern "C" int dg_implicit_step(dg_mesh* mesh, double* u, double t, double dt, c
     DG_LAUNCH_CHECK("k_lincomb");
     if (o.precond != DG_PC_NONE && o.precond_refresh == DG_REFRESH_STAGE) {
       const auto p0 = std::chrono::steady_clock::now();
-      rc = pc_setup(mesh, S, o.precond, U, ti, ci, s);
+      rc = pc_setup(mesh, S, o.precond, U, ti, ci, s, o.jv_prec == DG_PREC_F32);
       st.precond_ms += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - p0).count();
       if (rc) return finish(rc);
     }
@@ -2195,7 +2200,7 @@ extern "C" int dg_implicit_step(dg_mesh* mesh, double* u, double t, double dt, c
       if (it == o.max_newton) break;
       if (o.precond != DG_PC_NONE && o.precond_refresh == DG_REFRESH_NEWTON) {
         const auto p0 = std::chrono::steady_clock::now();
-        rc = pc_setup(mesh, S, o.precond, U, ti, ci, s);
+        rc = pc_setup(mesh, S, o.precond, U, ti, ci, s, o.jv_prec == DG_PREC_F32);
         st.precond_ms += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - p0).count();
         if (rc) return finish(rc);
       }
