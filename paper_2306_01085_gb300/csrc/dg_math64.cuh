@@ -4,7 +4,9 @@
 // while table look-ups and integer instructions are nearly free beside it.
 //   exp_fast, exp_pm_fast, power_fast   fixed point (dg_exp_fx.cuh), no FP64 instruction; outside its ranges
 //                                       (and for Inf, NaN) CUDA's exp and log
-//   recip_fast     4 FP64 instructions, from the hardware's reciprocal seed and two Newton steps, error below 1 ulp
+//   recip_fast     4 FP64 instructions: two Newton-Raphson steps y + y (1 - x y) from the hardware's seed, which is good
+//                  to 2^-20; the second leaves 2^-80 before its rounding, so the error is below 0.5 + 2^-20 ulp
+//                  (a division is correctly rounded); outside 2^-991 <= |x| < 2^993 the division itself
 #pragma once
 
 #include <cuda_runtime.h>
