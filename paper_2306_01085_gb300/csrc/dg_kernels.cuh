@@ -96,20 +96,6 @@ __device__ __forceinline__ R line(const R* __restrict__ A, const R* __restrict__
   return acc;
 }
 
-// the same pass accumulated into acc (NEG: subtracted), one FMA chain
-template <int N, bool T, bool NEG, typename R, int CM = CM_NATIVE>
-__device__ __forceinline__ R line_fma(const R* __restrict__ A, const R* __restrict__ in, int g, int dir, R acc) {
-  const int st = pt_stride<N>(dir);
-  const int i = (g / st) % N;
-  const int base = g - i * st;
-#pragma unroll
-  for (int k = 0; k < N; ++k) {
-    const R a = T ? A[k * N + i] : A[i * N + k];
-    acc = cm_fma<CM>(NEG ? -a : a, in[base + k * st], acc);
-  }
-  return acc;
-}
-
 // Gauss point index of (face phi, face point f, index k along the face normal)
 template <int N>
 __device__ __forceinline__ int face_vol_point(int phi, int f, int k) {
@@ -129,11 +115,6 @@ __device__ __forceinline__ int vol_face_point(int g, int axis) {
   if (axis == 0) return i1 + N * i2;
   if (axis == 1) return i0 + N * i2;
   return i0 + N * i1;
-}
-
-template <int N>
-__device__ __forceinline__ int axis_index(int g, int axis) {
-  return axis == 0 ? g % N : (axis == 1 ? (g / N) % N : g / (N * N));
 }
 
 template <typename R>
