@@ -23,7 +23,10 @@ namespace dg {
 template <int N>
 struct Blk {
   static constexpr int NP = N * N * N, NF = N * N;
-  static constexpr int T = Grp<N>::T, GP = N <= 3 ? 8 : N == 4 ? 4 : 2;      // threads per column, columns in flight
+  // threads per column, columns in flight. k_blocks with half as many, these, twice as many: degree 1 (27,648 elements)
+  // 6.15, 6.13, 10.4 ms; degree 2 (6,912) 20.8, 14.5, 15.1; degree 3 (1,296) 12.8, 12.6, 12.3; degree 4 (384) 26.4,
+  // 19.3, 16.3. Two CTAs per SM fit at degree 2 (74 KB each), one at 3 and 4
+  static constexpr int T = Grp<N>::T, GP = N <= 3 ? 8 : N == 4 ? 4 : 2;
   static constexpr long long JV = 400LL * NP, JF = 600LL * NF;               // doubles per element
   // cells of a column: gradient [9 + 3][NP] + [18][NF], then the reference fluxes [15][NP]; face fluxes [30][NF]
   static constexpr int W = 12 * NP + 18 * NF > 15 * NP ? 12 * NP + 18 * NF : 15 * NP;

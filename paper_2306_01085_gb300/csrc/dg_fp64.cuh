@@ -1113,14 +1113,16 @@ __global__ void __launch_bounds__(128, NC == 2 ? 4 : 5)
 // launches
 // --------------------------------------------------------------------------------------------
 // threads per CTA: groups of a warp or less share a CTA of four warps once that still gives every SM
-// several CTAs; with fewer elements one warp per CTA spreads them over all SMs
+// several CTAs; with fewer elements one warp per CTA spreads them over all SMs (Jv, one warp against four per CTA:
+// 3,072 degree-1 elements 113 against 122 us, 6,912 219 and 218, 98,304 2409 and 2279; degree 2, 1,536 elements 162.6
+// and 163.3, 6,912 556 and 551, 98,304 6742 and 6616)
 template <int N>
 constexpr int groups64_max() { return Grp<N>::T > 32 ? 1 : 128 / Grp<N>::T; }   // groups of the largest CTA
 template <int N>
 inline int threads64(long long groups) {
   if constexpr (Grp<N>::T > 32) return Grp<N>::T;
   const long long warps = (groups * Grp<N>::T + 31) / 32;
-  return warps <= 152 * 16 ? 32 : 128;
+  return warps <= NUM_SMS * 16 ? 32 : 128;
 }
 
 }  // namespace dg

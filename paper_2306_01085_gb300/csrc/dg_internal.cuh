@@ -253,6 +253,8 @@ struct Driver {
   static int residual_p(dg_mesh* m, double t, double* r, double* jv, bool tangent, cudaStream_t s, double stage_c);
 };
 
+constexpr int NUM_SMS = 152;   // of a GB300
+
 // smallest |c| of J_G = M - c J_r that the FP64 kernels take together with M (they hold M / c)
 constexpr double STAGE_C_MIN = 1e-200;
 

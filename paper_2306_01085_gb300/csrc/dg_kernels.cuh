@@ -1191,7 +1191,7 @@ static int run_faces(dg_mesh* m, cudaStream_t s, bool vout = true) {
   const long long work = m->nfaces * NF;
   // FP64: small CTAs, whose last wave leaves fewer SMs idle (one warp while the faces cannot fill every SM;
   // an 8x8x6 degree-2 stage solve 88.7 -> 80 ms against CTAs of 128)
-  const int threads = !std::is_same<R, double>::value ? 128 : work <= 152 * 512 ? 32 : 64;
+  const int threads = !std::is_same<R, double>::value ? 128 : work <= NUM_SMS * 512 ? 32 : 64;
   const unsigned blocks = (unsigned)((work + threads - 1) / threads);
   const WorkT<R> w = work_of<R>(m);
   prof_begin(m, s, KK_FACES);

@@ -119,7 +119,7 @@ __global__ void k_gemm_finish(long long total, int N, int splits, const float* _
 // splits of K: enough for one CTA per SM, each with at least four K tiles
 static int gemm_splits(int M, int N, int K) {
   const int tiles = ((N + GBN - 1) / GBN) * ((M + GBM - 1) / GBM);
-  return std::max(1, std::min((152 + tiles - 1) / tiles, K / (4 * GBK)));
+  return std::max(1, std::min((NUM_SMS + tiles - 1) / tiles, K / (4 * GBK)));
 }
 static size_t gemm_part_floats(int M, int N, int K) {
   const int sp = gemm_splits(M, N, K);
@@ -519,10 +519,10 @@ static int ensure_batch(Mlp* M, int batch) {
   if (err == cudaSuccess) err = cudaMalloc(&M->dh, (H > (size_t)batch * M->n_in ? H : (size_t)batch * M->n_in) * 4);
   if (err == cudaSuccess) err = cudaMalloc(&M->loss_part, sizeof(double) * batch);
   // partial sums of the split products, for every batch up to this one: fewer rows may split more, no more than
-  // 152 tiles of 64 rows at all
+  // NUM_SMS tiles of 64 rows at all
   const int Hd = M->hidden, O = M->n_out, I = M->n_in;
   size_t part = 1;
-  for (long long rows = GBM; rows < (long long)batch + GBM && rows <= 153 * GBM; rows += GBM) {
+  for (long long rows = GBM; rows < (long long)batch + GBM && rows <= (NUM_SMS + 1) * GBM; rows += GBM) {
     const int nb = (int)std::min(rows, (long long)batch);
     part = std::max(part, std::max(gemm_part_floats(nb, Hd, Hd), gemm_part_floats(nb, Hd, O)));
   }

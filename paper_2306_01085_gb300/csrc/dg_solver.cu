@@ -107,7 +107,7 @@ static int dirk_tableau(int stages, double A[3][3], double c[3]) {
 // ------------------------------------------------------------------------------------------
 // vector kernels (FP64); reductions use a fixed grid and a fixed summation order
 // ------------------------------------------------------------------------------------------
-constexpr int RED_BLOCKS = 304;   // 2 x 152 SMs
+constexpr int RED_BLOCKS = 2 * NUM_SMS;
 constexpr int RED_THREADS = 256;
 constexpr int MAXK = 64;          // largest restart + 1
 constexpr int RB_MAX = 16;        // largest reduced basis
@@ -1481,7 +1481,7 @@ static void update_dot_f32v(long long n, int k, const float* V, const double* h,
 
 static void scale_to_f32(long long n, const double* x, double a, const double* den, float* out, double* wide,
                          cudaStream_t s) {
-  k_scale_to_f32<<<std::min(grid_for(n / 2), 4u * 152u), 256, 0, s>>>(
+  k_scale_to_f32<<<std::min(grid_for(n / 2), 4u * (unsigned)NUM_SMS), 256, 0, s>>>(
       n / 2, reinterpret_cast<const double2*>(x), a, den, reinterpret_cast<float2*>(out), reinterpret_cast<double2*>(wide));
 }
 
@@ -1714,7 +1714,7 @@ static int rb_orthonormalise(dg_mesh* m, Solver* S, cudaStream_t s) {
     if (!std::isfinite(n0) || !std::isfinite(nf)) return fail(DG_ENAN, "reduced basis: non-finite Newton update");
     if (!(n0 > 0.0) || !(nf > 1e-20 * n0)) continue;
     prof_begin(m, s, KK_BLAS);
-    k_scale_dev<<<std::min(grid_for(n), 4u * 152u), 256, 0, s>>>(n, w, S->hdev + 2 * MAXK - 1, w);
+    k_scale_dev<<<std::min(grid_for(n), 4u * (unsigned)NUM_SMS), 256, 0, s>>>(n, w, S->hdev + 2 * MAXK - 1, w);
     prof_end(m, s);
     DG_LAUNCH_CHECK("k_scale_dev");
     ++r;
@@ -1966,7 +1966,7 @@ static int gmres(dg_mesh* m, Solver* S, const dg_solver_opts& o, const double* U
         k_mdot_finish<<<k + 1, 32, 0, s>>>(S->partial, S->hdev + MAXK);
         update_dot(n, k + 1, V, S->hdev + MAXK, w, S->partial, false, s, f32gs);
         k_mdot_finish<<<1, 32, 0, s>>>(S->partial, S->hdev + MAXK + k + 1);
-        k_scale_dev<<<std::min(grid_for(n), 4u * 152u), 256, 0, s>>>(n, w, S->hdev + MAXK + k + 1, V + (long long)(k + 1) * n);
+        k_scale_dev<<<std::min(grid_for(n), 4u * (unsigned)NUM_SMS), 256, 0, s>>>(n, w, S->hdev + MAXK + k + 1, V + (long long)(k + 1) * n);
       }
       prof_end(m, s);
       DG_LAUNCH_CHECK("arnoldi");
