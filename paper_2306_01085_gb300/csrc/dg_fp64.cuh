@@ -871,8 +871,11 @@ __device__ __noinline__ void volume_slow(const XOps<N>& so, long long e, long lo
 
 // stage_c != 0 (NC = 2): the tangent output is the DIRK stage operator J_G v = M v - stage_c J_r v. It is
 // formed as -stage_c (J_r v - M v / stage_c), with -|J| u_dot / stage_c added to the tangent's source.
-// CTAs per SM: latency of the pointwise physics against spills (Jv of a 16x16x8 degree-4 shell: 3 CTAs 1135 us, 4
-// 1066, 5 1160; r of a 21x21x9 degree-3 shell: 3 CTAs 748, 4 685, 5 651).
+// CTAs per SM: latency of the pointwise physics against spills (Jv of a 16x16x8 degree-4 shell: 3 CTAs 1144 us, 4
+// 1078, 5 1150; r of a 21x21x9 degree-3 shell: 3 CTAs 736, 4 689, 5 657).
+// The physics is evaluated once for the twin too: a point out of range forms its reference fluxes in FP64, the others
+// convert their products when their element is refused (residual of 12,288 degree-2 elements with composition, every one
+// refused: 1505 us, 2183 with a second evaluation; ordinary calls 0.4 to 2 % of this kernel for the branch).
 template <int N, int NC>
 __global__ void __launch_bounds__(128, NC == 2 ? 4 : 5)
     k_volume64(long long E, const Ops* __restrict__ ops, PhysT<double> P, Sun64 sun, const double* __restrict__ gu,

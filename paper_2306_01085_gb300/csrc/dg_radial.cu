@@ -469,8 +469,8 @@ struct Band {
   static constexpr int KL = 9 * N - 1, KU = 9 * N - 1, LD = 2 * KL + KU + 1;
 };
 
-// CTAs per SM: latency of the pointwise physics against spills (16,384 columns, Jv: 2 CTAs 1.29 ms, 3 1.08, 4 1.05;
-// 2,475 columns, r: 3 CTAs 160 us, the last 8 CTAs alone in a second wave, 4 121; probes: 4 0.90 ms, 5 0.82)
+// CTAs per SM: latency of the pointwise physics against spills (16,384 columns, Jv: 2 CTAs 1.33 ms, 3 1.12, 4 1.09;
+// 2,475 columns, r: 3 CTAs 153 us, the last 8 CTAs alone in a second wave, 4 125; probes: 4 0.90 ms, 5 0.82)
 template <int N, int NC, bool PROBE, typename R>
 __global__ void __launch_bounds__(128, PROBE ? 5 : 4) k_rvol(int E, long long nc, ROps<R> O, RPhys<R> P, RGeo<R> g, RPrm<R> prm, R t,
                        const double* __restrict__ u, const double* __restrict__ v, const R* __restrict__ qg,
